@@ -25,6 +25,7 @@ import paper_2609_39816_b200 as fmm
 _DTYPE = {"f32": torch.float32, "bf16": torch.bfloat16}
 _BYTES = {"f32": 4, "bf16": 2, "e4m3": 1}
 _GRID = {"strassen222": (2, 7), "strassen444": (4, 49)}   # blocks per side, products
+_CODE_BOUND = {"strassen444": 31, "strassen222": 63, "": 127}   # largest int8 code whose block sums still fit int8
 _PRODUCTS_BF16, _REUSE_BHAT = fmm.FLAG_PRODUCTS_BF16, fmm.FLAG_REUSE_BHAT
 
 
@@ -147,27 +148,17 @@ def _bytes(n):
     return torch.empty(n, dtype=torch.uint8, device="cuda")
 
 
-def prepare(case, seed):
+def _operands(case, seed):
+    """What the call works on, made from the seed alone: (X, signs) for a rotation, (A, B) in fp32 or the storage type
+    for a product; B is [N, K] in the weight layout, else [K, N]."""
     gen = torch.Generator(device="cuda")
     gen.manual_seed(seed)
-    state = {"case": case}
     if case["path"] == "rotate":
-        state["X"] = _activations(gen, case["rows"], case["K"], True).to(_DTYPE[case["storage"]])
-        state["signs"] = (torch.randint(0, 2, (case["K"],), device="cuda", generator=gen) * 2 - 1).to(torch.int8)
-        state["out"] = torch.empty_like(state["X"])
-        return state
+        X = _activations(gen, case["rows"], case["K"], True).to(_DTYPE[case["storage"]])
+        return X, (torch.randint(0, 2, (case["K"],), device="cuda", generator=gen) * 2 - 1).to(torch.int8)
     M, K, N = case["M"], case["K"], case["N"]
-    state["s"] = s = fmm.scheme_builtin(case["scheme"]) if case["scheme"] else None
-    state["C"] = torch.empty((M, N), dtype=_DTYPE[case["output"]], device="cuda")
     if case["path"] == "int8":
-        G, bound = K // 128, {"strassen444": 31, "strassen222": 63, "": 127}[case["scheme"]]
-        state.update(bound=bound, A=_activations(gen, M, K, False),
-                     cA=torch.empty((M, K), dtype=torch.int8, device="cuda"), dA=torch.empty((M, G), device="cuda"),
-                     cB=torch.empty((N, K), dtype=torch.int8, device="cuda"), dB=torch.empty((N, G), device="cuda"),
-                     ws=_bytes(fmm.int8_gemm_workspace(s, M, K, N)))
-        W = 0.02 * torch.randn(N, K, device="cuda", generator=gen)
-        fmm.int8_quantize(W, bound, state["cB"], state["dB"])
-        return state
+        return _activations(gen, M, K, False), 0.02 * torch.randn(N, K, device="cuda", generator=gen)
     td = _DTYPE[case["storage"]]
     if case["path"] == "sweep" and case["gauges"] == "signs":   # the ensemble's operands: U[0, 1]
         A = torch.rand(M, K, device="cuda", generator=gen)
@@ -175,7 +166,28 @@ def prepare(case, seed):
     else:
         A = _activations(gen, M, K, case["product"] == "e4m3")
         B = 0.02 * torch.randn(*((N, K) if case["weight_layout"] else (K, N)), device="cuda", generator=gen)
-    state["A"], state["B"] = A.to(td), B.to(td)
+    return A.to(td), B.to(td)
+
+
+def prepare(case, seed):
+    state = {"case": case}
+    if case["path"] == "rotate":
+        state["X"], state["signs"] = _operands(case, seed)
+        state["out"] = torch.empty_like(state["X"])
+        return state
+    M, K, N = case["M"], case["K"], case["N"]
+    state["s"] = s = fmm.scheme_builtin(case["scheme"]) if case["scheme"] else None
+    state["C"] = torch.empty((M, N), dtype=_DTYPE[case["output"]], device="cuda")
+    if case["path"] == "int8":
+        G, bound = K // 128, _CODE_BOUND[case["scheme"]]
+        A, W = _operands(case, seed)
+        state.update(bound=bound, A=A,
+                     cA=torch.empty((M, K), dtype=torch.int8, device="cuda"), dA=torch.empty((M, G), device="cuda"),
+                     cB=torch.empty((N, K), dtype=torch.int8, device="cuda"), dB=torch.empty((N, G), device="cuda"),
+                     ws=_bytes(fmm.int8_gemm_workspace(s, M, K, N)))
+        fmm.int8_quantize(W, bound, state["cB"], state["dB"])
+        return state
+    state["A"], state["B"] = _operands(case, seed)
 
     def desc(flags=0):
         return fmm.GemmDesc.make(M, K, N, case["storage"], case["product"], case["output"], weight_layout=case["weight_layout"],
@@ -260,3 +272,41 @@ def tolerance(case):
     if case["output"] == "bf16":
         return {"rel": 6e-4, "max": 0.016}      # seen: 1.5e-4 and one unit (fp64 sums of the same block sums)
     return {"rel": 1.5e-5, "max": 6e-5}         # seen: 3.7e-6, 1.3e-5
+
+
+def _quantised(X, bound):
+    """Codes and scales of groups of 128 along a row, as the quantiser's specification rounds them (fp32)."""
+    x = X.view(X.shape[0], -1, 128)
+    amax = x.abs().amax(dim=2)
+    d = torch.where(amax == 0, torch.ones_like(amax), amax / bound)
+    return torch.round(x / d[:, :, None]), d
+
+
+def exact(case, seed):
+    """fp64 products of the operands.  Nothing for what measures rounding itself (squared errors, ratios, codes), and
+    nothing for a product whose block sums were rounded to e4m3: that rounding is up to a tenth of the result."""
+    if case["path"] == "rotate":
+        X, signs = _operands(case, seed)
+        h = case["h"]
+        v = (X.double() * signs).reshape(-1, h)
+        stride = 1
+        while stride < h:
+            a, b = v.view(-1, h // (2 * stride), 2, stride).unbind(2)
+            v = torch.stack([a + b, a - b], dim=2).reshape(-1, h)
+            stride *= 2
+        return (v / math.sqrt(h)).view(X.shape)
+    A, B = _operands(case, seed)
+    if case["path"] == "int8":
+        bound = _CODE_BOUND[case["scheme"]]
+        (cA, dA), (cB, dB) = _quantised(A, bound), _quantised(B, bound)
+        a = (cA.double() * dA.double()[:, :, None]).view(A.shape)
+        b = (cB.double() * dB.double()[:, :, None]).view(B.shape)
+        return {"codes": None, "scales": dA.double(), "C": a @ b.T}
+    B = B.T if case["weight_layout"] else B
+    rounded = case["product"] == "e4m3"
+    if case["path"] == "gemm":
+        return None if rounded else A.double() @ B.double()
+    C = A.double() @ B.double()
+    if case["path"] == "audit":
+        return {"C": None if rounded else C, "Ccl": None if rounded else C, "Cstar": C, "errors": None}
+    return {"ratios": None, "e_classical": None, "norm": float(torch.linalg.norm(C))}
