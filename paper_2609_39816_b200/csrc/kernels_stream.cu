@@ -1,6 +1,7 @@
 // Streaming kernels of the scheme GEMM: encode (block sums -> product dtype), transpose,
 // decode (+ error reduction), Frobenius error, fp64 reference.  All are HBM-bound passes;
 // each thread moves 16-byte vectors and the grid covers the data once.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
@@ -20,6 +21,7 @@ int64_t& fmm_launch_counter() {
 
 namespace {
 
+namespace cg = cooperative_groups;
 
 template <typename SrcT, typename DstT, bool kAmaxOnly, int kEncSplit, bool kM3, bool kDense = false>
 __global__ void __launch_bounds__(kEncThreads)
@@ -374,61 +376,183 @@ __global__ void __launch_bounds__(256) frob_err_kernel(const OutT* __restrict__ 
 }
 
 // ------------------------------------------------------------------------------------------
-// fp64 reference product: 128 x 128 tile per block of 256 threads, 8 x 8 outputs per thread (rows ty + 16 a,
-// columns tx + 16 b: a half-warp reads 16 consecutive doubles of the staged operands), inner index ascending,
-// one fused multiply-add per term; operands converted to fp64 when they are staged.
+// fp64 reference product on the fp64 tensor path (mma.sync m16n8k8: tcgen05 has no fp64 kind).  A 64 x 64 tile per block
+// of four warps, a warp forms 32 x 32 of it; operands are converted to fp64 once, when they are staged.
+// What bounds it: the fp64 pipe (37 TFLOP/s from registers on this chip, by mma.sync and nearly by plain fused
+// multiply-adds).  Four blocks per SM hide the staging (16 inner indices ahead, in registers); the fragments are read
+// without bank conflicts (row strides of 4 mod 16 doubles).
+// Few tiles: a cluster of 2, 4 or 8 blocks shares one tile, each block takes a contiguous share of the inner dimension,
+// and the partial sums meet in distributed shared memory, added in ascending order of the shares.
 // ------------------------------------------------------------------------------------------
-constexpr int kExT = 128, kExK = 16;
+constexpr int kExT = 64, kExK = 16, kExThreads = 128, kExBlocksPerSm = 4;
+constexpr int kExLdK = kExK + 4, kExLdN = kExT + 4;      // row strides of [row][k] and [k][column] staging
+constexpr int kExOperand = kExT * kExLdK;                // doubles per staged operand tile (the larger of the two forms)
+static_assert(kExK * kExLdN <= kExOperand && 4 * kExOperand >= kExT * kExT, "staging");
+
+// VE consecutive elements of a line of X starting at element `at` of `len`: one 16-byte load where the line is aligned and
+// the vector lies inside it, else element by element, zeros beyond the end
 template <typename T>
-__global__ void __launch_bounds__(256) exact_f64_kernel(const T* __restrict__ A, int64_t lda,
-                                                        const T* __restrict__ B, int64_t ldb, int b_weight,
-                                                        int64_t M, int64_t K, int64_t N, double* __restrict__ C) {
-  __shared__ double As[kExK][kExT];
-  __shared__ double Bs[kExK][kExT];
-  const int64_t m0 = (int64_t)blockIdx.y * kExT, n0 = (int64_t)blockIdx.x * kExT;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[8][8];
+__device__ __forceinline__ uint4 exact_fetch(const T* __restrict__ line, int64_t at, int64_t len, bool line_ok, bool vec) {
+  constexpr int VE = 16 / (int)sizeof(T);
+  uint4 raw = make_uint4(0u, 0u, 0u, 0u);
+  if (line_ok) {
+    if (vec && at + VE <= len) {
+      raw = __ldg(reinterpret_cast<const uint4*>(line + at));
+    } else {
+      alignas(16) T e[VE];
 #pragma unroll
-  for (int a = 0; a < 8; ++a)
+      for (int j = 0; j < VE; ++j) e[j] = at + j < len ? line[at + j] : (T)0.0f;
+      raw = *reinterpret_cast<const uint4*>(e);
+    }
+  }
+  return raw;
+}
+template <typename T>
+__device__ __forceinline__ void exact_stage(double* dst, const uint4& raw) {
+  constexpr int VE = 16 / (int)sizeof(T);
+  float2 v[VE / 2];
+  Vec16<T>::unpack(raw, v);
 #pragma unroll
-    for (int b = 0; b < 8; ++b) acc[a][b] = 0.0;
-  for (int64_t k0 = 0; k0 < K; k0 += kExK) {
-    for (int i = threadIdx.x; i < kExT * kExK; i += 256) {
-      {  // A tile: consecutive threads along the inner dimension
-        const int kk = i & (kExK - 1), r = i >> 4;
-        const int64_t row = m0 + r, t = k0 + kk;
-        As[kk][r] = (row < M && t < K) ? (double)(float)A[row * lda + t] : 0.0;
-      }
-      if (b_weight) {
-        const int kk = i & (kExK - 1), c = i >> 4;
-        const int64_t col = n0 + c, t = k0 + kk;
-        Bs[kk][c] = (col < N && t < K) ? (double)(float)B[col * ldb + t] : 0.0;
+  for (int j = 0; j < VE / 2; ++j) *reinterpret_cast<double2*>(dst + 2 * j) = make_double2((double)v[j].x, (double)v[j].y);
+}
+__device__ __forceinline__ void mma_f64(double (&c)[4], const double (&a)[4], const double (&b)[2]) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k8.row.col.f64.f64.f64.f64 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+d"(c[0]), "+d"(c[1]), "+d"(c[2]), "+d"(c[3])
+      : "d"(a[0]), "d"(a[1]), "d"(a[2]), "d"(a[3]), "d"(b[0]), "d"(b[1]));
+}
+
+template <typename T, bool kWeight>
+__global__ void __launch_bounds__(kExThreads, kExBlocksPerSm)
+exact_f64_kernel(const T* __restrict__ A, int64_t lda, const T* __restrict__ B, int64_t ldb, int64_t M, int64_t K, int64_t N,
+                 double* __restrict__ C, int64_t tiles_n, int split, int vec_a, int vec_b) {
+  constexpr int VE = 16 / (int)sizeof(T), kLoads = kExT * kExK / VE / kExThreads;   // 16-byte vectors per thread and operand
+  __shared__ __align__(16) double sm[2][2][kExOperand];
+  const int64_t tile = blockIdx.x / split;
+  const int share = (int)(blockIdx.x - tile * split);
+  const int64_t m0 = tile / tiles_n * kExT, n0 = tile % tiles_n * kExT;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = lane >> 2, t = lane & 3, wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
+  const int64_t steps = (K + kExK - 1) / kExK;
+  const int64_t s0 = steps * share / split, s1 = steps * (share + 1) / split;
+
+  double acc[2][4][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.0;
+
+  uint4 ra[kLoads], rb[kLoads];
+  constexpr int kVecK = kExK / VE, kVecN = kExT / VE;
+  auto fetch = [&](int64_t step) {
+    const int64_t k0 = step * kExK;
+#pragma unroll
+    for (int u = 0; u < kLoads; ++u) {
+      const int i = tid + u * kExThreads;
+      const int row = i / kVecK, kv = (i % kVecK) * VE;
+      ra[u] = exact_fetch(A + (m0 + row) * lda, k0 + kv, K, m0 + row < M, vec_a != 0);
+      if constexpr (kWeight) {
+        rb[u] = exact_fetch(B + (n0 + row) * ldb, k0 + kv, K, n0 + row < N, vec_b != 0);
       } else {
-        const int c = i & (kExT - 1), kk = i >> 7;
-        const int64_t col = n0 + c, t = k0 + kk;
-        Bs[kk][c] = (col < N && t < K) ? (double)(float)B[t * ldb + col] : 0.0;
+        const int kk = i / kVecN, nv = (i % kVecN) * VE;
+        rb[u] = exact_fetch(B + (k0 + kk) * ldb, n0 + nv, N, k0 + kk < K, vec_b != 0);
       }
     }
-    __syncthreads();
+  };
+  auto stage = [&](int buf) {
 #pragma unroll
-    for (int kk = 0; kk < kExK; ++kk) {
-      double a[8], b[8];
-#pragma unroll
-      for (int x = 0; x < 8; ++x) { a[x] = As[kk][ty + 16 * x]; b[x] = Bs[kk][tx + 16 * x]; }
-#pragma unroll
-      for (int x = 0; x < 8; ++x)
-#pragma unroll
-        for (int y = 0; y < 8; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
+    for (int u = 0; u < kLoads; ++u) {
+      const int i = tid + u * kExThreads;
+      const int row = i / kVecK, kv = (i % kVecK) * VE;
+      exact_stage<T>(&sm[buf][0][row * kExLdK + kv], ra[u]);
+      if constexpr (kWeight) exact_stage<T>(&sm[buf][1][row * kExLdK + kv], rb[u]);
+      else exact_stage<T>(&sm[buf][1][(i / kVecN) * kExLdN + (i % kVecN) * VE], rb[u]);
     }
+  };
+  if (s0 < s1) { fetch(s0); stage(0); }
+  __syncthreads();
+  for (int64_t s = s0; s < s1; ++s) {
+    const int buf = (int)(s - s0) & 1;
+    if (s + 1 < s1) fetch(s + 1);
+    const double* As = sm[buf][0];
+    const double* Bs = sm[buf][1];
+#pragma unroll
+    for (int k = 0; k < kExK; k += 8) {
+      double a[2][4], b[4][2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) a[i][e] = As[(wm + i * 16 + g + (e & 1) * 8) * kExLdK + k + t + (e >> 1) * 4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          b[j][e] = kWeight ? Bs[(wn + j * 8 + g) * kExLdK + k + t + e * 4] : Bs[(k + t + e * 4) * kExLdN + wn + j * 8 + g];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) mma_f64(acc[i][j], a[i], b[j]);
+    }
+    if (s + 1 < s1) stage(buf ^ 1);     // the other buffer's readers passed the barrier of the step before
     __syncthreads();
   }
+
+  if (split == 1) {
 #pragma unroll
-  for (int x = 0; x < 8; ++x)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int y = 0; y < 8; ++y) {
-      const int64_t row = m0 + ty + 16 * x, col = n0 + tx + 16 * y;
-      if (row < M && col < N) C[row * N + col] = acc[x][y];
-    }
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int64_t row = m0 + wm + i * 16 + g + (e >> 1) * 8, col = n0 + wn + j * 8 + 2 * t + (e & 1);
+          if (row < M && col < N) C[row * N + col] = acc[i][j][e];
+        }
+    return;
+  }
+  // partial sums of this share, then rows [share * 64 / split, ...) of the tile summed over the cluster
+  cg::cluster_group cluster = cg::this_cluster();
+  double* part = &sm[0][0][0];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) part[(wm + i * 16 + g + (e >> 1) * 8) * kExT + wn + j * 8 + 2 * t + (e & 1)] = acc[i][j][e];
+  cluster.sync();
+  const int rows = kExT / split;
+  for (int i = tid; i < rows * kExT; i += kExThreads) {
+    const int at = share * rows * kExT + i;
+    double sum = *cluster.map_shared_rank(part + at, 0);
+    for (int c = 1; c < split; ++c) sum += *cluster.map_shared_rank(part + at, c);
+    const int64_t row = m0 + at / kExT, col = n0 + at % kExT;
+    if (row < M && col < N) C[row * N + col] = sum;
+  }
+  cluster.sync();     // no block leaves while its partial sums may still be read
+}
+
+template <typename T, bool kWeight>
+cudaError_t launch_exact_t(const T* A, int64_t lda, const T* B, int64_t ldb, int64_t M, int64_t K, int64_t N, double* C,
+                           cudaStream_t st) {
+  const int64_t tiles_n = (N + kExT - 1) / kExT, tiles = (M + kExT - 1) / kExT * tiles_n;
+  // blocks of one tile: as many as still run at once, while a share keeps at least 128 inner indices (a share of 64
+  // costs as much in the exchange as it saves)
+  int split = 1;
+  while (split < 8 && tiles * split * 2 <= 148 * kExBlocksPerSm && K >= (int64_t)split * 2 * 128) split *= 2;
+  if (tiles * split > 0x7fffffff) return cudaErrorInvalidValue;
+  auto aligned = [](const void* p, int64_t ld) { return (reinterpret_cast<uintptr_t>(p) % 16 == 0) && (ld * (int64_t)sizeof(T)) % 16 == 0; };
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(tiles * split)); cfg.blockDim = dim3(kExThreads); cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, exact_f64_kernel<T, kWeight>, A, lda, B, ldb, M, K, N, C, tiles_n, split,
+                                     (int)aligned(A, lda), (int)aligned(B, ldb));
+  if (e != cudaSuccess) return e;
+  ++fmm_launch_counter();
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -648,13 +772,11 @@ cudaError_t launch_frob_err_fixed_grid(int output, const void* C, int64_t ldc, c
 
 cudaError_t launch_exact_f64(int storage, const void* A, int64_t lda, const void* B, int64_t ldb,
                              int b_weight_layout, int64_t M, int64_t K, int64_t N, double* C, cudaStream_t st) {
-  dim3 grid((unsigned)((N + kExT - 1) / kExT), (unsigned)((M + kExT - 1) / kExT));
   if (storage == FMM_F32)
-    exact_f64_kernel<float><<<grid, 256, 0, st>>>((const float*)A, lda, (const float*)B, ldb, b_weight_layout, M, K, N, C);
-  else if (storage == FMM_BF16)
-    exact_f64_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)A, lda, (const __nv_bfloat16*)B, ldb, b_weight_layout, M, K, N, C);
-  else
-    return cudaErrorInvalidValue;
-  ++fmm_launch_counter();
-  return cudaGetLastError();
+    return b_weight_layout ? launch_exact_t<float, true>((const float*)A, lda, (const float*)B, ldb, M, K, N, C, st)
+                           : launch_exact_t<float, false>((const float*)A, lda, (const float*)B, ldb, M, K, N, C, st);
+  if (storage == FMM_BF16)
+    return b_weight_layout ? launch_exact_t<__nv_bfloat16, true>((const __nv_bfloat16*)A, lda, (const __nv_bfloat16*)B, ldb, M, K, N, C, st)
+                           : launch_exact_t<__nv_bfloat16, false>((const __nv_bfloat16*)A, lda, (const __nv_bfloat16*)B, ldb, M, K, N, C, st);
+  return cudaErrorInvalidValue;
 }
