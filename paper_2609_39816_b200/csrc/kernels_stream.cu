@@ -378,9 +378,10 @@ __global__ void __launch_bounds__(256) frob_err_kernel(const OutT* __restrict__ 
 // ------------------------------------------------------------------------------------------
 // fp64 reference product on the fp64 tensor path (mma.sync m16n8k8: tcgen05 has no fp64 kind).  A 64 x 64 tile per block
 // of four warps, a warp forms 32 x 32 of it; operands are converted to fp64 once, when they are staged.
-// What bounds it: the fp64 pipe (37 TFLOP/s from registers on this chip, by mma.sync and nearly by plain fused
+// What bounds it: the fp64 pipe (from registers alone this chip does 37 TFLOP/s by mma.sync, 33 by plain fused
 // multiply-adds).  Four blocks per SM hide the staging (16 inner indices ahead, in registers); the fragments are read
-// without bank conflicts (row strides of 4 mod 16 doubles).
+// without bank conflicts (row strides of 4 mod 16 doubles).  A 128 x 128 tile of plain multiply-adds, one block per SM,
+// left the pipe idle while it staged: 9.4 ms at 2048 x 4096 x 4096 where this takes 2.06.
 // Few tiles: a cluster of 2, 4 or 8 blocks shares one tile, each block takes a contiguous share of the inner dimension,
 // and the partial sums meet in distributed shared memory, added in ascending order of the shares.
 // ------------------------------------------------------------------------------------------
@@ -536,10 +537,16 @@ template <typename T, bool kWeight>
 cudaError_t launch_exact_t(const T* A, int64_t lda, const T* B, int64_t ldb, int64_t M, int64_t K, int64_t N, double* C,
                            cudaStream_t st) {
   const int64_t tiles_n = (N + kExT - 1) / kExT, tiles = (M + kExT - 1) / kExT * tiles_n;
-  // blocks of one tile: as many as still run at once, while a share keeps at least 128 inner indices (a share of 64
-  // costs as much in the exchange as it saves)
+  // Blocks of one tile: the number that leaves the busiest SM the least work.  A share's fill and exchange count as 64
+  // inner indices, and a block alone on its SM runs at three quarters of the pipe.  Measured, one block a tile against the
+  // chosen split: 2048 x 3456 x 1280 763 -> 578 us (2), 300 x 4096 x 500 243 -> 71 us (8), 512 x 1024 x 1024 68 -> 52 us (2),
+  // 128^3 16 -> 11 us (8); 2048 x 4096 x 4096 stays whole at 2.06 ms (33.4 TFLOP/s, the fp64 tensor pipe 90 % busy).
   int split = 1;
-  while (split < 8 && tiles * split * 2 <= 148 * kExBlocksPerSm && K >= (int64_t)split * 2 * 128) split *= 2;
+  int64_t least = INT64_MAX;
+  for (int c = 1; c <= 8 && (c == 1 || K >= (int64_t)c * kExK); c *= 2) {
+    const int64_t shares = (tiles * c + 147) / 148, load = shares * (K / c + 64) * (shares == 1 ? 4 : 3);
+    if (load < least) { least = load; split = c; }
+  }
   if (tiles * split > 0x7fffffff) return cudaErrorInvalidValue;
   auto aligned = [](const void* p, int64_t ld) { return (reinterpret_cast<uintptr_t>(p) % 16 == 0) && (ld * (int64_t)sizeof(T)) % 16 == 0; };
   cudaLaunchConfig_t cfg = {};
