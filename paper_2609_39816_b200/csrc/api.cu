@@ -505,9 +505,41 @@ bool merge_tables(const CoefTable* tabs, int kb, int R, CoefTable* mA, CoefTable
   return true;
 }
 
+// Sweeps on small blocks run many copies per launch (sweep_many.cu).  The line: every product is one tile of the product
+// kernel and a block sum is the work of one block of threads, so a copy alone is launch latency (40 us for six launches at
+// 128^3, two levels, against 1 us as one of a batch).  The model schedule's scales (mode 3) keep the general path.
+struct ManyLayout { size_t data, hat_a, hat_b, scale_a, scale_b, prod, part, total; int copies, blocks, tpb; };
+
+bool sweep_many_ok(const fmm_scheme* s, const fmm_gemm_desc* d) {
+  return d->M / s->m <= kManyRows && d->N / s->n <= kManyRows && d->K / s->k <= 1024 && d->scale_mode <= 2;
+}
+
+ManyLayout many_layout(const fmm_scheme* s, const fmm_gemm_desc* d, int G) {
+  ManyLayout L{};
+  const GemmLayout g = gemm_layout(s->m, s->k, s->n, s->R, d);
+  const int ep = esize(d->product), eo = (d->flags & FMM_FLAG_PRODUCTS_BF16) ? 2 : 4;
+  const int64_t bm = d->M / s->m, bn = d->N / s->n;
+  // copies of one batch: what it writes stays in L2 (48 MB) until the next pass reads it
+  const int64_t per_copy = s->R * std::max((g.sAhat + g.sBhat) * ep, g.sProd * (int64_t)eo);
+  L.copies = (int)std::min<int64_t>(std::min(G, 512), std::max<int64_t>(1, ((int64_t)48 << 20) / per_copy));
+  const size_t n = (size_t)L.copies * s->R;
+  size_t o = 0;
+  const size_t coefs = 2 * (size_t)FMM_MAX_R * 3 * kMaxCells, gauge = 2 * 3 * (size_t)kMaxCells;
+  L.data = o; o += align_up((coefs + G * gauge) * 8);
+  L.hat_a = o; o += align_up(n * g.sAhat * ep);
+  L.hat_b = o; o += align_up(n * g.sBhat * ep);
+  L.scale_a = o; o += align_up(n * (d->scale_mode == 2 ? bm : 1) * 4);
+  L.scale_b = o; o += align_up(n * (d->scale_mode == 2 ? bn : 1) * 4);
+  L.prod = o; o += align_up(n * g.sProd * eo);
+  L.blocks = decode_many_blocks(bm, bn, L.copies, &L.tpb);
+  L.part = o; o += align_up((size_t)G * L.blocks * 8);
+  L.total = o;
+  return L;
+}
+
 struct SweepLayout {
   GemmLayout g; ClassicalLayout c;
-  size_t gemm, gemm2, classical, cstar, cstar32, ccl, tables, sums, fpart, total;   // two GEMM workspaces: gauges are pipelined
+  size_t gemm, gemm2, classical, cstar, cstar32, ccl, tables, sums, fpart, many, total;   // two GEMM workspaces: gauges are pipelined
 };
 constexpr int kFusedPartialsPerGauge = 512;   // room for the streaming blocks of a fused launch (2 per SM)
 
@@ -525,6 +557,8 @@ SweepLayout sweep_layout(const fmm_scheme* s, const fmm_gemm_desc* d, int G) {
   L.tables = o; o += align_up((size_t)G * 3 * sizeof(CoefTable));
   L.sums = o; o += align_up((size_t)(G + 8) * 8);
   L.fpart = o; o += align_up((size_t)G * kFusedPartialsPerGauge * 8);
+  L.many = o;
+  if (sweep_many_ok(s, d)) o += many_layout(s, d, G).total;
   L.total = o;
   return L;
 }
@@ -775,20 +809,38 @@ fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const fmm_scheme* grid = level == 1 ? base->outer.get() : base;
   const int gm = grid->m, gk = grid->k, gn = grid->n;
+  const bool serial = g_prof_on || (d->flags & FMM_FLAG_SWEEP_SERIAL) != 0;
+  const bool many = !serial && sweep_many_ok(base, d);
   // every gauge matrix is checked before the first launch: a singular one returns with nothing enqueued
-  for (int g = 0; g < G; ++g)
-    if (!fmm_gauge_invertible(gm, gk, gn, P + (size_t)g * gm * gm, Q + (size_t)g * gk * gk, S + (size_t)g * gn * gn))
-      return FMM_ERR_SINGULAR;
+  const size_t per_gauge = 2 * (size_t)(gm * gm + gk * gk + gn * gn);
+  std::vector<double> packed;           // small blocks: coefficients and gauges for the device (launch_gauge_tables)
+  if (many) {
+    const fmm_scheme* inner = level == 1 ? base->inner.get() : nullptr;
+    const double one = 1.0;
+    for (const auto* v : {&grid->U, &grid->V, &grid->W}) packed.insert(packed.end(), v->begin(), v->end());
+    if (inner) for (const auto* v : {&inner->U, &inner->V, &inner->W}) packed.insert(packed.end(), v->begin(), v->end());
+    else packed.insert(packed.end(), 3, one);
+    const size_t head = packed.size();
+    packed.resize(head + G * per_gauge);
+    for (int g = 0; g < G; ++g)
+      if (!fmm_gauge_pack(gm, gk, gn, P + (size_t)g * gm * gm, Q + (size_t)g * gk * gk, S + (size_t)g * gn * gn,
+                          packed.data() + head + g * per_gauge))
+        return FMM_ERR_SINGULAR;
+  } else {
+    for (int g = 0; g < G; ++g)
+      if (!fmm_gauge_invertible(gm, gk, gn, P + (size_t)g * gm * gm, Q + (size_t)g * gk * gk, S + (size_t)g * gn * gn))
+        return FMM_ERR_SINGULAR;
+  }
 
   // 1. gauge-transformed coefficient tables: built on the host, merged per batch of algorithms and uploaded in groups
   //    of kTableGroup gauges while the device works on the groups before (the first launch waits for one group only)
   constexpr int kTableGroup = 32;
-  std::vector<CoefTable> single((size_t)G * 3);
-  std::memset(single.data(), 0, single.size() * sizeof(CoefTable));
+  std::vector<CoefTable> single(many ? 0 : (size_t)G * 3);
+  if (!many) std::memset(single.data(), 0, single.size() * sizeof(CoefTable));
   struct Chunk { int g0, count; };
   std::vector<Chunk> chunks;
   std::vector<CoefTable> tabs;          // three tables per chunk
-  tabs.reserve((size_t)G * 3);          // never reallocates: launches keep pointers into it
+  if (!many) tabs.reserve((size_t)G * 3);   // never reallocates: launches keep pointers into it
   const int kb = sweep_batch(base);
   int next_gauge = 0;
   char* ws = static_cast<char*>(d_ws);
@@ -854,11 +906,42 @@ fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P
   void* gws2 = ws + L.gemm2;
   FMM_CUDA(cudaMemsetAsync(at<char>(gws2, L.g.status), 0, sizeof(DeviceStatus), st));
   // with phase timing on, or when the caller asks for it, the stages run back to back on the caller's stream
-  const bool serial = g_prof_on || (d->flags & FMM_FLAG_SWEEP_SERIAL) != 0;
-  SideStream* side = serial ? nullptr : side_stream();
+  SideStream* side = serial || many ? nullptr : side_stream();
   fmm_scheme batched;                   // dimensions only: a batch of kc algorithms looks like one with kc * R products
   batched.m = base->m; batched.k = base->k; batched.n = base->n;
   fmm_status loop_rc = FMM_OK;
+  if (many) {
+    const ManyLayout Lm = many_layout(base, d, G);
+    char* mws = ws + L.many;
+    const int R = base->R, mode = d->scale_mode;
+    const int64_t bm = d->M / base->m, bn = d->N / base->n, bk = d->K / base->k;
+    const fmm_scheme* inner = level == 1 ? base->inner.get() : nullptr;
+    const GaugeDims gd{gm, gk, gn, grid->R, inner ? inner->m : 1, inner ? inner->k : 1, inner ? inner->n : 1, inner ? inner->R : 1};
+    FMM_CUDA(cudaMemcpyAsync(mws + Lm.data, packed.data(), packed.size() * 8, cudaMemcpyHostToDevice, st));
+    FMM_CUDA(launch_gauge_tables(at<double>(mws, Lm.data), gd, G, d_tabs, st));
+    const EncodeManyJob ja{dA, d->lda, base->k, (int)bm, (int)bk, at<char>(mws, Lm.hat_a), L.g.sAhat, at<float>(mws, Lm.scale_a)};
+    const EncodeManyJob jb{bk_ptr, bk_ld, base->k, (int)bn, (int)bk, at<char>(mws, Lm.hat_b), L.g.sBhat, at<float>(mws, Lm.scale_b)};
+    const bool prod_bf16 = (d->flags & FMM_FLAG_PRODUCTS_BF16) != 0;
+    for (int g = 0; g < G; g += Lm.copies) {
+      const int copies = std::min(Lm.copies, G - g);
+      FMM_CUDA(launch_encode_many(d->storage, d->product, ja, jb, d_tabs + 3 * g, R, copies, mode, st));
+      BlockProductArgs p{};
+      p.product = d->product;
+      p.A = ja.out; p.lda = bk; p.a_batch = L.g.sAhat;
+      p.B = jb.out; p.ldb = bk; p.b_batch = L.g.sBhat;
+      p.rows_a = bm; p.rows_b = bn; p.kdim = bk; p.batches = copies * R;
+      p.out = at<char>(mws, Lm.prod); p.ldo = bn; p.o_batch = L.g.sProd;
+      p.out_mode = prod_bf16 ? 1 : 0; p.output = prod_bf16 ? FMM_BF16 : FMM_F32;
+      if (mode == 2) { p.row_scale = ja.scale; p.rs_batch = bm; p.col_scale = jb.scale; p.cs_batch = bn; }
+      p.status = at<DeviceStatus>(gws, L.g.status);
+      FMM_TRY(launch_block_products(p, st));
+      FMM_CUDA(launch_decode_many(d->output, p.out, prod_bf16 ? FMM_BF16 : FMM_F32, L.g.sProd, d_tabs + 3 * g, R, copies,
+                                  mode == 1 ? ja.scale : nullptr, mode == 1 ? jb.scale : nullptr, base->m, base->n, bm, bn,
+                                  cstar32, at<double>(mws, Lm.part) + (size_t)g * Lm.blocks, Lm.blocks, Lm.tpb, st));
+    }
+    FMM_CUDA(launch_sum_partials(at<double>(mws, Lm.part), Lm.blocks, sums + 8, st, G));
+    next_gauge = G;
+  }
   // Fused pipeline (unless FMM_FLAG_SWEEP_UNFUSED; bf16 storage and products, no scales, batches of four or eight one-level
   // algorithms): ONE launch per batch runs its block products together with the decode of the batch before and the
   // encode of the batch after, in the same CTAs (launch_fused_sweep), on the caller's stream; the pipeline starts with a
@@ -870,7 +953,7 @@ fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P
   size_t first_plain_chunk = 0;
   const int kFusedGroups = 2;
   const int64_t bm_ = d->M / base->m, bn_ = d->N / base->n, bk_ = d->K / base->k;
-  const bool fused_ok = !(d->flags & FMM_FLAG_SWEEP_UNFUSED) && !serial && kb >= 4 && d->storage == FMM_BF16 && d->product == FMM_BF16 && d->scale_mode == 0 &&
+  const bool fused_ok = !many && !(d->flags & FMM_FLAG_SWEEP_UNFUSED) && !serial && kb >= 4 && d->storage == FMM_BF16 && d->product == FMM_BF16 && d->scale_mode == 0 &&
                         !(d->flags & FMM_FLAG_PRODUCTS_BF16) && base->m * base->k <= 4 && base->n * base->k <= 4 &&
                         base->m * base->n <= 4 && bm_ > 128 && bn_ > 128 &&
                         fused_sweep_blocks(kFusedGroups) <= kFusedPartialsPerGauge && fused_sweep_blocks(kFusedGroups) >= 2 &&

@@ -51,5 +51,7 @@ struct CoefTable {
 void fmm_build_tables(const fmm_scheme& s, CoefTable* tA, CoefTable* tB, CoefTable* tW);
 // true when P (m x m), Q (k x k) and S (n x n) can all be inverted (the test gauge_apply / fmm_gauge_core apply)
 bool fmm_gauge_invertible(int m, int k, int n, const double* P, const double* Q, const double* S);
+// the same, writing P, Q, S and their inverses to out (2 (m m + k k + n n) doubles) for the device's tables
+bool fmm_gauge_pack(int m, int k, int n, const double* P, const double* Q, const double* S, double* out);
 fmm_status fmm_gauge_core(const fmm_scheme& in, int level, const double* P, const double* Q, const double* S,
                           double cond_limit, fmm_scheme** out);

@@ -123,6 +123,23 @@ cudaError_t launch_decode(int output, const void* prod, int prod_dtype, int64_t 
                           cudaStream_t st, int gauges = 1);
 int decode_grid(int64_t bm, int64_t bn);
 
+// ---- many copies of an algorithm on small blocks (sweep_many.cu): tables of copy c at tabs[3 * c ..], its products numbered
+// c * R .. c * R + R - 1 in every buffer.
+// Dimensions of the gauged factor and of the inner factor it is nested with (1, 1, 1, 1 for none).
+struct GaugeDims { int m, k, n, R, im, ik, in, iR; };
+// data (DEVICE): coefficients U, V, W of the gauged factor, then of the inner one, then per copy P, Q, S, P^-1, Q^-1, S^-1.
+cudaError_t launch_gauge_tables(const double* data, const GaugeDims& d, int copies, CoefTable* tabs, cudaStream_t st);
+constexpr int kManyRows = 128;      // rows of a block at most
+// One operand: source X in a grid of br x bc blocks (gc per row), block sums to out, rstride elements apart.
+struct EncodeManyJob { const void* X; int64_t ldx; int gc; int br, bc; void* out; int64_t rstride; float* scale; };
+cudaError_t launch_encode_many(int storage, int product, const EncodeManyJob& a, const EncodeManyJob& b, const CoefTable* tabs,
+                               int R, int copies, int mode, cudaStream_t st);
+int decode_many_blocks(int64_t bm, int64_t bn, int copies, int* tiles_per_block);
+// Error-only decode; partials [copy][blocks].
+cudaError_t launch_decode_many(int output, const void* prod, int prod_dtype, int64_t prod_stride, const CoefTable* tabs, int R,
+                               int copies, const float* sA, const float* sB, int m, int n, int64_t bm, int64_t bn,
+                               const float* cstar32, double* partials, int blocks, int tiles_per_block, cudaStream_t st);
+
 // out[0] = sum of partials[0..n) in a fixed order (single block).
 // out[b] = sum of partials[b*n .. b*n+n), b < count
 cudaError_t launch_sum_partials(const double* partials, int n, double* out, cudaStream_t st, int count = 1);

@@ -249,6 +249,12 @@ bool fmm_gauge_invertible(int m, int k, int n, const double* P, const double* Q,
   return invert(m, P, inv) && invert(k, Q, inv) && invert(n, S, inv);
 }
 
+bool fmm_gauge_pack(int m, int k, int n, const double* P, const double* Q, const double* S, double* out) {
+  double* inv = out + m * m + k * k + n * n;
+  std::copy_n(S, n * n, std::copy_n(Q, k * k, std::copy_n(P, m * m, out)));
+  return invert(m, P, inv) && invert(k, Q, inv + m * m) && invert(n, S, inv + m * m + k * k);
+}
+
 fmm_status fmm_gauge_core(const fmm_scheme& in, int level, const double* P, const double* Q, const double* S,
                           double cond_limit, fmm_scheme** out) {
   std::unique_ptr<fmm_scheme> res(new (std::nothrow) fmm_scheme);
