@@ -73,13 +73,14 @@ __device__ __forceinline__ unsigned long long global_timer_ns() {
 // Bounded wait.  Returns false when the CTA is aborting (this wait or another one gave up).
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, int where,
                                           DeviceStatus* status, unsigned long long limit_ns) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const unsigned long long t0 = global_timer_ns();
+  unsigned long long t0 = 0;      // the clock is read every 64 polls only: a read takes longer than most waits
   for (uint32_t it = 1;; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
     if ((it & 63u) == 0u) {
       if (*abort_flag) return false;
-      if (global_timer_ns() - t0 > limit_ns) {
+      const unsigned long long now = global_timer_ns();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > limit_ns) {
         *abort_flag = 1;
         if (status != nullptr) {
           atomicExch(&status->code, (int)FMM_ERR_TIMEOUT);
@@ -137,6 +138,25 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32]) {
       : "memory");
 }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&v)[16]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+                 "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+               : "r"(taddr) : "memory");
+}
+// these waits name the registers of the loads that they complete: no use of them can be scheduled before
+__device__ __forceinline__ void tc_wait_ld16(uint32_t (&v)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                 "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]) :: "memory");
+}
+__device__ __forceinline__ void tc_wait_ld32(uint32_t (&v)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]),
+                 "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]),
+                 "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
+                 "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31]) :: "memory");
+}
 
 // Shared-memory matrix descriptor of a K-major tile stored as rows of 128 bytes with the 128-byte
 // swizzle (what TMA writes with CU_TENSOR_MAP_SWIZZLE_128B): start address (>>4), leading byte offset
@@ -1004,6 +1024,137 @@ __device__ __forceinline__ void tc_mma_i8(uint32_t d_tmem, uint64_t a_desc, uint
 // packed forms are used only where merging is impossible (multiply after multiply) or harmless (an exact subtraction).
 constexpr int kInt8Threads = 576;   // 18 warps: TMA, MMA, and 16 rescale warps (four per TMEM lane quarter, 32 columns each)
 
+// The rescale role of the group-scaled int8 kernels (warps 2..17): waits for a group's accumulator, converts it, applies
+// the two scales and adds to the tile's fp32 sums, which a thread holds for one row and 32 columns.
+struct RescaleCtx {
+  uint32_t tfull0, tempty0;     // accumulator barriers of the kAcc buffers (consecutive)
+  uint32_t sfull, sempty;       // the tile's column scales are staged / no longer read (16 arrivals each)
+  uint32_t tmem_base;
+  float* scale_sm;              // [group][128] column scales of the current tile
+  volatile int* abort_flag;
+  DeviceStatus* status;
+  unsigned long long limit;
+  void* out;
+  const float* dAt; const float* dBt;   // [G][M] and [G][N]
+  int M, N, G;
+  long long ldc;
+  int out_bf16, wide;
+};
+struct RescaleTile { int row0, rows, col0, cols; bool plus, minus; };   // first row and column of the tile in C, its extents
+
+// kMinus: a buffer is two accumulators side by side; the group's integer is the first minus the second, of those that
+// the tile says were written
+template <int kAcc, bool kMinus, typename TileOf>
+__device__ __forceinline__ void int8_rescale_role(const RescaleCtx& c, const int warp, const int lane, const int total_tiles,
+                                                  const TileOf tile_of) {
+  constexpr int BN = 128, PN = 32, kBufCols = kMinus ? 2 * BN : BN;
+  constexpr int kMaxGroupsStaged = Int8Layout::kMaxGroupsStaged;
+  const int quad = warp & 3;             // TMEM lanes [32*quad, 32*quad+32) are the ones this warp may read
+  const int part = (warp - 2) >> 2;      // which 32 of the tile's 128 columns
+  int acc = 0;
+  uint32_t acc_phase = 0;
+  uint32_t scale_phase = 0;
+  bool ok = true;
+  for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+    const RescaleTile t = tile_of(tile);
+    const int row = t.row0 + quad * 32 + lane;
+    const bool row_ok = quad * 32 + lane < t.rows;
+    const int cols_here = t.cols - part * PN;             // of this warp's 32 columns, those inside the tile
+    float2 sum[PN / 2];
+#pragma unroll
+    for (int j = 0; j < PN / 2; ++j) sum[j] = make_float2(0.0f, 0.0f);
+    // column scales of this tile: [group][128] into shared memory (zero beyond its edge), by the 512 rescale threads
+    const bool staged = c.G <= kMaxGroupsStaged;
+    if (staged) {
+      // bounded waits on mbarriers, not a named barrier: a warp that gives up elsewhere must not strand the others
+      ok = mbar_wait(c.sempty, scale_phase ^ 1u, c.abort_flag, 0x64, c.status, c.limit);   // previous tile's readers are done
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      const int et = threadIdx.x - 64;                  // 0 .. 511
+      for (int i = et; i < c.G * (BN / 4); i += 512) {
+        const int g = i / (BN / 4), c4 = (i - g * (BN / 4)) * 4;
+        const float4 val = c4 < t.cols ? *reinterpret_cast<const float4*>(c.dBt + (long long)g * c.N + t.col0 + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
+        *reinterpret_cast<float4*>(c.scale_sm + g * BN + c4) = val;
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(c.sfull);              // release: this warp's share is written
+      ok = mbar_wait(c.sfull, scale_phase, c.abort_flag, 0x65, c.status, c.limit);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+    }
+    float da_next = row_ok ? c.dAt[row] : 0.0f;
+    for (int g = 0; g < c.G; ++g) {
+      // the row scale does not depend on the products: the next group's is fetched a step ahead
+      const float da = da_next;
+      if (g + 1 < c.G) da_next = row_ok ? c.dAt[(long long)(g + 1) * c.M + row] : 0.0f;
+      const float* dbp = staged ? c.scale_sm + g * BN + part * PN : c.dBt + (long long)g * c.N + t.col0 + part * PN;
+      ok = mbar_wait(c.tfull0 + 8u * acc, acc_phase, c.abort_flag, 0x63, c.status, c.limit);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
+      uint32_t v[32];
+      const uint32_t taddr = c.tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * kBufCols + part * PN);
+      if (!kMinus || t.plus) {
+        tc_ld32(taddr, v);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = 0u;
+      }
+      if constexpr (kMinus) {
+        if (t.minus) {       // sixteen columns at a time: 96 registers a thread
+          uint32_t m[16];
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            tc_ld16(taddr + BN + 16 * half, m);
+            tc_wait_ld16(m);
+            if (half == 0) tc_wait_ld32(v);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[16 * half + j] -= m[j];
+          }
+        }
+      }
+      tc_wait_ld32(v);
+      // the accumulator is in registers: hand the buffer back before the arithmetic
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(c.tempty0 + 8u * acc);
+      if (++acc == kAcc) { acc = 0; acc_phase ^= 1u; }
+      const float2 da2 = make_float2(da, da);
+      const float2 neg_magic = make_float2(-12582912.0f, -12582912.0f);
+#pragma unroll
+      for (int j = 0; j < PN; ++j) {
+        // exact int -> float for |P| < 2^22 (a group product is at most 128 * 127^2): add the integer to the bits
+        // of 1.5 * 2^23, subtract that constant (exact).  Then two separately rounded multiplications and a
+        // separately rounded addition, as the specification orders them.
+        v[j] += 0x4B400000u;
+      }
+#pragma unroll
+      for (int q4 = 0; q4 < PN / 4; ++q4) {
+        float2 p0 = make_float2(__uint_as_float(v[q4 * 4 + 0]), __uint_as_float(v[q4 * 4 + 1]));
+        float2 p1 = make_float2(__uint_as_float(v[q4 * 4 + 2]), __uint_as_float(v[q4 * 4 + 3]));
+        p0 = __fadd2_rn(p0, neg_magic); p1 = __fadd2_rn(p1, neg_magic);
+        p0 = __fmul2_rn(p0, da2); p1 = __fmul2_rn(p1, da2);
+        const float4 db = (staged || q4 * 4 < cols_here) ? *reinterpret_cast<const float4*>(dbp + q4 * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+        p0 = __fmul2_rn(p0, make_float2(db.x, db.y)); p1 = __fmul2_rn(p1, make_float2(db.z, db.w));
+        sum[q4 * 2].x = __fadd_rn(sum[q4 * 2].x, p0.x); sum[q4 * 2].y = __fadd_rn(sum[q4 * 2].y, p0.y);
+        sum[q4 * 2 + 1].x = __fadd_rn(sum[q4 * 2 + 1].x, p1.x); sum[q4 * 2 + 1].y = __fadd_rn(sum[q4 * 2 + 1].y, p1.y);
+      }
+    }
+    if (!ok) break;
+    if (staged) {                                        // this warp no longer reads the tile's scales
+      __syncwarp();
+      if (lane == 0) mbar_arrive(c.sempty);
+      scale_phase ^= 1u;
+    }
+    if (row_ok && cols_here > 0) {
+      uint32_t w[32];
+#pragma unroll
+      for (int j = 0; j < PN / 2; ++j) { w[2 * j] = __float_as_uint(sum[j].x); w[2 * j + 1] = __float_as_uint(sum[j].y); }
+      store_row_chunk(c.out, (long long)row * c.ldc + t.col0 + part * PN, min(32, cols_here), w, 1, c.out_bf16, 1.0f, c.wide != 0);
+    }
+  }
+}
+
 __global__ void __launch_bounds__(kInt8Threads, 1)
 int8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                        void* __restrict__ out, Int8Params p, DeviceStatus* status) {
@@ -1118,90 +1269,13 @@ int8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
       }
     }
   } else {
-    // ------------------------------------------------------------ rescale and accumulate (warps 2..17)
-    const int quad = warp & 3;             // TMEM lanes [32*quad, 32*quad+32) are the ones this warp may read
-    const int part = (warp - 2) >> 2;      // which 32 of the tile's 128 columns
-    constexpr int PN = 32;
-    int acc = 0;
-    uint32_t acc_phase = 0;
-    uint32_t scale_phase = 0;
-    bool ok = true;
-    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+    const RescaleCtx rc{bar_base + 8u * (2 * L::kStages), bar_base + 8u * (2 * L::kStages + kAcc), sfull_bar, sempty_bar,
+                        tmem_base, scale_sm, abort_flag, status, p.wait_limit_ns, out, p.dAt, p.dBt, p.M, p.N, p.G,
+                        p.ldc, p.out_bf16, p.wide};
+    int8_rescale_role<kAcc, false>(rc, warp, lane, total_tiles, [&](int tile) {
       const int tm = tile / p.tiles_n, tn = tile - tm * p.tiles_n;
-      const int row = tm * BM + quad * 32 + lane;
-      const bool row_ok = row < p.M;
-      const int col_base = tn * BN + part * PN;
-      float2 sum[PN / 2];
-#pragma unroll
-      for (int j = 0; j < PN / 2; ++j) sum[j] = make_float2(0.0f, 0.0f);
-      // column scales of this tile: [group][128] into shared memory (zero beyond N), by the 512 rescale threads
-      const bool staged = p.G <= L::kMaxGroupsStaged;
-      if (staged) {
-        // bounded waits on mbarriers, not a named barrier: a warp that gives up elsewhere must not strand the others
-        ok = mbar_wait(sempty_bar, scale_phase ^ 1u, abort_flag, 0x64, status, p.wait_limit_ns);   // previous tile's readers are done
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        const int et = threadIdx.x - 64;                  // 0 .. 511
-        for (int i = et; i < p.G * (BN / 4); i += 512) {
-          const int g = i / (BN / 4), c4 = (i - g * (BN / 4)) * 4;
-          const int col = tn * BN + c4;
-          const float4 val = col < p.N ? *reinterpret_cast<const float4*>(p.dBt + (long long)g * p.N + col) : make_float4(0.f, 0.f, 0.f, 0.f);
-          *reinterpret_cast<float4*>(scale_sm + g * BN + c4) = val;
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(sfull_bar);            // release: this warp's share is written
-        ok = mbar_wait(sfull_bar, scale_phase, abort_flag, 0x65, status, p.wait_limit_ns);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-      }
-      float da_next = row_ok ? p.dAt[row] : 0.0f;
-      for (int g = 0; g < p.G; ++g) {
-        // the row scale does not depend on the products: the next group's is fetched a step ahead
-        const float da = da_next;
-        if (g + 1 < p.G) da_next = row_ok ? p.dAt[(long long)(g + 1) * p.M + row] : 0.0f;
-        const float* dbp = staged ? scale_sm + g * BN + part * PN : p.dBt + (long long)g * p.N + col_base;
-        ok = mbar_wait(tfull_bar(acc), acc_phase, abort_flag, 0x63, status, p.wait_limit_ns);
-        ok = __all_sync(0xffffffffu, ok);
-        if (!ok) break;
-        tc_fence_after();
-        uint32_t v[32];
-        tc_ld32(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN + part * PN), v);
-        tc_wait_ld();
-        // the accumulator is in registers: hand the buffer back before the arithmetic
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(tempty_bar(acc));
-        if (++acc == kAcc) { acc = 0; acc_phase ^= 1u; }
-        const float2 da2 = make_float2(da, da);
-        const float2 neg_magic = make_float2(-12582912.0f, -12582912.0f);
-#pragma unroll
-        for (int q4 = 0; q4 < PN / 4; ++q4) {
-          // exact int -> float for |P| < 2^22 (a group product is at most 128 * 127^2): add the integer to the bits
-          // of 1.5 * 2^23, subtract that constant (exact).  Then two separately rounded multiplications and a
-          // separately rounded addition, as the specification orders them.
-          float2 p0 = make_float2(__uint_as_float(v[q4 * 4 + 0] + 0x4B400000u), __uint_as_float(v[q4 * 4 + 1] + 0x4B400000u));
-          float2 p1 = make_float2(__uint_as_float(v[q4 * 4 + 2] + 0x4B400000u), __uint_as_float(v[q4 * 4 + 3] + 0x4B400000u));
-          p0 = __fadd2_rn(p0, neg_magic); p1 = __fadd2_rn(p1, neg_magic);
-          p0 = __fmul2_rn(p0, da2); p1 = __fmul2_rn(p1, da2);
-          const float4 db = (staged || col_base + q4 * 4 < p.N) ? *reinterpret_cast<const float4*>(dbp + q4 * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-          p0 = __fmul2_rn(p0, make_float2(db.x, db.y)); p1 = __fmul2_rn(p1, make_float2(db.z, db.w));
-          sum[q4 * 2].x = __fadd_rn(sum[q4 * 2].x, p0.x); sum[q4 * 2].y = __fadd_rn(sum[q4 * 2].y, p0.y);
-          sum[q4 * 2 + 1].x = __fadd_rn(sum[q4 * 2 + 1].x, p1.x); sum[q4 * 2 + 1].y = __fadd_rn(sum[q4 * 2 + 1].y, p1.y);
-        }
-      }
-      if (!ok) break;
-      if (staged) {                                        // this warp no longer reads the tile's scales
-        __syncwarp();
-        if (lane == 0) mbar_arrive(sempty_bar);
-        scale_phase ^= 1u;
-      }
-      if (row_ok && col_base < p.N) {
-        uint32_t w[32];
-#pragma unroll
-        for (int j = 0; j < PN / 2; ++j) { w[2 * j] = __float_as_uint(sum[j].x); w[2 * j + 1] = __float_as_uint(sum[j].y); }
-        store_row_chunk(out, (long long)row * p.ldc + col_base, min(32, p.N - col_base), w, 1, p.out_bf16, 1.0f, p.wide != 0);
-      }
-    }
+      return RescaleTile{tm * BM, min(BM, p.M - tm * BM), tn * BN, min(BN, p.N - tn * BN), true, false};
+    });
   }
 
   tc_fence_before();
@@ -1468,46 +1542,30 @@ fmm_status launch_int8_group_gemm(const int8_t* cA, const int8_t* cB, const floa
 fmm_status launch_int8_certified(const Int8CertArgs& a, cudaStream_t st) {
   using L = CertLayout;
   if (a.h != 32 && a.h != 64 && a.h != 128) return FMM_ERR_SHAPE;
-  if (a.m * a.n > L::kMaxBlocks || a.R > FMM_MAX_R || a.n_entries > L::kMaxEntries) return FMM_ERR_LIMIT;
-  if (a.bm * a.G > 0x7fffffff || a.bn * a.G > 0x7fffffff || a.M > 0x7fffffff || a.N > 0x7fffffff) return FMM_ERR_SHAPE;
-  const int per = BKB / a.h;
-  const int row_stages = (a.R + per - 1) / per;
-  CUtensorMap ma, mb;
-  if (!make_operand_map(&ma, true, a.Ahat, a.bm * a.G, BKB, BKB, a.bm * a.G * BKB, row_stages, BM)) return FMM_ERR_CUDA;
-  if (!make_operand_map(&mb, true, a.Bhat, a.bn * a.G, BKB, BKB, a.bn * a.G * BKB, row_stages, L::BN)) return FMM_ERR_CUDA;
+  if (a.m * a.n > kMaxCells || a.R > FMM_MAX_R) return FMM_ERR_LIMIT;
+  if (a.M > 0x7fffffff || a.N > 0x7fffffff) return FMM_ERR_SHAPE;
   CertParams p{};
-  p.M = (int)a.M; p.N = (int)a.N; p.m = a.m; p.n = a.n; p.bm = (int)a.bm; p.bn = (int)a.bn;
-  p.G = a.G; p.R = a.R; p.h = a.h; p.per = per; p.ksteps = a.h / UMMA_KB;
-  int8_certified_passes(a.R, per, &p.passes, &p.pass_len);
+  p.M = (int)a.M; p.N = (int)a.N; p.n = a.n; p.blocks = a.m * a.n; p.bm = (int)a.bm; p.bn = (int)a.bn;
+  p.G = a.G; p.ksteps = a.h / UMMA_KB;
   p.tiles_m = (int)((a.bm + BM - 1) / BM);
   p.tiles_n = (int)((a.bn + L::BN - 1) / L::BN);
   p.ldc = a.ldc; p.out_bf16 = a.output == FMM_BF16;
-  p.dAt = a.dAt; p.dBt = a.dBt;
-  p.entries = a.d_entries; p.pass_off = a.d_pass_off; p.owned = a.d_owned; p.n_entries = a.n_entries;
+  const int es = p.out_bf16 ? 2 : 4;
+  p.wide = (reinterpret_cast<uintptr_t>(a.C) % 32 == 0) && ((a.ldc * es) % 32 == 0) && ((a.bn * es) % 32 == 0);
+  p.Ahat = a.Ahat; p.Bhat = a.Bhat; p.dAt = a.dAt; p.dBt = a.dBt; p.tab_w = a.d_tab_w;
   p.wait_limit_ns = kDefaultWaitLimitNs;
-  const long long total = (long long)p.tiles_m * p.tiles_n;
+  const long long total = (long long)p.tiles_m * p.tiles_n * p.blocks;
   if (total <= 0) return FMM_OK;
+  if (total > 0x7fffffff) return FMM_ERR_SHAPE;
   const int sms = sm_count();
   if (sms <= 0) return FMM_ERR_CUDA;
   const int grid = (int)(total < sms ? total : sms);
   static unsigned long long smem_ok = 0;
   if (fmm_allow_dynamic_smem(int8_certified_kernel, L::kTotal, &smem_ok) != cudaSuccess) return FMM_ERR_CUDA;
-  int8_certified_kernel<<<grid, kCertThreads, L::kTotal, st>>>(ma, mb, a.C, p, a.status);
+  if (launch_dependent(int8_certified_kernel, dim3(grid), dim3(kInt8Threads), (size_t)L::kTotal, st, a.C, p, a.status) != cudaSuccess)
+    return FMM_ERR_CUDA;
   ++fmm_launch_counter();
   return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
-}
-
-int int8_certified_tile_columns() { return CertLayout::BN; }
-int int8_certified_decode_warps() { return CertLayout::kParts; }
-
-// The R products of a group go through TMEM in ceil(R / kPass) passes of equal length (a multiple of the products per
-// ring stage), the last one taking the remainder, when that fits a buffer; otherwise in passes of kPass.
-void int8_certified_passes(int R, int per, int* passes, int* pass_len) {
-  const int n = (R + CertLayout::kPass - 1) / CertLayout::kPass;
-  int len = R / n / per * per;
-  if (len == 0 || R - len * (n - 1) > CertLayout::kPass) len = CertLayout::kPass;
-  *passes = n;
-  *pass_len = len;
 }
 
 fmm_status launch_block_products(const BlockProductArgs& a, cudaStream_t st) {

@@ -375,67 +375,97 @@ cudaError_t launch_encode_split(const int8_t* codes, int64_t K, int gr, int gc, 
 }
 
 // ------------------------------------------------------------------------------------------
-// Block sums of int8 codes as int8 (certificate (i): |sum| <= 127), packed for the one-kernel certified realisation:
-// rows of 128 bytes that hold per = 128 / h products side by side, product r at byte (r % per) * h of row
-// (group, p) of slab r / per.  One thread forms, for one (group, row position) and four consecutive inner indices t,
-// the sums of every product (the same staging as encode_split_kernel).
+// Block sums of int8 codes as int8 (certificate (i): |sum| <= 127) in the order in which int8_certified_kernel's MMAs read
+// them: [product][group][32-index step][tile of 128 rows][2][128 rows][16 bytes], rows past the block's end zero.  One
+// thread forms, for one (group, row position) and 16 consecutive inner indices, the sums of every product, and turns the
+// scales of its rows to group-major.  Four codes are one 32-bit number with signed digits of base 256 (exact while the
+// digits of a result fit int8), so a list entry is one multiply-add for four sums; the pass is bound by its writes:
+// 138 MB for a 4096 x 11008 weight.  With a multiply-add per code and 4-byte stores, two launches, it took 203 us at
+// 2048 x 4096 x 11008.
 // ------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSplitThreads)
-encode_codes_kernel(const int8_t* __restrict__ codes, int64_t K, int gc, int64_t br, int G, int h,
-                    const CoefTable* __restrict__ d_tab, int8_t* __restrict__ out, int64_t nquad) {
+constexpr int kCodesThreads = 256;
+struct CodesJob {
+  const int8_t* codes; const float* scales; const CoefTable* tab; int8_t* out; float* scales_t;
+  int gr, gc, tiles, blocks; int64_t br;      // grid, 128-row tiles of a block, thread blocks of the job, rows of a block
+};
+__device__ __forceinline__ uint32_t digits_of(uint32_t bytes) { return (bytes ^ 0x80808080u) - 0x80808080u; }
+__device__ __forceinline__ uint32_t bytes_of(uint32_t digits) { return (digits + 0x80808080u) ^ 0x80808080u; }
+
+__global__ void __launch_bounds__(kCodesThreads)
+encode_codes_kernel(const CodesJob ja, const CodesJob jb, int64_t K, int G, int h) {
+  grid_launch_dependents();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int R = d_tab->R, ncell = d_tab->ncell;
-  const int total = d_tab->off[R];
-  int* off = reinterpret_cast<int*>(smem_raw);
-  int2* ent = reinterpret_cast<int2*>(smem_raw + ((size_t)(R + 1) * 4 + 15) / 16 * 16);
-  uint32_t* stage = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(ent) + (size_t)total * 8);
-  for (int i = threadIdx.x; i <= R; i += kSplitThreads) off[i] = d_tab->off[i];
-  for (int i = threadIdx.x; i < total; i += kSplitThreads)
-    ent[i] = make_int2(d_tab->cell[i], __float2int_rn(d_tab->coef[i]));
-  stage[ncell * kSplitThreads + threadIdx.x] = 0u;                    // the padding cell
-  const int64_t idx = (int64_t)blockIdx.x * kSplitThreads + threadIdx.x;
-  const bool live = idx < nquad;
-  const int qpr = h / 4;
-  const int64_t rowp = live ? idx / qpr : 0;                          // (group, p)
-  const int t = live ? (int)(idx - rowp * qpr) * 4 : 0;
-  const int64_t g = rowp / br, p = rowp - g * br;
-  for (int c = 0; c < ncell; ++c) {
-    const int gi = c / gc, gj = c - gi * gc;
-    stage[c * kSplitThreads + threadIdx.x] =
-        live ? *reinterpret_cast<const uint32_t*>(codes + ((int64_t)gi * br + p) * K + g * kGroup + gj * h + t) : 0u;
-  }
-  __syncthreads();
-  if (!live) return;
-  const int per = kGroup / h;
-  const int64_t slab = (int64_t)G * br * kGroup;                      // bytes of one slab of `per` products
-  for (int r = 0; r < R; ++r) {
-    int s0 = 0, s1 = 0, s2 = 0, s3 = 0;
-    for (int e = off[r]; e < off[r + 1]; ++e) {
-      const int2 en = ent[e];
-      const uint32_t wv = stage[en.x * kSplitThreads + threadIdx.x];
-      s0 += en.y * (int)(int8_t)(wv & 0xffu);
-      s1 += en.y * (int)(int8_t)((wv >> 8) & 0xffu);
-      s2 += en.y * (int)(int8_t)((wv >> 16) & 0xffu);
-      s3 += en.y * (int)(int8_t)(wv >> 24);
+  const bool second = (int)blockIdx.x >= ja.blocks;
+  const CodesJob& j = second ? jb : ja;
+  const int bid = (int)blockIdx.x - (second ? ja.blocks : 0);
+  const int R = j.tab->R, ncell = j.tab->ncell;
+  const int total = j.tab->off[R];
+  uint4* stage = reinterpret_cast<uint4*>(smem_raw);                 // [cell][thread], the padding cell last
+  int2* ent = reinterpret_cast<int2*>(stage + (ncell + 1) * kCodesThreads);
+  int* off = reinterpret_cast<int*>(ent + total);
+  const int tid = threadIdx.x;
+  for (int i = tid; i <= R; i += kCodesThreads) off[i] = j.tab->off[i];
+  for (int i = tid; i < total; i += kCodesThreads) ent[i] = make_int2(j.tab->cell[i] * kCodesThreads, __float2int_rn(j.tab->coef[i]));
+  const int chunks = h / 16, rows_here = kCodesThreads / chunks, per_group = j.tiles * 128 / rows_here;
+  const int g = bid / per_group, p = (bid - g * per_group) * rows_here + tid / chunks, c = tid % chunks;
+  const bool live = p < j.br;
+  for (int x0 = 0; x0 < ncell; x0 += 4) {          // four cells' loads in flight
+    uint2 lo[4], hi[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      lo[u] = hi[u] = make_uint2(0u, 0u);
+      if (live && x0 + u < ncell) {
+        const int gi = (x0 + u) / j.gc, gj = x0 + u - gi * j.gc;
+        const uint2* src = reinterpret_cast<const uint2*>(j.codes + ((int64_t)gi * j.br + p) * K + (int64_t)g * kGroup + gj * h + c * 16);
+        lo[u] = __ldg(src); hi[u] = __ldg(src + 1);     // the codes are 8-byte aligned
+      }
     }
-    const uint32_t packed = ((uint32_t)s0 & 0xffu) | (((uint32_t)s1 & 0xffu) << 8) | (((uint32_t)s2 & 0xffu) << 16) |
-                            (((uint32_t)s3 & 0xffu) << 24);
-    *reinterpret_cast<uint32_t*>(out + (r / per) * slab + rowp * kGroup + (r % per) * h + t) = packed;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (x0 + u < ncell)
+        stage[(x0 + u) * kCodesThreads + tid] = make_uint4(digits_of(lo[u].x), digits_of(lo[u].y), digits_of(hi[u].x), digits_of(hi[u].y));
+  }
+  stage[ncell * kCodesThreads + tid] = make_uint4(0u, 0u, 0u, 0u);
+  if (live && c == 0 && blockIdx.y == 0)
+    for (int gi = 0; gi < j.gr; ++gi)
+      j.scales_t[((int64_t)g * j.gr + gi) * j.br + p] = j.scales[((int64_t)gi * j.br + p) * G + g];
+  __syncthreads();
+  const int64_t step = (int64_t)j.tiles * 4096;                       // bytes of one 32-index step of a (product, group)
+  int8_t* dst = j.out + ((int64_t)g * (h / 32) + (c >> 1)) * step + (int64_t)(p >> 7) * 4096 + (c & 1) * 2048 + (p & 127) * 16;
+  const int64_t rstride = (int64_t)G * (h / 32) * step;
+  const int r0 = R * (int)blockIdx.y / (int)gridDim.y, r1 = R * ((int)blockIdx.y + 1) / (int)gridDim.y;
+  dst += r0 * rstride;
+  for (int r = r0; r < r1; ++r, dst += rstride) {
+    uint4 s = make_uint4(0u, 0u, 0u, 0u);
+    for (int e = off[r]; e < off[r + 1]; e += 2) {      // lists are padded to whole pairs
+      const int4 en = *reinterpret_cast<const int4*>(&ent[e]);
+      const uint4 v = stage[en.x + tid], u = stage[en.z + tid];
+      const uint32_t w = (uint32_t)en.y, x = (uint32_t)en.w;
+      s.x += w * v.x; s.y += w * v.y; s.z += w * v.z; s.w += w * v.w;
+      s.x += x * u.x; s.y += x * u.y; s.z += x * u.z; s.w += x * u.w;
+    }
+    *reinterpret_cast<uint4*>(dst) = make_uint4(bytes_of(s.x), bytes_of(s.y), bytes_of(s.z), bytes_of(s.w));
   }
 }
 
-cudaError_t launch_encode_codes(const int8_t* codes, int64_t K, int gr, int gc, int64_t br, int G, int h,
-                                const CoefTable* d_tab, const CoefTable* h_tab, int8_t* out, cudaStream_t st) {
-  const int64_t nquad = (int64_t)G * br * (h / 4);
-  const size_t smem = ((size_t)(h_tab->R + 1) * 4 + 15) / 16 * 16 + (size_t)h_tab->off[h_tab->R] * 8 +
-                      (size_t)(gr * gc + 1) * kSplitThreads * 4;
-  if (smem > 96 * 1024) return cudaErrorInvalidValue;
+cudaError_t launch_encode_codes(CodesJob a, CodesJob b, const CoefTable& h_a, const CoefTable& h_b, int64_t K, int G, int h, cudaStream_t st) {
+  size_t smem = 0;
+  for (const CoefTable* t : {&h_a, &h_b})
+    smem = std::max(smem, (size_t)(t->ncell + 1) * kCodesThreads * 16 + (size_t)t->off[t->R] * 8 + (size_t)(t->R + 1) * 4);
+  const int rows = kCodesThreads / (h / 16);
+  int64_t grid = 0;
+  for (CodesJob* j : {&a, &b}) {
+    const int64_t n = (int64_t)G * (j->tiles * 128 / rows);
+    if (n > 0x3fffffff) return cudaErrorInvalidValue;
+    j->blocks = (int)n;
+    grid += n;
+  }
   static unsigned long long smem_ok = 0;
   cudaError_t e = fmm_allow_dynamic_smem(encode_codes_kernel, 96 * 1024, &smem_ok);
   if (e != cudaSuccess) return e;
-  const int64_t grid = (nquad + kSplitThreads - 1) / kSplitThreads;
-  if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  encode_codes_kernel<<<(unsigned)grid, kSplitThreads, smem, st>>>(codes, K, gc, br, G, h, d_tab, out, nquad);
+  // few blocks: the products are shared out too (each part reads the codes again)
+  const unsigned parts = grid < 148 ? 4 : grid < 296 ? 2 : 1;
+  encode_codes_kernel<<<dim3((unsigned)grid, parts), kCodesThreads, smem, st>>>(a, b, K, G, h);
   ++fmm_launch_counter();
   return cudaGetLastError();
 }
@@ -511,8 +541,8 @@ struct Int8Layout {
 
 // Workspace of the one-kernel certified realisation
 struct CertWs {
-  size_t status, tabA, tabB, entries, pass_off, owned, dAt, dBt, ahat, bhat, total;
-  size_t max_entries;
+  size_t head, dAt, dBt, ahat, bhat, total;     // head: status block and the three kernel tables, as packed on the host
+  int tiles_m, tiles_n;                         // 128-row tiles of a block of A and of B
 };
 
 // the classical algorithm <1,1,1;1> as a scheme
@@ -536,20 +566,15 @@ fmm_status int8_shape_ok(const fmm_scheme& s, int64_t M, int64_t K, int64_t N) {
 CertWs cert_layout(const fmm_scheme& s, int64_t M, int64_t K, int64_t N) {
   CertWs L{};
   const int G = (int)(K / kGroup), h = kGroup / s.k, per = kGroup / h;
-  const int64_t bm = M / s.m, bn = N / s.n;
-  const int slabs = (s.R + per - 1) / per;
-  L.max_entries = (size_t)s.R * s.m * s.n;
+  L.tiles_m = (int)((M / s.m + 127) / 128);
+  L.tiles_n = (int)((N / s.n + 127) / 128);
+  const size_t sums = (size_t)((s.R + per - 1) / per) * per * G * h * 128;   // bytes of all block sums per tile of 128 rows
   size_t o = 0;
-  L.status = o; o += align_up(sizeof(DeviceStatus));
-  L.tabA = o; o += align_up(sizeof(CoefTable));
-  L.tabB = o; o += align_up(sizeof(CoefTable));
-  L.entries = o; o += align_up(L.max_entries * 8);
-  L.pass_off = o; o += align_up((size_t)(FMM_MAX_R + 1) * FMM_MAX_GRID * FMM_MAX_GRID * 4);
-  L.owned = o; o += align_up(FMM_MAX_GRID * FMM_MAX_GRID * 4);
+  L.head = o; o += align_up(kPackedStatusBytes + 3 * fmm_packed_table_stride());
   L.dAt = o; o += align_up((size_t)M * G * 4);
   L.dBt = o; o += align_up((size_t)N * G * 4);
-  L.ahat = o; o += align_up((size_t)slabs * G * bm * kGroup + 128 * kGroup);   // + one tile of rows: boxes may read past the end
-  L.bhat = o; o += align_up((size_t)slabs * G * bn * kGroup + 128 * kGroup);
+  L.ahat = o; o += align_up(sums * L.tiles_m);
+  L.bhat = o; o += align_up(sums * L.tiles_n);
   L.total = o;
   return L;
 }
@@ -720,79 +745,29 @@ size_t int8_gemm_materialised_workspace(const fmm_scheme* s, int64_t M, int64_t 
   return int8_layout(sc, M, K, N).total;
 }
 
-// The certified realisation in one kernel: block sums of the codes as int8 (two launches), scales transposed to
-// group-major (two launches), then int8_certified_kernel.
+// The certified realisation: one copy of the tables, one launch for the block sums of both operands (and the scales turned
+// to group-major), one for everything else.
 static fmm_status int8_certified_one_kernel(const fmm_scheme& sc, const int8_t* d_cA, const float* d_dA, const int8_t* d_cB,
                                             const float* d_dB, int64_t M, int64_t K, int64_t N, int output, void* d_C,
                                             int64_t ldc, void* d_ws, size_t ws_bytes, cudaStream_t st) {
   const CertWs L = cert_layout(sc, M, K, N);
   if (!d_ws || (reinterpret_cast<uintptr_t>(d_ws) & 255u) || ws_bytes < L.total) return FMM_ERR_WORKSPACE;
-  if ((reinterpret_cast<uintptr_t>(d_cA) % 4) || (reinterpret_cast<uintptr_t>(d_cB) % 4)) return FMM_ERR_SHAPE;
-  const int64_t bm = M / sc.m, bn = N / sc.n;
   const int h = kGroup / sc.k, G = (int)(K / kGroup);
-  FMM_CUDA(cudaMemsetAsync(at<char>(d_ws, L.status), 0, sizeof(DeviceStatus), st));
-  std::unique_ptr<CoefTable> hA(new CoefTable), hB(new CoefTable);
-  std::memset(hA.get(), 0, sizeof(CoefTable)); std::memset(hB.get(), 0, sizeof(CoefTable));
-  fmm_build_tables(sc, hA.get(), hB.get(), nullptr);
-  FMM_CUDA(cudaMemcpyAsync(at<char>(d_ws, L.tabA), hA.get(), sizeof(CoefTable), cudaMemcpyHostToDevice, st));
-  FMM_CUDA(cudaMemcpyAsync(at<char>(d_ws, L.tabB), hB.get(), sizeof(CoefTable), cudaMemcpyHostToDevice, st));
-  // Decode lists.  Every block of C is owned by one of four decode warps (per TMEM lane quarter); the blocks are dealt
-  // out longest list first to the warp with the least work so far that still has a free slot.  The lists are then laid
-  // out by (warp, pass of products, owned block, ascending r); an entry is (TMEM column of the product inside its
-  // pass, integer w).
-  const int blocks = sc.m * sc.n;
-  int passes = 0, pass = 0;
-  int8_certified_passes(sc.R, kGroup / h, &passes, &pass);
-  const int kParts = int8_certified_decode_warps(), kOwn = FMM_MAX_GRID * FMM_MAX_GRID / kParts, kBN = int8_certified_tile_columns();
-  std::vector<int> nnz(blocks, 0), order(blocks), owned(kParts * kOwn, -1), load(kParts, 0), used(kParts, 0);
-  for (int d = 0; d < blocks; ++d)
-    for (int r = 0; r < sc.R; ++r) nnz[d] += sc.W[(size_t)r * blocks + d] != 0.0;
-  for (int d = 0; d < blocks; ++d) order[d] = d;
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return nnz[x] > nnz[y]; });
-  for (int d : order) {
-    int best = -1;
-    for (int q = 0; q < kParts; ++q)
-      if (used[q] < kOwn && (best < 0 || load[q] < load[best])) best = q;
-    owned[best * kOwn + used[best]++] = d;
-    load[best] += nnz[d];
-  }
-  std::vector<int2> ent;
-  std::vector<int> poff;
-  for (int q = 0; q < kParts; ++q)
-    for (int ps = 0; ps < passes; ++ps)
-      for (int b = 0; b < kOwn; ++b) {
-        poff.push_back((int)ent.size());
-        const int d = owned[q * kOwn + b];
-        if (d < 0) continue;
-        for (int r = ps * pass; r < (ps == passes - 1 ? sc.R : (ps + 1) * pass); ++r) {
-          const double w = sc.W[(size_t)r * blocks + d];
-          if (w != 0.0) ent.push_back(make_int2((r - ps * pass) * kBN, (int)std::lrint(w)));
-        }
-      }
-  poff.push_back((int)ent.size());
-  if (ent.size() > L.max_entries) return FMM_ERR_LIMIT;
-  if (!ent.empty())
-    FMM_CUDA(cudaMemcpyAsync(at<char>(d_ws, L.entries), ent.data(), ent.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
-  FMM_CUDA(cudaMemcpyAsync(at<char>(d_ws, L.pass_off), poff.data(), poff.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-  FMM_CUDA(cudaMemcpyAsync(at<char>(d_ws, L.owned), owned.data(), owned.size() * sizeof(int), cudaMemcpyHostToDevice, st));
+  const std::vector<unsigned char>& packed = fmm_packed_tables(sc);
+  const size_t tab = L.head + kPackedStatusBytes, stride = fmm_packed_table_stride();
+  FMM_CUDA(cudaMemcpyAsync(at<char>(d_ws, L.head), packed.data(), packed.size(), cudaMemcpyHostToDevice, st));
+  const CodesJob ja{d_cA, d_dA, at<CoefTable>(d_ws, tab), at<int8_t>(d_ws, L.ahat), at<float>(d_ws, L.dAt), sc.m, sc.k, L.tiles_m, 0, M / sc.m};
+  const CodesJob jb{d_cB, d_dB, at<CoefTable>(d_ws, tab + stride), at<int8_t>(d_ws, L.bhat), at<float>(d_ws, L.dBt), sc.n, sc.k, L.tiles_n, 0, N / sc.n};
   {
     ProfScope ps(0, st);
-    FMM_CUDA(launch_encode_codes(d_cA, K, sc.m, sc.k, bm, G, h, at<CoefTable>(d_ws, L.tabA), hA.get(), at<int8_t>(d_ws, L.ahat), st));
-    FMM_CUDA(launch_encode_codes(d_cB, K, sc.n, sc.k, bn, G, h, at<CoefTable>(d_ws, L.tabB), hB.get(), at<int8_t>(d_ws, L.bhat), st));
-    transpose_scales_kernel<<<stream_blocks(M * G, 256), 256, 0, st>>>(d_dA, M, G, at<float>(d_ws, L.dAt));
-    ++fmm_launch_counter();
-    transpose_scales_kernel<<<stream_blocks(N * G, 256), 256, 0, st>>>(d_dB, N, G, at<float>(d_ws, L.dBt));
-    ++fmm_launch_counter();
-    FMM_CUDA(cudaGetLastError());
+    FMM_CUDA(launch_encode_codes(ja, jb, *fmm_packed_table(sc, 0), *fmm_packed_table(sc, 1), K, G, h, st));
   }
   Int8CertArgs a{};
-  a.Ahat = at<int8_t>(d_ws, L.ahat); a.Bhat = at<int8_t>(d_ws, L.bhat);
-  a.m = sc.m; a.n = sc.n; a.R = sc.R; a.h = h; a.bm = bm; a.bn = bn; a.G = G; a.M = M; a.N = N;
-  a.dAt = at<float>(d_ws, L.dAt); a.dBt = at<float>(d_ws, L.dBt);
-  a.d_entries = at<int2>(d_ws, L.entries); a.d_pass_off = at<int>(d_ws, L.pass_off); a.d_owned = at<int>(d_ws, L.owned); a.n_entries = (int)ent.size();
-  a.output = output; a.C = d_C; a.ldc = ldc; a.status = at<DeviceStatus>(d_ws, L.status);
+  a.Ahat = ja.out; a.Bhat = jb.out;
+  a.m = sc.m; a.n = sc.n; a.R = sc.R; a.h = h; a.bm = ja.br; a.bn = jb.br; a.G = G; a.M = M; a.N = N;
+  a.dAt = ja.scales_t; a.dBt = jb.scales_t; a.d_tab_w = at<CoefTable>(d_ws, tab + 2 * stride);
+  a.output = output; a.C = d_C; a.ldc = ldc; a.status = at<DeviceStatus>(d_ws, L.head);
   ProfScope ps(2, st);
-  // the host tables were copied from pageable memory: those copies are complete when cudaMemcpyAsync returns
   return launch_int8_certified(a, st);
 }
 
