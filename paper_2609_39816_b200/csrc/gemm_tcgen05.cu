@@ -1044,11 +1044,10 @@ struct RescaleTile { int row0, rows, col0, cols; bool plus, minus; };   // first
 
 // kMinus: a buffer is two accumulators side by side; the group's integer is the first minus the second, of those that
 // the tile says were written
-template <int kAcc, bool kMinus, typename TileOf>
+template <int kAcc, int kMaxGroupsStaged, bool kMinus, typename TileOf>
 __device__ __forceinline__ void int8_rescale_role(const RescaleCtx& c, const int warp, const int lane, const int total_tiles,
                                                   const TileOf tile_of) {
   constexpr int BN = 128, PN = 32, kBufCols = kMinus ? 2 * BN : BN;
-  constexpr int kMaxGroupsStaged = Int8Layout::kMaxGroupsStaged;
   const int quad = warp & 3;             // TMEM lanes [32*quad, 32*quad+32) are the ones this warp may read
   const int part = (warp - 2) >> 2;      // which 32 of the tile's 128 columns
   int acc = 0;
@@ -1100,20 +1099,23 @@ __device__ __forceinline__ void int8_rescale_role(const RescaleCtx& c, const int
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = 0u;
       }
-      if constexpr (kMinus) {
-        if (t.minus) {       // sixteen columns at a time: 96 registers a thread
-          uint32_t m[16];
+      // exact int -> float for |P| < 2^22 (a group product is at most 128 * 127^2): add the integer to the bits of
+      // 1.5 * 2^23, subtract that constant (exact)
+      if (kMinus && t.minus) {       // sixteen columns at a time: 96 registers a thread
+        uint32_t m[16];
 #pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            tc_ld16(taddr + BN + 16 * half, m);
-            tc_wait_ld16(m);
-            if (half == 0) tc_wait_ld32(v);
+        for (int half = 0; half < 2; ++half) {
+          tc_ld16(taddr + BN + 16 * half, m);
+          tc_wait_ld16(m);
+          if (half == 0) tc_wait_ld32(v);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) v[16 * half + j] -= m[j];
-          }
+          for (int j = 0; j < 16; ++j) v[16 * half + j] += 0x4B400000u - m[j];
         }
+      } else {
+        tc_wait_ld32(v);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] += 0x4B400000u;
       }
-      tc_wait_ld32(v);
       // the accumulator is in registers: hand the buffer back before the arithmetic
       tc_fence_before();
       __syncwarp();
@@ -1121,13 +1123,7 @@ __device__ __forceinline__ void int8_rescale_role(const RescaleCtx& c, const int
       if (++acc == kAcc) { acc = 0; acc_phase ^= 1u; }
       const float2 da2 = make_float2(da, da);
       const float2 neg_magic = make_float2(-12582912.0f, -12582912.0f);
-#pragma unroll
-      for (int j = 0; j < PN; ++j) {
-        // exact int -> float for |P| < 2^22 (a group product is at most 128 * 127^2): add the integer to the bits
-        // of 1.5 * 2^23, subtract that constant (exact).  Then two separately rounded multiplications and a
-        // separately rounded addition, as the specification orders them.
-        v[j] += 0x4B400000u;
-      }
+      // two separately rounded multiplications and a separately rounded addition, as the specification orders them
 #pragma unroll
       for (int q4 = 0; q4 < PN / 4; ++q4) {
         float2 p0 = make_float2(__uint_as_float(v[q4 * 4 + 0]), __uint_as_float(v[q4 * 4 + 1]));
@@ -1272,7 +1268,7 @@ int8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     const RescaleCtx rc{bar_base + 8u * (2 * L::kStages), bar_base + 8u * (2 * L::kStages + kAcc), sfull_bar, sempty_bar,
                         tmem_base, scale_sm, abort_flag, status, p.wait_limit_ns, out, p.dAt, p.dBt, p.M, p.N, p.G,
                         p.ldc, p.out_bf16, p.wide};
-    int8_rescale_role<kAcc, false>(rc, warp, lane, total_tiles, [&](int tile) {
+    int8_rescale_role<kAcc, L::kMaxGroupsStaged, false>(rc, warp, lane, total_tiles, [&](int tile) {
       const int tm = tile / p.tiles_n, tn = tile - tm * p.tiles_n;
       return RescaleTile{tm * BM, min(BM, p.M - tm * BM), tn * BN, min(BN, p.N - tn * BN), true, false};
     });

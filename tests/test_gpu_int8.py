@@ -287,3 +287,18 @@ def test_fine_group_control_on_the_device():
     want = oracle.int8_finegroup_control(oracle.strassen(), c3a, d3a, c3b, d3b, call=128, od="bf16")
     assert np.array_equal(C3.double().cpu().numpy(), want)
     assert lib.int8_finegroup_control_workspace(s2, 30, 128, 32, 128) == 0      # rows do not split into four blocks
+
+
+@pytest.mark.parametrize("M,K,N", [(8, 7424, 32), (516, 640, 1056), (1024, 7296, 512), (4, 128, 4128)])
+def test_certified_at_the_edges_of_its_tiles_and_rings(M, K, N):
+    """The certified realisation against the classical kernel, both bit-exact by the specification: blocks one row past a
+    tile of 128 and 8 columns past two of them, 57 and 58 groups (column scales staged for 56), one group, and <1,1,1;2>
+    with weights of 3 and -2 (repeated MMAs into both accumulators, four steps of K per product)."""
+    lib = fmm()
+    At, A, Bt, B = _inputs(71, M, K, N)
+    one = oracle.Scheme(np.ones((2, 1, 1)), np.ones((2, 1, 1)), np.array([3.0, -2.0]).reshape(2, 1, 1))
+    for o, b in ((S2, 31), (S1, 63), (one, 31)):
+        cA, dA = _quantize(lib, At, b)
+        cB, dB = _quantize(lib, Bt, b)
+        assert np.array_equal(_gemm(lib, _lib_scheme(lib, o), b, cA, dA, cB, dB, torch.float32),
+                              _gemm(lib, None, b, cA, dA, cB, dB, torch.float32))
