@@ -176,6 +176,12 @@ fmm_status encode_operand(const fmm_gemm_desc* d, const void* X, int64_t ldx, in
                           float* scale, bool b_side, cudaStream_t st) {
   const int mode = d->scale_mode;   // 0 none, 1 per encoded tensor, 2 per row of it, 3 model schedule (128-groups)
   const EncodeOperand o{X, ldx, gr, gc, br, bc, d_tab, h_tab, hat, hat_stride, amax, scale, b_side ? 128 : 1, b_side ? 1 : 0};
+  cudaError_t e = cudaSuccess;
+  if (fmm_encode_pattern(d->storage, d->product, b_side ? nullptr : &o, b_side ? &o : nullptr, mode, amax,
+                         scale_words(mode, h_tab->R, br, bc, b_side) * 4, st, &e)) {
+    FMM_CUDA(e);
+    return FMM_OK;
+  }
   if (mode != 0) {
     FMM_CUDA(cudaMemsetAsync(amax, 0, scale_words(mode, h_tab->R, br, bc, b_side) * 4, st));
     FMM_CUDA(launch_encode_pair(d->storage, d->product, o, nullptr, true, mode, st));
@@ -232,6 +238,11 @@ fmm_status stage_encode_pair(const SchemeRun& r, const void* A, const void* Bk, 
                          at<unsigned>(r.ws, r.L.amaxB), r.sB(), 128, 1};
   ProfScope ps(0, st);
   const int mode = d->scale_mode;
+  cudaError_t e = cudaSuccess;
+  if (fmm_encode_pattern(d->storage, d->product, &oa, &ob, mode, at<char>(r.ws, r.L.amaxA), r.L.sA - r.L.amaxA, st, &e)) {
+    FMM_CUDA(e);
+    return FMM_OK;
+  }
   if (mode != 0) {
     // amaxA and amaxB are neighbours in the workspace: one memset clears both
     FMM_CUDA(cudaMemsetAsync(at<char>(r.ws, r.L.amaxA), 0, r.L.sA - r.L.amaxA, st));

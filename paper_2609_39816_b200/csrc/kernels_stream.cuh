@@ -86,6 +86,12 @@ struct EncodeOperand {
 cudaError_t launch_encode_pair(int storage, int product, const EncodeOperand& a, const EncodeOperand* b, bool amax_only,
                                int use_scale, cudaStream_t st);
 
+// The whole encode of one or both operands (a or b may be null; amax passes included) for tables of the two-level Strassen
+// pattern (encode_pattern.cu).  False, with nothing enqueued, where it has no kernel for the tables, types or mode; else
+// *err is the launches' result.  clear: the amax words of the operands (zeroed first where they are accumulated).
+bool fmm_encode_pattern(int storage, int product, const EncodeOperand* a, const EncodeOperand* b, int mode, void* clear,
+                        size_t clear_bytes, cudaStream_t st, cudaError_t* err);
+
 // One operand of an encode launch.  A launch carries up to two (A and B of one product): blocks [0, a.blocks) work
 // on the first, the rest on the second, so both operands are encoded side by side without a second stream.
 struct EncodeJob {
