@@ -337,7 +337,14 @@ fmm_status stage_decode(const SchemeRun& r, void* C, const float* cstar32, doubl
   ProfScope ps(3, st);
   int np = 0;
   const bool per_product = r.d->scale_mode == 1;   // mode 2: the products already carry their scales
-  FMM_CUDA(launch_decode(r.d->output, at<char>(r.ws, r.L.prod), (r.d->flags & FMM_FLAG_PRODUCTS_BF16) ? FMM_BF16 : FMM_F32,
+  cudaError_t e = cudaSuccess;
+  if (gauges == 1 &&
+      fmm_decode_pattern(r.d->output, at<char>(r.ws, r.L.prod), (r.d->flags & FMM_FLAG_PRODUCTS_BF16) ? FMM_BF16 : FMM_F32, r.L.sProd,
+                         r.hW, per_product ? r.sA() : nullptr, per_product ? r.sB() : nullptr, r.d->M / s->m, r.d->N / s->n, C,
+                         r.d->ldc, cstar32, at<double>(r.ws, r.L.partials), &np, 148 * 4, st, &e))
+    FMM_CUDA(e);
+  else
+    FMM_CUDA(launch_decode(r.d->output, at<char>(r.ws, r.L.prod), (r.d->flags & FMM_FLAG_PRODUCTS_BF16) ? FMM_BF16 : FMM_F32,
                          r.L.sProd, r.dW, r.hW, s->R, per_product ? r.sA() : nullptr,
                          per_product ? r.sB() : nullptr, s->m, s->n,
                          r.d->M / s->m, r.d->N / s->n, C, r.d->ldc, cstar32, at<double>(r.ws, r.L.partials), &np, st, gauges));

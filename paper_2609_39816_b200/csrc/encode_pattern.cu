@@ -17,21 +17,13 @@
 #include <utility>
 
 #include "kernels_stream.cuh"
+#include "strassen_pattern.cuh"
 #include "stream_bodies.cuh"
 
 namespace {
 
-constexpr int kProducts = 49, kCells = 16;
 constexpr int kPatThreads = 128;
 
-// nonzero places of the one-level algorithm's coefficients, as (row, column) bits 2 * row + column of U (A) and V (B)
-constexpr unsigned char kU[7] = {0b1001, 0b1100, 0b0001, 0b1000, 0b0011, 0b0101, 0b1010};
-constexpr unsigned char kV[7] = {0b1001, 0b0001, 0b1010, 0b0101, 0b1000, 0b0011, 0b1100};
-
-struct Pattern {
-  int off[kProducts + 1] = {};
-  unsigned char cell[kProducts * kCells] = {};
-};
 // lists in the order of fmm_build_tables: ascending (row, column) of the coefficient matrix; B is stored transposed
 constexpr Pattern make_pattern(bool b_side, bool dense) {
   Pattern p;
@@ -47,7 +39,6 @@ constexpr Pattern make_pattern(bool b_side, bool dense) {
   return p;
 }
 template <bool kB, bool kDense> struct Pat { static constexpr Pattern value = make_pattern(kB, kDense); };
-constexpr int kMaxEntries = 336;
 static_assert(Pat<false, true>::value.off[kProducts] == kMaxEntries && Pat<true, true>::value.off[kProducts] == kMaxEntries, "pattern");
 
 struct PatCoefs { float a[kMaxEntries], b[kMaxEntries]; };
@@ -58,6 +49,9 @@ struct PatJob {
 };
 
 enum PatPass { kPlain, kAmax, kScaled, kGroupAmax, kGroupScaled };
+// blocks per SM that the register allocation aims at: measured 97 / 83 / 79 us (4 / 5 / 6) for kGroupAmax, 198 / 183 / 184 for
+// kGroupScaled, within 3 % elsewhere
+constexpr int pat_blocks_per_sm(int pass) { return pass == kGroupAmax ? 6 : pass == kPlain ? 4 : 5; }
 
 constexpr int E = 4, NP = 2;          // values of a thread: 16 cells x 4 fp32 registers
 __device__ __forceinline__ float4 load_values(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
@@ -66,9 +60,6 @@ __device__ __forceinline__ float4 load_values(const __nv_bfloat16* p) {
   return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xFFFF0000u), __uint_as_float(r.y << 16),
                      __uint_as_float(r.y & 0xFFFF0000u));
 }
-
-template <int... i, typename F>
-__device__ __forceinline__ void for_each(std::integer_sequence<int, i...>, F&& f) { (f(std::integral_constant<int, i>{}), ...); }
 
 __device__ __forceinline__ float max3(float a, float b, float c) {        // drops NaN, as fmaxf
   float d;
@@ -80,8 +71,8 @@ __device__ __forceinline__ float max3(float a, float b, float c) {        // dro
 // and x r (1 - 2^-21) enclose fl(x / scale), whose distance from x r is below 2^-22 of it, and rounding to e4m3 is
 // monotone: where the two give one code it is that of x / scale.  Otherwise (a few in a million) the division is made.
 template <typename DstT>
-__device__ __noinline__ void store_exactly(DstT* dst, float2 a0, float2 a1, const unsigned* amax_bits) {
-  const float amax = __uint_as_float(*amax_bits), sc = amax > 0.0f ? __fdiv_rn(amax, 448.0f) : 1.0f;
+__device__ __noinline__ void store_exactly(DstT* dst, float2 a0, float2 a1, const unsigned* amax_bits, int64_t at) {
+  const float amax = __uint_as_float(amax_bits[at]), sc = amax > 0.0f ? __fdiv_rn(amax, 448.0f) : 1.0f;
   const float2 q[2] = {make_float2(__fdiv_rn(a0.x, sc), __fdiv_rn(a0.y, sc)), make_float2(__fdiv_rn(a1.x, sc), __fdiv_rn(a1.y, sc))};
   store_vec<2>(dst, q, false);
 }
@@ -89,6 +80,29 @@ __device__ __forceinline__ unsigned codes_of(const float2 (&a)[2], float f) {
   const float2 ff = make_float2(f, f);
   return (unsigned)__nv_cvt_float2_to_fp8x2(__fmul2_rn(a[0], ff), __NV_SATFINITE, __NV_E4M3) |
          ((unsigned)__nv_cvt_float2_to_fp8x2(__fmul2_rn(a[1], ff), __NV_SATFINITE, __NV_E4M3) << 16);
+}
+
+// stores with an L2 eviction priority chosen at run time: one instruction where a choice of two stores is a branch
+__device__ __forceinline__ uint64_t evict_first_policy() {
+  uint64_t p;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+__device__ __forceinline__ uint64_t evict_normal_policy() {
+  uint64_t p;
+  asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
+__device__ __forceinline__ void store_hint(__nv_fp8_storage_t* p, unsigned v, uint64_t policy) {
+  asm volatile("st.global.L2::cache_hint.b32 [%0], %1, %2;" ::"l"(p), "r"(v), "l"(policy) : "memory");
+}
+__device__ __forceinline__ void store_hint(__nv_fp8_storage_t* p, const float2 (&a)[2], uint64_t policy) {
+  store_hint(p, codes_of(a, 1.0f), policy);
+}
+__device__ __forceinline__ void store_hint(__nv_bfloat16* p, const float2 (&a)[2], uint64_t policy) {
+  const __nv_bfloat162 lo = __floats2bfloat162_rn(a[0].x, a[0].y), hi = __floats2bfloat162_rn(a[1].x, a[1].y);
+  asm volatile("st.global.L2::cache_hint.v2.b32 [%0], {%1, %2}, %3;"
+               ::"l"(p), "r"(*reinterpret_cast<const uint32_t*>(&lo)), "r"(*reinterpret_cast<const uint32_t*>(&hi)), "l"(policy) : "memory");
 }
 
 struct PatSmem {
@@ -143,18 +157,26 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
       x[c] = live ? load_values(src + (int64_t)(c / 4) * j.br * j.ldx + (int64_t)(c % 4) * j.bc) : make_float4(0.f, 0.f, 0.f, 0.f);
     DstT* dst = static_cast<DstT*>(j.out) + (int64_t)p * j.bc + t;
     const int64_t row_groups = kB ? (j.br + 127) >> 7 : j.br;       // scale blocks of 128 x 128 (B) or 1 x 128 (A)
-    // scales on groups: lane l keeps the largest magnitude, or the scale's reciprocal, of products l and l + 32
+    const uint64_t policy = j.evict_first ? evict_first_policy() : evict_normal_policy();
+    (void)policy;
+    // scales on groups: lane l keeps the largest magnitude, or the two factors about the scale's reciprocal, of products l
+    // and l + 32
     constexpr int kKeep = kGroups ? (kProducts + kLanes - 1) / kLanes : 1;
     const int64_t sidx = (kB ? p >> 7 : p) * (int64_t)gk + (t >> 7), sstep = row_groups * gk;
     const int gl = lane & (kLanes - 1);
     unsigned keep[kKeep] = {};
+    float lower[kKeep] = {};
+    (void)lower;
     if constexpr (kPass == kGroupScaled) {
 #pragma unroll
       for (int u = 0; u < kKeep; ++u)
         if (p_live && u * kLanes + gl < kProducts) {
           const float amax = __uint_as_float(j.amax_bits[sidx + (u * kLanes + gl) * sstep]);
           const float sc = amax > 0.0f ? __fdiv_rn(amax, 448.0f) : 1.0f;
-          keep[u] = __float_as_uint(__frcp_rn(sc));
+          const float f = __frcp_rn(sc);
+          keep[u] = __float_as_uint(f * (1.0f + 4.76837158203125e-7f));
+          // (an infinite reciprocal would make NaN of zeros on both sides: its lower factor is 0 instead)
+          lower[u] = f <= 3.4e38f ? f * (1.0f - 4.76837158203125e-7f) : 0.0f;
           if (!kB || (p & 127) == 0) j.scale_out[sidx + (u * kLanes + gl) * sstep] = sc;
         }
     }
@@ -199,18 +221,14 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
           for (int i = 0; i < NP; ++i) acc[i] = __fmul2_rn(__fmul2_rn(acc[i], make_float2(f.x, f.x)), make_float2(f.y, f.y));
         }
         if constexpr (kPass == kGroupScaled) {
-          const float f = __uint_as_float(__shfl_sync(0xffffffffu, keep[r / kLanes], r % kLanes));
-          const unsigned code = codes_of(acc, f * (1.0f + 4.76837158203125e-7f));
-          // (an infinite reciprocal would make NaN of zeros on both sides: its lower factor is 0 instead)
-          const unsigned other = codes_of(acc, f <= 3.4e38f ? f * (1.0f - 4.76837158203125e-7f) : 0.0f);
-          DstT* to = dst + r * j.rstride;
+          const unsigned code = codes_of(acc, __uint_as_float(__shfl_sync(0xffffffffu, keep[r / kLanes], r % kLanes)));
+          const unsigned other = codes_of(acc, __shfl_sync(0xffffffffu, lower[r / kLanes], r % kLanes));
           if (live) {
-            if (code != other) store_exactly(to, acc[0], acc[1], &j.amax_bits[sidx + r * sstep]);
-            else if (j.evict_first) __stcs(reinterpret_cast<unsigned*>(to), code);
-            else *reinterpret_cast<unsigned*>(to) = code;
+            if (code != other) store_exactly(dst + r * j.rstride, acc[0], acc[1], j.amax_bits + sidx, r * sstep);
+            else store_hint(dst + r * j.rstride, code, policy);
           }
         } else {
-          if (live) store_vec<NP>(dst + r * j.rstride, acc, j.evict_first != 0);
+          if (live) store_hint(dst + r * j.rstride, acc, policy);
         }
       }
     });
@@ -232,7 +250,7 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
 
 // blocks [0, ja.blocks) work on A, the rest on B
 template <typename SrcT, typename DstT, bool kDense, int kPass>
-__global__ void __launch_bounds__(kPatThreads, 4)
+__global__ void __launch_bounds__(kPatThreads, pat_blocks_per_sm(kPass))
 encode_pattern_kernel(const __grid_constant__ PatJob ja, const __grid_constant__ PatJob jb, const __grid_constant__ PatCoefs coefs) {
   grid_launch_dependents();   // the block products may set up while this grid drains; they wait before reading
   __shared__ PatSmem sm;

@@ -128,6 +128,11 @@ cudaError_t launch_decode(int output, const void* prod, int prod_dtype, int64_t 
                           int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials, int* n_partials,
                           cudaStream_t st, int gauges = 1);
 int decode_grid(int64_t bm, int64_t bn);
+// The same for tables of the two-level Strassen pattern (decode_pattern.cu), result or error; at most max_partials partial
+// sums.  False, with nothing enqueued, where it has no kernel; else *err is the launch's result.
+bool fmm_decode_pattern(int output, const void* prod, int prod_dtype, int64_t prod_stride, const CoefTable* h_tab, const float* sA,
+                        const float* sB, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
+                        int* n_partials, int max_partials, cudaStream_t st, cudaError_t* err);
 
 // ---- many copies of an algorithm on small blocks (sweep_many.cu): tables of copy c at tabs[3 * c ..], its products numbered
 // c * R .. c * R + R - 1 in every buffer.
