@@ -1024,6 +1024,55 @@ __device__ __forceinline__ void tc_mma_i8(uint32_t d_tmem, uint64_t a_desc, uint
 // packed forms are used only where merging is impossible (multiply after multiply) or harmless (an exact subtraction).
 constexpr int kInt8Threads = 576;   // 18 warps: TMA, MMA, and 16 rescale warps (four per TMEM lane quarter, 32 columns each)
 
+// The MMA role of the group-scaled kernels (warp 1): four MMAs of K = 32 bytes per group of 128 into a fresh accumulator.  All
+// lanes run the loop with warp-uniform control flow and one elected lane issues.
+template <int kAcc, typename L, typename Mma>
+__device__ __forceinline__ void group_mma_loop(const int lane, const int total_tiles, const int G, unsigned char* smem, const uint32_t bar_base,
+                                               const uint32_t tmem_base, volatile int* abort_flag, DeviceStatus* status,
+                                               const unsigned long long limit, const int where_full, const int where_empty, const Mma mma) {
+  auto full_bar = [&](int s) { return bar_base + 8u * s; };
+  auto empty_bar = [&](int s) { return bar_base + 8u * (L::kStages + s); };
+  auto tfull_bar = [&](int b) { return bar_base + 8u * (2 * L::kStages + b); };
+  auto tempty_bar = [&](int b) { return bar_base + 8u * (2 * L::kStages + kAcc + b); };
+  const uint32_t drain_bar = bar_base + 8u * (2 * L::kStages + 2 * kAcc);
+  const uint64_t desc_fixed = make_smem_desc(0);        // everything but the start address
+  const uint32_t ring_lo = (smem_u32(smem) & 0x3FFFFu) >> 4;
+  int stage = 0;
+  uint32_t phase = 0;
+  int acc = 0;
+  uint32_t acc_phase = 0;
+  bool ok = true;
+  for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+    for (int g = 0; g < G; ++g) {
+      ok = mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, where_empty, status, limit) &&
+           mbar_wait(full_bar(stage), phase, abort_flag, where_full, status, limit);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t d_tmem = tmem_base + (uint32_t)(acc * L::BN);
+      const uint64_t da = desc_fixed | (uint64_t)(ring_lo + (uint32_t)(stage * (L::kStageBytes >> 4)));
+      const uint64_t db = da + (uint64_t)(L::kABytes >> 4);
+      if (elect_one()) {
+#pragma unroll
+        for (int k = 0; k < BKB / UMMA_KB; ++k)
+          mma(d_tmem, da + (uint64_t)(k * (UMMA_KB >> 4)), db + (uint64_t)(k * (UMMA_KB >> 4)), k != 0 ? 1u : 0u);
+        tc_commit(empty_bar(stage));
+        tc_commit(tfull_bar(acc));
+      }
+      __syncwarp();
+      if (++stage == L::kStages) { stage = 0; phase ^= 1u; }
+      if (++acc == kAcc) { acc = 0; acc_phase ^= 1u; }
+    }
+  }
+  if (!ok && lane == 0) {     // wait (bounded) for MMAs in flight before TMEM is freed
+    tc_commit(drain_bar);
+    const unsigned long long t0 = global_timer_ns();
+    while (!mbar_try_wait(drain_bar, 0)) {
+      if (global_timer_ns() - t0 > 20000000ull) break;
+    }
+  }
+}
+
 // The rescale role of the group-scaled int8 kernels (warps 2..17): waits for a group's accumulator, converts it, applies
 // the two scales and adds to the tile's fp32 sums, which a thread holds for one row and 32 columns.
 struct RescaleCtx {
@@ -1228,42 +1277,10 @@ int8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer: one fresh accumulator per group
-    if (lane == 0) {
-      // int32 accumulator (c format 2), signed 8-bit A and B (format 1), K-major, N >> 3, M >> 4
-      constexpr uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-      int stage = 0;
-      uint32_t phase = 0;
-      int acc = 0;
-      uint32_t acc_phase = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        for (int g = 0; g < p.G; ++g) {
-          ok = mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, 0x52, status, p.wait_limit_ns);
-          if (!ok) break;
-          ok = mbar_wait(full_bar(stage), phase, abort_flag, 0x51, status, p.wait_limit_ns);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-          const uint32_t sa = smem_u32(smem + stage * L::kStageBytes);
-          const uint64_t da = make_smem_desc(sa);
-          const uint64_t db = make_smem_desc(sa + L::kABytes);
-#pragma unroll
-          for (int k = 0; k < BKB / UMMA_KB; ++k)
-            tc_mma_i8(d_tmem, da + (uint64_t)(k * (UMMA_KB >> 4)), db + (uint64_t)(k * (UMMA_KB >> 4)), idesc, k != 0 ? 1u : 0u);
-          tc_commit(empty_bar(stage));
-          tc_commit(tfull_bar(acc));
-          if (++stage == L::kStages) { stage = 0; phase ^= 1u; }
-          if (++acc == kAcc) { acc = 0; acc_phase ^= 1u; }
-        }
-      }
-      if (!ok) {
-        tc_commit(drain_bar);
-        const unsigned long long t0 = global_timer_ns();
-        while (!mbar_try_wait(drain_bar, 0)) {
-          if (global_timer_ns() - t0 > 20000000ull) break;
-        }
-      }
-    }
+    // int32 accumulator (c format 2), signed 8-bit A and B (format 1), K-major, N >> 3, M >> 4
+    constexpr uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+    group_mma_loop<kAcc, L>(lane, total_tiles, p.G, smem, bar_base, tmem_base, abort_flag, status, p.wait_limit_ns, 0x51, 0x52,
+                            [&](uint32_t d, uint64_t a, uint64_t b, uint32_t acc) { tc_mma_i8(d, a, b, idesc, acc); });
   } else {
     const RescaleCtx rc{bar_base + 8u * (2 * L::kStages), bar_base + 8u * (2 * L::kStages + kAcc), sfull_bar, sempty_bar,
                         tmem_base, scale_sm, abort_flag, status, p.wait_limit_ns, out, p.dAt, p.dBt, p.M, p.N, p.G,
@@ -1289,6 +1306,14 @@ int8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
 // s_A[row][g] * s_B[column block][g] and adds it to its fp32 running sums (one fused multiply-add per element and group);
 // after the last group one rounding to the output dtype (bf16 when the product kernel "returns each product in bf16").
 // One CTA per 128 x 128 tile of one product, so a tile's columns lie in one 128-column scale block.
+// The scales of a tile's rows are staged in shared memory, a tile ahead: read where they lie, every group costs a warp 32
+// cache lines (the scales of a row are neighbours), more than the group's arithmetic.
+struct Fp8Layout : Int8Layout {
+  static constexpr int kMaxGroups = 64;                                  // staged up to this many groups
+  static constexpr int kScaleLd = BM + 1;                                // [group][row], padded against bank conflicts
+  static constexpr int kScaleFloats = kMaxGroups * (kScaleLd + 1);       // rows' scales, then the column block's
+  static constexpr int kTotal = kStages * kStageBytes + kBarBytes + 2 * kScaleFloats * 4 + 1024;
+};
 struct Fp8GroupParams {
   int rows_a, rows_b, G, batches;   // extents of one product, 128-groups along K, number of products
   int tiles_m, tiles_n;
@@ -1303,7 +1328,7 @@ __global__ void __launch_bounds__(kInt8Threads, 1)
 fp8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                       void* __restrict__ out, Fp8GroupParams p, DeviceStatus* status) {
   grid_launch_dependents();
-  using L = Int8Layout;             // same tile, ring and barrier block (the scale staging area is unused here)
+  using L = Fp8Layout;
   constexpr int BN = L::BN;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
@@ -1322,12 +1347,17 @@ fp8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_mem + 8 * (2 * L::kStages + 2 * kAcc + 1));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_mem + 8 * (2 * L::kStages + 2 * kAcc + 1) + 8);
 
+  auto sfull_bar = [&](int b) { return bar_base + 8u * (2 * L::kStages + 2 * kAcc + 3 + b); };    // scales of a tile are staged (16 warps)
+  auto sempty_bar = [&](int b) { return bar_base + 8u * (2 * L::kStages + 2 * kAcc + 5 + b); };   // and no longer read
+  float* scale_sm = reinterpret_cast<float*>(bar_mem + L::kBarBytes);
+
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr uint32_t kTmemCols = kAcc * BN;
   if (threadIdx.x == 0) {
     for (int s = 0; s < L::kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
     for (int b = 0; b < kAcc; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 16); }
     mbar_init(drain_bar, 1);
+    for (int b = 0; b < 2; ++b) { mbar_init(sfull_bar(b), 16); mbar_init(sempty_bar(b), 16); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1377,41 +1407,9 @@ fp8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer: one fresh accumulator per group
-    if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc(true, BN);
-      int stage = 0;
-      uint32_t phase = 0;
-      int acc = 0;
-      uint32_t acc_phase = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        for (int g = 0; g < p.G; ++g) {
-          ok = mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, 0x82, status, p.wait_limit_ns);
-          if (!ok) break;
-          ok = mbar_wait(full_bar(stage), phase, abort_flag, 0x81, status, p.wait_limit_ns);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-          const uint32_t sa = smem_u32(smem + stage * L::kStageBytes);
-          const uint64_t da = make_smem_desc(sa);
-          const uint64_t db = make_smem_desc(sa + L::kABytes);
-#pragma unroll
-          for (int k = 0; k < BKB / UMMA_KB; ++k)
-            tc_mma<true>(d_tmem, da + (uint64_t)(k * (UMMA_KB >> 4)), db + (uint64_t)(k * (UMMA_KB >> 4)), idesc, k != 0 ? 1u : 0u);
-          tc_commit(empty_bar(stage));
-          tc_commit(tfull_bar(acc));
-          if (++stage == L::kStages) { stage = 0; phase ^= 1u; }
-          if (++acc == kAcc) { acc = 0; acc_phase ^= 1u; }
-        }
-      }
-      if (!ok) {
-        tc_commit(drain_bar);
-        const unsigned long long t0 = global_timer_ns();
-        while (!mbar_try_wait(drain_bar, 0)) {
-          if (global_timer_ns() - t0 > 20000000ull) break;
-        }
-      }
-    }
+    constexpr uint32_t idesc = make_idesc(true, BN);
+    group_mma_loop<kAcc, L>(lane, total_tiles, p.G, smem, bar_base, tmem_base, abort_flag, status, p.wait_limit_ns, 0x81, 0x82,
+                            [&](uint32_t d, uint64_t a, uint64_t b, uint32_t acc) { tc_mma<true>(d, a, b, idesc, acc); });
   } else {
     // ------------------------------------------------------------ scale and accumulate (warps 2..17)
     const int quad = warp & 3;
@@ -1420,10 +1418,49 @@ fp8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
+    const bool staged = p.G <= L::kMaxGroups;
+    // asynchronous copies of this thread's share of a tile's scales
+    auto stage_scales = [&](int tile, int buf) {
+      const int r = tile / tiles_per_batch;
+      const int rem = tile - r * tiles_per_batch;
+      const int tm = rem / p.tiles_n, tn = rem - tm * p.tiles_n;
+      const float* rows = p.sA + (long long)r * p.sa_batch + (long long)tm * BM * p.G;
+      const float* cols = p.sB + (long long)r * p.sb_batch + (long long)tn * p.G;
+      const uint32_t dst = smem_u32(scale_sm + buf * L::kScaleFloats);
+      const int live = min(BM, p.rows_a - tm * BM) * p.G;
+      for (int i = (int)threadIdx.x - 64; i < live; i += 512) {
+        const int row = i / p.G, g = i - row * p.G;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4u * (uint32_t)(g * L::kScaleLd + row)), "l"(rows + i) : "memory");
+      }
+      for (int g = (int)threadIdx.x - 64; g < p.G; g += 512)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4u * (uint32_t)(L::kMaxGroups * L::kScaleLd + g)), "l"(cols + g) : "memory");
+    };
+    auto scales_ready = [&](int buf) {        // this warp's share has landed
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(sfull_bar(buf));
+    };
+    int buf = 0;
+    uint32_t buf_phase = 0;
+    if (staged && (int)blockIdx.x < total_tiles) {
+      stage_scales(blockIdx.x, 0);
+      scales_ready(0);
+    }
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
       const int r = tile / tiles_per_batch;
       const int rem = tile - r * tiles_per_batch;
       const int tm = rem / p.tiles_n, tn = rem - tm * p.tiles_n;
+      const bool more = staged && tile + (int)gridDim.x < total_tiles;
+      if (staged) {
+        ok = mbar_wait(sfull_bar(buf), buf_phase, abort_flag, 0x95, status, p.wait_limit_ns);
+        // the other buffer's readers (the tile before) are done; nobody has read buffer 1 before the first tile
+        if (more) ok = mbar_wait(sempty_bar(buf ^ 1), buf == 0 ? buf_phase ^ 1u : buf_phase, abort_flag, 0x94, status, p.wait_limit_ns) && ok;
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        if (more) stage_scales(tile + (int)gridDim.x, buf ^ 1);
+      }
+      const float* sc_rows = scale_sm + buf * L::kScaleFloats + quad * 32 + lane;
+      const float* sc_cols = scale_sm + buf * L::kScaleFloats + L::kMaxGroups * L::kScaleLd;
       const int row = tm * BM + quad * 32 + lane;
       const bool row_ok = row < p.rows_a;
       const int col_base = tn * BN + part * PN;
@@ -1432,20 +1469,15 @@ fp8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
       float2 sum[PN / 2];
 #pragma unroll
       for (int j = 0; j < PN / 2; ++j) sum[j] = make_float2(0.0f, 0.0f);
-      // the scales do not depend on the products: they are fetched two groups ahead of their use
-      float s_next = row_ok ? sa_row[0] * sb_blk[0] : 0.0f;
-      float s_next2 = (row_ok && p.G > 1) ? sa_row[1] * sb_blk[1] : 0.0f;
       for (int g = 0; g < p.G; ++g) {
-        const float sc = s_next;
-        s_next = s_next2;
-        if (g + 2 < p.G) s_next2 = row_ok ? sa_row[g + 2] * sb_blk[g + 2] : 0.0f;
+        const float sc = staged ? sc_rows[g * L::kScaleLd] * sc_cols[g] : row_ok ? sa_row[g] * sb_blk[g] : 0.0f;
         ok = mbar_wait(tfull_bar(acc), acc_phase, abort_flag, 0x93, status, p.wait_limit_ns);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after();
         uint32_t v[32];
         tc_ld32(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN + part * PN), v);
-        tc_wait_ld();
+        tc_wait_ld32(v);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(tempty_bar(acc));
@@ -1454,8 +1486,15 @@ fp8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
 #pragma unroll
         for (int j = 0; j < PN / 2; ++j)      // one fused multiply-add per element, two elements per instruction
           sum[j] = __ffma2_rn(make_float2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1])), sc2, sum[j]);
+        if (more && g == 0) scales_ready(buf ^ 1);
       }
       if (!ok) break;
+      if (staged) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(sempty_bar(buf));
+        buf ^= 1;
+        if (buf == 0) buf_phase ^= 1u;
+      }
       if (row_ok && col_base < p.rows_b) {
         uint32_t w[32];
 #pragma unroll
@@ -1464,6 +1503,7 @@ fp8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
                         p.out_bf16, 1.0f, p.wide != 0);
       }
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");     // none in flight unless the loop was left early
   }
 
   tc_fence_before();
@@ -1479,7 +1519,7 @@ fp8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
 }  // namespace
 
 fmm_status launch_fp8_group_gemm(const Fp8GroupArgs& a, cudaStream_t st) {
-  using L = Int8Layout;
+  using L = Fp8Layout;
   if (a.rows_a > 0x7fffffff || a.rows_b > 0x7fffffff || a.kdim <= 0 || a.kdim > 0x3fffffff) return FMM_ERR_SHAPE;
   CUtensorMap ma, mb;
   if (!make_operand_map(&ma, true, a.A, a.rows_a, a.kdim, a.lda, a.a_batch, a.batches, BM)) return FMM_ERR_CUDA;
