@@ -10,8 +10,10 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <numeric>
 
 #include "../../include/fmm_b200.h"
 #include "kernels_stream.cuh"
@@ -34,26 +36,29 @@ __device__ __forceinline__ void copy_bytes(void* dst, const void* src) {
   }
 }
 
-// raw storage values and their sign bytes -> fp32 pairs with the sign applied (an exact flip of the sign bit)
+// sign bytes -> one mask word per 32 bits of raw values (the sign bits to flip)
 template <typename T, int E>
-__device__ __forceinline__ void load_signed(const T* raw, const signed char* sg, bool has_signs, bool live, float2* v) {
+__device__ __forceinline__ void sign_masks(const signed char* sg, bool has_signs, uint32_t* mask) {
+#pragma unroll
+  for (int p = 0; p < E * (int)sizeof(T) / 4; ++p) {
+    if constexpr (sizeof(T) == 2)
+      mask[p] = has_signs ? (((uint32_t)(unsigned char)sg[2 * p] & 0x80u) << 8) | (((uint32_t)(unsigned char)sg[2 * p + 1] & 0x80u) << 24) : 0u;
+    else
+      mask[p] = has_signs ? ((uint32_t)(unsigned char)sg[p] & 0x80u) << 24 : 0u;
+  }
+}
+// raw storage values with their signs applied (an exact flip of the sign bit) -> fp32 pairs
+template <typename T, int E>
+__device__ __forceinline__ void load_signed(const T* raw, const uint32_t* mask, float2* v) {
 #pragma unroll
   for (int p = 0; p < E / 2; ++p) {
-    uint32_t x0, x1;
     if constexpr (sizeof(T) == 2) {
-      const uint32_t two = reinterpret_cast<const uint32_t*>(raw)[p];      // bf16 pair: fp32 bits are the halves shifted up
-      x0 = two << 16;
-      x1 = two & 0xffff0000u;
+      const uint32_t two = reinterpret_cast<const uint32_t*>(raw)[p] ^ mask[p];   // bf16 pair: fp32 bits are the halves shifted up
+      v[p] = make_float2(__uint_as_float(two << 16), __uint_as_float(two & 0xffff0000u));
     } else {
-      x0 = reinterpret_cast<const uint32_t*>(raw)[2 * p];
-      x1 = reinterpret_cast<const uint32_t*>(raw)[2 * p + 1];
+      v[p] = make_float2(__uint_as_float(reinterpret_cast<const uint32_t*>(raw)[2 * p] ^ mask[2 * p]),
+                         __uint_as_float(reinterpret_cast<const uint32_t*>(raw)[2 * p + 1] ^ mask[2 * p + 1]));
     }
-    if (has_signs) {
-      const uint32_t s0 = (uint32_t)(unsigned char)sg[2 * p], s1 = (uint32_t)(unsigned char)sg[2 * p + 1];
-      x0 ^= (s0 & 0x80u) << 24;
-      x1 ^= (s1 & 0x80u) << 24;
-    }
-    v[p] = live ? make_float2(__uint_as_float(x0), __uint_as_float(x1)) : make_float2(0.0f, 0.0f);
   }
 }
 __device__ __forceinline__ void store_pair(float2 x, float* y) { y[0] = x.x; y[1] = x.y; }
@@ -61,75 +66,84 @@ __device__ __forceinline__ void store_pair(float2 x, __nv_bfloat16* y) {
   *reinterpret_cast<__nv_bfloat162*>(y) = __float22bfloat162_rn(x);
 }
 
-// E elements per lane, L = h / E lanes per h-block (a power of two <= 32), 32 / L blocks per warp pass; a warp takes U
-// passes per loop iteration and issues all their loads before it transforms the first (bytes in flight).
-template <typename T, int E, int U>
+// E elements per lane, L = h / E lanes per h-block (a power of two <= 32), 32 / L blocks per warp pass.  The number of warps W
+// is chosen so that W passes are a whole number of rows: a lane then stays in its columns, its signs become mask words once
+// and for all, and a step is a constant distance in X and Y.  A warp keeps the loads of its next kAhead passes in flight
+// while it transforms one.  8192 x 13824 bf16: h = 128 100 -> 87 us (5.2 TB/s), h = 64 113 -> 95, h = 512 124 -> 113, against
+// passes that worked out their position and signs and loaded before they transformed.  What bounds it now: the lane
+// exchanges (48 shuffles for 16 values a lane at h = 128) beside the memory system.
+template <typename T, int E, int kAhead>
 __global__ void __launch_bounds__(kRotThreads)
-hadamard_rotate_kernel(const T* __restrict__ X, int64_t ldx, int64_t n_blocks, int blocks_per_row, int h,
-                       const signed char* __restrict__ signs, float inv_sqrt_h, T* __restrict__ Y, int64_t ldy) {
+hadamard_rotate_kernel(const T* X, int64_t n_blocks, int blocks_per_row, int h, const signed char* __restrict__ signs,
+                       float inv_sqrt_h, T* Y, int64_t ldx, int64_t ldy, int64_t W, int64_t step_x, int64_t step_y) {
   const int L = h / E;
   const int lane = threadIdx.x & 31;
   const int l = lane & (L - 1);            // lane inside its block
   const int sub = lane / L;                // which of the warp's blocks
   const int per_warp = 32 / L;
-  const int64_t warps = (int64_t)gridDim.x * (kRotThreads / 32);
-  const int64_t warp0 = (int64_t)blockIdx.x * (kRotThreads / 32) + (threadIdx.x >> 5);
+  const int64_t warp = (int64_t)blockIdx.x * (kRotThreads / 32) + (threadIdx.x >> 5);
+  if (warp >= W) return;
+  int64_t b = warp * per_warp + sub;
+  const int64_t row = b / blocks_per_row;
+  const int col = (int)(b - row * blocks_per_row) * h + l * E;
+  const T* src = X + row * ldx + col;
+  T* dst = Y + row * ldy + col;
+  uint32_t mask[E * sizeof(T) / 4];
+  {
+    alignas(16) signed char sg[E];
+    if (signs != nullptr) copy_bytes<E>(sg, signs + col);
+    sign_masks<T, E>(sg, signs != nullptr, mask);
+  }
+  alignas(16) T raw[kAhead + 1][E];
+  const int64_t step_b = W * per_warp;
+#pragma unroll
+  for (int a = 0; a < kAhead; ++a)
+    if (b + a * step_b < n_blocks) copy_bytes<E * (int)sizeof(T)>(raw[a], src + a * step_x);
   const int64_t passes = (n_blocks + per_warp - 1) / per_warp;
-  for (int64_t first = warp0 * U; first < passes; first += warps * U) {     // whole warps iterate together (shuffles below)
-    alignas(16) T raw[U][E];
-    alignas(16) signed char sg[U][E];
-    int64_t off_y[U];
-    bool live[U];
+#pragma unroll 1
+  for (int64_t pass = warp; pass < passes; pass += W) {     // whole warps iterate together (shuffles below)
+    if (b + kAhead * step_b < n_blocks) copy_bytes<E * (int)sizeof(T)>(raw[kAhead], src + kAhead * step_x);
+    float2 v[E / 2];          // (even, odd) neighbours: strides >= 2 and the lane exchanges run as packed fp32 pairs
+    load_signed<T, E>(raw[0], mask, v);
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int64_t b = (first + u) * per_warp + sub;
-      live[u] = first + u < passes && b < n_blocks;
-      const int64_t row = live[u] ? b / blocks_per_row : 0;
-      const int col = live[u] ? (int)(b - row * blocks_per_row) * h + l * E : 0;
-      off_y[u] = row * ldy + col;
-      if (live[u]) {
-        copy_bytes<E * (int)sizeof(T)>(raw[u], X + row * ldx + col);
-        if (signs != nullptr) copy_bytes<E>(sg[u], signs + col);
-      }
+    for (int p = 0; p < E / 2; ++p) {          // stride 1: inside each pair
+      const float a = v[p].x, c = v[p].y;
+      v[p] = make_float2(__fadd_rn(a, c), __fsub_rn(a, c));
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      float2 v[E / 2];          // (even, odd) neighbours: strides >= 2 and the lane exchanges run as packed fp32 pairs
-      load_signed<T, E>(raw[u], sg[u], signs != nullptr, live[u], v);
+    for (int s = 1; s < E / 2; s <<= 1) {      // strides 2 .. E/2 (pair index stride s)
 #pragma unroll
-      for (int p = 0; p < E / 2; ++p) {          // stride 1: inside each pair
-        const float a = v[p].x, c = v[p].y;
-        v[p] = make_float2(__fadd_rn(a, c), __fsub_rn(a, c));
-      }
-#pragma unroll
-      for (int s = 1; s < E / 2; s <<= 1) {      // strides 2 .. E/2 (pair index stride s)
-#pragma unroll
-        for (int p = 0; p < E / 2; ++p) {
-          if ((p & s) == 0) {
-            const float2 a = v[p], c = v[p + s];
-            v[p] = __fadd2_rn(a, c);
-            v[p + s] = __ffma2_rn(c, make_float2(-1.0f, -1.0f), a);     // a - c, one rounding
-          }
+      for (int p = 0; p < E / 2; ++p) {
+        if ((p & s) == 0) {
+          const float2 a = v[p], c = v[p + s];
+          v[p] = __fadd2_rn(a, c);
+          v[p + s] = __ffma2_rn(c, make_float2(-1.0f, -1.0f), a);     // a - c, one rounding
         }
-      }
-      for (int s = 1; s < L; s <<= 1) {          // strides E .. h/2: partner lane l ^ s; fma(v, +-1, o) = o +- v exactly once rounded
-        const float sgn = (l & s) != 0 ? -1.0f : 1.0f;
-        const float2 sg2 = make_float2(sgn, sgn);
-#pragma unroll
-        for (int p = 0; p < E / 2; ++p) {
-          float2 o;
-          o.x = __shfl_xor_sync(0xffffffffu, v[p].x, s);
-          o.y = __shfl_xor_sync(0xffffffffu, v[p].y, s);
-          v[p] = __ffma2_rn(v[p], sg2, o);
-        }
-      }
-      if (live[u]) {
-        const float2 r2 = make_float2(inv_sqrt_h, inv_sqrt_h);
-#pragma unroll
-        for (int p = 0; p < E / 2; ++p) store_pair(__fmul2_rn(v[p], r2), &raw[u][2 * p]);
-        copy_bytes<E * (int)sizeof(T)>(Y + off_y[u], raw[u]);
       }
     }
+    for (int s = 1; s < L; s <<= 1) {          // strides E .. h/2: partner lane l ^ s; fma(v, +-1, o) = o +- v exactly once rounded
+      const float sgn = (l & s) != 0 ? -1.0f : 1.0f;
+      const float2 sg2 = make_float2(sgn, sgn);
+#pragma unroll
+      for (int p = 0; p < E / 2; ++p) {
+        float2 o;
+        o.x = __shfl_xor_sync(0xffffffffu, v[p].x, s);
+        o.y = __shfl_xor_sync(0xffffffffu, v[p].y, s);
+        v[p] = __ffma2_rn(v[p], sg2, o);
+      }
+    }
+    if (b < n_blocks) {
+      alignas(16) T out[E];
+      const float2 r2 = make_float2(inv_sqrt_h, inv_sqrt_h);
+#pragma unroll
+      for (int p = 0; p < E / 2; ++p) store_pair(__fmul2_rn(v[p], r2), &out[2 * p]);
+      copy_bytes<E * (int)sizeof(T)>(dst, out);
+    }
+#pragma unroll
+    for (int a = 0; a < kAhead; ++a)
+#pragma unroll
+      for (int e = 0; e < E; ++e) raw[a][e] = raw[a + 1][e];
+    b += step_b; src += step_x; dst += step_y;
   }
 }
 
@@ -137,20 +151,27 @@ template <typename T, int E>
 cudaError_t launch_rotate(const void* X, int64_t ldx, int64_t rows, int64_t K, int h, const signed char* signs, void* Y,
                           int64_t ldy, cudaStream_t st) {
   constexpr int kBytes = E * (int)sizeof(T);
-  constexpr int U = kBytes >= 64 ? 1 : (kBytes >= 32 ? 2 : 4);
-  const int64_t n_blocks = rows * (K / h);
-  const int per_warp = 32 / (h / E);
+  constexpr int kAhead = kBytes >= 64 ? 1 : (kBytes >= 32 ? 2 : 3);
+  const int bpr = (int)(K / h), per_warp = 32 / (h / E);
+  const int64_t n_blocks = rows * bpr;
   const int64_t passes = (n_blocks + per_warp - 1) / per_warp;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return cudaErrorInvalidDevice;
-  const int64_t per_block = (int64_t)(kRotThreads / 32) * U;
-  const int64_t want = (passes + per_block - 1) / per_block;
-  const int64_t cap = (int64_t)sms * 8;                        // full occupancy; grid-stride beyond it
-  const unsigned grid = (unsigned)(want < cap ? want : cap);
+  // as many warps as run at once (24 or 32 an SM by the registers): with a few more, the last of them run alone (bf16, h = 128,
+  // 24 fit: 87 us at 24, 97 at 32)
+  static const int blocks_per_sm = [] {
+    int n = 0;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, hadamard_rotate_kernel<T, E, kAhead>, kRotThreads, 0) == cudaSuccess && n > 0 ? n : 1;
+  }();
+  const int64_t unit = bpr / std::gcd(bpr, per_warp);                     // passes that make up whole rows
+  const int64_t cap = std::max<int64_t>(1, (int64_t)sms * blocks_per_sm * (kRotThreads / 32) / unit);
+  const int64_t W = unit * std::min(cap, (passes + unit - 1) / unit);
+  const int64_t rows_step = W * per_warp / bpr;
   const float inv = (float)(1.0 / std::sqrt((double)h));
-  hadamard_rotate_kernel<T, E, U><<<grid, kRotThreads, 0, st>>>((const T*)X, ldx, n_blocks, (int)(K / h), h, signs, inv,
-                                                                 (T*)Y, ldy);
+  const int64_t grid = (W + kRotThreads / 32 - 1) / (kRotThreads / 32);
+  hadamard_rotate_kernel<T, E, kAhead><<<(unsigned)grid, kRotThreads, 0, st>>>((const T*)X, n_blocks, bpr, h, signs, inv, (T*)Y, ldx, ldy, W,
+                                                                               rows_step * ldx, rows_step * ldy);
   ++fmm_launch_counter();
   return cudaGetLastError();
 }
