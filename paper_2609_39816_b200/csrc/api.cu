@@ -801,11 +801,9 @@ fmm_status error_frobenius(const fmm_gemm_desc* d, const void* dC, const double*
   FMM_TRY(check_ws(d_ws, ws_bytes, error_frobenius_workspace()));
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   double* pe = at<double>(d_ws, 0);
-  double* pr = pe + kMaxStreamPartials;
-  int np = 0;
-  FMM_CUDA(launch_frob_err(d->output, dC, d->ldc, dCstar, d->M, d->N, pe, pr, &np, st));
-  FMM_CUDA(launch_sum_partials(pe, np, d_out, st));
-  FMM_CUDA(launch_sum_partials(pr, np, d_out + 1, st));
+  int np = stream_grid(d->M * d->N);        // partial sums of each of the two, one array behind the other
+  FMM_CUDA(launch_frob_err(d->output, dC, d->ldc, dCstar, d->M, d->N, pe, pe + np, &np, st));
+  FMM_CUDA(launch_sum_partials(pe, np, d_out, st, 2));
   return FMM_OK;
 }
 

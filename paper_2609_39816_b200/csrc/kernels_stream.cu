@@ -281,22 +281,50 @@ cudaError_t launch_encode_t(const EncodeOperand& a, const EncodeOperand* b, bool
 }
 
 // ------------------------------------------------------------------------------------------
-// transpose (only when B is given K x N): 32 x 32 tiles through padded shared memory
+// transpose (only when B is given K x N): tiles of 64 columns and 32 words of K (64 bf16 or 32 fp32 values) through shared
+// memory, 16-byte loads along N (element by element where B is not aligned) and 32 bytes a thread along K.  A bf16 pair of
+// neighbouring K is put together on the way in, so the tile is made of words.  K is a multiple of 16, N of 8.
 // ------------------------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(256) transpose_kernel(const T* __restrict__ B, int64_t ldb, int64_t K, int64_t N,
-                                                        T* __restrict__ Bt) {
-  __shared__ T tile[32][33];
-  const int64_t n0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  for (int r = ty; r < 32; r += 8) {
-    const int64_t kk = k0 + r, nn = n0 + tx;
-    if (kk < K && nn < N) tile[r][tx] = B[kk * ldb + nn];
+                                                        T* __restrict__ Bt, int vec) {
+  constexpr int kPer = 4 / (int)sizeof(T);            // values of a word
+  constexpr int VE = 16 / (int)sizeof(T);             // values of a vector
+  constexpr int kVecs = 64 / VE;                      // vectors of a tile's row
+  __shared__ uint32_t tile[64][33];
+  const int64_t n0 = (int64_t)blockIdx.x * 64, k0 = (int64_t)blockIdx.y * (32 * kPer);
+  const int tid = threadIdx.x;
+#pragma unroll
+  for (int i = tid; i < 32 * kVecs; i += 256) {
+    const int kw = i / kVecs, nv = i - kw * kVecs;
+    alignas(16) T e[kPer][VE] = {};
+#pragma unroll
+    for (int h = 0; h < kPer; ++h) {
+      const int64_t k = k0 + kw * kPer + h, n = n0 + nv * VE;
+      if (k < K && n < N) {
+        const T* src = B + k * ldb + n;
+        if (vec) {
+          *reinterpret_cast<uint4*>(e[h]) = __ldcs(reinterpret_cast<const uint4*>(src));
+        } else {
+#pragma unroll
+          for (int j = 0; j < VE; ++j) e[h][j] = src[j];
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < VE; ++j)
+      tile[nv * VE + j][kw] = kPer == 2 ? (uint32_t)e[0][j] | ((uint32_t)e[kPer - 1][j] << 16) : (uint32_t)e[0][j];
   }
   __syncthreads();
-  for (int r = ty; r < 32; r += 8) {
-    const int64_t nn = n0 + r, kk = k0 + tx;
-    if (kk < K && nn < N) Bt[nn * K + kk] = tile[tx][r];
+  const int n = tid >> 2, w0 = (tid & 3) * 8;
+  const int64_t k = k0 + w0 * kPer;
+  if (n0 + n < N && k < K) {                          // eight words: 16 bf16 or 8 fp32, inside K as a whole
+    uint32_t w[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) w[j] = tile[n][w0 + j];
+    uint4* dst = reinterpret_cast<uint4*>(Bt + (n0 + n) * K + k);
+    dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
   }
 }
 
@@ -333,6 +361,7 @@ decode_batch_kernel(const ProdT* __restrict__ prod, const CoefTable* __restrict_
 __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restrict__ partials, int n,
                                                            double* __restrict__ out) {
   __shared__ double red[8];
+  grid_dependency_wait();     // the partial sums come from the previous kernel of the stream
   double v = 0.0;
   for (int i = threadIdx.x; i < n; i += 256) v += partials[(size_t)blockIdx.x * n + i];
   const double tot = block_sum_double(v, red);
@@ -342,8 +371,10 @@ __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restr
 __global__ void __launch_bounds__(256) cstar_prepare_kernel(const double* __restrict__ cstar, int64_t count,
                                                             float* __restrict__ cstar32,
                                                             double* __restrict__ partials) {
+  grid_launch_dependents();
   __shared__ double red[8];
   double s = 0.0;
+#pragma unroll 4
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < count; i += (int64_t)gridDim.x * 256) {
     const double v = cstar[i];
     cstar32[i] = (float)v;
@@ -357,15 +388,21 @@ template <typename OutT>
 __global__ void __launch_bounds__(256) frob_err_kernel(const OutT* __restrict__ C, int64_t ldc,
                                                        const double* __restrict__ cstar, int64_t M, int64_t N,
                                                        double* __restrict__ part_err, double* __restrict__ part_ref) {
+  grid_launch_dependents();
   __shared__ double red[8];
   double e = 0.0, s = 0.0;
-  const int64_t count = M * N;
-  for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < count; i += (int64_t)gridDim.x * 256) {
-    const int64_t r = i / N, c = i - r * N;
+  // positions advance by a constant (rows, columns) step: one division a thread
+  const int64_t count = M * N, step = (int64_t)gridDim.x * 256, step_r = step / N, step_c = step - step_r * N;
+  int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x, r = i / N, c = i - r * N;
+#pragma unroll 4
+  for (; i < count; i += step) {
     const double v = cstar[i];
     const double d = (double)(float)C[r * ldc + c] - v;
     e += d * d;
     s += v * v;
+    r += step_r;
+    c += step_c;
+    if (c >= N) { c -= N; ++r; }
   }
   const double te = block_sum_double(e, red);
   if (threadIdx.x == 0) part_err[blockIdx.x] = te;
@@ -618,11 +655,13 @@ cudaError_t launch_encode(int storage, int product, const void* X, int64_t ldx, 
 
 cudaError_t launch_transpose(int elem_bytes, const void* B, int64_t ldb, int64_t K, int64_t N, void* Bt,
                              cudaStream_t st) {
-  dim3 grid((unsigned)((N + 31) / 32), (unsigned)((K + 31) / 32));
+  const dim3 grid((unsigned)((N + 63) / 64), (unsigned)((K * elem_bytes + 127) / 128));
+  const int vec = reinterpret_cast<uintptr_t>(B) % 16 == 0 && (ldb * elem_bytes) % 16 == 0;
+  if (K % 16 || N % 8) return cudaErrorInvalidValue;
   if (elem_bytes == 2)
-    transpose_kernel<uint16_t><<<grid, 256, 0, st>>>((const uint16_t*)B, ldb, K, N, (uint16_t*)Bt);
+    transpose_kernel<uint16_t><<<grid, 256, 0, st>>>((const uint16_t*)B, ldb, K, N, (uint16_t*)Bt, vec);
   else if (elem_bytes == 4)
-    transpose_kernel<uint32_t><<<grid, 256, 0, st>>>((const uint32_t*)B, ldb, K, N, (uint32_t*)Bt);
+    transpose_kernel<uint32_t><<<grid, 256, 0, st>>>((const uint32_t*)B, ldb, K, N, (uint32_t*)Bt, vec);
   else
     return cudaErrorInvalidValue;
   ++fmm_launch_counter();
@@ -729,7 +768,8 @@ cudaError_t launch_decode(int output, const void* prod, int prod_dtype, int64_t 
 }
 
 cudaError_t launch_sum_partials(const double* partials, int n, double* out, cudaStream_t st, int count) {
-  sum_partials_kernel<<<count, 256, 0, st>>>(partials, n, out);
+  const cudaError_t e = launch_dependent(sum_partials_kernel, dim3(count), dim3(256), 0, st, partials, n, out);
+  if (e != cudaSuccess) return e;
   ++fmm_launch_counter();
   return cudaGetLastError();
 }
