@@ -628,7 +628,8 @@ __device__ __forceinline__ void pair_roles(const int warp, const int lane, const
         __syncwarp();
         if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
       }
-      if (!ok && lane == 0) {
+      // a commit tracks the MMAs of the lane that executes it: the elected lane issued them, so it drains them
+      if (!ok && elect_one()) {
         asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(drain_bar)
                      : "memory");
         const unsigned long long t0 = global_timer_ns();
@@ -1027,7 +1028,7 @@ constexpr int kInt8Threads = 576;   // 18 warps: TMA, MMA, and 16 rescale warps 
 // The MMA role of the group-scaled kernels (warp 1): four MMAs of K = 32 bytes per group of 128 into a fresh accumulator.  All
 // lanes run the loop with warp-uniform control flow and one elected lane issues.
 template <int kAcc, typename L, typename Mma>
-__device__ __forceinline__ void group_mma_loop(const int lane, const int total_tiles, const int G, unsigned char* smem, const uint32_t bar_base,
+__device__ __forceinline__ void group_mma_loop(const int total_tiles, const int G, unsigned char* smem, const uint32_t bar_base,
                                                const uint32_t tmem_base, volatile int* abort_flag, DeviceStatus* status,
                                                const unsigned long long limit, const int where_full, const int where_empty, const Mma mma) {
   auto full_bar = [&](int s) { return bar_base + 8u * s; };
@@ -1064,7 +1065,9 @@ __device__ __forceinline__ void group_mma_loop(const int lane, const int total_t
       if (++acc == kAcc) { acc = 0; acc_phase ^= 1u; }
     }
   }
-  if (!ok && lane == 0) {     // wait (bounded) for MMAs in flight before TMEM is freed
+  // wait (bounded) for MMAs in flight before TMEM is freed; a commit tracks the MMAs of the lane that executes it, so the
+  // elected lane, which issued them, drains them
+  if (!ok && elect_one()) {
     tc_commit(drain_bar);
     const unsigned long long t0 = global_timer_ns();
     while (!mbar_try_wait(drain_bar, 0)) {
@@ -1279,7 +1282,7 @@ int8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     // ------------------------------------------------------------ MMA issuer: one fresh accumulator per group
     // int32 accumulator (c format 2), signed 8-bit A and B (format 1), K-major, N >> 3, M >> 4
     constexpr uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-    group_mma_loop<kAcc, L>(lane, total_tiles, p.G, smem, bar_base, tmem_base, abort_flag, status, p.wait_limit_ns, 0x51, 0x52,
+    group_mma_loop<kAcc, L>(total_tiles, p.G, smem, bar_base, tmem_base, abort_flag, status, p.wait_limit_ns, 0x51, 0x52,
                             [&](uint32_t d, uint64_t a, uint64_t b, uint32_t acc) { tc_mma_i8(d, a, b, idesc, acc); });
   } else {
     const RescaleCtx rc{bar_base + 8u * (2 * L::kStages), bar_base + 8u * (2 * L::kStages + kAcc), sfull_bar, sempty_bar,
@@ -1408,7 +1411,7 @@ fp8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer: one fresh accumulator per group
     constexpr uint32_t idesc = make_idesc(true, BN);
-    group_mma_loop<kAcc, L>(lane, total_tiles, p.G, smem, bar_base, tmem_base, abort_flag, status, p.wait_limit_ns, 0x81, 0x82,
+    group_mma_loop<kAcc, L>(total_tiles, p.G, smem, bar_base, tmem_base, abort_flag, status, p.wait_limit_ns, 0x81, 0x82,
                             [&](uint32_t d, uint64_t a, uint64_t b, uint32_t acc) { tc_mma<true>(d, a, b, idesc, acc); });
   } else {
     // ------------------------------------------------------------ scale and accumulate (warps 2..17)

@@ -324,3 +324,23 @@ def test_permuted_products_are_the_same_algorithm(lib):
     for bad in ([0] * 49, list(range(48)) + [49], list(range(48)) + [-1]):
         with pytest.raises(lib.FmmError):
             lib.scheme_permute_products(s2, bad)
+
+
+def test_drain_commits_come_from_the_lane_that_issues_the_mmas():
+    """A tcgen05.commit tracks the MMAs of the lane that executes it.  Where an elected lane issues them, the commit on
+    the abort path (after which tensor memory is freed) has to be the elected lane's too."""
+    csrc = os.path.join(ROOT, "paper_2609_39816_b200", "csrc")
+    drains = 0
+    for name in ("gemm_tcgen05.cu", "int8_certified.inc"):
+        with open(os.path.join(csrc, name)) as f:
+            lines = f.read().split("\n")
+        for i, line in enumerate(lines):
+            if not re.search(r"tc_commit\(drain_bar\)|tcgen05\.commit.*\(drain_bar\)", line):
+                continue
+            drains += 1
+            # the roles of a kernel start with a comparison of the warp's index, or the function that holds one role
+            start = max(j for j in range(i) if "warp == 1" in lines[j] or "group_mma_loop(" in lines[j])
+            body = lines[start:i]
+            issued_by_elected = any("elect_one()" in x and "!ok" not in x for x in body)
+            assert ("elect_one()" in lines[i - 1]) == issued_by_elected, (name, i + 1)
+    assert drains == 4
