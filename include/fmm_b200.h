@@ -89,9 +89,10 @@ typedef enum { FMM_F32 = 0, FMM_BF16 = 1, FMM_E4M3 = 2 } fmm_dtype;
 
 #define FMM_FLAG_SWEEP_SERIAL 4 /* error_sweep only: run the stages of every gauge back to back on the caller's
                                  stream instead of pipelining consecutive gauges over the library's helper
-                                 streams.  Same results bit for bit (the arithmetic and the order of every sum
-                                 are the same); slower.  For callers that want one stream only, and for checking
-                                 the pipelined path against.                                              */
+                                 streams.  Same results bit for bit as the pipeline's (the arithmetic and the order
+                                 of every sum are the same); slower.  For callers that want one stream only, and for
+                                 checking the pipelined path against.  Sweeps on small blocks (see error_sweep) run
+                                 on the caller's stream in any case: the flag changes nothing there.       */
 
 #define FMM_FLAG_SWEEP_UNFUSED 16 /* error_sweep only: do not use the fused launches.  By default, where it applies (bf16
                                  storage and products, no scales, one-level algorithms on a 2 x 2 grid, blocks larger
@@ -101,7 +102,8 @@ typedef enum { FMM_F32 = 0, FMM_BF16 = 1, FMM_E4M3 = 2 } fmm_dtype;
                                  Every algorithm's C is the same bits either way; its error sum is added over another
                                  partition of the outputs (ratios agree to 1e-8; each path is bit-reproducible run to
                                  run).  With this flag such sweeps take the three-stream pipeline that all other
-                                 sweeps use.                                                                    */
+                                 sweeps use, but for those on small blocks (see error_sweep), which the flag does
+                                 not change.                                                                    */
 #define FMM_FLAG_ROUND_PER_LEVEL 8 /* scheme_gemm on a handle made by scheme_kron (or "strassen444"): round the block
                                  sums at EVERY level.  The outer factor's block sums of A (and of B) are scaled
                                  and rounded to the product dtype; the inner factor's block sums are formed of
@@ -461,7 +463,8 @@ const char* fmm_status_string(fmm_status st);
 int64_t fmm_launch_count(void);
 
 /* Phase timing.  While enabled, every device call brackets each step of the path with CUDA events on
- * the caller's stream (events only; no synchronisation, no change to the kernels).  Phases:
+ * the caller's stream (events only; no synchronisation, no change to the kernels; error_sweep runs its stages back to
+ * back on the caller's stream, as with FMM_FLAG_SWEEP_SERIAL).  Phases:
  *   0 encode A   1 encode B (incl. the transpose of a K x N operand)   2 block products (scheme)
  *   3 decode (+ error reduction)   4 block products of classical_gemm   5 everything else.
  * fmm_profile_collect synchronises the recorded events, adds their durations (milliseconds) to ms[8]

@@ -826,7 +826,7 @@ fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P
   const fmm_scheme* grid = level == 1 ? base->outer.get() : base;
   const int gm = grid->m, gk = grid->k, gn = grid->n;
   const bool serial = g_prof_on || (d->flags & FMM_FLAG_SWEEP_SERIAL) != 0;
-  const bool many = !serial && sweep_many_ok(base, d);
+  const bool many = sweep_many_ok(base, d);     // on the caller's stream alone: the same kernels and sums with and without `serial`
   // every gauge matrix is checked before the first launch: a singular one returns with nothing enqueued
   const size_t per_gauge = 2 * (size_t)(gm * gm + gk * gk + gn * gn);
   std::vector<double> packed;           // small blocks: coefficients and gauges for the device (launch_gauge_tables)
@@ -933,14 +933,20 @@ fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P
     const int64_t bm = d->M / base->m, bn = d->N / base->n, bk = d->K / base->k;
     const fmm_scheme* inner = level == 1 ? base->inner.get() : nullptr;
     const GaugeDims gd{gm, gk, gn, grid->R, inner ? inner->m : 1, inner ? inner->k : 1, inner ? inner->n : 1, inner ? inner->R : 1};
-    FMM_CUDA(cudaMemcpyAsync(mws + Lm.data, packed.data(), packed.size() * 8, cudaMemcpyHostToDevice, st));
-    FMM_CUDA(launch_gauge_tables(at<double>(mws, Lm.data), gd, G, d_tabs, st));
+    {
+      ProfScope ps(5, st);
+      FMM_CUDA(cudaMemcpyAsync(mws + Lm.data, packed.data(), packed.size() * 8, cudaMemcpyHostToDevice, st));
+      FMM_CUDA(launch_gauge_tables(at<double>(mws, Lm.data), gd, G, d_tabs, st));
+    }
     const EncodeManyJob ja{dA, d->lda, base->k, (int)bm, (int)bk, at<char>(mws, Lm.hat_a), L.g.sAhat, at<float>(mws, Lm.scale_a)};
     const EncodeManyJob jb{bk_ptr, bk_ld, base->k, (int)bn, (int)bk, at<char>(mws, Lm.hat_b), L.g.sBhat, at<float>(mws, Lm.scale_b)};
     const bool prod_bf16 = (d->flags & FMM_FLAG_PRODUCTS_BF16) != 0;
     for (int g = 0; g < G; g += Lm.copies) {
       const int copies = std::min(Lm.copies, G - g);
-      FMM_CUDA(launch_encode_many(d->storage, d->product, ja, jb, d_tabs + 3 * g, R, copies, mode, st));
+      {
+        ProfScope ps(0, st);
+        FMM_CUDA(launch_encode_many(d->storage, d->product, ja, jb, d_tabs + 3 * g, R, copies, mode, st));
+      }
       BlockProductArgs p{};
       p.product = d->product;
       p.A = ja.out; p.lda = bk; p.a_batch = L.g.sAhat;
@@ -950,7 +956,11 @@ fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P
       p.out_mode = prod_bf16 ? 1 : 0; p.output = prod_bf16 ? FMM_BF16 : FMM_F32;
       if (mode == 2) { p.row_scale = ja.scale; p.rs_batch = bm; p.col_scale = jb.scale; p.cs_batch = bn; }
       p.status = at<DeviceStatus>(gws, L.g.status);
-      FMM_TRY(launch_block_products(p, st));
+      {
+        ProfScope ps(2, st);
+        FMM_TRY(launch_block_products(p, st));
+      }
+      ProfScope ps(3, st);
       FMM_CUDA(launch_decode_many(d->output, p.out, prod_bf16 ? FMM_BF16 : FMM_F32, L.g.sProd, d_tabs + 3 * g, R, copies,
                                   mode == 1 ? ja.scale : nullptr, mode == 1 ? jb.scale : nullptr, base->m, base->n, bm, bn,
                                   cstar32, at<double>(mws, Lm.part) + (size_t)g * Lm.blocks, Lm.blocks, Lm.tpb, st));

@@ -1,7 +1,9 @@
-"""Sweeps on small blocks (many copies per launch) against the same call with its stages back to back: one copy at a time
-through the general kernels, tables built on the host.  Block sums, scales and products are the same operations in the same
-order, so two ratios differ by the order of their error sums alone: at most M N additions in fp32 per thread share, below
-64 roundings of 2^-24 in a square, half of that in its root; 1e-5 bounds it."""
+"""Sweeps on small blocks (many copies per launch, tables built on the device) against the same algorithms one at a time:
+gauge_apply on the host, scheme_gemm, classical_gemm, and the errors against the fp64 reference in fp64.  Block sums, scales,
+products and sums over the products are the same operations in the same order, so the results are the same bits and two
+ratios differ by the reference (its fp32 copy: 2^-24 of its norm) and by the fp32 sums of squares (at most 16 tiles of 16
+a thread, and the rounding of each square) alone.  The flags that choose among the general paths, and phase timing, change
+no bit."""
 import numpy as np
 import pytest
 import torch
@@ -40,17 +42,45 @@ def test_many_copies(name, level, M, K, N, G, storage, product, mode, weight, fl
     grid = (2, 2, 2) if level == 1 else s.dims[:3]
     P, Q, S = _gauges(grid, G, M + N)
 
+    O = "f32" if storage == "f32" else "bf16"
+
+    def desc(extra=0):
+        return lib.GemmDesc.make(M, K, N, storage, product, O, weight_layout=weight, scale_mode=mode, flags=flags | extra)
+
     def call(extra):
-        d = lib.GemmDesc.make(M, K, N, storage, product, "f32" if storage == "f32" else "bf16", weight_layout=weight,
-                              scale_mode=mode, flags=flags | extra)
+        d = desc(extra)
         ws = gu.workspace(lib.error_sweep_workspace(s, d, G))
         ws.fill_(0xFF)
         return lib.error_sweep(s, level, P, Q, S, d, At, Bt, ws)
 
     many, sm = call(0)
-    serial, ss = call(lib.FLAG_SWEEP_SERIAL)
-    assert np.all(np.isfinite(serial)) and np.all(np.abs(many - serial) <= 1e-5 * serial + 1e-12)
-    assert sm["e_classical_rel"] == ss["e_classical_rel"] and sm["norm_ref"] == ss["norm_ref"]
+    for extra in (lib.FLAG_SWEEP_SERIAL, lib.FLAG_SWEEP_UNFUSED):
+        other, so = call(extra)
+        assert np.array_equal(many, other) and sm == so
+    lib.profile_enable(True)
+    try:
+        timed, st = call(0)
+        lib.profile_collect()
+    finally:
+        lib.profile_enable(False)
+    assert np.array_equal(many, timed) and sm == st
+
+    d = desc()
+    Cs = torch.empty(M, N, dtype=torch.float64, device="cuda")
+    lib.exact_gemm_f64(d, At, Bt, Cs)
+    norm = Cs.norm().item()
+
+    def error_of(run, ws_bytes):
+        C = torch.empty(M, N, dtype=torch.float32 if O == "f32" else torch.bfloat16, device="cuda")
+        run(C, gu.workspace(ws_bytes))
+        return (C.double() - Cs).norm().item()
+
+    e_cl = error_of(lambda C, ws: lib.classical_gemm(d, At, Bt, C, ws), lib.classical_gemm_workspace(d))
+    for g in range(G):
+        sg = lib.gauge_apply(s, P[g], Q[g], S[g], level=level)
+        e = error_of(lambda C, ws: lib.scheme_gemm(sg, d, At, Bt, C, ws), lib.scheme_gemm_workspace(sg, d))
+        bound = 2.0 ** -24 * (norm / e + (16 * 16 + 4) / 2) + 1e-12
+        assert abs(many[g] * e_cl / e - 1) <= bound, (g, many[g], e / e_cl, bound)
 
 
 def test_singular_gauge_launches_nothing():
