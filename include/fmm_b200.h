@@ -320,8 +320,8 @@ size_t error_sweep_workspace(const fmm_scheme* base, const fmm_gemm_desc* d, int
  * count_gt2 counts the comparable ratios above 2.
  * Execution: equivalent algorithms share their operands, so up to eight of them (as many as fit the table limits:
  * products of the batch <= FMM_MAX_R) run as one encode, one product launch and one error-only decode.  On small
- * blocks (at most 128 x 128, 1024 inner indices, scale modes 0 to 2) up to 512 copies run that way, and their
- * coefficients are transformed on the device.  Every
+ * blocks (up to 128 x 64 x 128 or 8 x 1024 x 8 in any sweep, up to 128 x 1024 x 128 where copies are many; scale modes
+ * 0 to 2) up to 512 copies run that way, and their coefficients are transformed on the device.  Every
  * algorithm's arithmetic and summation order are those of a scheme_gemm call on it, and the call is bit-reproducible
  * run to run.                                                                                              */
 fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P, const double* Q,

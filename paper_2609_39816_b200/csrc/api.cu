@@ -523,14 +523,8 @@ bool merge_tables(const CoefTable* tabs, int kb, int R, CoefTable* mA, CoefTable
   return true;
 }
 
-// Sweeps on small blocks run many copies per launch (sweep_many.cu).  The line: every product is one tile of the product
-// kernel and a block sum is the work of one block of threads, so a copy alone is launch latency (40 us for six launches at
-// 128^3, two levels, against 1 us as one of a batch).  The model schedule's scales (mode 3) keep the general path.
+// Sweeps on small blocks run many copies per launch (sweep_many.cu).
 struct ManyLayout { size_t data, hat_a, hat_b, scale_a, scale_b, prod, part, total; int copies, blocks, tpb; };
-
-bool sweep_many_ok(const fmm_scheme* s, const fmm_gemm_desc* d) {
-  return d->M / s->m <= kManyRows && d->N / s->n <= kManyRows && d->K / s->k <= 1024 && d->scale_mode <= 2;
-}
 
 ManyLayout many_layout(const fmm_scheme* s, const fmm_gemm_desc* d, int G) {
   ManyLayout L{};
@@ -555,6 +549,21 @@ ManyLayout many_layout(const fmm_scheme* s, const fmm_gemm_desc* d, int G) {
   return L;
 }
 
+// The line between them.  A block sum is the work of one block of threads here, so a launch takes as long as one thread's
+// walk over a block; against it stand the launches (and tables built on the host) of the general path's batches that one
+// launch replaces.  Measured, sweeps of 1 to 256 copies, blocks of 4 x 1024 to 128 x 1024, scale modes 0, 1 and 2 (time here
+// over time there): up to 8192 elements a block one batch is at par (0.83 to 1.13); 128 x 256 is 1.02 to 1.41 for one
+// batch, 0.77 to 1.01 for two, 0.63 to 0.97 for four; 128 x 512 is 0.81 to 1.07 for eight of one-level Strassen, 0.47 to
+// 1.27 for sixteen of two-level (general gauges of the outer factor at the upper end), 0.35 to 0.85 for 128 and more;
+// 128 x 1024 is 1.3 to 1.7 for eight of one-level, 0.60 to 0.89 for 32, and 1.0 to 5.5 for two-level Strassen, of which a
+// launch holds three copies at most.  The model schedule's scales (mode 3) keep the general path.
+bool sweep_many_ok(const fmm_scheme* s, const fmm_gemm_desc* d, int G) {
+  const int64_t bm = d->M / s->m, bn = d->N / s->n, bk = d->K / s->k;
+  if (bm > kManyRows || bn > kManyRows || bk > 1024 || d->scale_mode > 2) return false;
+  const int64_t kb = sweep_batch(s), batches = (G + kb - 1) / kb, work = std::max(bm, bn) * bk;
+  return work <= (batches == 1 ? 8192 : std::max<int64_t>(32768, 8192 * batches)) && work <= 32768 * (int64_t)many_layout(s, d, G).copies;
+}
+
 struct SweepLayout {
   GemmLayout g; ClassicalLayout c;
   size_t gemm, gemm2, classical, cstar, cstar32, ccl, tables, sums, fpart, many, total;   // two GEMM workspaces: gauges are pipelined
@@ -576,7 +585,7 @@ SweepLayout sweep_layout(const fmm_scheme* s, const fmm_gemm_desc* d, int G) {
   L.sums = o; o += align_up((size_t)(G + 8) * 8);
   L.fpart = o; o += align_up((size_t)G * kFusedPartialsPerGauge * 8);
   L.many = o;
-  if (sweep_many_ok(s, d)) o += many_layout(s, d, G).total;
+  if (sweep_many_ok(s, d, G)) o += many_layout(s, d, G).total;
   L.total = o;
   return L;
 }
@@ -826,7 +835,7 @@ fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P
   const fmm_scheme* grid = level == 1 ? base->outer.get() : base;
   const int gm = grid->m, gk = grid->k, gn = grid->n;
   const bool serial = g_prof_on || (d->flags & FMM_FLAG_SWEEP_SERIAL) != 0;
-  const bool many = sweep_many_ok(base, d);     // on the caller's stream alone: the same kernels and sums with and without `serial`
+  const bool many = sweep_many_ok(base, d, G);     // on the caller's stream alone: the same kernels and sums with and without `serial`
   // every gauge matrix is checked before the first launch: a singular one returns with nothing enqueued
   const size_t per_gauge = 2 * (size_t)(gm * gm + gk * gk + gn * gn);
   std::vector<double> packed;           // small blocks: coefficients and gauges for the device (launch_gauge_tables)

@@ -24,11 +24,13 @@ CASES = [
     ("strassen444", 0, 128, 128, 128, 5, "f32", "e4m3", 2, False, 0),
     ("strassen444", 0, 64, 64, 64, 1, "f32", "e4m3", 1, False, 0),
     ("strassen444", 1, 20, 192, 160, 7, "bf16", "bf16", 0, True, 0),
-    ("strassen444", 1, 512, 4096, 512, 33, "bf16", "e4m3", 1, True, 0),      # largest blocks, more copies than one batch
+    ("strassen444", 1, 512, 1024, 512, 33, "bf16", "e4m3", 1, True, 0),      # 128 x 256 blocks, more copies than a launch holds
+    ("strassen222", 0, 256, 2048, 256, 136, "bf16", "e4m3", 1, True, 0),     # the largest blocks
     ("strassen444", 0, 4, 64, 32, 3, "f32", "bf16", 0, False, 2),            # one-row blocks, products rounded to bf16
     ("strassen222", 0, 256, 96, 208, 9, "f32", "bf16", 0, True, 0),
     ("strassen222", 0, 34, 64, 48, 2, "bf16", "e4m3", 2, True, 0),
-    ("classical111", 0, 128, 1024, 128, 2, "f32", "e4m3", 1, False, 0),
+    ("classical111", 0, 128, 64, 128, 2, "f32", "e4m3", 1, False, 0),
+    ("classical111", 0, 128, 1024, 128, 2, "f32", "e4m3", 1, False, 0),      # too large for two copies: the general path
 ]
 
 
@@ -81,6 +83,29 @@ def test_many_copies(name, level, M, K, N, G, storage, product, mode, weight, fl
         e = error_of(lambda C, ws: lib.scheme_gemm(sg, d, At, Bt, C, ws), lib.scheme_gemm_workspace(sg, d))
         bound = 2.0 ** -24 * (norm / e + (16 * 16 + 4) / 2) + 1e-12
         assert abs(many[g] * e_cl / e - 1) <= bound, (g, many[g], e / e_cl, bound)
+
+
+# encode launches of a sweep: one per launch of many copies, or one per batch of the general path
+@pytest.mark.parametrize("name,level,M,K,N,G,encodes", [
+    ("strassen444", 0, 128, 128, 128, 5, 1), ("strassen222", 0, 256, 128, 256, 8, 1),     # 8192 elements a block: any sweep
+    ("strassen222", 0, 256, 512, 256, 16, 1), ("strassen444", 1, 512, 2048, 512, 8, 2),   # four and eight times, more batches
+    ("strassen444", 1, 512, 2048, 512, 7, 7),                                             # 7 are too few for that
+    ("strassen444", 1, 512, 4096, 512, 4, 4), ("strassen222", 0, 256, 2048, 256, 16, 2),  # the largest blocks, few copies
+    ("strassen222", 0, 256, 2048, 256, 136, 6),                                           # and seventeen batches of copies
+])
+def test_line_between_the_paths(name, level, M, K, N, G, encodes):
+    lib = gu.fmm()
+    s = lib.scheme_builtin(name)
+    A, B = torch.randn(M, K, device="cuda").bfloat16(), torch.randn(N, K, device="cuda").bfloat16()
+    P, Q, S = _gauges((2, 2, 2), G, 1) if level else _gauges(s.dims[:3], G, 1)
+    d = lib.GemmDesc.make(M, K, N, "bf16", "e4m3", "bf16", weight_layout=True, scale_mode=1)
+    ws = gu.workspace(lib.error_sweep_workspace(s, d, G))
+    lib.profile_enable(True)
+    try:
+        lib.error_sweep(s, level, P, Q, S, d, A, B, ws)
+        assert lib.profile_collect()["encode_a"][1] == encodes
+    finally:
+        lib.profile_enable(False)
 
 
 def test_singular_gauge_launches_nothing():
