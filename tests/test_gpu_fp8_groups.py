@@ -21,7 +21,7 @@ def _codes(x, rows):
     return (q.double() * s.double()).view(pad.shape)[:M, :K]
 
 
-@pytest.mark.parametrize("M,K,N", [(130, 8192, 136), (129, 8320, 264), (4, 16, 8), (1664, 272, 1800)])
+@pytest.mark.parametrize("M,K,N", [(130, 8192, 136), (129, 8320, 264), (4, 16, 8), (1664, 272, 1800), (1664, 8336, 1800)])
 def test_group_gemm(M, K, N):
     lib = gu.fmm()
     gen = torch.Generator(device="cuda").manual_seed(K)
