@@ -37,7 +37,8 @@ __device__ __forceinline__ float4 load_quad(const __nv_bfloat16* p) {
   return staged_quad(reinterpret_cast<const unsigned char*>(&raw), p);
 }
 
-// kErr: the squared error against cstar32 instead of the result, one partial sum per block of threads
+// kErr: the squared error against cstar32 instead of the result, one partial sum per block of threads; sixteen squares (a row
+// of cells) are added in fp32, those sums in fp64
 template <typename OutT, typename ProdT, bool kErr, bool kDense>
 __global__ void __launch_bounds__(kPatThreads, 4)
 decode_pattern_kernel(const ProdT* __restrict__ prod, int64_t rstride, const __grid_constant__ PatCoefs coefs,
@@ -55,7 +56,7 @@ decode_pattern_kernel(const ProdT* __restrict__ prod, int64_t rstride, const __g
   });
   __syncthreads();
   const int vpr = bn >> 2, nvec = bm * vpr;
-  float err = 0.0f;
+  double total = 0.0;
 #pragma unroll 1
   for (int s = 0; s < steps; ++s) {
     const int idx = (blockIdx.x * steps + s) * kPatThreads + tid;
@@ -76,6 +77,7 @@ decode_pattern_kernel(const ProdT* __restrict__ prod, int64_t rstride, const __g
       });
     });
     const int64_t ld = kErr ? 4 * (int64_t)bn : ldc;
+    float err = 0.0f;
 #pragma unroll
     for (int c = 0; c < kCells; ++c) {
       const int64_t at = ((int64_t)(c / 4) * bm + p) * ld + (int64_t)(c % 4) * bn + q;
@@ -86,13 +88,14 @@ decode_pattern_kernel(const ProdT* __restrict__ prod, int64_t rstride, const __g
         const float d2 = round_out(x.z, (OutT*)nullptr) - cs.z, d3 = round_out(x.w, (OutT*)nullptr) - cs.w;
         err = __fmaf_rn(d0, d0, err); err = __fmaf_rn(d1, d1, err);
         err = __fmaf_rn(d2, d2, err); err = __fmaf_rn(d3, d3, err);
+        if (c % 4 == 3) { total += (double)err; err = 0.0f; }
       } else {
         store4(C + at, x);
       }
     }
   }
   if constexpr (kErr) {
-    const double tot = block_sum_double((double)err, red);
+    const double tot = block_sum_double(total, red);
     if (tid == 0) partials[blockIdx.x] = tot;
   }
 }

@@ -446,7 +446,9 @@ __device__ __forceinline__ float4 staged_quad(const unsigned char* p, const __nv
   return make_float4(__low2float(lo), __high2float(lo), __low2float(hi), __high2float(hi));
 }
 
-template <typename OutT, bool kStore, bool kErr, int kDecSplit, typename ProdT>
+// kFold: a thread's error sum goes to fp64 after every tile (its share of a tile is at most sixteen squares), for launches
+// whose blocks walk many tiles
+template <typename OutT, bool kStore, bool kErr, int kDecSplit, typename ProdT, bool kFold = false>
 __device__ __forceinline__ void decode_body(const StreamRole role, unsigned char* smem_raw, const ProdT* __restrict__ prod, const CoefTable* __restrict__ d_tab, int R,
               const float* __restrict__ sA, const float* __restrict__ sB, int n, int64_t bm, int64_t bn,
               OutT* __restrict__ C, int64_t ldc, const float* __restrict__ cstar32, int64_t ldcs,
@@ -488,12 +490,14 @@ __device__ __forceinline__ void decode_body(const StreamRole role, unsigned char
   const int64_t cs_src = (int64_t)(g / n) * bm * ldcs + (int64_t)(g % n) * bn;
 
   float err = 0.0f;
+  double folded = 0.0;
   for (int it = 0; it < tiles_per_block; ++it) {
     const int idx = (role.bid * tiles_per_block + it) * kDecPos + pq;
     const bool live = idx < nvec;
     const int p = live ? idx / vec_per_row : 0;
     const int q = live ? (idx - p * vec_per_row) << 2 : 0;
     if (it > 0) role.sync();               // previous tile's readers are done with the stage
+    if (kFold) { folded += (double)err; err = 0.0f; }
     {
       const ProdT* src = prod + (int64_t)p * bn + q;
       const int nbytes = live ? kVecBytes : 0;  // 0 source bytes -> the destination bytes are zero-filled
@@ -567,11 +571,11 @@ __device__ __forceinline__ void decode_body(const StreamRole role, unsigned char
   }
   if (kErr) {
     if (gauges == 1) {
-      const double tot = block_sum_double(role, (double)err, sm.red);
+      const double tot = block_sum_double(role, folded + (double)err, sm.red);
       if (role.tid == 0) partials[role.bid] = tot;
     } else {
       // one sum per algorithm: warps with the same (g % gauges); partials laid out [algorithm][block]
-      double v = (double)err;
+      double v = folded + (double)err;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
       const int warp = role.tid >> 5;

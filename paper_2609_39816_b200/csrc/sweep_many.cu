@@ -205,7 +205,7 @@ decode_many_kernel(const ProdT* __restrict__ prod, const CoefTable* __restrict__
   const size_t copy = blockIdx.y;
   const float* a = sA ? sA + copy * R : nullptr;
   const float* b = sB ? sB + copy * R : nullptr;
-  decode_body<OutT, false, true, 4, ProdT>(StreamRole{(int)threadIdx.x, (int)blockIdx.x, (int)gridDim.x, 0}, smem_raw,
+  decode_body<OutT, false, true, 4, ProdT, true>(StreamRole{(int)threadIdx.x, (int)blockIdx.x, (int)gridDim.x, 0}, smem_raw,
                                            prod + copy * R * rstride, tabs + 3 * copy + 2, R, a, b, n, bm, bn, nullptr, 0,
                                            cstar32, n * bn, partials + copy * gridDim.x, tiles_per_block, rstride, 1);
 }
