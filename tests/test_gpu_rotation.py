@@ -144,3 +144,32 @@ def test_rotation_experiment_on_the_device(lib):
         want_plain, want_rot = gold[case]
         assert abs(plain - want_plain) < 0.10 * want_plain and abs(rot - want_rot) < 0.06 * want_rot, (case, plain, rot)
         assert (rot < plain) == (case == "uniform_offset")
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("rows,K,h", [(3001, 13824, 128), (2999, 13824, 512), (4097, 1344, 64), (24001, 5 * 1024, 1024), (9001, 11 * 256, 256),
+                                      (40001, 7 * 16, 16)])
+def test_many_passes_on_odd_numbers_of_blocks(lib, dtype, rows, K, h):
+    """Operands of several passes a warp whose rows are no power of two of blocks long, so that a pass ends inside a row and
+    a lane's columns and signs have to hold for all of its rows; padded leading dimensions, out of place and in place.  Every
+    element against the transform in fp64 on the device, under the bound of this file's head."""
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    T = torch.float32 if dtype == "f32" else torch.bfloat16
+    X = torch.randn(rows, K + 8, device="cuda", generator=g).to(T)
+    signs = (torch.randint(0, 2, (K,), device="cuda", generator=g) * 2 - 1).to(torch.int8)
+    out = torch.full((rows, K + 24), 7.0, dtype=T, device="cuda")
+    lib.hadamard_rotate(X[:, :K], signs, h, out=out[:, :K])
+    assert bool((out[:, K:] == 7.0).all())
+    for r0 in range(0, rows, 4096):            # in slices: the reference is fp64
+        x = X[r0:r0 + 4096, :K].double() * signs
+        blk = x.reshape(-1, h).norm(dim=1).repeat_interleave(h).view(x.shape)
+        v, stride = x.reshape(-1, h), 1
+        while stride < h:
+            a, b = v.view(-1, h // (2 * stride), 2, stride).unbind(2)
+            v = torch.stack([a + b, a - b], dim=2).reshape(-1, h)
+            stride *= 2
+        want = (v / math.sqrt(h)).view(x.shape)
+        bound = (math.log2(h) + 2) * 2.0 ** -24 * blk + (2.0 ** -22 if dtype == "f32" else 2.0 ** -8) * want.abs()
+        assert bool(((out[r0:r0 + 4096, :K].double() - want).abs() <= bound).all())
+    lib.hadamard_rotate(X[:, :K], signs, h, out=X[:, :K])
+    assert torch.equal(X[:, :K], out[:, :K])
