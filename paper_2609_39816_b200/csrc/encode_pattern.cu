@@ -45,7 +45,7 @@ struct PatCoefs { float a[kMaxEntries], b[kMaxEntries]; };
 
 struct PatJob {
   const void* X; int64_t ldx; int br, bc; void* out; int64_t rstride;
-  unsigned* amax_bits; float* scale_out; const float* pre_scale; int evict_first; int blocks;
+  unsigned* amax_bits; float* scale_out; int evict_first; int blocks;
 };
 
 enum PatPass { kPlain, kAmax, kScaled, kGroupAmax, kGroupScaled };
@@ -130,7 +130,7 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
     if (tid < kProducts) {
       const float s = pow2_scale_448(__uint_as_float(j.amax_bits[tid])), inv = 1.0f / s;   // s: at most 2^120
       sm.factor[tid] = isfinite(inv) ? make_float2(inv, 1.0f) : make_float2(0x1p127f, 0x1p-127f / s);
-      if (bid == 0 && j.scale_out) j.scale_out[tid] = j.pre_scale ? s * j.pre_scale[0] : s;   // powers of two: exact
+      if (bid == 0 && j.scale_out) j.scale_out[tid] = s;
     }
     __syncthreads();
   }
@@ -277,7 +277,7 @@ bool matches(const CoefTable& t, const Pattern& p, float* coefs) {
 
 PatJob make_pat_job(const EncodeOperand& o, int dst_bytes) {
   const bool evict = (int64_t)o.h_tab->R * o.out_stride * dst_bytes > ((int64_t)48 << 20);   // as encode_kernel
-  return PatJob{o.X, o.ldx, (int)o.br, (int)o.bc, o.out, o.out_stride, o.amax_bits, o.scale, o.pre_scale, evict ? 1 : 0, 0};
+  return PatJob{o.X, o.ldx, (int)o.br, (int)o.bc, o.out, o.out_stride, o.amax_bits, o.scale, evict ? 1 : 0, 0};
 }
 
 int pat_blocks(const PatJob& j, int pass) {
