@@ -2,7 +2,9 @@
 // position.  It walks the 49 products in order, one 16-byte load each, and adds a product to the two to four cells (up to
 // eight for a general outer gauge) that it feeds, whose fp32 sums stay in registers: the multiply-add chains of
 // decode_kernel in the same order, without its staging in shared memory, its barriers and its table walk.
-// What bounds it: reading the products; the loads of the products ahead are in flight while one is added.
+// What bounds it: reading the products; the loads of the products ahead are in flight while one is added (4096^3: 43 us,
+// 239 MB at 5.5 TB/s).  It stores results of the scheme and its sign variants, and adds up errors of these and of general
+// gauges of the outer factor from fp32 products; a general gauge's result and errors of bf16 products stay with decode_kernel.
 #include <cstring>
 
 #include "kernels_stream.cuh"

@@ -6,9 +6,10 @@
 // no table walk, no staging in shared memory, no unpacking per list entry.  The sums are encode_kernel's: the same fp32
 // multiply-add chains in the same order (its padding entries, zero times zero, are left out: they add nothing), the same
 // scales and roundings.
-// What bounds it: the writes of the plain bf16 pass, instruction issue elsewhere.  The code is straight, 49 products long for
-// each operand, so everything rare is kept out of it: with the exact divisions inline the warps waited for
-// instructions (12 of them per issue) and the scaled pass took 219 us instead of 93 at the sizes below.
+// What bounds it: the writes of the plain bf16 pass, instruction issue elsewhere.  Both operands, kernel times: bf16 at 4096^3
+// 42 us (272 MB, 6.5 TB/s); e4m3 with a scale per block sum at 2048 x 4096 x 12288 56 us for the maxima and 73 for the codes;
+// model schedule at 2048 x 11008 x 4096 79 and 189 us.  The code is straight, 49 products long for each operand, so everything
+// rare is kept out of it: with the exact divisions inline the model schedule's codes take 206 us.
 //
 // With scales on groups of 128 inner indices (scale mode 3) the 32 lanes of a warp hold one group: they find its largest
 // magnitude by shuffles (A) or one reduction per block of threads (B), and keep the group's 49 scales between them.
@@ -49,8 +50,8 @@ struct PatJob {
 };
 
 enum PatPass { kPlain, kAmax, kScaled, kGroupAmax, kGroupScaled };
-// blocks per SM that the register allocation aims at: measured 97 / 83 / 79 us (4 / 5 / 6) for kGroupAmax, 198 / 183 / 184 for
-// kGroupScaled, within 3 % elsewhere
+// blocks per SM that the register allocation aims at: at the sizes above, 4 / 5 / 6 give 95 / 82 / 79 us for kGroupAmax,
+// 207 / 190 / 192 for kGroupScaled, 41 / 41 / 43 for kPlain, and differ by 1 % in the other two
 constexpr int pat_blocks_per_sm(int pass) { return pass == kGroupAmax ? 6 : pass == kPlain ? 4 : 5; }
 
 constexpr int E = 4, NP = 2;          // values of a thread: 16 cells x 4 fp32 registers
@@ -295,8 +296,9 @@ cudaError_t launch_pass(PatJob a, PatJob b, bool have_a, bool have_b, const PatC
   return cudaGetLastError();
 }
 
-// Which (types, pattern, mode) have a kernel: what the library's own schemes, schedules and sweeps use; the rest stays with
-// encode_kernel.  kGroups: the model schedule's passes too.
+// Which (types, pattern, mode) have a kernel: bf16 without scales and e4m3 with a scale per block sum, both patterns; the model
+// schedule for the scheme and its sign variants (kGroups).  The rest (scale mode 2, e4m3 without scales, the model schedule
+// under a general gauge of the outer factor) stays with encode_kernel.
 template <typename SrcT, typename DstT, bool kDense, bool kGroups>
 bool run_pattern(const PatJob& a, const PatJob& b, bool have_a, bool have_b, const PatCoefs& c, int mode, void* clear,
                  size_t clear_bytes, cudaStream_t st, cudaError_t* e) {

@@ -577,7 +577,7 @@ cudaError_t launch_exact_t(const T* A, int64_t lda, const T* B, int64_t ldb, int
   // Blocks of one tile: the number that leaves the busiest SM the least work.  A share's fill and exchange count as 64
   // inner indices, and a block alone on its SM runs at three quarters of the pipe.  Measured, one block a tile against the
   // chosen split: 2048 x 3456 x 1280 763 -> 578 us (2), 300 x 4096 x 500 243 -> 71 us (8), 512 x 1024 x 1024 68 -> 52 us (2),
-  // 128^3 16 -> 11 us (8); 2048 x 4096 x 4096 stays whole at 2.06 ms (33.4 TFLOP/s, the fp64 tensor pipe 90 % busy).
+  // 128^3 16 -> 11 us (8); 2048 x 4096 x 4096 stays whole at 2.06 ms (33.4 TFLOP/s, the fp64 tensor pipe 92 % busy).
   int split = 1;
   int64_t least = INT64_MAX;
   for (int c = 1; c <= 8 && (c == 1 || K >= (int64_t)c * kExK); c *= 2) {

@@ -69,8 +69,8 @@ __device__ __forceinline__ void store_pair(float2 x, __nv_bfloat16* y) {
 // E elements per lane, L = h / E lanes per h-block (a power of two <= 32), 32 / L blocks per warp pass.  The number of warps W
 // is chosen so that W passes are a whole number of rows: a lane then stays in its columns, its signs become mask words once
 // and for all, and a step is a constant distance in X and Y.  A warp keeps the loads of its next kAhead passes in flight
-// while it transforms one.  8192 x 13824 bf16: h = 128 100 -> 87 us (5.2 TB/s), h = 64 113 -> 95, h = 512 124 -> 113, against
-// passes that worked out their position and signs and loaded before they transformed.  What bounds it now: the lane
+// while it transforms one.  8192 x 13824 bf16, L2 flushed before each: h = 128 102 -> 90 us (5.0 TB/s), h = 64 116 -> 100,
+// h = 512 126 -> 115, against passes that worked out their position and signs and loaded before they transformed.  What bounds it now: the lane
 // exchanges (48 shuffles for 16 values a lane at h = 128) beside the memory system.
 template <typename T, int E, int kAhead>
 __global__ void __launch_bounds__(kRotThreads)
@@ -160,7 +160,7 @@ cudaError_t launch_rotate(const void* X, int64_t ldx, int64_t rows, int64_t K, i
   if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return cudaErrorInvalidDevice;
   // as many warps as run at once (24 or 32 an SM by the registers): with a few more, the last of them run alone (bf16, h = 128,
-  // 24 fit: 87 us at 24, 97 at 32)
+  // 24 fit: a tenth slower at 32)
   static const int blocks_per_sm = [] {
     int n = 0;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, hadamard_rotate_kernel<T, E, kAhead>, kRotThreads, 0) == cudaSuccess && n > 0 ? n : 1;

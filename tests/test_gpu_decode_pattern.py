@@ -36,3 +36,34 @@ def test_decode_of_the_products(M, K, N, output, product, mode, flags):
     size = np.einsum("rij,rpq->ipjq", np.abs(w), np.abs(P)).reshape(M, N)
     bound = 16 * 2.0 ** -24 * size + (2.0 ** -8 * np.abs(want) * 1.01 if output == "bf16" else 0.0)
     assert np.all(np.abs(C.double().cpu().numpy() - want) <= bound + 1e-30)
+
+
+@pytest.mark.parametrize("product,mode", [("bf16", 0), ("e4m3", 1)])
+@pytest.mark.parametrize("level", [0, 1])
+@pytest.mark.parametrize("M,K,N", [(2308, 64, 2336), (1036, 128, 1056)])
+def test_error_sums_of_the_products(M, K, N, level, product, mode):
+    """The error form, sparse (sign gauges) and dense (general gauges of the outer factor), where a block of threads walks
+    two tiles and its last one is partial (577 x 584 blocks), and one tile: ratios against scheme_gemm on the gauged handle,
+    its squared error in fp64.  They differ by the reference's fp32 copy, 2^-24 of its norm, and by fp32 sums of sixteen
+    squares."""
+    lib = gu.fmm()
+    s = lib.scheme_builtin("strassen444")
+    A, _ = gu.storage_pair(gen.activations_outlier(4, 1, M, K, frac=0.05, factor=30.0), "bf16")
+    W, _ = gu.storage_pair(np.ascontiguousarray(gen.weights(4, 2, K, N).T), "bf16")
+    rng = np.random.default_rng(M)
+    if level == 0:
+        P, Q, S = (np.stack([np.eye(4), np.diag(rng.choice([-1.0, 1.0], 4))]) for _ in range(3))
+    else:
+        P, Q, S = (np.stack([np.eye(2), rng.standard_normal((2, 2)) + 2 * np.eye(2)]) for _ in range(3))
+    d = lib.GemmDesc.make(M, K, N, "bf16", product, "bf16", weight_layout=True, scale_mode=mode)
+    Cs = torch.empty(M, N, dtype=torch.float64, device="cuda")
+    lib.exact_gemm_f64(d, A, W, Cs)
+    ratios, summ = lib.error_sweep(s, level, P, Q, S, d, A, W, gu.workspace(lib.error_sweep_workspace(s, d, 2)), Cstar=Cs)
+    norm = Cs.norm().item()
+    for g in range(2):
+        sg = lib.gauge_apply(s, P[g], Q[g], S[g], level=level)
+        C = torch.empty(M, N, dtype=torch.bfloat16, device="cuda")
+        lib.scheme_gemm(sg, d, A, W, C, gu.workspace(lib.scheme_gemm_workspace(sg, d)))
+        e = (C.double() - Cs).norm().item()
+        bound = 2.0 ** -24 * (norm / e + (16 + 4) / 2) + 1e-12
+        assert abs(ratios[g] * summ["e_classical_rel"] * norm / e - 1) <= bound
