@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <mutex>
@@ -145,6 +146,8 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&v)[16]) {
                  "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
                : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t (&v)[16]) { tc_ld16(taddr, v); }
+__device__ __forceinline__ void tc_ld(uint32_t taddr, uint32_t (&v)[32]) { tc_ld32(taddr, v); }
 // these waits name the registers of the loads that they complete: no use of them can be scheduled before
 __device__ __forceinline__ void tc_wait_ld16(uint32_t (&v)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
@@ -158,6 +161,9 @@ __device__ __forceinline__ void tc_wait_ld32(uint32_t (&v)[32]) {
                  "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]),
                  "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31]) :: "memory");
 }
+
+__device__ __forceinline__ void tc_wait_ld(uint32_t (&v)[16]) { tc_wait_ld16(v); }
+__device__ __forceinline__ void tc_wait_ld(uint32_t (&v)[32]) { tc_wait_ld32(v); }
 
 // Shared-memory matrix descriptor of a K-major tile stored as rows of 128 bytes with the 128-byte
 // swizzle (what TMA writes with CU_TENSOR_MAP_SWIZZLE_128B): start address (>>4), leading byte offset
@@ -979,64 +985,167 @@ fmm_status launch_fused_t(const FusedSweepArgs& f, cudaStream_t st) {
 }
 
 
-// ---------------------------------------------------------------- group-scaled int8 GEMM
-// The classical int8 operator of the quantisation specification (Appendix D) as one kernel:
-//     C[t][j] = rnd_O( sum over groups g, ascending, of (float(P_g[t][j]) * dA[t][g]) * dB[j][g] ),
-//     P_g = exact integer product of the int8 codes of group g (128 inner indices).
-// One CTA owns a 128 x 128 output tile.  Warp 0 streams, per group, the 128 x 128-byte code tiles of A and B (one
-// 128-byte swizzle span = one group) through a shared-memory ring; one lane of warp 1 issues four tcgen05.mma
-// kind::i8 (K = 32 each) per group into one of two int32 accumulator buffers in TMEM, a FRESH accumulator per group;
-// warps 2-5 read the finished group's accumulator, convert it exactly to fp32, apply the two scales with two separate
-// roundings, and add to 128 fp32 accumulators per thread (one output row each); after the last group one rounding to
-// the output dtype.  The MMA of group g+1 overlaps the rescale of group g.
-struct Int8Layout {
-  static constexpr int BN = 128;
-  static constexpr int kStages = 4;
-  static constexpr int kABytes = BM * BKB;
-  static constexpr int kBBytes = BN * BKB;
-  static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kBarBytes = 256;
-  static constexpr int kMaxGroupsStaged = 64;                 // column scales of a tile staged in shared memory up to this many groups
-  static constexpr int kScaleBytes = kMaxGroupsStaged * BN * 4;
-  static constexpr int kTotal = kStages * kStageBytes + kBarBytes + kScaleBytes + 1024;
+// ---------------------------------------------------------------- group-scaled GEMMs: common parts
+// Three kernels whose scales change every 128 inner indices: the classical int8 operator, the block products of the model
+// schedule (e4m3) and the certified int8 realisation (int8_certified.inc).  Every group has an accumulator of its own in
+// TMEM; sixteen rescale warps read it, scale it and add it to fp32 sums in registers, in ascending group order, while the
+// MMAs of the next groups run.  Two forms:
+//   single  one CTA per 128 x 128 tile, four accumulators, 32 columns a rescale warp;
+//   pair    two CTAs per 256 x 256 tile (cta_group::2; a CTA's TMEM holds its 128 rows), two accumulators of 256 columns,
+//           64 columns a warp: what a group costs a warp whatever its width (the wait, the vote, the hand-back, the scales)
+//           is paid once for twice the columns, and a CTA copies half the operand bytes per output.
+template <bool kPair> struct GroupShape {
+  static constexpr int kRows = kPair ? 2 * BM : BM;   // rows of a tile
+  static constexpr int BN = kPair ? 256 : 128;        // columns of a tile
+  static constexpr int kAcc = 512 / BN;               // accumulators: all of TMEM
+  static constexpr int PN = BN / 4;                   // columns of a rescale warp
+  static constexpr int kUnits = kPair ? 2 : 1;        // CTAs of a tile
+  static constexpr int kLoad = kPair ? 16 : 32;       // columns of a TMEM load: with 64 sums a thread, 32 more spill
 };
-
-struct Int8Params {
-  int M, N, G;                  // rows of A, rows of B (= output columns), groups of 128 along K
-  int tiles_m, tiles_n;
-  long long ldc;
-  int out_bf16;
-  int wide;                     // every output row starts on a 32-byte boundary
-  const float* dAt;             // [G][M] row scales, group-major
-  const float* dBt;             // [G][N] column scales, group-major
-  unsigned long long wait_limit_ns;
-};
-
-__device__ __forceinline__ void tc_mma_i8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
+constexpr int kRescaleWarps = 16;    // four per TMEM lane quarter
+// Warps before the rescale warps: copies and MMA.  kMove: a whole warpgroup of them, so that registers can move from it to the
+// rescale warps (20 warps start with 96 each: 128 x 32 + 512 x 112 = 640 x 96).
+template <bool kMove> constexpr int kFirstRescale = kMove ? 4 : 2;
+template <bool kMove> constexpr int kGroupThreads = 32 * (kFirstRescale<kMove> + kRescaleWarps);
+template <bool kMove> __device__ __forceinline__ void more_registers() {
+  if constexpr (kMove) asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
+}
+template <bool kMove> __device__ __forceinline__ void fewer_registers() {
+  if constexpr (kMove) asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
 }
 
-// Packed fp32 pairs (__fmul2_rn, __fadd2_rn): each lane one IEEE operation.  Measured on this toolchain: a packed
-// multiply followed by a packed add IS merged into a packed fused multiply-add, even when both are written with an
-// explicit rounding mode, so the accumulation that must round twice (product, then sum) uses scalar __fadd_rn; the
-// packed forms are used only where merging is impossible (multiply after multiply) or harmless (an exact subtraction).
-constexpr int kInt8Threads = 576;   // 18 warps: TMA, MMA, and 16 rescale warps (four per TMEM lane quarter, 32 columns each)
+// Barrier block behind the ring; in a pair `full` and `tempty` are used in the leader only.
+template <int kStages, int kAcc> struct GroupBars {
+  uint32_t base;
+  __device__ __forceinline__ uint32_t full(int s) const { return base + 8u * s; }                        // a ring stage has landed
+  __device__ __forceinline__ uint32_t empty(int s) const { return base + 8u * (kStages + s); }           // and has been read
+  __device__ __forceinline__ uint32_t tfull(int b) const { return base + 8u * (2 * kStages + b); }       // an accumulator is complete
+  __device__ __forceinline__ uint32_t tempty(int b) const { return base + 8u * (2 * kStages + kAcc + b); }   // and in registers
+  __device__ __forceinline__ uint32_t drain() const { return base + 8u * (2 * kStages + 2 * kAcc); }
+  __device__ __forceinline__ uint32_t sfull(int b) const { return drain() + 8u * (1 + b); }              // a tile's scales are staged
+  __device__ __forceinline__ uint32_t sempty(int b) const { return drain() + 8u * (3 + b); }             // and no longer read
+  static constexpr int kSlot = 8 * (2 * kStages + 2 * kAcc + 5);                                         // TMEM base, abort flag
+  static constexpr int kBytes = kSlot + 16;
+};
 
-// The MMA role of the group-scaled kernels (warp 1): four MMAs of K = 32 bytes per group of 128 into a fresh accumulator.  All
-// lanes run the loop with warp-uniform control flow and one elected lane issues.
-template <int kAcc, typename L, typename Mma>
-__device__ __forceinline__ void group_mma_loop(const int total_tiles, const int G, unsigned char* smem, const uint32_t bar_base,
-                                               const uint32_t tmem_base, volatile int* abort_flag, DeviceStatus* status,
-                                               const unsigned long long limit, const int where_full, const int where_empty, const Mma mma) {
-  auto full_bar = [&](int s) { return bar_base + 8u * s; };
-  auto empty_bar = [&](int s) { return bar_base + 8u * (L::kStages + s); };
-  auto tfull_bar = [&](int b) { return bar_base + 8u * (2 * L::kStages + b); };
-  auto tempty_bar = [&](int b) { return bar_base + 8u * (2 * L::kStages + kAcc + b); };
-  const uint32_t drain_bar = bar_base + 8u * (2 * L::kStages + 2 * kAcc);
+template <bool kPair> __device__ __forceinline__ void group_commit(uint32_t bar) {
+  if constexpr (kPair) tc_commit_pair(bar);
+  else tc_commit(bar);
+}
+// an arrival on a barrier that a pair keeps in its leader
+template <bool kPair> __device__ __forceinline__ void group_arrive(uint32_t bar) {
+  if constexpr (kPair) mbar_arrive_cluster(bar & kPeerBitMask);
+  else mbar_arrive(bar);
+}
+
+// Barriers, TMEM (all 512 columns) and the synchronisation that makes them visible; every thread calls it.
+template <bool kPair, int kStages, int kAcc>
+__device__ __forceinline__ uint32_t group_setup(const GroupBars<kStages, kAcc> b, unsigned char* bar_mem, const int warp) {
+  uint32_t* slot = reinterpret_cast<uint32_t*>(bar_mem + GroupBars<kStages, kAcc>::kSlot);
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) { mbar_init(b.full(s), 1); mbar_init(b.empty(s), 1); }
+    for (int a = 0; a < kAcc; ++a) { mbar_init(b.tfull(a), 1); mbar_init(b.tempty(a), GroupShape<kPair>::kUnits * kRescaleWarps); }
+    mbar_init(b.drain(), 1);
+    for (int i = 0; i < 2; ++i) { mbar_init(b.sfull(i), kRescaleWarps); mbar_init(b.sempty(i), kRescaleWarps); }
+    reinterpret_cast<volatile int*>(slot)[2] = 0;         // abort flag
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    if constexpr (kPair) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(512u) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(512u) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if constexpr (kPair) cluster_sync_all();      // both CTAs' barriers are initialised before anything signals across the pair
+  tc_fence_after();
+  return *slot;
+}
+template <bool kPair> __device__ __forceinline__ void group_teardown(const uint32_t tmem_base, const int warp) {
+  tc_fence_before();
+  __syncthreads();
+  if constexpr (kPair) cluster_sync_all();      // neither CTA frees TMEM or leaves while its partner may still touch it
+  if (warp == 1) {
+    tc_fence_after();
+    if constexpr (kPair) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+  }
+}
+
+// a commit that arrives in this CTA alone
+template <bool kPair> __device__ __forceinline__ void commit_here(uint32_t bar) {
+  if constexpr (kPair) asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+  else tc_commit(bar);
+}
+// bounded wait (20 ms) for a barrier's first phase
+__device__ __forceinline__ void wait_drained(uint32_t bar) {
+  const unsigned long long t0 = global_timer_ns();
+  while (!mbar_try_wait(bar, 0)) {
+    if (global_timer_ns() - t0 > 20000000ull) break;
+  }
+}
+
+// bounded wait for the most recent fill of every stage (those that were issued land before shared memory goes away)
+template <int kStages, int kAcc>
+__device__ __forceinline__ void drain_ring(const GroupBars<kStages, kAcc> b, const int stage, const uint32_t phase) {
+  for (int s = 0; s < kStages; ++s) {
+    const uint32_t last_parity = (s < stage) ? phase : (phase ^ 1u);
+    const unsigned long long t0 = global_timer_ns();
+    while (!mbar_try_wait(b.full(s), last_parity)) {
+      if (global_timer_ns() - t0 > 20000000ull) break;  // 20 ms
+    }
+  }
+}
+
+// The copies of the kernels whose operands are K-major code matrices (one lane of warp 0): per group a 128-row x 128-byte
+// tile of A and of B (in a pair this CTA's rows of A and its half of the tile's rows of B) into the ring.
+// at(tile, &row_a, &row_b, &batch): first rows of the tile.
+template <bool kPair, typename L, typename At>
+__device__ __forceinline__ void group_copy_loop(const CUtensorMap& map_a, const CUtensorMap& map_b, const int first, const int stride,
+                                                const int total_tiles, const int G, unsigned char* smem,
+                                                const GroupBars<L::kStages, GroupShape<kPair>::kAcc> b, const uint32_t rank,
+                                                volatile int* abort_flag, DeviceStatus* status, const unsigned long long limit,
+                                                const int where, const At at) {
+  int stage = 0;
+  uint32_t phase = 0;
+  bool ok = true;
+  for (int tile = first; tile < total_tiles && ok; tile += stride) {
+    int row_a, row_b, r;
+    at(tile, &row_a, &row_b, &r);
+    for (int g = 0; g < G; ++g) {
+      ok = mbar_wait(b.empty(stage), phase ^ 1u, abort_flag, where, status, limit);
+      if (!ok) break;
+      const uint32_t sa = smem_u32(smem + stage * L::kStageBytes);
+      if constexpr (kPair) {      // both CTAs' copies complete on the leader's barrier
+        const uint32_t lead_full = b.full(stage) & kPeerBitMask;
+        if (rank == 0) mbar_arrive_expect_tx(b.full(stage), 2u * (uint32_t)L::kStageBytes);
+        tma_load_3d_pair(sa, &map_a, lead_full, g * BKB, row_a + (int)rank * BM, r);
+        tma_load_3d_pair(sa + L::kABytes, &map_b, lead_full, g * BKB, row_b + (int)rank * BM, r);
+      } else {
+        mbar_arrive_expect_tx(b.full(stage), (uint32_t)L::kStageBytes);
+        tma_load_3d(sa, &map_a, b.full(stage), g * BKB, row_a, r);
+        tma_load_3d(sa + L::kABytes, &map_b, b.full(stage), g * BKB, row_b, r);
+      }
+      if (++stage == L::kStages) { stage = 0; phase ^= 1u; }
+    }
+  }
+  // in a pair the leader waits for both CTAs' copies; its partner cannot leave before it does (group_teardown)
+  if (!ok && rank == 0) drain_ring(b, stage, phase);
+}
+
+// The MMA role of the same kernels (warp 1, in a pair the leader's): four MMAs of K = 32 bytes per group of 128 into a fresh
+// accumulator.  All lanes run the loop with warp-uniform control flow and one elected lane issues.
+template <bool kPair, typename L, typename Mma>
+__device__ __forceinline__ void group_mma_loop(const int first, const int stride, const int total_tiles, const int G, unsigned char* smem,
+                                               const GroupBars<L::kStages, GroupShape<kPair>::kAcc> b, const uint32_t tmem_base,
+                                               volatile int* abort_flag, DeviceStatus* status, const unsigned long long limit,
+                                               const int where_full, const int where_empty, const Mma mma) {
+  constexpr int kAcc = GroupShape<kPair>::kAcc, BN = GroupShape<kPair>::BN;
   const uint64_t desc_fixed = make_smem_desc(0);        // everything but the start address
   const uint32_t ring_lo = (smem_u32(smem) & 0x3FFFFu) >> 4;
   int stage = 0;
@@ -1044,22 +1153,22 @@ __device__ __forceinline__ void group_mma_loop(const int total_tiles, const int 
   int acc = 0;
   uint32_t acc_phase = 0;
   bool ok = true;
-  for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
+  for (int tile = first; tile < total_tiles && ok; tile += stride) {
     for (int g = 0; g < G; ++g) {
-      ok = mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, where_empty, status, limit) &&
-           mbar_wait(full_bar(stage), phase, abort_flag, where_full, status, limit);
+      ok = mbar_wait(b.tempty(acc), acc_phase ^ 1u, abort_flag, where_empty, status, limit) &&
+           mbar_wait(b.full(stage), phase, abort_flag, where_full, status, limit);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      const uint32_t d_tmem = tmem_base + (uint32_t)(acc * L::BN);
+      const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
       const uint64_t da = desc_fixed | (uint64_t)(ring_lo + (uint32_t)(stage * (L::kStageBytes >> 4)));
       const uint64_t db = da + (uint64_t)(L::kABytes >> 4);
       if (elect_one()) {
 #pragma unroll
         for (int k = 0; k < BKB / UMMA_KB; ++k)
           mma(d_tmem, da + (uint64_t)(k * (UMMA_KB >> 4)), db + (uint64_t)(k * (UMMA_KB >> 4)), k != 0 ? 1u : 0u);
-        tc_commit(empty_bar(stage));
-        tc_commit(tfull_bar(acc));
+        group_commit<kPair>(b.empty(stage));
+        group_commit<kPair>(b.tfull(acc));
       }
       __syncwarp();
       if (++stage == L::kStages) { stage = 0; phase ^= 1u; }
@@ -1068,22 +1177,78 @@ __device__ __forceinline__ void group_mma_loop(const int total_tiles, const int 
   }
   // wait (bounded) for MMAs in flight before TMEM is freed; a commit tracks the MMAs of the lane that executes it, so the
   // elected lane, which issued them, drains them
+  const auto drain_tc_commit = [](uint32_t bar) { commit_here<kPair>(bar); };
+  const uint32_t drain_bar = b.drain();
   if (!ok && elect_one()) {
-    tc_commit(drain_bar);
-    const unsigned long long t0 = global_timer_ns();
-    while (!mbar_try_wait(drain_bar, 0)) {
-      if (global_timer_ns() - t0 > 20000000ull) break;
-    }
+    drain_tc_commit(drain_bar);
+    wait_drained(drain_bar);
   }
 }
 
-// The rescale role of the group-scaled int8 kernels (warps 2..17): waits for a group's accumulator, converts it, applies
-// the two scales and adds to the tile's fp32 sums, which a thread holds for one row and 32 columns.
+// ---------------------------------------------------------------- group-scaled int8 GEMM
+// The classical int8 operator of the quantisation specification (Appendix D) as one kernel:
+//     C[t][j] = rnd_O( sum over groups g, ascending, of (float(P_g[t][j]) * dA[t][g]) * dB[j][g] ),
+//     P_g = exact integer product of the int8 codes of group g (128 inner indices).
+// Warp 0 streams, per group, the 128 x 128-byte code tiles of A and B (one 128-byte swizzle span = one group) through a
+// shared-memory ring; warp 1 issues four tcgen05.mma kind::i8 (K = 32 each) per group into an int32 accumulator in TMEM;
+// the rescale warps convert it exactly to fp32, apply the two scales with two separate roundings, add with a third, and
+// round to the output dtype after the last group.
+struct Int8Layout {
+  static constexpr int kStages = 4;
+  static constexpr int kABytes = BM * BKB;
+  static constexpr int kBBytes = BM * BKB;                    // 128 rows of B in either form
+  static constexpr int kStageBytes = kABytes + kBBytes;
+  static constexpr int kBarBytes = 256;
+  static constexpr int kMaxGroupsStaged = 64;                 // column scales of a tile staged in shared memory up to this many groups
+  static constexpr int scale_bytes(bool pair) { return kMaxGroupsStaged * (pair ? 256 : 128) * 4; }
+  static constexpr int total(bool pair) { return kStages * kStageBytes + kBarBytes + scale_bytes(pair) + 1024; }
+};
+
+struct Int8Params {
+  int M, N, G;                  // rows of A, rows of B (= output columns), groups of 128 along K
+  int tiles_m, tiles_n;
+  long long ldc;
+  int out_bf16;
+  int wide;                     // every output row starts on a 32-byte boundary
+  float one;                    // 1.0f (see int8_rescale_role)
+  const float* dAt;             // [G][M] row scales, group-major
+  const float* dBt;             // [G][N] column scales, group-major
+  unsigned long long wait_limit_ns;
+};
+
+template <bool kPair>
+__device__ __forceinline__ void tc_mma_i8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  if constexpr (kPair)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
+}
+// int32 accumulator (c format 2), signed 8-bit A and B (format 1), K-major, N >> 3, M >> 4
+template <bool kPair> constexpr uint32_t kInt8Desc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GroupShape<kPair>::BN >> 3) << 17) |
+                                                     ((uint32_t)(GroupShape<kPair>::kRows >> 4) << 24);
+
+// The rescale role of the int8 kernels (warps 2..17): waits for a group's accumulator, converts it, applies the two scales
+// and adds to the tile's fp32 sums, which a thread holds for one row and PN columns.
+// Its arithmetic is three rounded operations per element and group, in the order of the specification, and sets the pace of
+// the classical kernel.  The multiplications run as packed pairs.  A packed multiply followed by a packed add (__fmul2_rn,
+// __fadd2_rn) IS merged into a fused multiply-add by this toolchain, even with explicit rounding modes; the addition is
+// therefore a fused multiply-add by a one that the compiler cannot see (fma(p, 1, s) rounds p + s once).  Integers become
+// floats by a conversion: adding them to the bits of 1.5 * 2^23 and subtracting that took an instruction and a half.
+// Classical, 2048 x 4096 x 11008: 266 us with scalar additions and the bit trick, 253 with the packed additions, 196 with
+// the conversion too, 192 with the staged scales in a loop of their own (128 x 128 tiles), 167 as pairs, 155 with the registers
+// that keep a pair's 64 sums a thread out of local memory.  What bounds it now: issue slots (60 %, 268 instructions per 64 columns
+// and group) and the latency of TMEM and scale loads behind four warps a scheduler.
 struct RescaleCtx {
-  uint32_t tfull0, tempty0;     // accumulator barriers of the kAcc buffers (consecutive)
+  uint32_t tfull0, tempty0;     // accumulator barriers of the buffers (consecutive)
   uint32_t sfull, sempty;       // the tile's column scales are staged / no longer read (16 arrivals each)
   uint32_t tmem_base;
-  float* scale_sm;              // [group][128] column scales of the current tile
+  float* scale_sm;              // [group][BN] column scales of the current tile
   volatile int* abort_flag;
   DeviceStatus* status;
   unsigned long long limit;
@@ -1092,37 +1257,39 @@ struct RescaleCtx {
   int M, N, G;
   long long ldc;
   int out_bf16, wide;
+  float one;
 };
-struct RescaleTile { int row0, rows, col0, cols; bool plus, minus; };   // first row and column of the tile in C, its extents
+struct RescaleTile { int row0, rows, col0, cols; bool any; };   // this CTA's first row and the first column of the tile in C, its
+                                                                // extents; any: an MMA wrote the accumulators
 
-// kMinus: a buffer is two accumulators side by side; the group's integer is the first minus the second, of those that
-// the tile says were written
-template <int kAcc, int kMaxGroupsStaged, bool kMinus, typename TileOf>
-__device__ __forceinline__ void int8_rescale_role(const RescaleCtx& c, const int warp, const int lane, const int total_tiles,
-                                                  const TileOf tile_of) {
-  constexpr int BN = 128, PN = 32, kBufCols = kMinus ? 2 * BN : BN;
+// kMove: the number of warps before the rescale warps; tile_at(k, &tile): the CTA's k-th tile, false after its last
+template <bool kPair, int kMaxGroupsStaged, bool kMove, typename TileAt>
+__device__ __forceinline__ void int8_rescale_role(const RescaleCtx& c, const int warp, const int lane, const TileAt tile_at) {
+  using S = GroupShape<kPair>;
+  constexpr int BN = S::BN, PN = S::PN, kLoad = S::kLoad;
   const int quad = warp & 3;             // TMEM lanes [32*quad, 32*quad+32) are the ones this warp may read
-  const int part = (warp - 2) >> 2;      // which 32 of the tile's 128 columns
+  const int part = (warp - kFirstRescale<kMove>) >> 2;      // which PN of the tile's columns
+  const float2 one2 = make_float2(c.one, c.one);
   int acc = 0;
   uint32_t acc_phase = 0;
   uint32_t scale_phase = 0;
   bool ok = true;
-  for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-    const RescaleTile t = tile_of(tile);
+  RescaleTile t;
+  for (int k = 0; ok && tile_at(k, &t); ++k) {
     const int row = t.row0 + quad * 32 + lane;
     const bool row_ok = quad * 32 + lane < t.rows;
-    const int cols_here = t.cols - part * PN;             // of this warp's 32 columns, those inside the tile
+    const int cols_here = t.cols - part * PN;             // of this warp's columns, those inside the tile
     float2 sum[PN / 2];
 #pragma unroll
     for (int j = 0; j < PN / 2; ++j) sum[j] = make_float2(0.0f, 0.0f);
-    // column scales of this tile: [group][128] into shared memory (zero beyond its edge), by the 512 rescale threads
+    // column scales of this tile: [group][BN] into shared memory (zero beyond its edge), by the 512 rescale threads
     const bool staged = c.G <= kMaxGroupsStaged;
     if (staged) {
       // bounded waits on mbarriers, not a named barrier: a warp that gives up elsewhere must not strand the others
       ok = mbar_wait(c.sempty, scale_phase ^ 1u, c.abort_flag, 0x64, c.status, c.limit);   // previous tile's readers are done
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
-      const int et = threadIdx.x - 64;                  // 0 .. 511
+      const int et = threadIdx.x - 32 * kFirstRescale<kMove>;                  // 0 .. 511
       for (int i = et; i < c.G * (BN / 4); i += 512) {
         const int g = i / (BN / 4), c4 = (i - g * (BN / 4)) * 4;
         const float4 val = c4 < t.cols ? *reinterpret_cast<const float4*>(c.dBt + (long long)g * c.N + t.col0 + c4) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -1134,173 +1301,130 @@ __device__ __forceinline__ void int8_rescale_role(const RescaleCtx& c, const int
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
     }
-    float da_next = row_ok ? c.dAt[row] : 0.0f;
-    for (int g = 0; g < c.G; ++g) {
-      // the row scale does not depend on the products: the next group's is fetched a step ahead
-      const float da = da_next;
-      if (g + 1 < c.G) da_next = row_ok ? c.dAt[(long long)(g + 1) * c.M + row] : 0.0f;
-      const float* dbp = staged ? c.scale_sm + g * BN + part * PN : c.dBt + (long long)g * c.N + t.col0 + part * PN;
-      ok = mbar_wait(c.tfull0 + 8u * acc, acc_phase, c.abort_flag, 0x63, c.status, c.limit);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
-      tc_fence_after();
-      uint32_t v[32];
-      const uint32_t taddr = c.tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * kBufCols + part * PN);
-      if (!kMinus || t.plus) {
-        tc_ld32(taddr, v);
-      } else {
+    const float* da_row = c.dAt + (row_ok ? row : 0);
+    auto add_groups = [&](auto from_smem) {
+      constexpr bool kStaged = decltype(from_smem)::value;
+      const float* db_sm = c.scale_sm + part * PN;                // column scales of group g
+      const float* db_gl = c.dBt + t.col0 + part * PN;
+      const float* da_at = da_row;
+      float da_next = *da_at;
+      for (int g = 0; g < c.G; ++g) {
+        // the row scale does not depend on the products: the next group's is fetched a step ahead
+        const float2 da2 = make_float2(da_next, da_next);
+        if (g + 1 < c.G) { da_at += c.M; da_next = *da_at; }
+        ok = mbar_wait(c.tfull0 + 8u * acc, acc_phase, c.abort_flag, 0x63, c.status, c.limit);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t taddr = c.tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN + part * PN);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = 0u;
-      }
-      // exact int -> float for |P| < 2^22 (a group product is at most 128 * 127^2): add the integer to the bits of
-      // 1.5 * 2^23, subtract that constant (exact)
-      if (kMinus && t.minus) {       // sixteen columns at a time: 96 registers a thread
-        uint32_t m[16];
+        for (int h = 0; h < PN / kLoad; ++h) {
+          uint32_t v[kLoad];
+          tc_ld(taddr + kLoad * h, v);
+          tc_wait_ld(v);
+          if (h == PN / kLoad - 1) {   // the accumulator is in registers: hand the buffer back before the arithmetic
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) group_arrive<kPair>(c.tempty0 + 8u * acc);
+          }
+          if (!t.any) {
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          tc_ld16(taddr + BN + 16 * half, m);
-          tc_wait_ld16(m);
-          if (half == 0) tc_wait_ld32(v);
+            for (int j = 0; j < kLoad; ++j) v[j] = 0u;
+          }
 #pragma unroll
-          for (int j = 0; j < 16; ++j) v[16 * half + j] += 0x4B400000u - m[j];
+          for (int q4 = 0; q4 < kLoad / 4; ++q4) {
+            const int j = h * (kLoad / 4) + q4;
+            float2 p0 = make_float2((float)(int)v[q4 * 4 + 0], (float)(int)v[q4 * 4 + 1]);
+            float2 p1 = make_float2((float)(int)v[q4 * 4 + 2], (float)(int)v[q4 * 4 + 3]);
+            p0 = __fmul2_rn(p0, da2); p1 = __fmul2_rn(p1, da2);
+            float4 db;
+            if constexpr (kStaged) db = *reinterpret_cast<const float4*>(db_sm + j * 4);
+            else db = j * 4 < cols_here ? *reinterpret_cast<const float4*>(db_gl + j * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+            p0 = __fmul2_rn(p0, make_float2(db.x, db.y)); p1 = __fmul2_rn(p1, make_float2(db.z, db.w));
+            sum[j * 2] = __ffma2_rn(p0, one2, sum[j * 2]);
+            sum[j * 2 + 1] = __ffma2_rn(p1, one2, sum[j * 2 + 1]);
+          }
         }
-      } else {
-        tc_wait_ld32(v);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] += 0x4B400000u;
+        db_sm += BN;
+        db_gl += c.N;
+        if (++acc == S::kAcc) { acc = 0; acc_phase ^= 1u; }
       }
-      // the accumulator is in registers: hand the buffer back before the arithmetic
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(c.tempty0 + 8u * acc);
-      if (++acc == kAcc) { acc = 0; acc_phase ^= 1u; }
-      const float2 da2 = make_float2(da, da);
-      const float2 neg_magic = make_float2(-12582912.0f, -12582912.0f);
-      // two separately rounded multiplications and a separately rounded addition, as the specification orders them
-#pragma unroll
-      for (int q4 = 0; q4 < PN / 4; ++q4) {
-        float2 p0 = make_float2(__uint_as_float(v[q4 * 4 + 0]), __uint_as_float(v[q4 * 4 + 1]));
-        float2 p1 = make_float2(__uint_as_float(v[q4 * 4 + 2]), __uint_as_float(v[q4 * 4 + 3]));
-        p0 = __fadd2_rn(p0, neg_magic); p1 = __fadd2_rn(p1, neg_magic);
-        p0 = __fmul2_rn(p0, da2); p1 = __fmul2_rn(p1, da2);
-        const float4 db = (staged || q4 * 4 < cols_here) ? *reinterpret_cast<const float4*>(dbp + q4 * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-        p0 = __fmul2_rn(p0, make_float2(db.x, db.y)); p1 = __fmul2_rn(p1, make_float2(db.z, db.w));
-        sum[q4 * 2].x = __fadd_rn(sum[q4 * 2].x, p0.x); sum[q4 * 2].y = __fadd_rn(sum[q4 * 2].y, p0.y);
-        sum[q4 * 2 + 1].x = __fadd_rn(sum[q4 * 2 + 1].x, p1.x); sum[q4 * 2 + 1].y = __fadd_rn(sum[q4 * 2 + 1].y, p1.y);
-      }
-    }
+    };
+    if (staged) add_groups(std::true_type{});
+    else add_groups(std::false_type{});
     if (!ok) break;
     if (staged) {                                        // this warp no longer reads the tile's scales
       __syncwarp();
       if (lane == 0) mbar_arrive(c.sempty);
       scale_phase ^= 1u;
     }
-    if (row_ok && cols_here > 0) {
-      uint32_t w[32];
 #pragma unroll
-      for (int j = 0; j < PN / 2; ++j) { w[2 * j] = __float_as_uint(sum[j].x); w[2 * j + 1] = __float_as_uint(sum[j].y); }
-      store_row_chunk(c.out, (long long)row * c.ldc + t.col0 + part * PN, min(32, cols_here), w, 1, c.out_bf16, 1.0f, c.wide != 0);
-    }
+    for (int h = 0; h < PN / 32; ++h)
+      if (row_ok && cols_here > 32 * h) {
+        uint32_t w[32];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) { w[2 * j] = __float_as_uint(sum[h * 16 + j].x); w[2 * j + 1] = __float_as_uint(sum[h * 16 + j].y); }
+        store_row_chunk(c.out, (long long)row * c.ldc + t.col0 + part * PN + 32 * h, min(32, cols_here - 32 * h), w, 1, c.out_bf16, 1.0f, c.wide != 0);
+      }
   }
 }
 
-__global__ void __launch_bounds__(kInt8Threads, 1)
-int8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                       void* __restrict__ out, Int8Params p, DeviceStatus* status) {
+template <bool kPair>
+__device__ __forceinline__ void int8_group_gemm_body(const CUtensorMap& map_a, const CUtensorMap& map_b, void* __restrict__ out,
+                                                     const Int8Params& p, DeviceStatus* status) {
   using L = Int8Layout;
-  constexpr int BN = L::BN;
+  using S = GroupShape<kPair>;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t base = (raw_addr + 1023u) & ~1023u;
   unsigned char* smem = smem_raw + (base - raw_addr);
   unsigned char* bar_mem = smem + L::kStages * L::kStageBytes;
-  const uint32_t bar_base = smem_u32(bar_mem);
-  auto full_bar = [&](int s) { return bar_base + 8u * s; };
-  auto empty_bar = [&](int s) { return bar_base + 8u * (L::kStages + s); };
-  constexpr int kAcc = 4;   // accumulator buffers: all 512 TMEM columns, so the MMAs run up to three groups ahead of the rescale
-  auto tfull_bar = [&](int b) { return bar_base + 8u * (2 * L::kStages + b); };
-  auto tempty_bar = [&](int b) { return bar_base + 8u * (2 * L::kStages + kAcc + b); };
-  const uint32_t drain_bar = bar_base + 8u * (2 * L::kStages + 2 * kAcc);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_mem + 8 * (2 * L::kStages + 2 * kAcc + 1));
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_mem + 8 * (2 * L::kStages + 2 * kAcc + 1) + 8);
+  using Bars = GroupBars<L::kStages, S::kAcc>;
+  static_assert(Bars::kBytes <= L::kBarBytes, "barrier block");
+  const Bars b{smem_u32(bar_mem)};
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_mem + Bars::kSlot + 8);
   float* scale_sm = reinterpret_cast<float*>(bar_mem + L::kBarBytes);   // [group][BN] column scales of the current tile
-  const uint32_t sfull_bar = bar_base + 8u * (2 * L::kStages + 2 * kAcc + 3);   // the tile's scales are staged (16 warps arrive)
-  const uint32_t sempty_bar = bar_base + 8u * (2 * L::kStages + 2 * kAcc + 4);  // the tile's scales are no longer read
-
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr uint32_t kTmemCols = kAcc * BN;
+  const uint32_t tmem_base = group_setup<kPair>(b, bar_mem, warp);
+  const uint32_t rank = kPair ? cluster_ctarank() : 0u;
+  grid_dependency_wait();           // the scales come from the previous kernel of the stream
+  const int total_tiles = p.tiles_m * p.tiles_n, first = (int)blockIdx.x / S::kUnits, stride = (int)gridDim.x / S::kUnits;
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < L::kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int b = 0; b < kAcc; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 16); }
-    mbar_init(drain_bar, 1);
-    mbar_init(sfull_bar, 16); mbar_init(sempty_bar, 16);
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
-
-  const int total_tiles = p.tiles_m * p.tiles_n;
-
+  if (warp < kFirstRescale<kPair>) fewer_registers<kPair>();
   if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        const int tm = tile / p.tiles_n, tn = tile - tm * p.tiles_n;
-        for (int g = 0; g < p.G; ++g) {
-          ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, 0x41, status, p.wait_limit_ns);
-          if (!ok) break;
-          const uint32_t sa = smem_u32(smem + stage * L::kStageBytes);
-          mbar_arrive_expect_tx(full_bar(stage), (uint32_t)L::kStageBytes);
-          tma_load_3d(sa, &map_a, full_bar(stage), g * BKB, tm * BM, 0);
-          tma_load_3d(sa + L::kABytes, &map_b, full_bar(stage), g * BKB, tn * BN, 0);
-          if (++stage == L::kStages) { stage = 0; phase ^= 1u; }
-        }
-      }
-      if (!ok) {
-        for (int s = 0; s < L::kStages; ++s) {
-          const uint32_t last_parity = (s < stage) ? phase : (phase ^ 1u);
-          const unsigned long long t0 = global_timer_ns();
-          while (!mbar_try_wait(full_bar(s), last_parity)) {
-            if (global_timer_ns() - t0 > 20000000ull) break;
-          }
-        }
-      }
-    }
+    if (lane == 0)
+      group_copy_loop<kPair, L>(map_a, map_b, first, stride, total_tiles, p.G, smem, b, rank, abort_flag, status, p.wait_limit_ns, 0x41,
+                                [&](int tile, int* row_a, int* row_b, int* r) {
+                                  const int tm = tile / p.tiles_n;
+                                  *row_a = tm * S::kRows; *row_b = (tile - tm * p.tiles_n) * S::BN; *r = 0;
+                                });
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer: one fresh accumulator per group
-    // int32 accumulator (c format 2), signed 8-bit A and B (format 1), K-major, N >> 3, M >> 4
-    constexpr uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-    group_mma_loop<kAcc, L>(total_tiles, p.G, smem, bar_base, tmem_base, abort_flag, status, p.wait_limit_ns, 0x51, 0x52,
-                            [&](uint32_t d, uint64_t a, uint64_t b, uint32_t acc) { tc_mma_i8(d, a, b, idesc, acc); });
-  } else {
-    const RescaleCtx rc{bar_base + 8u * (2 * L::kStages), bar_base + 8u * (2 * L::kStages + kAcc), sfull_bar, sempty_bar,
-                        tmem_base, scale_sm, abort_flag, status, p.wait_limit_ns, out, p.dAt, p.dBt, p.M, p.N, p.G,
-                        p.ldc, p.out_bf16, p.wide};
-    int8_rescale_role<kAcc, L::kMaxGroupsStaged, false>(rc, warp, lane, total_tiles, [&](int tile) {
-      const int tm = tile / p.tiles_n, tn = tile - tm * p.tiles_n;
-      return RescaleTile{tm * BM, min(BM, p.M - tm * BM), tn * BN, min(BN, p.N - tn * BN), true, false};
+    if (rank == 0)
+      group_mma_loop<kPair, L>(first, stride, total_tiles, p.G, smem, b, tmem_base, abort_flag, status, p.wait_limit_ns, 0x51, 0x52,
+                               [&](uint32_t d, uint64_t x, uint64_t y, uint32_t acc) { tc_mma_i8<kPair>(d, x, y, kInt8Desc<kPair>, acc); });
+  } else if (warp >= kFirstRescale<kPair>) {
+    more_registers<kPair>();
+    const RescaleCtx rc{b.tfull(0), b.tempty(0), b.sfull(0), b.sempty(0), tmem_base, scale_sm, abort_flag, status, p.wait_limit_ns, out,
+                        p.dAt, p.dBt, p.M, p.N, p.G, p.ldc, p.out_bf16, p.wide, p.one};
+    int8_rescale_role<kPair, L::kMaxGroupsStaged, kPair>(rc, warp, lane, [&](int k, RescaleTile* t) {
+      const int tile = first + k * stride;
+      if (tile >= total_tiles) return false;
+      const int tm = tile / p.tiles_n, tn = tile - tm * p.tiles_n, row0 = tm * S::kRows + (int)rank * BM;
+      *t = RescaleTile{row0, min(BM, p.M - row0), tn * S::BN, min(S::BN, p.N - tn * S::BN), true};
+      return true;
     });
   }
-
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
-  }
+  group_teardown<kPair>(tmem_base, warp);
+}
+__global__ void __launch_bounds__(kGroupThreads<false>, 1)
+int8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, void* __restrict__ out,
+                       const __grid_constant__ Int8Params p, DeviceStatus* status) {
+  int8_group_gemm_body<false>(map_a, map_b, out, p, status);
+}
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGroupThreads<true>, 1)
+int8_group_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, void* __restrict__ out,
+                            const __grid_constant__ Int8Params p, DeviceStatus* status) {
+  int8_group_gemm_body<true>(map_a, map_b, out, p, status);
 }
 
 // ---------------------------------------------------------------- group-scaled fp8 GEMM (model schedule)
@@ -1308,170 +1432,132 @@ int8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
 // 128 inner indices, e4m3 codes of B with one scale per 128 x 128 block.  As in the int8 kernel every 128-group gets a
 // fresh fp32 accumulator in TMEM (four kind::f8f6f4 MMAs of K = 32); the epilogue multiplies the finished group by
 // s_A[row][g] * s_B[column block][g] and adds it to its fp32 running sums (one fused multiply-add per element and group);
-// after the last group one rounding to the output dtype (bf16 when the product kernel "returns each product in bf16").
-// One CTA per 128 x 128 tile of one product, so a tile's columns lie in one 128-column scale block.
+// after the last group one rounding to the output dtype.  A rescale warp's columns lie in one 128-column scale block.
 // The scales of a tile's rows are staged in shared memory, a tile ahead: read where they lie, every group costs a warp 32
 // cache lines (the scales of a row are neighbours), more than the group's arithmetic.  Above kMaxGroups groups they are
-// read where they lie, two groups ahead of their use and in a loop of their own (classical_gemm, 2048 x 11008 x 4096, 86 groups:
-// 373 us fetched where they are used, 367 ahead of it beside the staged form in one loop, 343 so).
+// read where they lie, two groups ahead of their use and in a loop of their own (classical_gemm, 2048 x 11008 x 4096, 86 groups,
+// 128 x 128 tiles: 373 us fetched where they are used, 367 ahead of it beside the staged form in one loop, 343 so).
+// Pairs: 49 products of 512 x 2752 x 1024 119 -> 97 us (tensor pipe 44 % busy).  Registers moved to the rescale warps, as the int8
+// kernels do, make it slower (the call 191 -> 200 us): nothing that the loop touches is in local memory here.
 struct Fp8Layout : Int8Layout {
   static constexpr int kMaxGroups = 64;                                  // staged up to this many groups
   static constexpr int kScaleLd = BM + 1;                                // [group][row], padded against bank conflicts
-  static constexpr int kScaleFloats = kMaxGroups * (kScaleLd + 1);       // rows' scales, then the column block's
+  static constexpr int kScaleFloats = kMaxGroups * (kScaleLd + 2);       // rows' scales, then those of two column blocks
   static constexpr int kTotal = kStages * kStageBytes + kBarBytes + 2 * kScaleFloats * 4 + 1024;
 };
 struct Fp8GroupParams {
   int rows_a, rows_b, G, batches;   // extents of one product, 128-groups along K, number of products
-  int tiles_m, tiles_n;
+  int tiles_m, tiles_n, blocks_n;   // tiles; 128-column scale blocks
   long long ldo, o_batch;           // output strides in elements
   int out_bf16, wide;
   const float* sA; long long sa_batch;   // [batch][rows_a][G]
-  const float* sB; long long sb_batch;   // [batch][ceil(rows_b / 128)][G]
+  const float* sB; long long sb_batch;   // [batch][blocks_n][G]
   unsigned long long wait_limit_ns;
 };
 
-__global__ void __launch_bounds__(kInt8Threads, 1)
-fp8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-                      void* __restrict__ out, Fp8GroupParams p, DeviceStatus* status) {
-  grid_launch_dependents();
+template <bool kPair>
+__device__ __forceinline__ void fp8_group_gemm_body(const CUtensorMap& map_a, const CUtensorMap& map_b, void* __restrict__ out,
+                                                    const Fp8GroupParams& p, DeviceStatus* status) {
   using L = Fp8Layout;
-  constexpr int BN = L::BN;
+  using S = GroupShape<kPair>;
+  constexpr int BN = S::BN, PN = S::PN, kAcc = S::kAcc, kLoad = S::kLoad;
+  grid_launch_dependents();
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t base = (raw_addr + 1023u) & ~1023u;
   unsigned char* smem = smem_raw + (base - raw_addr);
   unsigned char* bar_mem = smem + L::kStages * L::kStageBytes;
-  const uint32_t bar_base = smem_u32(bar_mem);
-  auto full_bar = [&](int s) { return bar_base + 8u * s; };
-  auto empty_bar = [&](int s) { return bar_base + 8u * (L::kStages + s); };
-  // four accumulator buffers (all 512 TMEM columns): the MMAs of the next three groups run while the rescale warps wait
-  // for the tcgen05.ld of a finished one — that latency, not the arithmetic, sets the pace of this kernel
-  constexpr int kAcc = 4;
-  auto tfull_bar = [&](int b) { return bar_base + 8u * (2 * L::kStages + b); };
-  auto tempty_bar = [&](int b) { return bar_base + 8u * (2 * L::kStages + kAcc + b); };
-  const uint32_t drain_bar = bar_base + 8u * (2 * L::kStages + 2 * kAcc);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_mem + 8 * (2 * L::kStages + 2 * kAcc + 1));
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_mem + 8 * (2 * L::kStages + 2 * kAcc + 1) + 8);
-
-  auto sfull_bar = [&](int b) { return bar_base + 8u * (2 * L::kStages + 2 * kAcc + 3 + b); };    // scales of a tile are staged (16 warps)
-  auto sempty_bar = [&](int b) { return bar_base + 8u * (2 * L::kStages + 2 * kAcc + 5 + b); };   // and no longer read
+  using Bars = GroupBars<L::kStages, kAcc>;
+  const Bars b{smem_u32(bar_mem)};
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_mem + Bars::kSlot + 8);
   float* scale_sm = reinterpret_cast<float*>(bar_mem + L::kBarBytes);
-
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  constexpr uint32_t kTmemCols = kAcc * BN;
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < L::kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int b = 0; b < kAcc; ++b) { mbar_init(tfull_bar(b), 1); mbar_init(tempty_bar(b), 16); }
-    mbar_init(drain_bar, 1);
-    for (int b = 0; b < 2; ++b) { mbar_init(sfull_bar(b), 16); mbar_init(sempty_bar(b), 16); }
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = group_setup<kPair>(b, bar_mem, warp);
+  const uint32_t rank = kPair ? cluster_ctarank() : 0u;
   grid_dependency_wait();           // codes and scales come from the previous kernel of the stream
 
   const int tiles_per_batch = p.tiles_m * p.tiles_n;
-  const int total_tiles = tiles_per_batch * p.batches;
+  const int total_tiles = tiles_per_batch * p.batches, first = (int)blockIdx.x / S::kUnits, stride = (int)gridDim.x / S::kUnits;
+  auto position = [&](int tile, int* r, int* row0, int* tn) {      // product, first row of this CTA, column tile
+    *r = tile / tiles_per_batch;
+    const int rem = tile - *r * tiles_per_batch, tm = rem / p.tiles_n;
+    *row0 = tm * S::kRows + (int)rank * BM;
+    *tn = rem - tm * p.tiles_n;
+  };
   if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-        const int r = tile / tiles_per_batch;
-        const int rem = tile - r * tiles_per_batch;
-        const int tm = rem / p.tiles_n, tn = rem - tm * p.tiles_n;
-        for (int g = 0; g < p.G; ++g) {
-          ok = mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, 0x71, status, p.wait_limit_ns);
-          if (!ok) break;
-          const uint32_t sa = smem_u32(smem + stage * L::kStageBytes);
-          mbar_arrive_expect_tx(full_bar(stage), (uint32_t)L::kStageBytes);
-          tma_load_3d(sa, &map_a, full_bar(stage), g * BKB, tm * BM, r);
-          tma_load_3d(sa + L::kABytes, &map_b, full_bar(stage), g * BKB, tn * BN, r);
-          if (++stage == L::kStages) { stage = 0; phase ^= 1u; }
-        }
-      }
-      if (!ok) {
-        for (int s = 0; s < L::kStages; ++s) {
-          const uint32_t last_parity = (s < stage) ? phase : (phase ^ 1u);
-          const unsigned long long t0 = global_timer_ns();
-          while (!mbar_try_wait(full_bar(s), last_parity)) {
-            if (global_timer_ns() - t0 > 20000000ull) break;
-          }
-        }
-      }
-    }
+    if (lane == 0)
+      group_copy_loop<kPair, L>(map_a, map_b, first, stride, total_tiles, p.G, smem, b, rank, abort_flag, status, p.wait_limit_ns, 0x71,
+                                [&](int tile, int* row_a, int* row_b, int* r) {
+                                  int row0, tn;
+                                  position(tile, r, &row0, &tn);
+                                  *row_a = row0 - (int)rank * BM; *row_b = tn * BN;
+                                });
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer: one fresh accumulator per group
-    constexpr uint32_t idesc = make_idesc(true, BN);
-    group_mma_loop<kAcc, L>(total_tiles, p.G, smem, bar_base, tmem_base, abort_flag, status, p.wait_limit_ns, 0x81, 0x82,
-                            [&](uint32_t d, uint64_t a, uint64_t b, uint32_t acc) { tc_mma<true>(d, a, b, idesc, acc); });
+    // M >> 4 of the tile, N >> 3; formats as make_idesc
+    constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(S::kRows >> 4) << 24);
+    if (rank == 0)
+      group_mma_loop<kPair, L>(first, stride, total_tiles, p.G, smem, b, tmem_base, abort_flag, status, p.wait_limit_ns, 0x81, 0x82,
+                               [&](uint32_t d, uint64_t x, uint64_t y, uint32_t acc) {
+                                 if constexpr (kPair) tc_mma_pair<true>(d, x, y, idesc, acc);
+                                 else tc_mma<true>(d, x, y, idesc, acc);
+                               });
   } else {
-    // ------------------------------------------------------------ scale and accumulate (warps 2..17)
+    // ------------------------------------------------------------ scale and accumulate
     const int quad = warp & 3;
-    const int part = (warp - 2) >> 2;
-    constexpr int PN = 32;
+    const int part = (warp - kFirstRescale<false>) >> 2;
+    const int col_blk = part * PN / 128;          // which of the tile's scale blocks
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
     const bool staged = p.G <= L::kMaxGroups;
     // asynchronous copies of this thread's share of a tile's scales
     auto stage_scales = [&](int tile, int buf) {
-      const int r = tile / tiles_per_batch;
-      const int rem = tile - r * tiles_per_batch;
-      const int tm = rem / p.tiles_n, tn = rem - tm * p.tiles_n;
-      const float* rows = p.sA + (long long)r * p.sa_batch + (long long)tm * BM * p.G;
-      const float* cols = p.sB + (long long)r * p.sb_batch + (long long)tn * p.G;
+      int r, row0, tn;
+      position(tile, &r, &row0, &tn);
+      const float* rows = p.sA + (long long)r * p.sa_batch + (long long)row0 * p.G;
       const uint32_t dst = smem_u32(scale_sm + buf * L::kScaleFloats);
-      const int live = min(BM, p.rows_a - tm * BM) * p.G;
-      for (int i = (int)threadIdx.x - 64; i < live; i += 512) {
+      const int live = max(0, min(BM, p.rows_a - row0)) * p.G;
+      for (int i = (int)threadIdx.x - 32 * kFirstRescale<false>; i < live; i += 512) {
         const int row = i / p.G, g = i - row * p.G;
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4u * (uint32_t)(g * L::kScaleLd + row)), "l"(rows + i) : "memory");
       }
-      for (int g = (int)threadIdx.x - 64; g < p.G; g += 512)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4u * (uint32_t)(L::kMaxGroups * L::kScaleLd + g)), "l"(cols + g) : "memory");
+      const int blk0 = tn * (BN / 128), nblk = min(BN / 128, p.blocks_n - blk0);
+      const float* cols = p.sB + (long long)r * p.sb_batch + (long long)blk0 * p.G;
+      for (int i = (int)threadIdx.x - 32 * kFirstRescale<false>; i < nblk * p.G; i += 512) {
+        const int blk = i / p.G, g = i - blk * p.G;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst + 4u * (uint32_t)(L::kMaxGroups * (L::kScaleLd + blk) + g)), "l"(cols + i) : "memory");
+      }
     };
     auto scales_ready = [&](int buf) {        // this warp's share has landed
       asm volatile("cp.async.wait_all;" ::: "memory");
       __syncwarp();
-      if (lane == 0) mbar_arrive(sfull_bar(buf));
+      if (lane == 0) mbar_arrive(b.sfull(buf));
     };
     int buf = 0;
     uint32_t buf_phase = 0;
-    if (staged && (int)blockIdx.x < total_tiles) {
-      stage_scales(blockIdx.x, 0);
+    if (staged && first < total_tiles) {
+      stage_scales(first, 0);
       scales_ready(0);
     }
-    for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-      const int r = tile / tiles_per_batch;
-      const int rem = tile - r * tiles_per_batch;
-      const int tm = rem / p.tiles_n, tn = rem - tm * p.tiles_n;
-      const bool more = staged && tile + (int)gridDim.x < total_tiles;
+    for (int tile = first; tile < total_tiles && ok; tile += stride) {
+      int r, row0, tn;
+      position(tile, &r, &row0, &tn);
+      const bool more = staged && tile + stride < total_tiles;
       if (staged) {
-        ok = mbar_wait(sfull_bar(buf), buf_phase, abort_flag, 0x95, status, p.wait_limit_ns);
+        ok = mbar_wait(b.sfull(buf), buf_phase, abort_flag, 0x95, status, p.wait_limit_ns);
         // the other buffer's readers (the tile before) are done; nobody has read buffer 1 before the first tile
-        if (more) ok = mbar_wait(sempty_bar(buf ^ 1), buf == 0 ? buf_phase ^ 1u : buf_phase, abort_flag, 0x94, status, p.wait_limit_ns) && ok;
+        if (more) ok = mbar_wait(b.sempty(buf ^ 1), buf == 0 ? buf_phase ^ 1u : buf_phase, abort_flag, 0x94, status, p.wait_limit_ns) && ok;
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
-        if (more) stage_scales(tile + (int)gridDim.x, buf ^ 1);
+        if (more) stage_scales(tile + stride, buf ^ 1);
       }
       const float* sc_rows = scale_sm + buf * L::kScaleFloats + quad * 32 + lane;
-      const float* sc_cols = scale_sm + buf * L::kScaleFloats + L::kMaxGroups * L::kScaleLd;
-      const int row = tm * BM + quad * 32 + lane;
+      const float* sc_cols = scale_sm + buf * L::kScaleFloats + L::kMaxGroups * (L::kScaleLd + col_blk);
+      const int row = row0 + quad * 32 + lane;
       const bool row_ok = row < p.rows_a;
       const int col_base = tn * BN + part * PN;
       const float* sa_row = p.sA + (long long)r * p.sa_batch + (long long)(row_ok ? row : 0) * p.G;
-      const float* sb_blk = p.sB + (long long)r * p.sb_batch + (long long)tn * p.G;   // BN = 128 = one scale block of columns
+      const float* sb_blk = p.sB + (long long)r * p.sb_batch + (long long)min(tn * (BN / 128) + col_blk, p.blocks_n - 1) * p.G;
       float2 sum[PN / 2];
 #pragma unroll
       for (int j = 0; j < PN / 2; ++j) sum[j] = make_float2(0.0f, 0.0f);
@@ -1487,21 +1573,26 @@ fp8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
             s_next = s_next2;
             if (g + 2 < p.G) s_next2 = row_ok ? sa_row[g + 2] * sb_blk[g + 2] : 0.0f;
           }
-          ok = mbar_wait(tfull_bar(acc), acc_phase, abort_flag, 0x93, status, p.wait_limit_ns);
+          ok = mbar_wait(b.tfull(acc), acc_phase, abort_flag, 0x93, status, p.wait_limit_ns);
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
-          uint32_t v[32];
-          tc_ld32(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN + part * PN), v);
-          tc_wait_ld32(v);
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(tempty_bar(acc));
-          if (++acc == kAcc) { acc = 0; acc_phase ^= 1u; }
           const float2 sc2 = make_float2(sc, sc);
 #pragma unroll
-          for (int j = 0; j < PN / 2; ++j)      // one fused multiply-add per element, two elements per instruction
-            sum[j] = __ffma2_rn(make_float2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1])), sc2, sum[j]);
+          for (int h = 0; h < PN / kLoad; ++h) {
+            uint32_t v[kLoad];
+            tc_ld(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN + part * PN + kLoad * h), v);
+            tc_wait_ld(v);
+            if (h == PN / kLoad - 1) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) group_arrive<kPair>(b.tempty(acc));
+            }
+#pragma unroll
+            for (int j = 0; j < kLoad / 2; ++j)      // one fused multiply-add per element, two elements per instruction
+              sum[h * (kLoad / 2) + j] = __ffma2_rn(make_float2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1])), sc2, sum[h * (kLoad / 2) + j]);
+          }
+          if (++acc == kAcc) { acc = 0; acc_phase ^= 1u; }
           if (kStaged && more && g == 0) scales_ready(buf ^ 1);
         }
       };
@@ -1510,117 +1601,158 @@ fp8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
       if (!ok) break;
       if (staged) {
         __syncwarp();
-        if (lane == 0) mbar_arrive(sempty_bar(buf));
+        if (lane == 0) mbar_arrive(b.sempty(buf));
         buf ^= 1;
         if (buf == 0) buf_phase ^= 1u;
       }
-      if (row_ok && col_base < p.rows_b) {
-        uint32_t w[32];
 #pragma unroll
-        for (int j = 0; j < PN / 2; ++j) { w[2 * j] = __float_as_uint(sum[j].x); w[2 * j + 1] = __float_as_uint(sum[j].y); }
-        store_row_chunk(out, (long long)r * p.o_batch + (long long)row * p.ldo + col_base, min(32, p.rows_b - col_base), w, 1,
-                        p.out_bf16, 1.0f, p.wide != 0);
-      }
+      for (int h = 0; h < PN / 32; ++h)
+        if (row_ok && col_base + 32 * h < p.rows_b) {
+          uint32_t w[32];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) { w[2 * j] = __float_as_uint(sum[h * 16 + j].x); w[2 * j + 1] = __float_as_uint(sum[h * 16 + j].y); }
+          store_row_chunk(out, (long long)r * p.o_batch + (long long)row * p.ldo + col_base + 32 * h, min(32, p.rows_b - col_base - 32 * h), w, 1,
+                          p.out_bf16, 1.0f, p.wide != 0);
+        }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");     // none in flight unless the loop was left early
   }
-
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
-  }
+  group_teardown<kPair>(tmem_base, warp);
+}
+__global__ void __launch_bounds__(kGroupThreads<false>, 1)
+fp8_group_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, void* __restrict__ out,
+                      const __grid_constant__ Fp8GroupParams p, DeviceStatus* status) {
+  fp8_group_gemm_body<false>(map_a, map_b, out, p, status);
+}
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGroupThreads<false>, 1)
+fp8_group_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, void* __restrict__ out,
+                           const __grid_constant__ Fp8GroupParams p, DeviceStatus* status) {
+  fp8_group_gemm_body<true>(map_a, map_b, out, p, status);
 }
 
 #include "int8_certified.inc"
 
 }  // namespace
 
+// Pairs or single CTAs for a group-scaled kernel.  A pair's tile is four single ones on two SMs and takes kPairRound times as
+// long as a single one (measured 1.4 to 1.6 for the three kernels); pairs are taken where their rounds of the grid come out
+// shorter.  Calls, us, pairs / single: classical int8 2048 x 4096 x 11008 155 / 192, 464 x 1664 x 4160 27 / 21; certified two-level
+// 2048 x 4096 x 11008 340 / 420, 1040 x 2048 x 4160 106 / 91; model schedule, weights cached, 2048 x 11008 x 4096 191 / 209,
+// 512 x 4096 x 4096 63 / 54, classical 7848 x 4224 x 4576 430 / 495.
+constexpr double kPairRound = 1.5;
+bool group_pairs(int64_t rows_a, int64_t rows_b, int64_t batches, int sms) {
+  if (sms < 2) return false;
+  auto tiles = [&](int64_t t) { return ((rows_a + t - 1) / t) * ((rows_b + t - 1) / t) * batches; };
+  const int64_t pair_rounds = (tiles(256) + sms / 2 - 1) / (sms / 2), single_rounds = (tiles(128) + sms - 1) / sms;
+  return (double)pair_rounds * kPairRound < (double)single_rounds;
+}
+
+// The grid of a group-scaled kernel and its launch, with the CTAs of a pair in one cluster (a dimension of the kernel).
+template <typename Kernel, typename Params>
+fmm_status launch_group_kernel(Kernel kernel, int smem, unsigned long long* smem_ok, bool pair, int threads, long long tiles, int sms, cudaStream_t st,
+                               const CUtensorMap& ma, const CUtensorMap& mb, void* out, const Params& p, DeviceStatus* status) {
+  if (tiles <= 0) return FMM_OK;
+  if (tiles > 0x7fffffff - sms) return FMM_ERR_SHAPE;
+  const long long units = std::min<long long>(tiles, pair ? sms / 2 : sms);
+  if (fmm_allow_dynamic_smem(kernel, smem, smem_ok) != cudaSuccess) return FMM_ERR_CUDA;
+  if (launch_dependent(kernel, dim3((unsigned)(units * (pair ? 2 : 1))), dim3(threads), (size_t)smem, st, ma, mb, out, p, status) != cudaSuccess)
+    return FMM_ERR_CUDA;
+  ++fmm_launch_counter();
+  return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+}
+
 fmm_status launch_fp8_group_gemm(const Fp8GroupArgs& a, cudaStream_t st) {
   using L = Fp8Layout;
   if (a.rows_a > 0x7fffffff || a.rows_b > 0x7fffffff || a.kdim <= 0 || a.kdim > 0x3fffffff) return FMM_ERR_SHAPE;
+  const int sms = sm_count();
+  if (sms <= 0) return FMM_ERR_CUDA;
   CUtensorMap ma, mb;
   if (!make_operand_map(&ma, true, a.A, a.rows_a, a.kdim, a.lda, a.a_batch, a.batches, BM)) return FMM_ERR_CUDA;
-  if (!make_operand_map(&mb, true, a.B, a.rows_b, a.kdim, a.ldb, a.b_batch, a.batches, L::BN)) return FMM_ERR_CUDA;
+  if (!make_operand_map(&mb, true, a.B, a.rows_b, a.kdim, a.ldb, a.b_batch, a.batches, BM)) return FMM_ERR_CUDA;
+  const bool pair = group_pairs(a.rows_a, a.rows_b, a.batches, sms);
+  const int tile = pair ? 256 : 128;
   Fp8GroupParams p;
   p.rows_a = (int)a.rows_a; p.rows_b = (int)a.rows_b; p.G = (int)((a.kdim + BKB - 1) / BKB); p.batches = a.batches;   // a ragged last group is zero-filled by the copies
-  p.tiles_m = (int)((a.rows_a + BM - 1) / BM);
-  p.tiles_n = (int)((a.rows_b + L::BN - 1) / L::BN);
+  p.tiles_m = (int)((a.rows_a + tile - 1) / tile);
+  p.tiles_n = (int)((a.rows_b + tile - 1) / tile);
+  p.blocks_n = (int)((a.rows_b + 127) / 128);
   p.ldo = a.ldo; p.o_batch = a.o_batch; p.out_bf16 = a.output == FMM_BF16;
   const int es = p.out_bf16 ? 2 : 4;
   p.wide = (reinterpret_cast<uintptr_t>(a.out) % 32 == 0) && ((a.ldo * es) % 32 == 0) && ((a.o_batch * es) % 32 == 0);
   p.sA = a.sA; p.sa_batch = a.rows_a * p.G;
-  p.sB = a.sB; p.sb_batch = (long long)p.tiles_n * p.G;
+  p.sB = a.sB; p.sb_batch = (long long)p.blocks_n * p.G;
   p.wait_limit_ns = kDefaultWaitLimitNs;
   const long long total = (long long)p.tiles_m * p.tiles_n * p.batches;
-  if (total <= 0) return FMM_OK;
-  const int sms = sm_count();
-  if (sms <= 0) return FMM_ERR_CUDA;
-  const int grid = (int)(total < sms ? total : sms);
-  static unsigned long long smem_ok = 0;
-  if (fmm_allow_dynamic_smem(fp8_group_gemm_kernel, L::kTotal, &smem_ok) != cudaSuccess) return FMM_ERR_CUDA;
-  if (launch_dependent(fp8_group_gemm_kernel, dim3(grid), dim3(kInt8Threads), (size_t)L::kTotal, st, ma, mb, a.out, p, a.status) != cudaSuccess)
-    return FMM_ERR_CUDA;
-  ++fmm_launch_counter();
-  return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+  static unsigned long long smem_ok[2] = {0, 0};
+  if (pair) return launch_group_kernel(fp8_group_gemm_pair_kernel, L::kTotal, &smem_ok[1], true, kGroupThreads<false>, total, sms, st, ma, mb, a.out, p, a.status);
+  return launch_group_kernel(fp8_group_gemm_kernel, L::kTotal, &smem_ok[0], false, kGroupThreads<false>, total, sms, st, ma, mb, a.out, p, a.status);
 }
 
 fmm_status launch_int8_group_gemm(const int8_t* cA, const int8_t* cB, const float* dAt, const float* dBt, int64_t M,
                                   int64_t K, int64_t N, int output, void* C, int64_t ldc, DeviceStatus* status, cudaStream_t st) {
   using L = Int8Layout;
   if (M > 0x7fffffff || N > 0x7fffffff || K % BKB || K / BKB > 0x7fffffff) return FMM_ERR_SHAPE;
+  const int sms = sm_count();
+  if (sms <= 0) return FMM_ERR_CUDA;
   CUtensorMap ma, mb;
   if (!make_operand_map(&ma, true, cA, M, K, K, 0, 1, BM)) return FMM_ERR_CUDA;
-  if (!make_operand_map(&mb, true, cB, N, K, K, 0, 1, L::BN)) return FMM_ERR_CUDA;
+  if (!make_operand_map(&mb, true, cB, N, K, K, 0, 1, BM)) return FMM_ERR_CUDA;
+  const bool pair = group_pairs(M, N, 1, sms);
+  const int tile = pair ? 256 : 128;
   Int8Params p;
   p.M = (int)M; p.N = (int)N; p.G = (int)(K / BKB);
-  p.tiles_m = (int)((M + BM - 1) / BM);
-  p.tiles_n = (int)((N + L::BN - 1) / L::BN);
+  p.tiles_m = (int)((M + tile - 1) / tile);
+  p.tiles_n = (int)((N + tile - 1) / tile);
   p.ldc = ldc; p.out_bf16 = output == FMM_BF16;
   const int es = p.out_bf16 ? 2 : 4;
   p.wide = (reinterpret_cast<uintptr_t>(C) % 32 == 0) && ((ldc * es) % 32 == 0);
+  p.one = 1.0f;
   p.dAt = dAt; p.dBt = dBt;
   p.wait_limit_ns = kDefaultWaitLimitNs;
   const long long total = (long long)p.tiles_m * p.tiles_n;
-  if (total <= 0) return FMM_OK;
-  const int sms = sm_count();
-  if (sms <= 0) return FMM_ERR_CUDA;
-  const int grid = (int)(total < sms ? total : sms);
-  static unsigned long long smem_ok = 0;
-  if (fmm_allow_dynamic_smem(int8_group_gemm_kernel, L::kTotal, &smem_ok) != cudaSuccess) return FMM_ERR_CUDA;
-  int8_group_gemm_kernel<<<grid, kInt8Threads, L::kTotal, st>>>(ma, mb, C, p, status);
-  ++fmm_launch_counter();
-  return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+  static unsigned long long smem_ok[2] = {0, 0};
+  if (pair) return launch_group_kernel(int8_group_gemm_pair_kernel, L::total(true), &smem_ok[1], true, kGroupThreads<true>, total, sms, st, ma, mb, C, p, status);
+  return launch_group_kernel(int8_group_gemm_kernel, L::total(false), &smem_ok[0], false, kGroupThreads<false>, total, sms, st, ma, mb, C, p, status);
 }
 
 fmm_status launch_int8_certified(const Int8CertArgs& a, cudaStream_t st) {
-  using L = CertLayout;
-  if (a.h != 32 && a.h != 64 && a.h != 128) return FMM_ERR_SHAPE;
+    if (a.h != 32 && a.h != 64 && a.h != 128) return FMM_ERR_SHAPE;
   if (a.m * a.n > kMaxCells || a.R > FMM_MAX_R) return FMM_ERR_LIMIT;
   if (a.M > 0x7fffffff || a.N > 0x7fffffff) return FMM_ERR_SHAPE;
+  const int sms = sm_count();
+  if (sms <= 0) return FMM_ERR_CUDA;
+  const bool pair = group_pairs(a.bm, a.bn, a.m * a.n, sms);
+  const int tile = pair ? 256 : 128;
   CertParams p{};
   p.M = (int)a.M; p.N = (int)a.N; p.n = a.n; p.blocks = a.m * a.n; p.bm = (int)a.bm; p.bn = (int)a.bn;
   p.G = a.G; p.ksteps = a.h / UMMA_KB;
-  p.tiles_m = (int)((a.bm + BM - 1) / BM);
-  p.tiles_n = (int)((a.bn + L::BN - 1) / L::BN);
+  p.tiles_m = (int)((a.bm + tile - 1) / tile);
+  p.tiles_n = (int)((a.bn + tile - 1) / tile);
+  p.hat_tiles_m = (int)((a.bm + BM - 1) / BM);
+  p.hat_tiles_n = (int)((a.bn + BM - 1) / BM);
   p.ldc = a.ldc; p.out_bf16 = a.output == FMM_BF16;
   const int es = p.out_bf16 ? 2 : 4;
   p.wide = (reinterpret_cast<uintptr_t>(a.C) % 32 == 0) && ((a.ldc * es) % 32 == 0) && ((a.bn * es) % 32 == 0);
-  p.Ahat = a.Ahat; p.Bhat = a.Bhat; p.dAt = a.dAt; p.dBt = a.dBt; p.tab_w = a.d_tab_w;
+  p.one = 1.0f;
+  p.dAt = a.dAt; p.dBt = a.dBt; p.tab_w = a.d_tab_w;
   p.wait_limit_ns = kDefaultWaitLimitNs;
+  // blocks of C by the number of MMAs that a group of theirs takes, the most first
+  const CoefTable& t = *a.h_tab_w;
+  int cost[kMaxCells];
+  for (int d = 0; d < p.blocks; ++d) {
+    cost[d] = 0;
+    for (int e = t.off[d]; e < t.off[d + 1]; ++e) cost[d] += t.cell[e] < t.ncell ? (int)std::fabs(t.coef[e]) : 0;
+    p.order[d] = (unsigned char)d;
+  }
+  std::stable_sort(p.order, p.order + p.blocks, [&](unsigned char x, unsigned char y) { return cost[x] > cost[y]; });
   const long long total = (long long)p.tiles_m * p.tiles_n * p.blocks;
-  if (total <= 0) return FMM_OK;
-  if (total > 0x7fffffff) return FMM_ERR_SHAPE;
-  const int sms = sm_count();
-  if (sms <= 0) return FMM_ERR_CUDA;
-  const int grid = (int)(total < sms ? total : sms);
-  static unsigned long long smem_ok = 0;
-  if (fmm_allow_dynamic_smem(int8_certified_kernel, L::kTotal, &smem_ok) != cudaSuccess) return FMM_ERR_CUDA;
-  if (launch_dependent(int8_certified_kernel, dim3(grid), dim3(kInt8Threads), (size_t)L::kTotal, st, a.C, p, a.status) != cudaSuccess)
-    return FMM_ERR_CUDA;
-  ++fmm_launch_counter();
-  return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+  // block sums as rows of 4 KB (a tile of 128 rows, 32 inner indices), copied whole
+  CUtensorMap ma, mb;
+  if (!make_sums_map(&ma, a.Ahat, (int64_t)a.R * a.G * p.ksteps * p.hat_tiles_m)) return FMM_ERR_CUDA;
+  if (!make_sums_map(&mb, a.Bhat, (int64_t)a.R * a.G * p.ksteps * p.hat_tiles_n)) return FMM_ERR_CUDA;
+  static unsigned long long smem_ok[2] = {0, 0};
+  if (pair) return launch_group_kernel(int8_certified_pair_kernel, CertLayout<true>::kTotal, &smem_ok[1], true, kGroupThreads<true>, total, sms, st, ma, mb, a.C, p, a.status);
+  return launch_group_kernel(int8_certified_kernel, CertLayout<false>::kTotal, &smem_ok[0], false, kGroupThreads<true>, total, sms, st, ma, mb, a.C, p, a.status);
 }
 
 fmm_status launch_block_products(const BlockProductArgs& a, cudaStream_t st) {

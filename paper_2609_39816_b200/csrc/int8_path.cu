@@ -765,7 +765,7 @@ static fmm_status int8_certified_one_kernel(const fmm_scheme& sc, const int8_t* 
   Int8CertArgs a{};
   a.Ahat = ja.out; a.Bhat = jb.out;
   a.m = sc.m; a.n = sc.n; a.R = sc.R; a.h = h; a.bm = ja.br; a.bn = jb.br; a.G = G; a.M = M; a.N = N;
-  a.dAt = ja.scales_t; a.dBt = jb.scales_t; a.d_tab_w = at<CoefTable>(d_ws, tab + 2 * stride);
+  a.dAt = ja.scales_t; a.dBt = jb.scales_t; a.d_tab_w = at<CoefTable>(d_ws, tab + 2 * stride); a.h_tab_w = fmm_packed_table(sc, 2);
   a.output = output; a.C = d_C; a.ldc = ldc; a.status = at<DeviceStatus>(d_ws, L.head);
   ProfScope ps(2, st);
   return launch_int8_certified(a, st);

@@ -231,13 +231,13 @@ fmm_status launch_int8_group_gemm(const int8_t* cA, const int8_t* cB, const floa
 
 // The certified int8 realisation in one kernel (tcgen05 kind::i8 block products of the int8 block sums, combined in the
 // tensor cores' accumulators, group rescale in the epilogue).  Ahat, Bhat: int8 block sums in the order that
-// encode_codes_kernel writes, [R][G][h / 32][tile of 128 rows][2][128][16]; d_tab_w: the decode table (list d = the
-// products of C block d with their integer weights).  dAt [G][M], dBt [G][N]: scales, group-major.
+// encode_codes_kernel writes, [R][G][h / 32][tile of 128 rows][2][128][16]; tab_w (device and host): the decode table (list d =
+// the products of C block d with their integer weights).  dAt [G][M], dBt [G][N]: scales, group-major.
 struct Int8CertArgs {
   const int8_t* Ahat; const int8_t* Bhat;
   int m, n, R, h; int64_t bm, bn; int G; int64_t M, N;
   const float* dAt; const float* dBt;
-  const CoefTable* d_tab_w;
+  const CoefTable* d_tab_w; const CoefTable* h_tab_w;
   int output; void* C; int64_t ldc; DeviceStatus* status;
 };
 fmm_status launch_int8_certified(const Int8CertArgs& a, cudaStream_t st);
