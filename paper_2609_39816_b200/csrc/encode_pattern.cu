@@ -1,18 +1,22 @@
-// Encode for the two-level Strassen pattern: the places of the nonzero coefficients are known when this file is compiled,
-// their values are kernel parameters.  The built-in scheme and its sign variants have the pattern S (x) S (144 entries a
-// side); a general gauge of the outer factor fills the outer coefficients, dense (x) S (336 entries).
+// Encode for the two-level Strassen pattern: the places of the nonzero coefficients are known when this file is compiled.  The
+// built-in scheme and its sign variants have the pattern S (x) S (144 entries a side); a general gauge of the outer factor fills
+// the outer coefficients, dense (x) S (336 entries).  Values are kernel parameters; those of the built-in scheme are compiled in
+// for the passes with scales, whose sums are then additions (95 of pairs for 144 multiply-adds).
 //
 // A thread keeps four values of all sixteen cells in registers, as fp32, and forms the 49 block sums one after the other:
 // no table walk, no staging in shared memory, no unpacking per list entry.  The sums are encode_kernel's: the same fp32
 // multiply-add chains in the same order (its padding entries, zero times zero, are left out: they add nothing), the same
 // scales and roundings.
-// What bounds it: the writes of the plain bf16 pass, instruction issue elsewhere.  Both operands, kernel times: bf16 at 4096^3
-// 42 us (272 MB, 6.5 TB/s); e4m3 with a scale per block sum at 2048 x 4096 x 12288 56 us for the maxima and 73 for the codes;
-// model schedule at 2048 x 11008 x 4096 79 and 189 us.  The code is straight, 49 products long for each operand, so everything
-// rare is kept out of it: with the exact divisions inline the model schedule's codes take 206 us.
+// What bounds it: the writes of the plain bf16 pass, the latency of loads and instruction issue elsewhere.  Both operands, kernel
+// times: bf16 at 4096^3 45 us (272 MB); e4m3 with a scale per block sum at 2048 x 4096 x 12288 34 us for the maxima and 51 for the
+// codes (297 MB); model schedule at 2048 x 11008 x 4096 34 us for the maxima of B and 92 for the codes of both (342 MB).  The same
+// passes took 55, 71, 79 and 189 us when coefficients were read for every entry, every warp reduced every maximum, a store stood
+// behind a branch and worked out its address (together half of the instructions), and every quotient near a rounding boundary
+// went through divisions (see e4m3_quotient).  Copies of the next cells ahead into shared memory change nothing.
 //
-// With scales on groups of 128 inner indices (scale mode 3) the 32 lanes of a warp hold one group: they find its largest
-// magnitude by shuffles (A) or one reduction per block of threads (B), and keep the group's 49 scales between them.
+// With scales on groups of 128 inner indices (scale mode 3) the 32 lanes of a warp hold one group: for A, whose groups are one row, the
+// same pass finds a group's largest magnitudes and stores its codes; B takes a pass for each.
+#include <algorithm>
 #include <cstring>
 #include <type_traits>
 #include <utility>
@@ -31,10 +35,15 @@ constexpr Pattern make_pattern(bool b_side, bool dense) {
   int n = 0;
   for (int r = 0; r < kProducts; ++r) {
     const int out = b_side ? kV[r / 7] : kU[r / 7], in = b_side ? kV[r % 7] : kU[r % 7];
+    const int out_minus = b_side ? kVMinus[r / 7] : kUMinus[r / 7], in_minus = b_side ? kVMinus[r % 7] : kUMinus[r % 7];
     for (int x = 0; x < 4; ++x)
-      for (int y = 0; y < 4; ++y)
-        if ((dense || ((out >> (x / 2 * 2 + y / 2)) & 1)) && ((in >> (x % 2 * 2 + y % 2)) & 1))
+      for (int y = 0; y < 4; ++y) {
+        const int o = x / 2 * 2 + y / 2, i = x % 2 * 2 + y % 2;
+        if ((dense || ((out >> o) & 1)) && ((in >> i) & 1)) {
+          p.sign[n] = (signed char)((((dense ? 0 : out_minus >> o) ^ (in_minus >> i)) & 1) ? -1 : 1);
           p.cell[n++] = (unsigned char)(b_side ? y * 4 + x : x * 4 + y);
+        }
+      }
     p.off[r + 1] = n;
   }
   return p;
@@ -42,17 +51,26 @@ constexpr Pattern make_pattern(bool b_side, bool dense) {
 template <bool kB, bool kDense> struct Pat { static constexpr Pattern value = make_pattern(kB, kDense); };
 static_assert(Pat<false, true>::value.off[kProducts] == kMaxEntries && Pat<true, true>::value.off[kProducts] == kMaxEntries, "pattern");
 
+__device__ const Pattern kListsA = make_pattern(false, false), kListsB = make_pattern(true, false);    // for exact_codes
+
+// What the coefficients are: the built-in algorithm's (compiled in); any on the pattern S (x) S; those of a gauge of the outer factor
+// with the built-in inner one (28 numbers, [outer product][outer cell]); any on dense (x) S
+enum PatKind { kScheme, kSparse, kOuter, kDense };
+template <PatKind kKind> constexpr bool kIsDense = kKind == kOuter || kKind == kDense;
+
 struct PatCoefs { float a[kMaxEntries], b[kMaxEntries]; };
 
 struct PatJob {
   const void* X; int64_t ldx; int br, bc; void* out; int64_t rstride;
   unsigned* amax_bits; float* scale_out; int evict_first; int blocks;
+  int steps;      // positions that a thread works on, one after the other (kAmax, kGroupAmax, kGroupScaled)
 };
 
-enum PatPass { kPlain, kAmax, kScaled, kGroupAmax, kGroupScaled };
-// blocks per SM that the register allocation aims at: at the sizes above, 4 / 5 / 6 give 95 / 82 / 79 us for kGroupAmax,
-// 207 / 190 / 192 for kGroupScaled, 41 / 41 / 43 for kPlain, and differ by 1 % in the other two
-constexpr int pat_blocks_per_sm(int pass) { return pass == kGroupAmax ? 6 : pass == kPlain ? 4 : 5; }
+// Passes of an operand; the last three are the model schedule's: A in one (its groups lie within a warp), B in two
+enum PatPass { kNoPass, kPlain, kAmax, kScaled, kGroupOneRow, kGroupAmax, kGroupScaled };
+// blocks per SM that the register allocation aims at: at the sizes above, 3 for the passes that look for maxima (49 of them a
+// thread) take 50 us where 4 take 38; 4 / 5 / 6 for kScaled 66 / 51 / 58
+template <int kPass, PatKind kKind> constexpr int kPatBlocksPerSm = kPass == kPlain || ((kPass == kAmax || kPass == kGroupAmax) && kKind == kScheme) ? 4 : 5;
 
 constexpr int E = 4, NP = 2;          // values of a thread: 16 cells x 4 fp32 registers
 __device__ __forceinline__ float4 load_values(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
@@ -68,20 +86,14 @@ __device__ __forceinline__ float max3(float a, float b, float c) {        // dro
   return d;
 }
 
-// Codes of x / scale (the schedule's division, rounded to fp32 and then to e4m3) from the scale's reciprocal r.  x r (1 + 2^-21)
-// and x r (1 - 2^-21) enclose fl(x / scale), whose distance from x r is below 2^-22 of it, and rounding to e4m3 is
-// monotone: where the two give one code it is that of x / scale.  Otherwise (a few in a million) the division is made.
-template <typename DstT>
-__device__ __noinline__ void store_exactly(DstT* dst, float2 a0, float2 a1, const unsigned* amax_bits, int64_t at) {
-  const float amax = __uint_as_float(amax_bits[at]), sc = amax > 0.0f ? __fdiv_rn(amax, 448.0f) : 1.0f;
-  const float2 q[2] = {make_float2(__fdiv_rn(a0.x, sc), __fdiv_rn(a0.y, sc)), make_float2(__fdiv_rn(a1.x, sc), __fdiv_rn(a1.y, sc))};
-  store_vec<2>(dst, q, false);
+// e4m3 codes of four values: round to nearest even, saturate to +-448, NaN stays NaN
+__device__ __forceinline__ unsigned codes_of(const float2 (&a)[2]) {
+  unsigned codes;
+  asm("{\n\t.reg .b16 l, h;\n\tcvt.rn.satfinite.e4m3x2.f32 l, %2, %1;\n\tcvt.rn.satfinite.e4m3x2.f32 h, %4, %3;\n\tmov.b32 %0, {l, h};\n\t}"
+      : "=r"(codes) : "f"(a[0].x), "f"(a[0].y), "f"(a[1].x), "f"(a[1].y));
+  return codes;
 }
-__device__ __forceinline__ unsigned codes_of(const float2 (&a)[2], float f) {
-  const float2 ff = make_float2(f, f);
-  return (unsigned)__nv_cvt_float2_to_fp8x2(__fmul2_rn(a[0], ff), __NV_SATFINITE, __NV_E4M3) |
-         ((unsigned)__nv_cvt_float2_to_fp8x2(__fmul2_rn(a[1], ff), __NV_SATFINITE, __NV_E4M3) << 16);
-}
+__device__ __forceinline__ float group_scale(float amax) { return amax > 0.0f ? __fdiv_rn(amax, 448.0f) : 1.0f; }
 
 // stores with an L2 eviction priority chosen at run time: one instruction where a choice of two stores is a branch
 __device__ __forceinline__ uint64_t evict_first_policy() {
@@ -94,171 +106,279 @@ __device__ __forceinline__ uint64_t evict_normal_policy() {
   asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
-__device__ __forceinline__ void store_hint(__nv_fp8_storage_t* p, unsigned v, uint64_t policy) {
+__device__ __forceinline__ void store_hint(char* p, unsigned v, uint64_t policy) {
   asm volatile("st.global.L2::cache_hint.b32 [%0], %1, %2;" ::"l"(p), "r"(v), "l"(policy) : "memory");
 }
-__device__ __forceinline__ void store_hint(__nv_fp8_storage_t* p, const float2 (&a)[2], uint64_t policy) {
-  store_hint(p, codes_of(a, 1.0f), policy);
-}
-__device__ __forceinline__ void store_hint(__nv_bfloat16* p, const float2 (&a)[2], uint64_t policy) {
+__device__ __forceinline__ void store_hint(char* p, const float2 (&a)[2], uint64_t policy) {
   const __nv_bfloat162 lo = __floats2bfloat162_rn(a[0].x, a[0].y), hi = __floats2bfloat162_rn(a[1].x, a[1].y);
   asm volatile("st.global.L2::cache_hint.v2.b32 [%0], {%1, %2}, %3;"
                ::"l"(p), "r"(*reinterpret_cast<const uint32_t*>(&lo)), "r"(*reinterpret_cast<const uint32_t*>(&hi)), "l"(policy) : "memory");
 }
 
+// weights are rounded to bf16 before they are quantised under the model schedule
+__device__ __forceinline__ void through_bf16(float2 (&a)[NP]) {
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    const __nv_bfloat162 b = __floats2bfloat162_rn(a[i].x, a[i].y);
+    const uint32_t u = *reinterpret_cast<const uint32_t*>(&b);
+    a[i] = make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u));
+  }
+}
+
 struct PatSmem {
   unsigned amax[kProducts];
-  float2 factor[kProducts];     // kScaled: x / scale = (x * factor.x) * factor.y, both steps exact
+  // pairs (f, f, g, g).  kScaled: x / scale = (x * f) * g, both steps exact; groups: the scale's reciprocal and its negative
+  // (e4m3_quotient), of a warp's group (A) or the block's ([0], B)
+  float4 factors[kPatThreads / 32][kProducts];
 };
 
-template <typename SrcT, typename DstT, bool kB, bool kDense, int kPass>
+// The codes of product r by divisions, for scales that e4m3_quotient does not take: the sum of the cells at src (cell c at
+// offset cell_at(c)), through bf16 for weights, over the scale.
+template <typename SrcT, bool kB, typename CellAt>
+__device__ __noinline__ void exact_codes(const SrcT* src, const CellAt cell_at, const float* coefs, int r, float scale, char* dst) {
+  const Pattern& pat = kB ? kListsB : kListsA;
+  float2 a[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+  for (int e = pat.off[r]; e < pat.off[r + 1]; ++e) {
+    const float4 v = load_values(src + cell_at(pat.cell[e]));
+    const float w = coefs ? coefs[e] : (float)pat.sign[e];
+    a[0] = __ffma2_rn(make_float2(w, w), make_float2(v.x, v.y), a[0]);
+    a[1] = __ffma2_rn(make_float2(w, w), make_float2(v.z, v.w), a[1]);
+  }
+  if (kB) through_bf16(a);
+  const float2 q[2] = {make_float2(__fdiv_rn(a[0].x, scale), __fdiv_rn(a[0].y, scale)), make_float2(__fdiv_rn(a[1].x, scale), __fdiv_rn(a[1].y, scale))};
+  store_vec<2>(reinterpret_cast<__nv_fp8_storage_t*>(dst), q, false);
+}
+
+// The block sum of product r from a thread's cells: the chain of fused multiply-adds from zero, in list order.
+// kScheme: coefficients are 1 and -1, so the first step is the cell itself (cells hold no -0, as zero plus a cell would not)
+// and a chain of n terms takes n - 1 additions.
+template <bool kB, PatKind kKind, int r>
+__device__ __forceinline__ void block_sum(float2 (&acc)[NP], const float2 (&x)[kCells][NP], const float* coefs) {
+  using P = Pat<kB, kIsDense<kKind>>;
+  constexpr int e0 = P::value.off[r], n = P::value.off[r + 1] - e0;
+  if constexpr (kKind == kScheme) {
+    const float2 minus = make_float2(-1.0f, -1.0f);
+    constexpr int c0 = P::value.cell[e0], c1 = P::value.cell[e0 + (n > 1)];
+    constexpr bool lead_minus = P::value.sign[e0] < 0, then_plus = n > 1 && P::value.sign[e0 + (n > 1)] > 0;
+    static_assert(!lead_minus || n > 1, "a single term is positive");
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      if constexpr (lead_minus && then_plus)
+        acc[i] = __ffma2_rn(minus, x[c0][i], x[c1][i]);
+      else if constexpr (lead_minus)
+        acc[i] = __ffma2_rn(minus, x[c0][i], make_float2(0.0f, 0.0f));
+      else
+        acc[i] = x[c0][i];
+    }
+    constexpr int skip = lead_minus && then_plus ? 2 : 1;
+    for_each(std::make_integer_sequence<int, n - skip>{}, [&](auto ec) {
+      constexpr int e = e0 + skip + decltype(ec)::value, c = P::value.cell[e];
+#pragma unroll
+      for (int i = 0; i < NP; ++i) {
+        if constexpr (P::value.sign[e] > 0) acc[i] = __fadd2_rn(acc[i], x[c][i]);
+        else acc[i] = __ffma2_rn(minus, x[c][i], acc[i]);
+      }
+    });
+  } else {
+#pragma unroll
+    for (int i = 0; i < NP; ++i) acc[i] = make_float2(0.0f, 0.0f);
+    for_each(std::make_integer_sequence<int, n>{}, [&](auto ec) {
+      constexpr int e = e0 + decltype(ec)::value, c = P::value.cell[e];
+      float f;
+      if constexpr (kKind == kOuter) {
+        constexpr int oc = kB ? (c % 4) / 2 * 2 + c / 4 / 2 : c / 4 / 2 * 2 + (c % 4) / 2;      // outer cell, of the coefficient matrix
+        constexpr float sign = P::value.sign[e];
+        f = sign * coefs[r / 7 * 4 + oc];
+      } else {
+        f = coefs[e];
+      }
+      const float2 w = make_float2(f, f);
+#pragma unroll
+      for (int i = 0; i < NP; ++i) acc[i] = __ffma2_rn(w, x[c][i], acc[i]);
+    });
+  }
+}
+__device__ __forceinline__ void next(char*& dst, int64_t bytes) {
+  dst += bytes;
+  asm volatile("" : "+l"(dst));
+}
+// nothing that was computed from the cells so far is kept for later products
+__device__ __forceinline__ void hide(float2 (&x)[kCells][NP]) {
+#pragma unroll
+  for (int c = 0; c < kCells; ++c)
+#pragma unroll
+    for (int i = 0; i < NP; ++i) asm volatile("" : "+f"(x[c][i].x), "+f"(x[c][i].y));
+}
+
+template <typename SrcT, typename DstT, bool kB, PatKind kKind, int kPass>
 __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs, int bid, PatSmem& sm) {
-  constexpr bool kGroups = kPass == kGroupAmax || kPass == kGroupScaled;
+  constexpr bool kGroups = kPass == kGroupOneRow || kPass == kGroupAmax || kPass == kGroupScaled;
   constexpr bool kFindMax = kPass == kAmax || kPass == kGroupAmax;
-  constexpr bool kBlockMax = kPass == kAmax || (kPass == kGroupAmax && kB);   // one largest magnitude a product and block of threads
-  constexpr int kLanes = 128 / E;                     // lanes that hold one group of 128 inner indices
-  const int tid = threadIdx.x, lane = tid & 31;
+  constexpr bool kLoop = kFindMax || kPass == kGroupScaled;
+  constexpr bool kKeepMax = kFindMax && kKind == kScheme;     // maxima in registers until the end; coefficients leave no room for them
+  static_assert(128 / E == 32 && (kB || (kPass != kGroupAmax && kPass != kGroupScaled)), "a group's columns are a warp's");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const SrcT* __restrict__ X = static_cast<const SrcT*>(j.X);
-  const int gk = (j.bc + 127) >> 7;
-  // Positions.  Without groups: vector bid * 128 + tid of the block in row-major order.  With groups: columns of group
-  // bid % gk, kRowsPerStep rows.
-  constexpr int kRowsPerStep = kPatThreads / kLanes;
-  if (kBlockMax) {
+  const int gk = (j.bc + 127) >> 7, group = bid % gk, rows0 = bid / gk * (kPatThreads / 32) * (kLoop ? j.steps : 1);
+  const int64_t sstep = (int64_t)gk * (kB ? (j.br + 127) >> 7 : j.br);       // scale blocks of 128 x 128 (B) or 1 x 128 (A)
+  const int64_t sidx = (int64_t)(kB ? rows0 >> 7 : rows0 + warp) * gk + group;
+  if (kFindMax) {
     if (tid < kProducts) sm.amax[tid] = 0u;
     __syncthreads();
   }
   if (kPass == kScaled) {
     if (tid < kProducts) {
       const float s = pow2_scale_448(__uint_as_float(j.amax_bits[tid])), inv = 1.0f / s;   // s: at most 2^120
-      sm.factor[tid] = isfinite(inv) ? make_float2(inv, 1.0f) : make_float2(0x1p127f, 0x1p-127f / s);
+      sm.factors[0][tid] = isfinite(inv) ? make_float4(inv, inv, 1.0f, 1.0f)
+                                           : make_float4(0x1p127f, 0x1p127f, 0x1p-127f / s, 0x1p-127f / s);
       if (bid == 0 && j.scale_out) j.scale_out[tid] = s;
     }
     __syncthreads();
   }
-  {
+  bool odd = false;           // a scale that needs exact_codes
+  (void)odd;
+  if (kPass == kGroupScaled) {
+    if (tid < kProducts) {
+      const float scale = group_scale(__uint_as_float(j.amax_bits[sidx + tid * sstep])), r = e4m3_reciprocal(scale);
+      sm.factors[0][tid] = make_float4(r, r, -scale, -scale);
+      if ((rows0 & 127) == 0) j.scale_out[sidx + tid * sstep] = scale;
+      odd = !e4m3_scale_ok(scale);
+    }
+    odd = __syncthreads_or(odd) != 0;
+  }
+  const uint64_t policy = j.evict_first ? evict_first_policy() : evict_normal_policy();
+  (void)policy;
+  float largest[kKeepMax ? kProducts : 1] = {};
+  const int vpr = j.bc / E;
+#pragma unroll 1
+  for (int step = 0; step < (kLoop ? j.steps : 1); ++step) {
+    // Positions.  Without groups: vector (bid * steps + step) * 128 + tid of the block in row-major order.  With groups: columns of
+    // a group, a row per warp.
+    // Threads past the end repeat the last position: they store what its thread stores, and add nothing to a maximum.
     int p, t;
-    bool live;
     if (kGroups) {
-      p = bid / gk * kRowsPerStep + tid / kLanes;
-      t = (bid % gk) * 128 + (tid % kLanes) * E;
-      live = p < j.br && t < j.bc;
+      p = rows0 + step * (kPatThreads / 32) + warp;
+      if (kPass == kGroupOneRow && p >= j.br) return;             // whole warps
+      p = min(p, j.br - 1);
+      t = min(group * 128 + lane * E, j.bc - E);
     } else {
-      const int vpr = j.bc / E, idx = bid * kPatThreads + tid;
+      const int idx = (int)min((unsigned)(bid * (kLoop ? j.steps : 1) + step) * kPatThreads + tid, (unsigned)(j.br * vpr - 1));
       p = idx / vpr;
       t = (idx - p * vpr) * E;
-      live = p < j.br;
     }
-    const bool p_live = kGroups && p < j.br;      // the lane's group exists (its own columns may lie past the block's end)
-    (void)p_live;
-    if (!live && !(kGroups && p_live)) p = t = 0;
-    float4 x[kCells];
+    float2 x[kCells][NP];
     const SrcT* src = X + (int64_t)p * j.ldx + t;
 #pragma unroll
-    for (int c = 0; c < kCells; ++c)
-      x[c] = live ? load_values(src + (int64_t)(c / 4) * j.br * j.ldx + (int64_t)(c % 4) * j.bc) : make_float4(0.f, 0.f, 0.f, 0.f);
-    DstT* dst = static_cast<DstT*>(j.out) + (int64_t)p * j.bc + t;
-    const int64_t row_groups = kB ? (j.br + 127) >> 7 : j.br;       // scale blocks of 128 x 128 (B) or 1 x 128 (A)
-    const uint64_t policy = j.evict_first ? evict_first_policy() : evict_normal_policy();
-    (void)policy;
-    // scales on groups: lane l keeps the largest magnitude, or the two factors about the scale's reciprocal, of products l
-    // and l + 32
-    constexpr int kKeep = kGroups ? (kProducts + kLanes - 1) / kLanes : 1;
-    const int64_t sidx = (kB ? p >> 7 : p) * (int64_t)gk + (t >> 7), sstep = row_groups * gk;
-    const int gl = lane & (kLanes - 1);
-    unsigned keep[kKeep] = {};
-    float lower[kKeep] = {};
-    (void)lower;
-    if constexpr (kPass == kGroupScaled) {
+    for (int c = 0; c < kCells; ++c) {
+      const float4 v = load_values(src + (int64_t)(c / 4) * j.br * j.ldx + (int64_t)(c % 4) * j.bc);
+      x[c][0] = make_float2(v.x, v.y);
+      x[c][1] = make_float2(v.z, v.w);
+    }
+    if constexpr (kKind == kScheme && !kFindMax) {
 #pragma unroll
-      for (int u = 0; u < kKeep; ++u)
-        if (p_live && u * kLanes + gl < kProducts) {
-          const float amax = __uint_as_float(j.amax_bits[sidx + (u * kLanes + gl) * sstep]);
-          const float sc = amax > 0.0f ? __fdiv_rn(amax, 448.0f) : 1.0f;
-          const float f = __frcp_rn(sc);
-          keep[u] = __float_as_uint(f * (1.0f + 4.76837158203125e-7f));
-          // (an infinite reciprocal would make NaN of zeros on both sides: its lower factor is 0 instead)
-          lower[u] = f <= 3.4e38f ? f * (1.0f - 4.76837158203125e-7f) : 0.0f;
-          if (!kB || (p & 127) == 0) j.scale_out[sidx + (u * kLanes + gl) * sstep] = sc;
+      for (int c = 0; c < kCells; ++c)
+#pragma unroll
+        for (int i = 0; i < NP; ++i) x[c][i] = __fadd2_rn(x[c][i], make_float2(0.0f, 0.0f));      // -0 -> 0
+    }
+    // where this product's sums go: the address is carried from product to product, worked out anew it costs more than the sum
+    char* dst = static_cast<char*>(j.out) + ((int64_t)p * j.bc + t) * (int64_t)sizeof(DstT);
+    const int64_t rbytes = j.rstride * (int64_t)sizeof(DstT);
+    if constexpr (kPass == kGroupOneRow) {
+      // the largest magnitude of the warp's row of the group: lane l keeps those of products l and l + 32, and their factors
+      unsigned keep[2] = {0u, 0u};
+      for_each(std::make_integer_sequence<int, kProducts>{}, [&](auto rc) {
+        constexpr int r = decltype(rc)::value;
+        float2 acc[NP];
+        block_sum<kB, kKind, r>(acc, x, coefs);
+        const float a = max3(max3(0.0f, fabsf(acc[0].x), fabsf(acc[0].y)), fabsf(acc[1].x), fabsf(acc[1].y));     // drops NaN
+        const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(a));
+        if (lane == r % 32) keep[r / 32] = w;
+      });
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int r = u * 32 + lane;
+        if (r < kProducts) {
+          const float scale = group_scale(__uint_as_float(keep[u])), f = e4m3_reciprocal(scale);
+          sm.factors[warp][r] = make_float4(f, f, -scale, -scale);
+          j.scale_out[sidx + r * sstep] = scale;
+          odd = odd || !e4m3_scale_ok(scale);
         }
+      }
+      odd = __any_sync(0xffffffffu, odd);
+      __syncwarp();
+      // the sums are formed again: kept, they would go to local memory
+      hide(x);
+    }
+    if constexpr (kGroups && !kFindMax) {
+      if (odd) {
+        for (int r = 0; r < kProducts; ++r)
+          exact_codes<SrcT, kB>(src, [&](int c) { return (int64_t)(c / 4) * j.br * j.ldx + (int64_t)(c % 4) * j.bc; },
+                                kKind == kScheme ? nullptr : coefs, r, -sm.factors[kB ? 0 : warp][r].w, dst + r * rbytes);
+        continue;
+      }
     }
     for_each(std::make_integer_sequence<int, kProducts>{}, [&](auto rc) {
       constexpr int r = decltype(rc)::value;
-      constexpr int e0 = Pat<kB, kDense>::value.off[r], e1 = Pat<kB, kDense>::value.off[r + 1];
       float2 acc[NP];
+      block_sum<kB, kKind, r>(acc, x, coefs);
+      if constexpr (kPass == kGroupScaled) through_bf16(acc);
+      if constexpr (kFindMax && !kKeepMax) {
+        const float a = max3(max3(0.0f, fabsf(acc[0].x), fabsf(acc[0].y)), fabsf(acc[1].x), fabsf(acc[1].y));
+        const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(a));
+        if (lane == 0) atomicMax(&sm.amax[r], w);
+      } else if constexpr (kFindMax) {
+        largest[r] = max3(largest[r], fabsf(acc[0].x), fabsf(acc[0].y));
+        largest[r] = max3(largest[r], fabsf(acc[1].x), fabsf(acc[1].y));
+      } else if constexpr (kGroups) {
+        const float4 f = sm.factors[kB ? 0 : warp][r];
 #pragma unroll
-      for (int i = 0; i < NP; ++i) acc[i] = make_float2(0.0f, 0.0f);
-      for_each(std::make_integer_sequence<int, e1 - e0>{}, [&](auto ec) {
-        constexpr int e = e0 + decltype(ec)::value, c = Pat<kB, kDense>::value.cell[e];
-        const float2 w = make_float2(coefs[e], coefs[e]);
-        acc[0] = __ffma2_rn(w, make_float2(x[c].x, x[c].y), acc[0]);
-        acc[1] = __ffma2_rn(w, make_float2(x[c].z, x[c].w), acc[1]);
-      });
-      if constexpr (kGroups && kB) {       // weights are rounded to bf16 before they are quantised
-#pragma unroll
-        for (int i = 0; i < NP; ++i) {
-          acc[i].x = __bfloat162float(__float2bfloat16_rn(acc[i].x));
-          acc[i].y = __bfloat162float(__float2bfloat16_rn(acc[i].y));
-        }
-      }
-      if constexpr (kFindMax) {
-        float a = fmaxf(fabsf(acc[0].x), fabsf(acc[0].y));
-#pragma unroll
-        for (int i = 1; i < NP; ++i) a = max3(a, fabsf(acc[i].x), fabsf(acc[i].y));
-        a = fmaxf(a, 0.0f);                 // NaN in both of the first pair
-        // non-negative floats order like their bit patterns
-        if constexpr (kBlockMax) {
-          const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(a));
-          if (lane == 0) atomicMax(&sm.amax[r], w);
-        } else {
-          unsigned w = __float_as_uint(a);
-#pragma unroll
-          for (int o = kLanes / 2; o > 0; o >>= 1) w = max(w, __shfl_xor_sync(0xffffffffu, w, o));
-          if (gl == r % kLanes) keep[r / kLanes] = w;
-        }
+        for (int i = 0; i < NP; ++i) acc[i] = e4m3_quotient(acc[i], make_float2(f.x, f.y), make_float2(f.z, f.w));
+        store_hint(dst, codes_of(acc), policy);
+        next(dst, rbytes);
       } else {
         if constexpr (kPass == kScaled) {
-          const float2 f = sm.factor[r];
+          const float4 f = sm.factors[0][r];
 #pragma unroll
-          for (int i = 0; i < NP; ++i) acc[i] = __fmul2_rn(__fmul2_rn(acc[i], make_float2(f.x, f.x)), make_float2(f.y, f.y));
-        }
-        if constexpr (kPass == kGroupScaled) {
-          const unsigned code = codes_of(acc, __uint_as_float(__shfl_sync(0xffffffffu, keep[r / kLanes], r % kLanes)));
-          const unsigned other = codes_of(acc, __shfl_sync(0xffffffffu, lower[r / kLanes], r % kLanes));
-          if (live) {
-            if (code != other) store_exactly(dst + r * j.rstride, acc[0], acc[1], j.amax_bits + sidx, r * sstep);
-            else store_hint(dst + r * j.rstride, code, policy);
-          }
+          for (int i = 0; i < NP; ++i) acc[i] = __fmul2_rn(__fmul2_rn(acc[i], make_float2(f.x, f.y)), make_float2(f.z, f.w));
+          store_hint(dst, codes_of(acc), policy);
         } else {
-          if (live) store_hint(dst + r * j.rstride, acc, policy);
+          store_hint(dst, acc, policy);
         }
+        next(dst, rbytes);
       }
     });
-    if constexpr (kPass == kGroupAmax && !kB) {
-#pragma unroll
-      for (int u = 0; u < kKeep; ++u)
-        if (p_live && u * kLanes + gl < kProducts) j.amax_bits[sidx + (u * kLanes + gl) * sstep] = keep[u];
-    }
   }
-  if (kBlockMax) {
+  if constexpr (kKeepMax) {
+    for_each(std::make_integer_sequence<int, kProducts>{}, [&](auto rc) {
+      constexpr int r = decltype(rc)::value;
+      const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(largest[r]));      // non-negative floats order like their bit patterns
+      if (lane == 0) atomicMax(&sm.amax[r], w);
+    });
+  }
+  if constexpr (kFindMax) {
     __syncthreads();
-    if (tid < kProducts && sm.amax[tid] != 0u) {
-      const int64_t at = kPass == kAmax ? tid
-                                        : ((int64_t)tid * ((j.br + 127) >> 7) + (bid / gk * kRowsPerStep >> 7)) * gk + bid % gk;
-      atomicMax(&j.amax_bits[at], sm.amax[tid]);
+    if (tid < kProducts) {
+      unsigned w = sm.amax[tid];
+      // weights under the model schedule: the largest of the sums through bf16 (rounding keeps their order)
+      if (kPass == kGroupAmax) w = __float_as_uint(__bfloat162float(__float2bfloat16_rn(__uint_as_float(w))));
+      if (w != 0u) atomicMax(&j.amax_bits[kPass == kAmax ? tid : sidx + tid * sstep], w);
     }
   }
 }
 
-// blocks [0, ja.blocks) work on A, the rest on B
-template <typename SrcT, typename DstT, bool kDense, int kPass>
-__global__ void __launch_bounds__(kPatThreads, pat_blocks_per_sm(kPass))
+// blocks [0, ja.blocks) make pass kPassA over A, the rest kPassB over B (kNoPass: B alone)
+template <typename SrcT, typename DstT, PatKind kKind, int kPassA, int kPassB>
+__global__ void __launch_bounds__(kPatThreads, (kPatBlocksPerSm<kPassB, kKind>))
 encode_pattern_kernel(const __grid_constant__ PatJob ja, const __grid_constant__ PatJob jb, const __grid_constant__ PatCoefs coefs) {
   grid_launch_dependents();   // the block products may set up while this grid drains; they wait before reading
   __shared__ PatSmem sm;
-  if ((int)blockIdx.x < ja.blocks)
-    pattern_body<SrcT, DstT, false, kDense, kPass>(ja, coefs.a, blockIdx.x, sm);
-  else
-    pattern_body<SrcT, DstT, true, kDense, kPass>(jb, coefs.b, blockIdx.x - ja.blocks, sm);
+  if constexpr (kPassA != kNoPass) {
+    if ((int)blockIdx.x < ja.blocks) {
+      pattern_body<SrcT, DstT, false, kKind, kPassA>(ja, coefs.a, blockIdx.x, sm);
+      return;
+    }
+  }
+  pattern_body<SrcT, DstT, true, kKind, kPassB>(jb, coefs.b, blockIdx.x - ja.blocks, sm);
 }
 
 // the table's lists without their padding, if they are the pattern's
@@ -276,56 +396,98 @@ bool matches(const CoefTable& t, const Pattern& p, float* coefs) {
   return true;
 }
 
+// the numbers of a gauge of the outer factor, if the inner coefficients are the built-in ones: places of kOuter
+bool outer_numbers(const float* coefs, const Pattern& p, bool b_side, float* numbers) {
+  bool seen[28] = {};
+  for (int r = 0; r < kProducts; ++r)
+    for (int e = p.off[r]; e < p.off[r + 1]; ++e) {
+      const int c = p.cell[e], at = r / 7 * 4 + (b_side ? (c % 4) / 2 * 2 + c / 4 / 2 : c / 4 / 2 * 2 + (c % 4) / 2);
+      const float f = coefs[e] * (float)p.sign[e];
+      if (seen[at] && numbers[at] != f) return false;
+      numbers[at] = f;
+      seen[at] = true;
+    }
+  return true;
+}
+// are they the built-in algorithm's?
+bool is_scheme(const float* coefs, const Pattern& p) {
+  for (int e = 0; e < p.off[kProducts]; ++e)
+    if (coefs[e] != (float)p.sign[e]) return false;
+  return true;
+}
+
 PatJob make_pat_job(const EncodeOperand& o, int dst_bytes) {
   const bool evict = (int64_t)o.h_tab->R * o.out_stride * dst_bytes > ((int64_t)48 << 20);   // as encode_kernel
-  return PatJob{o.X, o.ldx, (int)o.br, (int)o.bc, o.out, o.out_stride, o.amax_bits, o.scale, evict ? 1 : 0, 0};
+  return PatJob{o.X, o.ldx, (int)o.br, (int)o.bc, o.out, o.out_stride, o.amax_bits, o.scale, evict ? 1 : 0, 0, 1};
 }
 
-int pat_blocks(const PatJob& j, int pass) {
-  const int64_t gk = (j.bc + 127) / 128, rows = kPatThreads * E / 128;
-  if (pass == kGroupAmax || pass == kGroupScaled) return (int)(gk * ((j.br + rows - 1) / rows));
-  return (int)(((int64_t)j.br * (j.bc / E) + kPatThreads - 1) / kPatThreads);
+// Blocks of a pass over an operand, and how many positions their threads work on.  Passes that keep 49 maxima a thread reduce them
+// at their end: one round of blocks over the SMs.  Without them positions are worth more as blocks of their own (dense coefficients, 2048
+// x 3456 x 1280: maxima 17 us, 22 in one round).  B's codes under the model schedule start with 49 scales: rows of a group share a
+// block, as many as still leave two rounds.  `share`: this operand's part of the launch.
+void set_blocks(PatJob& j, int pass, bool keep_maxima, double share) {
+  const int64_t gk = (j.bc + 127) / 128, want = (int64_t)(148 * 4 * share) + 1;
+  if (pass == kGroupOneRow) {
+    j.blocks = (int)(gk * ((j.br + 3) / 4));
+  } else if (pass == kGroupAmax || pass == kGroupScaled) {
+    j.steps = 1;
+    while (j.steps < 32 && gk * ((j.br + 8 * j.steps - 1) / (8 * j.steps)) >= 2 * want) j.steps *= 2;
+    j.blocks = (int)(gk * ((j.br + 4 * j.steps - 1) / (4 * j.steps)));      // 4 * steps divides 128: a block stays in a group
+  } else {
+    const int64_t tiles = ((int64_t)j.br * (j.bc / E) + kPatThreads - 1) / kPatThreads;
+    j.steps = pass == kAmax && keep_maxima ? (int)std::max<int64_t>(1, (tiles + want - 1) / want) : 1;
+    j.blocks = (int)((tiles + j.steps - 1) / j.steps);
+  }
 }
 
-template <typename SrcT, typename DstT, bool kDense, int kPass>
+template <typename SrcT, typename DstT, PatKind kKind, int kPassA, int kPassB>
 cudaError_t launch_pass(PatJob a, PatJob b, bool have_a, bool have_b, const PatCoefs& c, cudaStream_t st) {
-  a.blocks = have_a ? pat_blocks(a, kPass) : 0;
-  b.blocks = have_b ? pat_blocks(b, kPass) : 0;
-  encode_pattern_kernel<SrcT, DstT, kDense, kPass><<<a.blocks + b.blocks, kPatThreads, 0, st>>>(a, b, c);
+  const double na = have_a ? (double)a.br * a.bc : 0.0, nb = have_b ? (double)b.br * b.bc : 0.0;
+  if (have_a) set_blocks(a, kPassA, kKind == kScheme, na / (na + nb));
+  if (have_b) set_blocks(b, kPassB, kKind == kScheme, nb / (na + nb));
+  if (a.blocks + b.blocks == 0) return cudaSuccess;
+  encode_pattern_kernel<SrcT, DstT, kKind, kPassA, kPassB><<<a.blocks + b.blocks, kPatThreads, 0, st>>>(a, b, c);
   ++fmm_launch_counter();
   return cudaGetLastError();
 }
 
-// Which (types, pattern, mode) have a kernel: bf16 without scales and e4m3 with a scale per block sum, both patterns; the model
-// schedule for the scheme and its sign variants (kGroups).  The rest (scale mode 2, e4m3 without scales, the model schedule
+// Which (types, pattern, mode) have a kernel: bf16 without scales and e4m3 with a scale per block sum, all patterns; the model
+// schedule for the scheme and its sign variants.  The rest (scale mode 2, e4m3 without scales, the model schedule
 // under a general gauge of the outer factor) stays with encode_kernel.
-template <typename SrcT, typename DstT, bool kDense, bool kGroups>
+template <typename SrcT, typename DstT, PatKind kKind>
 bool run_pattern(const PatJob& a, const PatJob& b, bool have_a, bool have_b, const PatCoefs& c, int mode, void* clear,
                  size_t clear_bytes, cudaStream_t st, cudaError_t* e) {
   if constexpr (sizeof(DstT) == 2) {
     if (mode != 0) return false;
-    *e = launch_pass<SrcT, DstT, kDense, kPlain>(a, b, have_a, have_b, c, st);
+    *e = launch_pass<SrcT, DstT, kKind, kPlain, kPlain>(a, b, have_a, have_b, c, st);
     return true;
   } else if (mode == 1) {
     *e = cudaMemsetAsync(clear, 0, clear_bytes, st);
-    if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kDense, kAmax>(a, b, have_a, have_b, c, st);
-    if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kDense, kScaled>(a, b, have_a, have_b, c, st);
+    if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kAmax, kAmax>(a, b, have_a, have_b, c, st);
+    if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kScaled, kScaled>(a, b, have_a, have_b, c, st);
     return true;
-  } else if constexpr (kGroups) {
+  } else if constexpr (!kIsDense<kKind>) {
     if (mode != 3) return false;
-    *e = cudaMemsetAsync(clear, 0, clear_bytes, st);
-    if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kDense, kGroupAmax>(a, b, have_a, have_b, c, st);
-    if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kDense, kGroupScaled>(a, b, have_a, have_b, c, st);
+    *e = cudaSuccess;
+    if (have_b) {
+      *e = cudaMemsetAsync(clear, 0, clear_bytes, st);
+      if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kNoPass, kGroupAmax>(a, b, false, true, c, st);
+    }
+    if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kGroupOneRow, kGroupScaled>(a, b, have_a, have_b, c, st);
     return true;
   }
   return false;
 }
 
 template <typename SrcT, typename DstT>
-bool run_types(const PatJob& a, const PatJob& b, bool have_a, bool have_b, const PatCoefs& c, bool dense, int mode, void* clear,
+bool run_types(const PatJob& a, const PatJob& b, bool have_a, bool have_b, const PatCoefs& c, PatKind kind, int mode, void* clear,
                size_t clear_bytes, cudaStream_t st, cudaError_t* e) {
-  return dense ? run_pattern<SrcT, DstT, true, false>(a, b, have_a, have_b, c, mode, clear, clear_bytes, st, e)
-               : run_pattern<SrcT, DstT, false, true>(a, b, have_a, have_b, c, mode, clear, clear_bytes, st, e);
+  if constexpr (sizeof(DstT) == 1)
+    if (kind == kOuter) return run_pattern<SrcT, DstT, kOuter>(a, b, have_a, have_b, c, mode, clear, clear_bytes, st, e);
+  if (kind == kDense || kind == kOuter) return run_pattern<SrcT, DstT, kDense>(a, b, have_a, have_b, c, mode, clear, clear_bytes, st, e);
+  if constexpr (sizeof(DstT) == 1)
+    if (kind == kScheme) return run_pattern<SrcT, DstT, kScheme>(a, b, have_a, have_b, c, mode, clear, clear_bytes, st, e);
+  return run_pattern<SrcT, DstT, kSparse>(a, b, have_a, have_b, c, mode, clear, clear_bytes, st, e);
 }
 
 }  // namespace
@@ -344,12 +506,21 @@ bool fmm_encode_pattern(int storage, int product, const EncodeOperand* a, const 
     if (ok_a && ok_b) dense = d;
   }
   if (dense < 0) return false;
+  PatKind kind = dense ? kDense : kSparse;
+  if (!dense && (!a || is_scheme(c.a, Pat<false, false>::value)) && (!b || is_scheme(c.b, Pat<true, false>::value))) kind = kScheme;
+  if (dense && product == FMM_E4M3) {
+    PatCoefs numbers = {};
+    if ((!a || outer_numbers(c.a, Pat<false, true>::value, false, numbers.a)) && (!b || outer_numbers(c.b, Pat<true, true>::value, true, numbers.b))) {
+      kind = kOuter;
+      c = numbers;
+    }
+  }
   const int dst = product == FMM_E4M3 ? 1 : 2;
   const PatJob ja = a ? make_pat_job(*a, dst) : PatJob{}, jb = b ? make_pat_job(*b, dst) : PatJob{};
-  const bool ha = a != nullptr, hb = b != nullptr, f32 = storage == FMM_F32, dn = dense != 0;
+  const bool ha = a != nullptr, hb = b != nullptr, f32 = storage == FMM_F32;
   if (product == FMM_BF16)
-    return f32 ? run_types<float, __nv_bfloat16>(ja, jb, ha, hb, c, dn, mode, clear, clear_bytes, st, err)
-               : run_types<__nv_bfloat16, __nv_bfloat16>(ja, jb, ha, hb, c, dn, mode, clear, clear_bytes, st, err);
-  return f32 ? run_types<float, __nv_fp8_storage_t>(ja, jb, ha, hb, c, dn, mode, clear, clear_bytes, st, err)
-             : run_types<__nv_bfloat16, __nv_fp8_storage_t>(ja, jb, ha, hb, c, dn, mode, clear, clear_bytes, st, err);
+    return f32 ? run_types<float, __nv_bfloat16>(ja, jb, ha, hb, c, kind, mode, clear, clear_bytes, st, err)
+               : run_types<__nv_bfloat16, __nv_bfloat16>(ja, jb, ha, hb, c, kind, mode, clear, clear_bytes, st, err);
+  return f32 ? run_types<float, __nv_fp8_storage_t>(ja, jb, ha, hb, c, kind, mode, clear, clear_bytes, st, err)
+             : run_types<__nv_bfloat16, __nv_fp8_storage_t>(ja, jb, ha, hb, c, kind, mode, clear, clear_bytes, st, err);
 }

@@ -168,30 +168,32 @@ template <int NP> __device__ __forceinline__ void store_vec(__nv_fp8_storage_t* 
   }
 }
 
-// x / sc for values that are about to be rounded to e4m3, without eight IEEE divisions in the common case.  The exact
-// schedule is code = rnd_e4m3(fl32(x / sc)).  q = x * fl32(1 / sc) lies within 1.5 * 2^-23 (relative) of fl32(x / sc); rounding
-// to e4m3 is monotone, so if q (1 + 2^-21) and q (1 - 2^-21) round to the same code, so does fl32(x / sc), and q can stand
-// in for it.  Otherwise (a value that close to a rounding boundary: a few in a million) the vector is divided exactly.
+// x / s for values that are about to be rounded to e4m3, without an IEEE division each.  The schedule's code is
+// rnd_e4m3(fl(x / s)), so what counts is on which side of the nearest rounding boundary of e4m3 (a number of five significant
+// bits) fl(x / s) lies, or whether it is the boundary itself; with weights in bf16 one quotient in a few hundred is.
+// With r = fl(1 / s): q = fl(x r) is within two units of x / s in the last place; m is the number of five bits nearest to q;
+// d = x - m s is exact in one fused multiply-add (m s has 29 bits, the leading ones cancel).  fl(m + d r) then stands in for fl(x / s):
+// d r is off by less than 2^-24 of itself, and in units of 2^-27 of m s's binade d is a whole number and s / 2 units in the
+// last place of m a multiple of 2^-20 below 16, so the rounding to m or beside it goes wrong only if d is exactly half a unit,
+// which needs s to be a multiple of 1/8 of its binade, and r above 1 / s: there r is rounded towards zero instead.
+// For s from 2^-100 (below, d could underflow) to the largest float.
+__device__ __forceinline__ bool e4m3_scale_ok(float s) { return s >= 0x1p-100f && s <= 3.402823466e38f; }
+__device__ __forceinline__ float e4m3_reciprocal(float s) { return (__float_as_uint(s) & 0xFFFFFu) == 0u ? __frcp_rz(s) : __frcp_rn(s); }
+__device__ __forceinline__ float2 e4m3_quotient(float2 x, float2 r, float2 minus_s) {      // r, -s twice each
+  const float2 q = __fmul2_rn(x, r);
+  const float2 m = make_float2(__uint_as_float((__float_as_uint(q.x) + 0x40000u) & 0xFFF80000u),
+                               __uint_as_float((__float_as_uint(q.y) + 0x40000u) & 0xFFF80000u));
+  return __ffma2_rn(__ffma2_rn(m, minus_s, x), r, m);
+}
 template <int NP>
-__device__ __forceinline__ void divide_for_e4m3(float2 (&a)[NP], float sc) {
-  const float r = __frcp_rn(sc);
-  const float2 up = make_float2(1.0f + 4.76837158203125e-7f, 1.0f + 4.76837158203125e-7f);
-  const float2 dn = make_float2(1.0f - 4.76837158203125e-7f, 1.0f - 4.76837158203125e-7f);
-  float2 q[NP];
-  bool same = true;
+__device__ __forceinline__ void divide_for_e4m3(float2 (&a)[NP], float s) {
+  if (e4m3_scale_ok(s)) {
+    const float r = e4m3_reciprocal(s);
 #pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    q[i] = __fmul2_rn(a[i], make_float2(r, r));
-    const unsigned hi = __nv_cvt_float2_to_fp8x2(__fmul2_rn(q[i], up), __NV_SATFINITE, __NV_E4M3);
-    const unsigned lo = __nv_cvt_float2_to_fp8x2(__fmul2_rn(q[i], dn), __NV_SATFINITE, __NV_E4M3);
-    same = same && (hi == lo);
-  }
-  if (same) {
-#pragma unroll
-    for (int i = 0; i < NP; ++i) a[i] = q[i];
+    for (int i = 0; i < NP; ++i) a[i] = e4m3_quotient(a[i], make_float2(r, r), make_float2(-s, -s));
   } else {
 #pragma unroll
-    for (int i = 0; i < NP; ++i) { a[i].x = __fdiv_rn(a[i].x, sc); a[i].y = __fdiv_rn(a[i].y, sc); }
+    for (int i = 0; i < NP; ++i) { a[i].x = __fdiv_rn(a[i].x, s); a[i].y = __fdiv_rn(a[i].y, s); }
   }
 }
 
