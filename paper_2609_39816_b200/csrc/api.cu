@@ -170,15 +170,16 @@ T* at(void* ws, size_t off) { return reinterpret_cast<T*>(static_cast<char*>(ws)
 #define FMM_CUDA(x) do { if ((x) != cudaSuccess) return FMM_ERR_CUDA; } while (0)
 #define FMM_TRY(x) do { fmm_status _s = (x); if (_s != FMM_OK) return _s; } while (0)
 
-// Encode one operand: optional amax pass, then block sums -> product dtype.
+// Encode one operand: optional amax pass, then block sums -> product dtype.  status: zeroed on the way by the kernels of
+// fmm_encode_pattern (callers pass it only where those run).
 fmm_status encode_operand(const fmm_gemm_desc* d, const void* X, int64_t ldx, int gr, int gc, int64_t br, int64_t bc,
                           const CoefTable* d_tab, const CoefTable* h_tab, void* hat, int64_t hat_stride, unsigned* amax,
-                          float* scale, bool b_side, cudaStream_t st) {
+                          float* scale, bool b_side, int* status, cudaStream_t st) {
   const int mode = d->scale_mode;   // 0 none, 1 per encoded tensor, 2 per row of it, 3 model schedule (128-groups)
   const EncodeOperand o{X, ldx, gr, gc, br, bc, d_tab, h_tab, hat, hat_stride, amax, scale, b_side ? 128 : 1, b_side ? 1 : 0};
   cudaError_t e = cudaSuccess;
   if (fmm_encode_pattern(d->storage, d->product, b_side ? nullptr : &o, b_side ? &o : nullptr, mode, amax,
-                         scale_words(mode, h_tab->R, br, bc, b_side) * 4, st, &e)) {
+                         scale_words(mode, h_tab->R, br, bc, b_side) * 4, status, st, &e)) {
     FMM_CUDA(e);
     return FMM_OK;
   }
@@ -211,6 +212,7 @@ struct SchemeRun {
   void* ws;
   const CoefTable *hA, *hB, *hW;   // host tables (list lengths size the kernels' shared memory)
   const CoefTable *dA, *dB, *dW;   // device copies
+  int* status = nullptr;           // to be zeroed by the encode
   float* sA() const { return d->scale_mode != 0 ? at<float>(ws, L.sA) : nullptr; }
   float* sB() const { return d->scale_mode != 0 ? at<float>(ws, L.sB) : nullptr; }
 };
@@ -219,13 +221,13 @@ fmm_status stage_encode_a(const SchemeRun& r, const void* A, cudaStream_t st) {
   const fmm_scheme* s = r.s;
   ProfScope ps(0, st);
   return encode_operand(r.d, A, r.d->lda, s->m, s->k, r.d->M / s->m, r.d->K / s->k, r.dA, r.hA, at<char>(r.ws, r.L.ahat),
-                        r.L.sAhat, at<unsigned>(r.ws, r.L.amaxA), r.sA(), false, st);
+                        r.L.sAhat, at<unsigned>(r.ws, r.L.amaxA), r.sA(), false, r.status, st);
 }
 fmm_status stage_encode_b(const SchemeRun& r, const void* Bk, int64_t ldbk, cudaStream_t st) {
   const fmm_scheme* s = r.s;
   ProfScope ps(1, st);
   return encode_operand(r.d, Bk, ldbk, s->n, s->k, r.d->N / s->n, r.d->K / s->k, r.dB, r.hB, at<char>(r.ws, r.L.bhat),
-                        r.L.sBhat, at<unsigned>(r.ws, r.L.amaxB), r.sB(), true, st);
+                        r.L.sBhat, at<unsigned>(r.ws, r.L.amaxB), r.sB(), true, r.status, st);
 }
 // Both operands in one launch per pass (amax pass if scaled, then the encode pass), on one stream.
 fmm_status stage_encode_pair(const SchemeRun& r, const void* A, const void* Bk, int64_t ldbk, cudaStream_t st) {
@@ -239,7 +241,7 @@ fmm_status stage_encode_pair(const SchemeRun& r, const void* A, const void* Bk, 
   ProfScope ps(0, st);
   const int mode = d->scale_mode;
   cudaError_t e = cudaSuccess;
-  if (fmm_encode_pattern(d->storage, d->product, &oa, &ob, mode, at<char>(r.ws, r.L.amaxA), r.L.sA - r.L.amaxA, st, &e)) {
+  if (fmm_encode_pattern(d->storage, d->product, &oa, &ob, mode, at<char>(r.ws, r.L.amaxA), r.L.sA - r.L.amaxA, r.status, st, &e)) {
     FMM_CUDA(e);
     return FMM_OK;
   }
@@ -357,7 +359,7 @@ fmm_status stage_decode(const SchemeRun& r, void* C, const float* cstar32, doubl
 fmm_status run_scheme(const fmm_scheme* s, const fmm_gemm_desc* d, const GemmLayout& L, const CoefTable* hA,
                       const CoefTable* hB, const CoefTable* hW, const CoefTable* dA_tab, const CoefTable* dB_tab,
                       const CoefTable* dW_tab, const void* A, const void* Bsrc_kmajor, int64_t ldb_kmajor, void* C,
-                      const float* cstar32, double* err_out, void* ws, bool skip_b, cudaStream_t st) {
+                      const float* cstar32, double* err_out, void* ws, bool skip_b, bool zero_status, cudaStream_t st) {
   if (!dA_tab) {
     FMM_CUDA(cudaMemcpyAsync(at<char>(ws, L.tabA), hA, sizeof(CoefTable), cudaMemcpyHostToDevice, st));
     dA_tab = at<CoefTable>(ws, L.tabA);
@@ -370,7 +372,7 @@ fmm_status run_scheme(const fmm_scheme* s, const fmm_gemm_desc* d, const GemmLay
     FMM_CUDA(cudaMemcpyAsync(at<char>(ws, L.tabW), hW, sizeof(CoefTable), cudaMemcpyHostToDevice, st));
     dW_tab = at<CoefTable>(ws, L.tabW);
   }
-  const SchemeRun r{s, d, L, ws, hA, hB, hW, dA_tab, dB_tab, dW_tab};
+  const SchemeRun r{s, d, L, ws, hA, hB, hW, dA_tab, dB_tab, dW_tab, zero_status ? at<int>(ws, L.status) : nullptr};
   // encode A and encode B side by side: one launch whose blocks split between the two operands (they share nothing)
   if (d->flags & FMM_FLAG_ROUND_PER_LEVEL) {
     FMM_TRY(stage_encode_per_level(r, A, d->lda, false, st));
@@ -382,6 +384,18 @@ fmm_status run_scheme(const fmm_scheme* s, const fmm_gemm_desc* d, const GemmLay
   }
   FMM_TRY(stage_products(r, st));
   return stage_decode(r, C, cstar32, err_out, st);
+}
+
+// Do the kernels with compiled-in lists cover the whole of a scheme_gemm call?
+bool pattern_gemm(const fmm_scheme* s, const fmm_gemm_desc* d, bool skip_b) {
+  if (d->flags & FMM_FLAG_ROUND_PER_LEVEL) return false;
+  EncodeOperand a{}, b{};
+  a.br = d->M / s->m; b.br = d->N / s->n; a.bc = b.bc = d->K / s->k;
+  a.h_tab = fmm_packed_table(*s, 0); b.h_tab = fmm_packed_table(*s, 1);
+  const CoefTable* w = fmm_packed_table(*s, 2);
+  return a.h_tab->R == b.h_tab->R && a.h_tab->R == w->ncell &&
+         fmm_encode_pattern(d->storage, d->product, &a, skip_b ? nullptr : &b, d->scale_mode, nullptr, 0, nullptr, nullptr, nullptr) &&
+         fmm_decode_pattern(d->output, nullptr, 0, 0, w, nullptr, nullptr, a.br, b.br, nullptr, 0, nullptr, nullptr, nullptr, 1, nullptr, nullptr);
 }
 
 // B as a K-major matrix [N x K]: in place for the weight layout, else transposed into the workspace.
@@ -642,12 +656,15 @@ fmm_status scheme_gemm(const fmm_scheme* s, const fmm_gemm_desc* d, const void* 
   if (L.status != 0 || L.tabA != kPackedStatusBytes || L.tabB != L.tabA + fmm_packed_table_stride() ||
       L.tabW != L.tabB + fmm_packed_table_stride() || sizeof(DeviceStatus) > kPackedStatusBytes)
     return FMM_ERR_CUDA;
-  FMM_CUDA(cudaMemcpyAsync(d_ws, packed.data(), packed.size(), cudaMemcpyHostToDevice, st));
+  // kernels with compiled-in lists read no tables: the encode zeroes the status block, and there is nothing to copy (2.5 us and
+  // the wait for it; with launches that overlap their predecessor's end 256^3 from fp32 takes 16.0 us where it took 23.6)
+  const bool patterns = pattern_gemm(s, d, skip_b);
+  if (!patterns) FMM_CUDA(cudaMemcpyAsync(d_ws, packed.data(), packed.size(), cudaMemcpyHostToDevice, st));
   const void* bk_ptr; int64_t bk_ld;
   FMM_TRY(kmajor_b(d, dB, d_ws, L.bt, &bk_ptr, &bk_ld, skip_b, st));
   return run_scheme(s, d, L, fmm_packed_table(*s, 0), fmm_packed_table(*s, 1), fmm_packed_table(*s, 2),
                     at<CoefTable>(d_ws, L.tabA), at<CoefTable>(d_ws, L.tabB), at<CoefTable>(d_ws, L.tabW), dA, bk_ptr, bk_ld, dC,
-                    nullptr, nullptr, d_ws, skip_b, st);
+                    nullptr, nullptr, d_ws, skip_b, patterns, st);
 }
 
 fmm_status scheme_joint_round_weights(const fmm_scheme* s, const fmm_gemm_desc* d, const void* dB, int max_sweeps,

@@ -1,4 +1,4 @@
-// Decode for the two-level Strassen pattern (see encode_pattern.cu): a thread forms all sixteen cells of four columns of a
+// Decode for the patterns of encode_pattern.cu, described here for the two-level one: a thread forms all sixteen cells of four columns of a
 // position.  It walks the 49 products in order, one 16-byte load each, and adds a product to the two to four cells (up to
 // eight for a general outer gauge) that it feeds, whose fp32 sums stay in registers: the multiply-add chains of
 // decode_kernel in the same order, without its staging in shared memory, its barriers and its table walk.
@@ -20,10 +20,9 @@ constexpr Pattern make_pattern(bool dense) {
   Pattern p;
   int n = 0;
   for (int r = 0; r < kProducts; ++r) {
-    for (int x = 0; x < 4; ++x)
-      for (int y = 0; y < 4; ++y)
-        if ((dense || ((kW[r / 7] >> (x / 2 * 2 + y / 2)) & 1)) && ((kW[r % 7] >> (x % 2 * 2 + y % 2)) & 1))
-          p.cell[n++] = (unsigned char)(x * 4 + y);
+    for (int x = 0; x < kGrid; ++x)
+      for (int y = 0; y < kGrid; ++y)
+        if (is_entry(kW, r, x, y, dense)) p.cell[n++] = (unsigned char)(x * kGrid + y);
     p.off[r + 1] = n;
   }
   return p;
@@ -42,7 +41,7 @@ __device__ __forceinline__ float4 load_quad(const __nv_bfloat16* p) {
 // kErr: the squared error against cstar32 instead of the result, one partial sum per block of threads; sixteen squares (a row
 // of cells) are added in fp32, those sums in fp64
 template <typename OutT, typename ProdT, bool kErr, bool kDense>
-__global__ void __launch_bounds__(kPatThreads, 4)
+__global__ void __launch_bounds__(kPatThreads, kLevels == 2 ? 4 : 8)
 decode_pattern_kernel(const ProdT* __restrict__ prod, int64_t rstride, const __grid_constant__ PatCoefs coefs,
                       const float* __restrict__ sA, const float* __restrict__ sB, int bm, int bn, OutT* __restrict__ C, int64_t ldc,
                       const float* __restrict__ cstar32, double* __restrict__ partials, int steps) {
@@ -50,6 +49,7 @@ decode_pattern_kernel(const ProdT* __restrict__ prod, int64_t rstride, const __g
   __shared__ float w[P::value.off[kProducts]];
   __shared__ double red[8];
   const int tid = threadIdx.x;
+  grid_launch_dependents();
   grid_dependency_wait();     // the products (and scales) come from the previous kernel of the stream
   for_each(std::make_integer_sequence<int, kProducts>{}, [&](auto rc) {
     constexpr int r = decltype(rc)::value, e0 = P::value.off[r], n = P::value.off[r + 1] - e0;
@@ -78,11 +78,11 @@ decode_pattern_kernel(const ProdT* __restrict__ prod, int64_t rstride, const __g
         hi[c] = __ffma2_rn(ww, make_float2(v.z, v.w), hi[c]);
       });
     });
-    const int64_t ld = kErr ? 4 * (int64_t)bn : ldc;
+    const int64_t ld = kErr ? kGrid * (int64_t)bn : ldc;
     float err = 0.0f;
 #pragma unroll
     for (int c = 0; c < kCells; ++c) {
-      const int64_t at = ((int64_t)(c / 4) * bm + p) * ld + (int64_t)(c % 4) * bn + q;
+      const int64_t at = ((int64_t)(c / kGrid) * bm + p) * ld + (int64_t)(c % kGrid) * bn + q;
       const float4 x = make_float4(lo[c].x, lo[c].y, hi[c].x, hi[c].y);
       if constexpr (kErr) {
         const float4 cs = __ldg(reinterpret_cast<const float4*>(cstar32 + at));
@@ -143,10 +143,10 @@ bool launch_out(const void* prod, bool prod_bf16, int64_t rstride, const PatCoef
 
 }  // namespace
 
-bool fmm_decode_pattern(int output, const void* prod, int prod_dtype, int64_t prod_stride, const CoefTable* h_tab, const float* sA,
+bool FMM_PATTERN(fmm_decode)(int output, const void* prod, int prod_dtype, int64_t prod_stride, const CoefTable* h_tab, const float* sA,
                         const float* sB, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
                         int* n_partials, int max_partials, cudaStream_t st, cudaError_t* err) {
-  if ((C != nullptr) == (cstar32 != nullptr)) return false;
+  if (err != nullptr && (C != nullptr) == (cstar32 != nullptr)) return false;
   const int64_t nvec = bm * (bn >> 2), tiles = (nvec + kPatThreads - 1) / kPatThreads;
   if (nvec >= ((int64_t)1 << 31) - 4096) return false;          // positions are 32-bit
   PatCoefs c;
@@ -156,6 +156,7 @@ bool fmm_decode_pattern(int output, const void* prod, int prod_dtype, int64_t pr
     dense = true;
     if (!matches(*h_tab, Pat<true>::value, c.w)) return false;
   }
+  if (err == nullptr) return !dense;            // has a result of these tables a kernel?
   // an error launch has one partial sum per block: blocks walk several tiles where they are many
   const int64_t steps = cstar32 ? (tiles + max_partials - 1) / max_partials : 1, blocks = (tiles + steps - 1) / steps;
   const bool done = output == FMM_F32

@@ -1,4 +1,5 @@
-// Encode for the two-level Strassen pattern: the places of the nonzero coefficients are known when this file is compiled.  The
+// Encode for the patterns of Strassen's algorithm, described here for the two-level one (FMM_LEVELS 1: 7 products of 4 cells, the
+// algorithm's places or, under a general gauge, all): the places of the nonzero coefficients are known when this file is compiled.  The
 // built-in scheme and its sign variants have the pattern S (x) S (144 entries a side); a general gauge of the outer factor fills
 // the outer coefficients, dense (x) S (336 entries).  Values are kernel parameters; those of the built-in scheme are compiled in
 // for the passes with scales, whose sums are then additions (95 of pairs for 144 multiply-adds).
@@ -16,6 +17,9 @@
 //
 // With scales on groups of 128 inner indices (scale mode 3) the 32 lanes of a warp hold one group: for A, whose groups are one row, the
 // same pass finds a group's largest magnitudes and stores its codes; B takes a pass for each.
+//
+// One level (whole calls, against the table-driven kernels): 2048 x 4096 x 4096 bf16 119 -> 82 us, e4m3 with a scale per block sum 144 ->
+// 77, model schedule from fp32 280 -> 103; 64 x 4096 x 4096 under the model schedule, weights cached, 45 -> 16.
 #include <algorithm>
 #include <cstring>
 #include <type_traits>
@@ -34,16 +38,14 @@ constexpr Pattern make_pattern(bool b_side, bool dense) {
   Pattern p;
   int n = 0;
   for (int r = 0; r < kProducts; ++r) {
-    const int out = b_side ? kV[r / 7] : kU[r / 7], in = b_side ? kV[r % 7] : kU[r % 7];
-    const int out_minus = b_side ? kVMinus[r / 7] : kUMinus[r / 7], in_minus = b_side ? kVMinus[r % 7] : kUMinus[r % 7];
-    for (int x = 0; x < 4; ++x)
-      for (int y = 0; y < 4; ++y) {
-        const int o = x / 2 * 2 + y / 2, i = x % 2 * 2 + y % 2;
-        if ((dense || ((out >> o) & 1)) && ((in >> i) & 1)) {
-          p.sign[n] = (signed char)((((dense ? 0 : out_minus >> o) ^ (in_minus >> i)) & 1) ? -1 : 1);
-          p.cell[n++] = (unsigned char)(b_side ? y * 4 + x : x * 4 + y);
+    const int outer_minus = dense ? 0 : (b_side ? kVMinus : kUMinus)[kLevels == 2 ? r / 7 : r], inner_minus = kLevels == 2 ? (b_side ? kVMinus : kUMinus)[r % 7] : 0;
+    for (int x = 0; x < kGrid; ++x)
+      for (int y = 0; y < kGrid; ++y)
+        if (is_entry(b_side ? kV : kU, r, x, y, dense)) {
+          const int outer = kLevels == 2 ? x / 2 * 2 + y / 2 : x * 2 + y, inner = x % 2 * 2 + y % 2;
+          p.sign[n] = (signed char)((((outer_minus >> outer) ^ (inner_minus >> inner)) & 1) ? -1 : 1);
+          p.cell[n++] = (unsigned char)(b_side ? y * kGrid + x : x * kGrid + y);
         }
-      }
     p.off[r + 1] = n;
   }
   return p;
@@ -70,7 +72,7 @@ struct PatJob {
 enum PatPass { kNoPass, kPlain, kAmax, kScaled, kGroupOneRow, kGroupAmax, kGroupScaled };
 // blocks per SM that the register allocation aims at: at the sizes above, 3 for the passes that look for maxima (49 of them a
 // thread) take 50 us where 4 take 38; 4 / 5 / 6 for kScaled 66 / 51 / 58
-template <int kPass, PatKind kKind> constexpr int kPatBlocksPerSm = kPass == kPlain || ((kPass == kAmax || kPass == kGroupAmax) && kKind == kScheme) ? 4 : 5;
+template <int kPass, PatKind kKind> constexpr int kPatBlocksPerSm = kLevels == 1 ? 8 : kPass == kPlain || ((kPass == kAmax || kPass == kGroupAmax) && kKind == kScheme) ? 4 : 5;
 
 constexpr int E = 4, NP = 2;          // values of a thread: 16 cells x 4 fp32 registers
 __device__ __forceinline__ float4 load_values(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
@@ -270,7 +272,7 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
     const SrcT* src = X + (int64_t)p * j.ldx + t;
 #pragma unroll
     for (int c = 0; c < kCells; ++c) {
-      const float4 v = load_values(src + (int64_t)(c / 4) * j.br * j.ldx + (int64_t)(c % 4) * j.bc);
+      const float4 v = load_values(src + (int64_t)(c / kGrid) * j.br * j.ldx + (int64_t)(c % kGrid) * j.bc);
       x[c][0] = make_float2(v.x, v.y);
       x[c][1] = make_float2(v.z, v.w);
     }
@@ -285,7 +287,8 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
     const int64_t rbytes = j.rstride * (int64_t)sizeof(DstT);
     if constexpr (kPass == kGroupOneRow) {
       // the largest magnitude of the warp's row of the group: lane l keeps those of products l and l + 32, and their factors
-      unsigned keep[2] = {0u, 0u};
+      constexpr int kKeep = (kProducts + 31) / 32;
+      unsigned keep[kKeep] = {};
       for_each(std::make_integer_sequence<int, kProducts>{}, [&](auto rc) {
         constexpr int r = decltype(rc)::value;
         float2 acc[NP];
@@ -295,7 +298,7 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
         if (lane == r % 32) keep[r / 32] = w;
       });
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < kKeep; ++u) {
         const int r = u * 32 + lane;
         if (r < kProducts) {
           const float scale = group_scale(__uint_as_float(keep[u])), f = e4m3_reciprocal(scale);
@@ -312,7 +315,7 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
     if constexpr (kGroups && !kFindMax) {
       if (odd) {
         for (int r = 0; r < kProducts; ++r)
-          exact_codes<SrcT, kB>(src, [&](int c) { return (int64_t)(c / 4) * j.br * j.ldx + (int64_t)(c % 4) * j.bc; },
+          exact_codes<SrcT, kB>(src, [&](int c) { return (int64_t)(c / kGrid) * j.br * j.ldx + (int64_t)(c % kGrid) * j.bc; },
                                 kKind == kScheme ? nullptr : coefs, r, -sm.factors[kB ? 0 : warp][r].w, dst + r * rbytes);
         continue;
       }
@@ -369,8 +372,10 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
 // blocks [0, ja.blocks) make pass kPassA over A, the rest kPassB over B (kNoPass: B alone)
 template <typename SrcT, typename DstT, PatKind kKind, int kPassA, int kPassB>
 __global__ void __launch_bounds__(kPatThreads, (kPatBlocksPerSm<kPassB, kKind>))
-encode_pattern_kernel(const __grid_constant__ PatJob ja, const __grid_constant__ PatJob jb, const __grid_constant__ PatCoefs coefs) {
-  grid_launch_dependents();   // the block products may set up while this grid drains; they wait before reading
+encode_pattern_kernel(const __grid_constant__ PatJob ja, const __grid_constant__ PatJob jb, const __grid_constant__ PatCoefs coefs, int* status) {
+  grid_launch_dependents();   // the next kernel may set up while this grid drains; it waits before reading
+  grid_dependency_wait();     // the operands (and maxima) may come from the kernel before
+  if (status != nullptr && blockIdx.x == 0 && threadIdx.x < sizeof(DeviceStatus) / 4) status[threadIdx.x] = 0;
   __shared__ PatSmem sm;
   if constexpr (kPassA != kNoPass) {
     if ((int)blockIdx.x < ja.blocks) {
@@ -426,7 +431,7 @@ PatJob make_pat_job(const EncodeOperand& o, int dst_bytes) {
 // x 3456 x 1280: maxima 17 us, 22 in one round).  B's codes under the model schedule start with 49 scales: rows of a group share a
 // block, as many as still leave two rounds.  `share`: this operand's part of the launch.
 void set_blocks(PatJob& j, int pass, bool keep_maxima, double share) {
-  const int64_t gk = (j.bc + 127) / 128, want = (int64_t)(148 * 4 * share) + 1;
+  const int64_t gk = (j.bc + 127) / 128, want = (int64_t)(148 * (kLevels == 2 ? 4 : 8) * share) + 1;
   if (pass == kGroupOneRow) {
     j.blocks = (int)(gk * ((j.br + 3) / 4));
   } else if (pass == kGroupAmax || pass == kGroupScaled) {
@@ -441,39 +446,41 @@ void set_blocks(PatJob& j, int pass, bool keep_maxima, double share) {
 }
 
 template <typename SrcT, typename DstT, PatKind kKind, int kPassA, int kPassB>
-cudaError_t launch_pass(PatJob a, PatJob b, bool have_a, bool have_b, const PatCoefs& c, cudaStream_t st) {
+cudaError_t launch_pass(PatJob a, PatJob b, bool have_a, bool have_b, const PatCoefs& c, int* status, cudaStream_t st) {
   const double na = have_a ? (double)a.br * a.bc : 0.0, nb = have_b ? (double)b.br * b.bc : 0.0;
   if (have_a) set_blocks(a, kPassA, kKind == kScheme, na / (na + nb));
   if (have_b) set_blocks(b, kPassB, kKind == kScheme, nb / (na + nb));
   if (a.blocks + b.blocks == 0) return cudaSuccess;
-  encode_pattern_kernel<SrcT, DstT, kKind, kPassA, kPassB><<<a.blocks + b.blocks, kPatThreads, 0, st>>>(a, b, c);
+  const cudaError_t e = launch_dependent(encode_pattern_kernel<SrcT, DstT, kKind, kPassA, kPassB>, dim3(a.blocks + b.blocks), dim3(kPatThreads), 0, st,
+                                         a, b, c, status);
+  if (e != cudaSuccess) return e;
   ++fmm_launch_counter();
   return cudaGetLastError();
 }
 
 // Which (types, pattern, mode) have a kernel: bf16 without scales and e4m3 with a scale per block sum, all patterns; the model
 // schedule for the scheme and its sign variants.  The rest (scale mode 2, e4m3 without scales, the model schedule
-// under a general gauge of the outer factor) stays with encode_kernel.
+// under a general gauge) stays with encode_kernel.
 template <typename SrcT, typename DstT, PatKind kKind>
 bool run_pattern(const PatJob& a, const PatJob& b, bool have_a, bool have_b, const PatCoefs& c, int mode, void* clear,
-                 size_t clear_bytes, cudaStream_t st, cudaError_t* e) {
+                 size_t clear_bytes, int* status, cudaStream_t st, cudaError_t* e) {
   if constexpr (sizeof(DstT) == 2) {
     if (mode != 0) return false;
-    *e = launch_pass<SrcT, DstT, kKind, kPlain, kPlain>(a, b, have_a, have_b, c, st);
+    *e = launch_pass<SrcT, DstT, kKind, kPlain, kPlain>(a, b, have_a, have_b, c, status, st);
     return true;
   } else if (mode == 1) {
     *e = cudaMemsetAsync(clear, 0, clear_bytes, st);
-    if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kAmax, kAmax>(a, b, have_a, have_b, c, st);
-    if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kScaled, kScaled>(a, b, have_a, have_b, c, st);
+    if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kAmax, kAmax>(a, b, have_a, have_b, c, status, st);
+    if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kScaled, kScaled>(a, b, have_a, have_b, c, nullptr, st);
     return true;
   } else if constexpr (!kIsDense<kKind>) {
     if (mode != 3) return false;
     *e = cudaSuccess;
     if (have_b) {
       *e = cudaMemsetAsync(clear, 0, clear_bytes, st);
-      if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kNoPass, kGroupAmax>(a, b, false, true, c, st);
+      if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kNoPass, kGroupAmax>(a, b, false, true, c, nullptr, st);
     }
-    if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kGroupOneRow, kGroupScaled>(a, b, have_a, have_b, c, st);
+    if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kGroupOneRow, kGroupScaled>(a, b, have_a, have_b, c, status, st);
     return true;
   }
   return false;
@@ -481,20 +488,21 @@ bool run_pattern(const PatJob& a, const PatJob& b, bool have_a, bool have_b, con
 
 template <typename SrcT, typename DstT>
 bool run_types(const PatJob& a, const PatJob& b, bool have_a, bool have_b, const PatCoefs& c, PatKind kind, int mode, void* clear,
-               size_t clear_bytes, cudaStream_t st, cudaError_t* e) {
+               size_t clear_bytes, int* status, cudaStream_t st, cudaError_t* e) {
+  if constexpr (sizeof(DstT) == 1 && kLevels == 2)
+    if (kind == kOuter) return run_pattern<SrcT, DstT, kOuter>(a, b, have_a, have_b, c, mode, clear, clear_bytes, status, st, e);
+  if (kind == kDense || kind == kOuter) return run_pattern<SrcT, DstT, kDense>(a, b, have_a, have_b, c, mode, clear, clear_bytes, status, st, e);
   if constexpr (sizeof(DstT) == 1)
-    if (kind == kOuter) return run_pattern<SrcT, DstT, kOuter>(a, b, have_a, have_b, c, mode, clear, clear_bytes, st, e);
-  if (kind == kDense || kind == kOuter) return run_pattern<SrcT, DstT, kDense>(a, b, have_a, have_b, c, mode, clear, clear_bytes, st, e);
-  if constexpr (sizeof(DstT) == 1)
-    if (kind == kScheme) return run_pattern<SrcT, DstT, kScheme>(a, b, have_a, have_b, c, mode, clear, clear_bytes, st, e);
-  return run_pattern<SrcT, DstT, kSparse>(a, b, have_a, have_b, c, mode, clear, clear_bytes, st, e);
+    if (kind == kScheme) return run_pattern<SrcT, DstT, kScheme>(a, b, have_a, have_b, c, mode, clear, clear_bytes, status, st, e);
+  return run_pattern<SrcT, DstT, kSparse>(a, b, have_a, have_b, c, mode, clear, clear_bytes, status, st, e);
 }
 
 }  // namespace
 
-bool fmm_encode_pattern(int storage, int product, const EncodeOperand* a, const EncodeOperand* b, int mode, void* clear,
-                        size_t clear_bytes, cudaStream_t st, cudaError_t* err) {
-  if (mode == 2 || (storage != FMM_F32 && storage != FMM_BF16)) return false;
+bool FMM_PATTERN(fmm_encode)(int storage, int product, const EncodeOperand* a, const EncodeOperand* b, int mode, void* clear,
+                             size_t clear_bytes, int* status, cudaStream_t st, cudaError_t* err) {
+  if (storage != FMM_F32 && storage != FMM_BF16) return false;
+  if (product == FMM_BF16 ? mode != 0 : mode != 1 && mode != 3) return false;
   for (const EncodeOperand* o : {a, b})
     if (o && o->br * (o->bc / E) >= ((int64_t)1 << 31) - 4096) return false;      // positions are 32-bit
   PatCoefs c;
@@ -505,10 +513,11 @@ bool fmm_encode_pattern(int storage, int product, const EncodeOperand* a, const 
     const bool ok_b = !b || matches(*b->h_tab, d ? Pat<true, true>::value : Pat<true, false>::value, c.b);
     if (ok_a && ok_b) dense = d;
   }
-  if (dense < 0) return false;
+  if (dense < 0 || (dense == 1 && mode == 3)) return false;
+  if (err == nullptr) return true;
   PatKind kind = dense ? kDense : kSparse;
   if (!dense && (!a || is_scheme(c.a, Pat<false, false>::value)) && (!b || is_scheme(c.b, Pat<true, false>::value))) kind = kScheme;
-  if (dense && product == FMM_E4M3) {
+  if (dense && product == FMM_E4M3 && kLevels == 2) {
     PatCoefs numbers = {};
     if ((!a || outer_numbers(c.a, Pat<false, true>::value, false, numbers.a)) && (!b || outer_numbers(c.b, Pat<true, true>::value, true, numbers.b))) {
       kind = kOuter;
@@ -519,8 +528,8 @@ bool fmm_encode_pattern(int storage, int product, const EncodeOperand* a, const 
   const PatJob ja = a ? make_pat_job(*a, dst) : PatJob{}, jb = b ? make_pat_job(*b, dst) : PatJob{};
   const bool ha = a != nullptr, hb = b != nullptr, f32 = storage == FMM_F32;
   if (product == FMM_BF16)
-    return f32 ? run_types<float, __nv_bfloat16>(ja, jb, ha, hb, c, kind, mode, clear, clear_bytes, st, err)
-               : run_types<__nv_bfloat16, __nv_bfloat16>(ja, jb, ha, hb, c, kind, mode, clear, clear_bytes, st, err);
-  return f32 ? run_types<float, __nv_fp8_storage_t>(ja, jb, ha, hb, c, kind, mode, clear, clear_bytes, st, err)
-             : run_types<__nv_bfloat16, __nv_fp8_storage_t>(ja, jb, ha, hb, c, kind, mode, clear, clear_bytes, st, err);
+    return f32 ? run_types<float, __nv_bfloat16>(ja, jb, ha, hb, c, kind, mode, clear, clear_bytes, status, st, err)
+               : run_types<__nv_bfloat16, __nv_bfloat16>(ja, jb, ha, hb, c, kind, mode, clear, clear_bytes, status, st, err);
+  return f32 ? run_types<float, __nv_fp8_storage_t>(ja, jb, ha, hb, c, kind, mode, clear, clear_bytes, status, st, err)
+             : run_types<__nv_bfloat16, __nv_fp8_storage_t>(ja, jb, ha, hb, c, kind, mode, clear, clear_bytes, status, st, err);
 }

@@ -288,6 +288,8 @@ cudaError_t launch_encode_t(const EncodeOperand& a, const EncodeOperand* b, bool
 template <typename T>
 __global__ void __launch_bounds__(256) transpose_kernel(const T* __restrict__ B, int64_t ldb, int64_t K, int64_t N,
                                                         T* __restrict__ Bt, int vec) {
+  grid_launch_dependents();
+  grid_dependency_wait();
   constexpr int kPer = 4 / (int)sizeof(T);            // values of a word
   constexpr int VE = 16 / (int)sizeof(T);             // values of a vector
   constexpr int kVecs = 64 / VE;                      // vectors of a tile's row
@@ -658,12 +660,12 @@ cudaError_t launch_transpose(int elem_bytes, const void* B, int64_t ldb, int64_t
   const dim3 grid((unsigned)((N + 63) / 64), (unsigned)((K * elem_bytes + 127) / 128));
   const int vec = reinterpret_cast<uintptr_t>(B) % 16 == 0 && (ldb * elem_bytes) % 16 == 0;
   if (K % 16 || N % 8) return cudaErrorInvalidValue;
+  cudaError_t e = cudaErrorInvalidValue;
   if (elem_bytes == 2)
-    transpose_kernel<uint16_t><<<grid, 256, 0, st>>>((const uint16_t*)B, ldb, K, N, (uint16_t*)Bt, vec);
+    e = launch_dependent(transpose_kernel<uint16_t>, grid, dim3(256), 0, st, (const uint16_t*)B, ldb, K, N, (uint16_t*)Bt, vec);
   else if (elem_bytes == 4)
-    transpose_kernel<uint32_t><<<grid, 256, 0, st>>>((const uint32_t*)B, ldb, K, N, (uint32_t*)Bt, vec);
-  else
-    return cudaErrorInvalidValue;
+    e = launch_dependent(transpose_kernel<uint32_t>, grid, dim3(256), 0, st, (const uint32_t*)B, ldb, K, N, (uint32_t*)Bt, vec);
+  if (e != cudaSuccess) return e;
   ++fmm_launch_counter();
   return cudaGetLastError();
 }

@@ -86,11 +86,18 @@ struct EncodeOperand {
 cudaError_t launch_encode_pair(int storage, int product, const EncodeOperand& a, const EncodeOperand* b, bool amax_only,
                                int use_scale, cudaStream_t st);
 
-// The whole encode of one or both operands (a or b may be null; amax passes included) for tables of the two-level Strassen
-// pattern (encode_pattern.cu).  False, with nothing enqueued, where it has no kernel for the tables, types or mode; else
-// *err is the launches' result.  clear: the amax words of the operands (zeroed first where they are accumulated).
-bool fmm_encode_pattern(int storage, int product, const EncodeOperand* a, const EncodeOperand* b, int mode, void* clear,
-                        size_t clear_bytes, cudaStream_t st, cudaError_t* err);
+// The whole encode of one or both operands (a or b may be null; amax passes included) for tables of the pattern of Strassen's
+// algorithm, nested once or plain (encode_pattern.cu).  False, with nothing enqueued, where it has no kernel for the tables, types
+// or mode; else *err is the launches' result.  clear: the amax words of the operands (zeroed first where they are accumulated);
+// status: a DeviceStatus that the launches zero, or null.  With err null nothing is enqueued: the answer alone.
+bool fmm_encode_two_level(int storage, int product, const EncodeOperand* a, const EncodeOperand* b, int mode, void* clear,
+                          size_t clear_bytes, int* status, cudaStream_t st, cudaError_t* err);
+bool fmm_encode_one_level(int storage, int product, const EncodeOperand* a, const EncodeOperand* b, int mode, void* clear,
+                          size_t clear_bytes, int* status, cudaStream_t st, cudaError_t* err);
+inline bool fmm_encode_pattern(int storage, int product, const EncodeOperand* a, const EncodeOperand* b, int mode, void* clear,
+                               size_t clear_bytes, int* status, cudaStream_t st, cudaError_t* err) {
+  return ((a ? a : b)->h_tab->R == 7 ? fmm_encode_one_level : fmm_encode_two_level)(storage, product, a, b, mode, clear, clear_bytes, status, st, err);
+}
 
 // One operand of an encode launch.  A launch carries up to two (A and B of one product): blocks [0, a.blocks) work
 // on the first, the rest on the second, so both operands are encoded side by side without a second stream.
@@ -128,11 +135,21 @@ cudaError_t launch_decode(int output, const void* prod, int prod_dtype, int64_t 
                           int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials, int* n_partials,
                           cudaStream_t st, int gauges = 1);
 int decode_grid(int64_t bm, int64_t bn);
-// The same for tables of the two-level Strassen pattern (decode_pattern.cu), result or error; at most max_partials partial
-// sums.  False, with nothing enqueued, where it has no kernel; else *err is the launch's result.
-bool fmm_decode_pattern(int output, const void* prod, int prod_dtype, int64_t prod_stride, const CoefTable* h_tab, const float* sA,
-                        const float* sB, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
-                        int* n_partials, int max_partials, cudaStream_t st, cudaError_t* err);
+// The same for the patterns that fmm_encode_pattern takes (decode_pattern.cu), result or error; at most max_partials partial
+// sums.  False, with nothing enqueued, where it has no kernel; else *err is the launch's result.  With err null: would a result
+// of these tables have one?
+bool fmm_decode_two_level(int output, const void* prod, int prod_dtype, int64_t prod_stride, const CoefTable* h_tab, const float* sA,
+                          const float* sB, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
+                          int* n_partials, int max_partials, cudaStream_t st, cudaError_t* err);
+bool fmm_decode_one_level(int output, const void* prod, int prod_dtype, int64_t prod_stride, const CoefTable* h_tab, const float* sA,
+                          const float* sB, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
+                          int* n_partials, int max_partials, cudaStream_t st, cudaError_t* err);
+inline bool fmm_decode_pattern(int output, const void* prod, int prod_dtype, int64_t prod_stride, const CoefTable* h_tab, const float* sA,
+                               const float* sB, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
+                               int* n_partials, int max_partials, cudaStream_t st, cudaError_t* err) {
+  return (h_tab->ncell == 7 ? fmm_decode_one_level : fmm_decode_two_level)(output, prod, prod_dtype, prod_stride, h_tab, sA, sB, bm, bn, C, ldc,
+                                                                           cstar32, partials, n_partials, max_partials, st, err);
+}
 
 // ---- many copies of an algorithm on small blocks (sweep_many.cu): tables of copy c at tabs[3 * c ..], its products numbered
 // c * R .. c * R + R - 1 in every buffer.
