@@ -3,10 +3,10 @@
 // sums of a fast algorithm round.  Here H = diag(signs) . blockdiag(H_h, ..., H_h) / sqrt(h), H_h Sylvester's
 // Hadamard matrix, applied to rows whose inner dimension is contiguous (A as stored; B in its [N, K] layout).
 //
-// A streaming pass (one read, one write per element): a group of h / E lanes of a warp owns one h-block, each lane
-// E consecutive elements.  The transform is the fast Walsh-Hadamard recursion in fp32, strides ascending —
-// strides below E inside a lane's registers, the rest with xor shuffles — then one multiplication by
-// fl(1 / sqrt(h)) and one rounding to the storage type.
+// A streaming pass (one read, one write per element) in fp32, then one multiplication by fl(1 / sqrt(h)) and one rounding to the
+// storage type.  Two forms of the fast Walsh-Hadamard recursion: fp32, and bf16 with h below 32, strides ascending — a group of
+// h / E lanes of a warp owns one h-block, each lane E consecutive elements, strides below E inside a lane's registers, the rest with
+// xor shuffles; and bf16 with h from 32 on, sixteen points by the tensor cores (hadamard_rotate_mma_kernel).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -69,9 +69,7 @@ __device__ __forceinline__ void store_pair(float2 x, __nv_bfloat16* y) {
 // E elements per lane, L = h / E lanes per h-block (a power of two <= 32), 32 / L blocks per warp pass.  The number of warps W
 // is chosen so that W passes are a whole number of rows: a lane then stays in its columns, its signs become mask words once
 // and for all, and a step is a constant distance in X and Y.  A warp keeps the loads of its next kAhead passes in flight
-// while it transforms one.  8192 x 13824 bf16, L2 flushed before each: h = 128 102 -> 90 us (5.0 TB/s), h = 64 116 -> 100,
-// h = 512 126 -> 115, against passes that worked out their position and signs and loaded before they transformed.  What bounds it now: the lane
-// exchanges (48 shuffles for 16 values a lane at h = 128) beside the memory system.
+// while it transforms one.  8192 x 8192 fp32, h = 128, L2 flushed before each: 92 us (5.8 TB/s).  What bounds it: the lane exchanges beside the memory system.
 template <typename T, int E, int kAhead>
 __global__ void __launch_bounds__(kRotThreads)
 hadamard_rotate_kernel(const T* X, int64_t n_blocks, int blocks_per_row, int h, const signed char* __restrict__ signs,
@@ -177,20 +175,191 @@ cudaError_t launch_rotate(const void* X, int64_t ldx, int64_t rows, int64_t K, i
   return cudaGetLastError();
 }
 
+// ------------------------------------------------------------------------------------------
+// bf16, h from 32 to 1024: bits 0, 1, 3 and 4 of the column are transformed by mma.sync (m16n8k16 with a matrix of 1 and -1: exact
+// products, fp32 sums of sixteen), the rest by packed additions, none of the seven lower bits by a lane exchange.  (tcgen05 would
+// take the operand through shared memory and the result through tensor memory, for a contraction of sixteen.)
+// A warp works on 16 x 128 values: 16 rows where h <= 128; beyond, the row index of the fragment also counts the 128-column parts of
+// an h-block, bit 7 in a lane's two rows, bits 8 and 9 in the lane (one exchange of all values each).  A lane loads and stores 16 bytes
+// at columns 8 t + 32 q of its two rows g and g + 8 (lane = 4 g + t): as a fragment, word w of such a vector is K index 2 t of the
+// half w % 2, for the value of bit 2 that w / 2 says; results come out in the same places.  Rows and columns past the end are zeros.
+// The number of warps is a multiple of the parts of a row: a warp stays in its columns, and the signs stay in registers.
+// What bounds it: the memory system.  8192 x 13824, L2 flushed before each, against the other form: h = 32 94 -> 77 us, 64 98 -> 77,
+// 128 90 -> 77 (5.9 TB/s), 256 101 -> 84, 512 115 -> 94; 8192 x 4096, h = 1024 52 -> 38.  The distance from 64-bit results is the
+// rounding to bf16 in either (1.661e-3); outputs that round otherwise than the 64-bit result: 6.0e-7 of them at h = 128 (5.8e-7 before).
+// ------------------------------------------------------------------------------------------
+constexpr int kMmaThreads = 128;
+
+__device__ __forceinline__ void mma_16(float2 (&d)[2], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+               : "=f"(d[0].x), "=f"(d[0].y), "=f"(d[1].x), "=f"(d[1].y)
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
+}
+__device__ __forceinline__ void butterfly(float2& a, float2& b) {
+  const float2 x = a;
+  a = __fadd2_rn(x, b);
+  b = __ffma2_rn(b, make_float2(-1.0f, -1.0f), x);      // x - b, one rounding
+}
+
+template <int kH>
+__global__ void __launch_bounds__(kMmaThreads, 3)
+hadamard_rotate_mma_kernel(const __nv_bfloat16* X, int64_t rows, int64_t K, const signed char* __restrict__ signs, float inv_sqrt_h,
+                           __nv_bfloat16* Y, int64_t ldx, int64_t ldy, int col_parts, int64_t row_step, int64_t warps) {
+  constexpr int kParts = kH > 128 ? kH / 128 : 1, kRows = 16 / kParts;     // 128-column parts of an h-block, rows of a warp's unit
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int64_t warp = (int64_t)blockIdx.x * (kMmaThreads / 32) + (threadIdx.x >> 5);
+  if (warp >= warps) return;
+  int64_t row[2], at_x[2], at_y[2];
+  int col[2];
+  uint32_t mask[kParts > 1 ? 2 : 1][4][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {             // fragment row g + 8 i: bit 7 is its bit 3, bit 8 its bit 2, bit 9 its bit 1
+    const int part = kParts == 1 ? 0 : i + (kParts >= 4 ? 2 * ((g >> 2) & 1) : 0) + (kParts >= 8 ? 4 * ((g >> 1) & 1) : 0);
+    row[i] = warp / col_parts * kRows + ((g + 8 * i) & (kRows - 1));
+    col[i] = ((int)(warp % col_parts) * kParts + part) * 128 + 8 * t;
+    at_x[i] = row[i] * ldx + col[i];
+    at_y[i] = row[i] * ldy + col[i];
+    if (i == 0 || kParts > 1) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        alignas(8) signed char sg[8] = {};
+        if (signs != nullptr && col[i] + 32 * q < K) *reinterpret_cast<uint2*>(sg) = *reinterpret_cast<const uint2*>(signs + col[i] + 32 * q);
+        sign_masks<__nv_bfloat16, 8>(sg, true, mask[i][q]);
+      }
+    }
+  }
+  // the matrix of a half: K index 2 t + j, column g: j meets bit 0 of the result, t its bits 3 and 4; the other half of K meets bit 1
+  const uint32_t odd = __popc(t & (g >> 1)) & 1u;
+  const uint32_t b = (odd ? 0xBF80u : 0x3F80u) | ((odd ^ (g & 1u)) ? 0xBF800000u : 0x3F800000u), minus_b = b ^ 0x80008000u;
+  uint4 raw[2][4];
+  auto load = [&]() {
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        raw[i][q] = row[i] < rows && col[i] + 32 * q < K ? *reinterpret_cast<const uint4*>(X + at_x[i] + 32 * q) : make_uint4(0u, 0u, 0u, 0u);
+  };
+  load();
+  const int64_t step_x = row_step * ldx, step_y = row_step * ldy;
+#pragma unroll 1
+  for (int64_t first = warp / col_parts * kRows; first < rows; first += row_step) {
+    float2 v[4][2][2][2];                   // [q][bit 2][bit 1][fragment row], pairs of bit 0
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const uint32_t* w0 = reinterpret_cast<const uint32_t*>(&raw[0][q]) + 2 * c;
+        const uint32_t* w1 = reinterpret_cast<const uint32_t*>(&raw[1][q]) + 2 * c;
+        const uint32_t (&m0)[4] = mask[0][q];
+        const uint32_t (&m1)[4] = mask[kParts > 1 ? 1 : 0][q];
+        const uint32_t a[4] = {w0[0] ^ m0[2 * c], w1[0] ^ m1[2 * c], w0[1] ^ m0[2 * c + 1], w1[1] ^ m1[2 * c + 1]};
+        mma_16(v[q][c][0], a, b, b);
+        mma_16(v[q][c][1], a, b, minus_b);
+      }
+    const bool here[2] = {row[0] < rows, row[1] < rows};
+    row[0] += row_step; row[1] += row_step;
+    at_x[0] += step_x; at_x[1] += step_x;
+    load();                                 // the next unit's, under this one's additions
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) butterfly(v[q][0][n][i], v[q][1][n][i]);      // bit 2
+#pragma unroll
+    for (int s = 1; s < 4 && 32 * s < kH; s <<= 1)                                  // bits 5 and 6
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if ((q & s) == 0)
+#pragma unroll
+          for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int n = 0; n < 2; ++n)
+#pragma unroll
+              for (int i = 0; i < 2; ++i) butterfly(v[q][c][n][i], v[q + s][c][n][i]);
+    if constexpr (kParts > 1) {                                                     // bit 7
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int n = 0; n < 2; ++n) butterfly(v[q][c][n][0], v[q][c][n][1]);
+    }
+#pragma unroll
+    for (int s = 16; s >= 8 && 8192 / s <= kH; s >>= 1) {                           // bits 8 and 9: partner's lane; fma(v, +-1, o) = o +- v
+      const float sgn = (lane & s) != 0 ? -1.0f : 1.0f;
+      const float2 sg2 = make_float2(sgn, sgn);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+              float2 o;
+              o.x = __shfl_xor_sync(0xffffffffu, v[q][c][n][i].x, s);
+              o.y = __shfl_xor_sync(0xffffffffu, v[q][c][n][i].y, s);
+              v[q][c][n][i] = __ffma2_rn(v[q][c][n][i], sg2, o);
+            }
+    }
+    const float2 r2 = make_float2(inv_sqrt_h, inv_sqrt_h);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        alignas(16) __nv_bfloat16 out[8];
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int n = 0; n < 2; ++n) store_pair(__fmul2_rn(v[q][c][n][i], r2), &out[4 * c + 2 * n]);
+        if (here[i] && col[i] + 32 * q < K) *reinterpret_cast<uint4*>(Y + at_y[i] + 32 * q) = *reinterpret_cast<const uint4*>(out);
+      }
+      at_y[i] += step_y;
+    }
+  }
+}
+
+template <int kH>
+cudaError_t launch_rotate_mma(const void* X, int64_t ldx, int64_t rows, int64_t K, const signed char* signs, void* Y, int64_t ldy, cudaStream_t st) {
+  constexpr int kWidth = kH > 128 ? kH : 128, kRows = 16 * 128 / kWidth;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return cudaErrorInvalidDevice;
+  const int64_t col_parts = (K + kWidth - 1) / kWidth, groups = (rows + kRows - 1) / kRows;
+  const int64_t cap = std::max<int64_t>(1, (int64_t)sms * 3 * (kMmaThreads / 32) / col_parts), at_once = std::min(cap, groups), warps = at_once * col_parts;
+  hadamard_rotate_mma_kernel<kH><<<(unsigned)((warps + kMmaThreads / 32 - 1) / (kMmaThreads / 32)), kMmaThreads, 0, st>>>(
+      (const __nv_bfloat16*)X, rows, K, signs, (float)(1.0 / std::sqrt((double)kH)), (__nv_bfloat16*)Y, ldx, ldy, (int)col_parts, at_once * kRows, warps);
+  ++fmm_launch_counter();
+  return cudaGetLastError();
+}
+
 // elements per lane: 16 bytes where the block is long enough, more once a block outgrows 32 lanes
 template <typename T>
 cudaError_t launch_rotate_t(const void* X, int64_t ldx, int64_t rows, int64_t K, int h, const signed char* signs, void* Y,
                             int64_t ldy, cudaStream_t st) {
   constexpr int kVec = 16 / (int)sizeof(T);          // 4 (fp32) or 8 (bf16)
+  if constexpr (sizeof(T) == 2) {
+    switch (h) {
+      case 32: return launch_rotate_mma<32>(X, ldx, rows, K, signs, Y, ldy, st);
+      case 64: return launch_rotate_mma<64>(X, ldx, rows, K, signs, Y, ldy, st);
+      case 128: return launch_rotate_mma<128>(X, ldx, rows, K, signs, Y, ldy, st);
+      case 256: return launch_rotate_mma<256>(X, ldx, rows, K, signs, Y, ldy, st);
+      case 512: return launch_rotate_mma<512>(X, ldx, rows, K, signs, Y, ldy, st);
+      case 1024: return launch_rotate_mma<1024>(X, ldx, rows, K, signs, Y, ldy, st);
+    }
+  }
   if (h == 2) return launch_rotate<T, 2>(X, ldx, rows, K, h, signs, Y, ldy, st);
   if (h == 4) return launch_rotate<T, 4>(X, ldx, rows, K, h, signs, Y, ldy, st);
-  if (h < 128) return launch_rotate<T, kVec>(X, ldx, rows, K, h, signs, Y, ldy, st);
-  // from 128 on, more elements per lane: every doubling trades a lane-exchange stage (a shuffle and an FMA per
+  if (h < 128 || sizeof(T) == 2) return launch_rotate<T, kVec>(X, ldx, rows, K, h, signs, Y, ldy, st);
+  // fp32 from 128 on, more elements per lane: every doubling trades a lane-exchange stage (a shuffle and an FMA per
   // element) for an in-register one (half a packed instruction per element) — the kernel is issue-bound
-  // (32 elements per lane lose more to register pressure than they save: 2.8 against 3.6 TB/s at h = 512, bf16)
-  if (h <= 32 * 2 * kVec) return launch_rotate<T, 2 * kVec>(X, ldx, rows, K, h, signs, Y, ldy, st);
-  if (h <= 32 * 16) return launch_rotate<T, 16>(X, ldx, rows, K, h, signs, Y, ldy, st);
-  return launch_rotate<T, 32>(X, ldx, rows, K, h, signs, Y, ldy, st);
+  if constexpr (sizeof(T) == 4) {
+    if (h <= 32 * 2 * kVec) return launch_rotate<T, 2 * kVec>(X, ldx, rows, K, h, signs, Y, ldy, st);
+    if (h <= 32 * 16) return launch_rotate<T, 16>(X, ldx, rows, K, h, signs, Y, ldy, st);
+    return launch_rotate<T, 32>(X, ldx, rows, K, h, signs, Y, ldy, st);
+  }
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace
