@@ -284,7 +284,9 @@ struct TileParams {
   unsigned long long wait_limit_ns;   // bound of every mbarrier wait
 };
 
-template <int BN, bool kFp8>
+// kPack > 1: blocks of at most 128 / kPack rows and columns, kPack products a tile.  Product p of a tile has rows and columns
+// [128 / kPack * p, ..) of it, the copies bring them with one box, and the blocks off the diagonal are not read.
+template <int BN, bool kFp8, int kPack>
 __global__ void __launch_bounds__(kNumThreads, 1)
 block_products_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                       void* __restrict__ out, const float* __restrict__ sA, const float* __restrict__ sB,
@@ -331,8 +333,9 @@ block_products_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
   grid_dependency_wait();     // operands and scales come from the previous kernel of the stream
 
   const int num_kb = (tp.kbytes + BKB - 1) / BKB;
+  static_assert(kPack == 1 || BN == BM, "square tiles");
   const int tiles_per_batch = tp.tiles_m * tp.tiles_n;
-  const int total_tiles = tiles_per_batch * tp.batches * tp.groups;
+  const int total_tiles = kPack > 1 ? (tp.batches + kPack - 1) / kPack : tiles_per_batch * tp.batches * tp.groups;
   const int kelems_per_stage = BKB / tp.elem_bytes;
 
   if (warp == 0) {
@@ -352,8 +355,8 @@ block_products_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
           const uint32_t sa = smem_u32(smem + stage * L::kStageBytes);
           const uint32_t sb = sa + L::kABytes;
           mbar_arrive_expect_tx(full_bar(stage), (uint32_t)L::kStageBytes);
-          tma_load_3d(sa, &map_a, full_bar(stage), kb * kelems_per_stage, g * tp.rows_a + tm * BM, r);
-          tma_load_3d(sb, &map_b, full_bar(stage), kb * kelems_per_stage, g * tp.rows_b + tn * BN, r);
+          tma_load_3d(sa, &map_a, full_bar(stage), kb * kelems_per_stage, kPack > 1 ? 0 : g * tp.rows_a + tm * BM, kPack > 1 ? tile * kPack : r);
+          tma_load_3d(sb, &map_b, full_bar(stage), kb * kelems_per_stage, kPack > 1 ? 0 : g * tp.rows_b + tn * BN, kPack > 1 ? tile * kPack : r);
           if (++stage == L::kStages) { stage = 0; phase ^= 1u; }
         }
       }
@@ -420,20 +423,21 @@ block_products_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_co
     float alpha = 1.0f;
     if (tp.out_mode == 1 && sA != nullptr && sB != nullptr) alpha = sA[0] * sB[0];
     for (int tile = blockIdx.x; tile < total_tiles && ok; tile += gridDim.x) {
-      const int r = tile / tiles_per_batch;     // index of the (batch, group) product
-      const int rem = tile - r * tiles_per_batch;
+      constexpr int kSide = 128 / kPack;            // rows (packed: and columns) of a product in the tile
+      const int r = kPack > 1 ? tile * kPack + quad * 32 / kSide : tile / tiles_per_batch;     // index of the (batch, group) product
+      const int rem = kPack > 1 ? 0 : tile - r * tiles_per_batch;
       const int tm = rem / tp.tiles_n, tn = rem - tm * tp.tiles_n;
       ok = mbar_wait(tfull_bar(acc), acc_phase, abort_flag, 0x23, status, tp.wait_limit_ns);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      const int row = tm * BM + quad * 32 + lane;
-      const bool row_ok = row < tp.rows_a;
+      const int row = tm * BM + (quad * 32 + lane) % kSide;
+      const bool row_ok = row < tp.rows_a && (kPack == 1 || r < tp.batches);
       const long long row_off = (long long)r * tp.o_batch + (long long)row * tp.ldo;
 #pragma unroll 1
-      for (int c = 0; c < BN / 32; ++c) {
+      for (int c = 0; c < BN / kPack / 32; ++c) {
         uint32_t v[32];
-        const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN + c * 32);
+        const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN + (kPack > 1 ? quad * 32 / kSide * kSide : 0) + c * 32);
         tc_ld32(taddr, v);
         tc_wait_ld();
         const int col0 = tn * BN + c * 32;
@@ -827,15 +831,15 @@ EncodeTiledFn get_encode_fn() {
   return fn;
 }
 
-// K-major operand [batches][rows][kdim] -> 3-D map, box {128 bytes of K, box_rows, 1}, 128-byte swizzle.
+// K-major operand [batches][rows][kdim] -> 3-D map, box {128 bytes of K, box_rows, box_batches}, 128-byte swizzle.
 bool make_operand_map(CUtensorMap* map, bool fp8, const void* ptr, int64_t rows, int64_t kdim, int64_t ld,
-                      int64_t batch_stride, int batches, int box_rows) {
+                      int64_t batch_stride, int batches, int box_rows, int box_batches = 1) {
   EncodeTiledFn fn = get_encode_fn();
   if (!fn) return false;
   const int es = fp8 ? 1 : 2;
   cuuint64_t dims[3] = {(cuuint64_t)kdim, (cuuint64_t)rows, (cuuint64_t)batches};
   cuuint64_t strides[2] = {(cuuint64_t)(ld * es), (cuuint64_t)((batches > 1 ? batch_stride : rows * ld) * es)};
-  cuuint32_t box[3] = {(cuuint32_t)(BKB / es), (cuuint32_t)box_rows, 1u};
+  cuuint32_t box[3] = {(cuuint32_t)(BKB / es), (cuuint32_t)box_rows, (cuuint32_t)box_batches};
   cuuint32_t estr[3] = {1u, 1u, 1u};
   CUresult rc = fn(map, fp8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
                    const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -859,13 +863,13 @@ int rows_32b_aligned(const BlockProductArgs& a) {
   return (reinterpret_cast<uintptr_t>(a.out) % 32 == 0) && ((a.ldo * es) % 32 == 0) && ((a.o_batch * es) % 32 == 0);
 }
 
-template <int BN, bool kFp8>
+template <int BN, bool kFp8, int kPack = 1>
 fmm_status launch_t(const BlockProductArgs& a, cudaStream_t st) {
   using L = SmemLayout<BN>;
   CUtensorMap ma, mb;
   const int groups = a.groups > 1 ? a.groups : 1;
-  if (!make_operand_map(&ma, kFp8, a.A, a.rows_a * groups, a.kdim, a.lda, a.a_batch, a.batches, BM)) return FMM_ERR_CUDA;
-  if (!make_operand_map(&mb, kFp8, a.B, a.rows_b * groups, a.kdim, a.ldb, a.b_batch, a.batches, BN)) return FMM_ERR_CUDA;
+  if (!make_operand_map(&ma, kFp8, a.A, a.rows_a * groups, a.kdim, a.lda, a.a_batch, a.batches, BM / kPack, kPack)) return FMM_ERR_CUDA;
+  if (!make_operand_map(&mb, kFp8, a.B, a.rows_b * groups, a.kdim, a.ldb, a.b_batch, a.batches, BN / kPack, kPack)) return FMM_ERR_CUDA;
   TileParams tp;
   tp.rows_a = (int)a.rows_a; tp.rows_b = (int)a.rows_b;
   tp.elem_bytes = kFp8 ? 1 : 2;
@@ -880,12 +884,12 @@ fmm_status launch_t(const BlockProductArgs& a, cudaStream_t st) {
   tp.row_scale = a.row_scale; tp.col_scale = a.col_scale; tp.rs_batch = a.rs_batch; tp.cs_batch = a.cs_batch;
   tp.selftest_no_producer = a.selftest_no_producer;
   tp.wait_limit_ns = a.wait_limit_ns ? a.wait_limit_ns : kDefaultWaitLimitNs;
-  const long long total = (long long)tp.tiles_m * tp.tiles_n * tp.batches * tp.groups;
+  const long long total = kPack > 1 ? ((long long)tp.batches + kPack - 1) / kPack : (long long)tp.tiles_m * tp.tiles_n * tp.batches * tp.groups;
   if (total <= 0) return FMM_OK;
   const int sms = sm_count();
   if (sms <= 0) return FMM_ERR_CUDA;
   const int grid = (int)(total < sms ? total : sms);
-  auto k = block_products_kernel<BN, kFp8>;
+  auto k = block_products_kernel<BN, kFp8, kPack>;
   static unsigned long long smem_ok = 0;   // per template instantiation, one bit per device
   if (fmm_allow_dynamic_smem(k, L::kTotal, &smem_ok) != cudaSuccess) return FMM_ERR_CUDA;
   if (launch_dependent(k, dim3(grid), dim3(kNumThreads), (size_t)L::kTotal, st, ma, mb, a.out, a.sA, a.sB, tp, a.status) != cudaSuccess)
@@ -1762,6 +1766,12 @@ fmm_status launch_block_products(const BlockProductArgs& a, cudaStream_t st) {
   // large problems: CTA pairs on 256 x 256 tiles (less L2 traffic per flop)
   if (a.rows_a > 128 && a.rows_b > 128 && !a.selftest_no_producer)
     return fp8 ? launch_pair<true>(a, st) : launch_pair<false>(a, st);
+  // small blocks, more products than SMs: several to a tile (8,400 products of 32 x 32 x 32, e4m3: 48 -> 20 us)
+  const int64_t side = std::max(a.rows_a, a.rows_b);
+  if (side <= 64 && a.groups <= 1 && a.batches > sm_count() && !a.selftest_no_producer) {
+    if (side <= 32) return fp8 ? launch_t<128, true, 4>(a, st) : launch_t<128, false, 4>(a, st);
+    return fp8 ? launch_t<128, true, 2>(a, st) : launch_t<128, false, 2>(a, st);
+  }
   // narrow problems use the 128-column tile (less padding, more tiles in flight)
   const bool narrow = a.rows_b <= 128;
   if (fp8) return narrow ? launch_t<128, true>(a, st) : launch_t<256, true>(a, st);
