@@ -195,12 +195,15 @@ fmm_status encode_operand(const fmm_gemm_desc* d, const void* X, int64_t ldx, in
 fmm_status quantize_operand(const fmm_gemm_desc* d, const void* X, int64_t ldx, int64_t rows, int64_t cols, void* hat,
                             unsigned* amax, float* scale, bool b_side, cudaStream_t st) {
   const int mode = d->scale_mode;
-  const int srows = b_side ? 128 : 1, bf16_first = b_side ? 1 : 0;   // model schedule only
+  if (mode == 3) {
+    FMM_CUDA(launch_quantize_groups(d->storage, X, ldx, rows, cols, hat, scale, b_side, st));
+    return FMM_OK;
+  }
   if (mode != 0) {
     FMM_CUDA(cudaMemsetAsync(amax, 0, scale_words(mode, 1, rows, cols, b_side) * 4, st));
-    FMM_CUDA(launch_quantize_plain(d->storage, d->product, X, ldx, rows, cols, hat, amax, scale, true, mode, srows, bf16_first, st));
+    FMM_CUDA(launch_quantize_plain(d->storage, d->product, X, ldx, rows, cols, hat, amax, scale, true, mode, st));
   }
-  FMM_CUDA(launch_quantize_plain(d->storage, d->product, X, ldx, rows, cols, hat, amax, scale, false, mode, srows, bf16_first, st));
+  FMM_CUDA(launch_quantize_plain(d->storage, d->product, X, ldx, rows, cols, hat, amax, scale, false, mode, st));
   return FMM_OK;
 }
 

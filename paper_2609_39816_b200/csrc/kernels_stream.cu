@@ -42,8 +42,7 @@ encode_kernel(const EncodeJob job_a, const EncodeJob job_b, int use_scale) {
 template <typename SrcT, typename DstT, bool kAmaxOnly>
 __global__ void __launch_bounds__(256)
 quantize_plain_kernel(const SrcT* __restrict__ X, int64_t ldx, int64_t rows, int64_t cols, DstT* __restrict__ out,
-                      unsigned* __restrict__ amax_bits, float* __restrict__ scale_out, int mode, int scale_rows,
-                      int bf16_first) {
+                      unsigned* __restrict__ amax_bits, float* __restrict__ scale_out, int mode) {
   constexpr int VE = Vec16<SrcT>::kElems;
   constexpr int NP = VE / 2;
   constexpr int kU = 4;
@@ -79,29 +78,11 @@ quantize_plain_kernel(const SrcT* __restrict__ X, int64_t ldx, int64_t rows, int
       const bool on = base + u * stride < nvec;
       float2 v[NP];
       Vec16<SrcT>::unpack(raw[u], v);
-      // model schedule (mode 3): one scale per 128 consecutive entries of a row, shared by scale_rows rows
-      const int64_t sidx3 = (row[u] / scale_rows) * ((cols + 127) >> 7) + (col[u] >> 7);
-      if (mode == 3 && bf16_first) {
-#pragma unroll
-        for (int i = 0; i < NP; ++i) {
-          v[i].x = __bfloat162float(__float2bfloat16_rn(v[i].x));
-          v[i].y = __bfloat162float(__float2bfloat16_rn(v[i].y));
-        }
-      }
       if (kAmaxOnly) {
         float a = 0.0f;
 #pragma unroll
         for (int i = 0; i < NP; ++i) a = fmaxf(a, fmaxf(fabsf(v[i].x), fabsf(v[i].y)));
-        if (mode == 3) {
-          constexpr int kLanesPerGroup = 128 / VE;
-          if ((vec_per_row & 31) == 0) {   // a warp's 32 consecutive vectors lie in one row
-            const unsigned mask = kLanesPerGroup == 32 ? 0xffffffffu : (0xffffu << (threadIdx.x & 16));
-            const unsigned wmax = __reduce_max_sync(mask, on ? __float_as_uint(a) : 0u);
-            if ((threadIdx.x & (kLanesPerGroup - 1)) == 0 && wmax != 0u) atomicMax(&amax_bits[sidx3], wmax);
-          } else if (on && a > 0.0f) {
-            atomicMax(&amax_bits[sidx3], __float_as_uint(a));
-          }
-        } else if (mode == 2) {
+        if (mode == 2) {
           if ((vec_per_row & 31) == 0) {   // a warp's 32 consecutive vectors lie in one row
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
@@ -113,17 +94,7 @@ quantize_plain_kernel(const SrcT* __restrict__ X, int64_t ldx, int64_t rows, int
           tmax = fmaxf(tmax, a);
         }
       } else if (on) {
-        if (mode == 3) {
-          const float amax = __uint_as_float(amax_bits[sidx3]);
-          const float sc = amax > 0.0f ? __fdiv_rn(amax, 448.0f) : 1.0f;
-          if constexpr (sizeof(DstT) == 1) {
-            divide_for_e4m3<NP>(v, sc);
-          } else {
-#pragma unroll
-            for (int i = 0; i < NP; ++i) { v[i].x = __fdiv_rn(v[i].x, sc); v[i].y = __fdiv_rn(v[i].y, sc); }
-          }
-          if ((col[u] & 127) == 0 && (row[u] % scale_rows) == 0 && scale_out) scale_out[sidx3] = sc;
-        } else if (mode == 2) {
+        if (mode == 2) {
           const float amax = __uint_as_float(amax_bits[row[u]]);
           const float sc = amax > 0.0f ? __fdiv_rn(amax, 448.0f) : 1.0f;
           if constexpr (sizeof(DstT) == 1) {
@@ -146,7 +117,7 @@ quantize_plain_kernel(const SrcT* __restrict__ X, int64_t ldx, int64_t rows, int
       }
     }
   }
-  if (kAmaxOnly && mode != 2 && mode != 3) {
+  if (kAmaxOnly && mode != 2) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
     if ((threadIdx.x & 31) == 0 && tmax > 0.0f) atomicMax(&s_amax, __float_as_uint(tmax));
@@ -155,18 +126,114 @@ quantize_plain_kernel(const SrcT* __restrict__ X, int64_t ldx, int64_t rows, int
   }
 }
 
+// The model schedule's control: codes and scales of groups of 128 columns of kRows rows (1: the input, 128: the weight, which goes
+// through bf16 first) in one pass.  A block holds 128 columns of 128 rows (weight) or 32 rows (input) in registers, a warp every
+// eighth row, a lane four values of each; maxima by warp reduction, for the weight over the block's warps too.
+// Two passes with an atomic maximum per 16 or 32 lanes (per lane where rows are no multiple of 32 vectors) took 64 + 6 us an operand
+// for 216 x 1472 fp32, where this takes 3 and 4.  classical_gemm, 2048 x 11008 x 4096 bf16: 332 -> 187 us (the weight 54, the input 26
+// of it); 2048 x 4096 x 12288 fp32 407 -> 179 (48 for the weight, 5.2 TB/s).  bf16 weights are bound by the quotients' instructions.
+template <typename SrcT, int kRows>
+__global__ void __launch_bounds__(256)
+quantize_groups_kernel(const SrcT* __restrict__ X, int64_t ldx, int64_t rows, int64_t cols, __nv_fp8_storage_t* __restrict__ out,
+                       float* __restrict__ scale_out) {
+  constexpr int kPer = kRows == 128 ? 16 : 4;            // rows of a warp
+  __shared__ unsigned block_max;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t gk = (cols + 127) >> 7, g = blockIdx.x % gk, row0 = blockIdx.x / gk * (8 * kPer) + warp, t = g * 128 + lane * 4;
+  if (kRows == 128) {
+    if (threadIdx.x == 0) block_max = 0u;
+    __syncthreads();
+  }
+  float2 v[kPer][2];
+  unsigned amax[kPer];
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    const int64_t row = row0 + 8 * i;
+    v[i][0] = v[i][1] = make_float2(0.0f, 0.0f);
+    if (row < rows && t < cols) {
+      if constexpr (sizeof(SrcT) == 4) {
+        const float4 raw = __ldcs(reinterpret_cast<const float4*>(X + row * ldx + t));
+        v[i][0] = make_float2(raw.x, raw.y);
+        v[i][1] = make_float2(raw.z, raw.w);
+      } else {
+        const uint2 raw = __ldcs(reinterpret_cast<const uint2*>(X + row * ldx + t));
+        v[i][0] = make_float2(__uint_as_float(raw.x << 16), __uint_as_float(raw.x & 0xFFFF0000u));
+        v[i][1] = make_float2(__uint_as_float(raw.y << 16), __uint_as_float(raw.y & 0xFFFF0000u));
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < kPer; ++i) {
+    if (kRows == 128 && sizeof(SrcT) == 4) {
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const float2 b = __bfloat1622float2(__floats2bfloat162_rn(v[i][k].x, v[i][k].y));
+        v[i][k] = b;
+      }
+    }
+    const float a = fmaxf(fmaxf(fabsf(v[i][0].x), fabsf(v[i][0].y)), fmaxf(fabsf(v[i][1].x), fabsf(v[i][1].y)));     // drops NaN
+    amax[i] = __float_as_uint(fmaxf(a, 0.0f));
+  }
+  if (kRows == 128) {
+    unsigned m = 0u;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) m = max(m, amax[i]);
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) atomicMax(&block_max, m);
+    __syncthreads();
+    m = block_max;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) amax[i] = m;
+    if (threadIdx.x == 0) scale_out[blockIdx.x / gk * gk + g] = m != 0u ? __fdiv_rn(__uint_as_float(m), 448.0f) : 1.0f;
+  } else {
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) amax[i] = __reduce_max_sync(0xffffffffu, amax[i]);
+  }
+  auto scale_of = [](unsigned m) { return m != 0u ? __fdiv_rn(__uint_as_float(m), 448.0f) : 1.0f; };
+  auto store = [&](int i) {
+    const int64_t row = row0 + 8 * i;
+    if (row < rows && t < cols) store_vec<2>(out + row * cols + t, v[i], false);
+  };
+  if (kRows == 128) {
+    const float s = scale_of(amax[0]);
+    if (e4m3_scale_ok(s)) {               // one reciprocal and one branch for the block's 64 values a thread
+      const float r = e4m3_reciprocal(s);
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        v[i][0] = e4m3_quotient(v[i][0], make_float2(r, r), make_float2(-s, -s));
+        v[i][1] = e4m3_quotient(v[i][1], make_float2(r, r), make_float2(-s, -s));
+        store(i);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        v[i][0] = make_float2(__fdiv_rn(v[i][0].x, s), __fdiv_rn(v[i][0].y, s));
+        v[i][1] = make_float2(__fdiv_rn(v[i][1].x, s), __fdiv_rn(v[i][1].y, s));
+        store(i);
+      }
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+      const float s = scale_of(amax[i]);
+      if (row0 + 8 * i < rows && lane == 0) scale_out[(row0 + 8 * i) * gk + g] = s;
+      divide_for_e4m3<2>(v[i], s);
+      store(i);
+    }
+  }
+}
+
 template <typename SrcT, typename DstT>
 static cudaError_t launch_quantize_plain_t(const void* X, int64_t ldx, int64_t rows, int64_t cols, void* out,
-                                           unsigned* amax_bits, float* scale, bool amax_only, int mode, int scale_rows,
-                                           int bf16_first, cudaStream_t st) {
+                                           unsigned* amax_bits, float* scale, bool amax_only, int mode, cudaStream_t st) {
   constexpr int VE = Vec16<SrcT>::kElems;
   const int64_t nvec = rows * (cols / VE);
   if (nvec == 0) return cudaSuccess;
   const int grid = (int)std::min<int64_t>((nvec + 256 * 4 - 1) / (256 * 4), 148 * 16);
   if (amax_only)
-    quantize_plain_kernel<SrcT, DstT, true><<<grid, 256, 0, st>>>((const SrcT*)X, ldx, rows, cols, (DstT*)out, amax_bits, scale, mode, scale_rows > 0 ? scale_rows : 1, bf16_first);
+    quantize_plain_kernel<SrcT, DstT, true><<<grid, 256, 0, st>>>((const SrcT*)X, ldx, rows, cols, (DstT*)out, amax_bits, scale, mode);
   else
-    quantize_plain_kernel<SrcT, DstT, false><<<grid, 256, 0, st>>>((const SrcT*)X, ldx, rows, cols, (DstT*)out, amax_bits, scale, mode, scale_rows > 0 ? scale_rows : 1, bf16_first);
+    quantize_plain_kernel<SrcT, DstT, false><<<grid, 256, 0, st>>>((const SrcT*)X, ldx, rows, cols, (DstT*)out, amax_bits, scale, mode);
   ++fmm_launch_counter();
   return cudaGetLastError();
 }
@@ -603,17 +670,29 @@ cudaError_t launch_exact_t(const T* A, int64_t lda, const T* B, int64_t ldb, int
 
 }  // namespace
 
+cudaError_t launch_quantize_groups(int storage, const void* X, int64_t ldx, int64_t rows, int64_t cols, void* out, float* scale, bool weight,
+                                   cudaStream_t st) {
+  const int64_t gk = (cols + 127) / 128, per = weight ? 128 : 32, blocks = gk * ((rows + per - 1) / per);
+  if (blocks > 0x7fffffff || (storage != FMM_F32 && storage != FMM_BF16)) return cudaErrorInvalidValue;
+  __nv_fp8_storage_t* codes = static_cast<__nv_fp8_storage_t*>(out);
+  if (storage == FMM_F32 && weight) quantize_groups_kernel<float, 128><<<(unsigned)blocks, 256, 0, st>>>((const float*)X, ldx, rows, cols, codes, scale);
+  else if (storage == FMM_F32) quantize_groups_kernel<float, 1><<<(unsigned)blocks, 256, 0, st>>>((const float*)X, ldx, rows, cols, codes, scale);
+  else if (weight) quantize_groups_kernel<__nv_bfloat16, 128><<<(unsigned)blocks, 256, 0, st>>>((const __nv_bfloat16*)X, ldx, rows, cols, codes, scale);
+  else quantize_groups_kernel<__nv_bfloat16, 1><<<(unsigned)blocks, 256, 0, st>>>((const __nv_bfloat16*)X, ldx, rows, cols, codes, scale);
+  ++fmm_launch_counter();
+  return cudaGetLastError();
+}
+
 cudaError_t launch_quantize_plain(int storage, int product, const void* X, int64_t ldx, int64_t rows, int64_t cols,
-                                  void* out, unsigned* amax_bits, float* scale, bool amax_only, int mode, int scale_rows,
-                                  int bf16_first, cudaStream_t st) {
+                                  void* out, unsigned* amax_bits, float* scale, bool amax_only, int mode, cudaStream_t st) {
   if (storage == FMM_F32 && product == FMM_BF16)
-    return launch_quantize_plain_t<float, __nv_bfloat16>(X, ldx, rows, cols, out, amax_bits, scale, amax_only, mode, scale_rows, bf16_first, st);
+    return launch_quantize_plain_t<float, __nv_bfloat16>(X, ldx, rows, cols, out, amax_bits, scale, amax_only, mode, st);
   if (storage == FMM_BF16 && product == FMM_BF16)
-    return launch_quantize_plain_t<__nv_bfloat16, __nv_bfloat16>(X, ldx, rows, cols, out, amax_bits, scale, amax_only, mode, scale_rows, bf16_first, st);
+    return launch_quantize_plain_t<__nv_bfloat16, __nv_bfloat16>(X, ldx, rows, cols, out, amax_bits, scale, amax_only, mode, st);
   if (storage == FMM_F32 && product == FMM_E4M3)
-    return launch_quantize_plain_t<float, __nv_fp8_storage_t>(X, ldx, rows, cols, out, amax_bits, scale, amax_only, mode, scale_rows, bf16_first, st);
+    return launch_quantize_plain_t<float, __nv_fp8_storage_t>(X, ldx, rows, cols, out, amax_bits, scale, amax_only, mode, st);
   if (storage == FMM_BF16 && product == FMM_E4M3)
-    return launch_quantize_plain_t<__nv_bfloat16, __nv_fp8_storage_t>(X, ldx, rows, cols, out, amax_bits, scale, amax_only, mode, scale_rows, bf16_first, st);
+    return launch_quantize_plain_t<__nv_bfloat16, __nv_fp8_storage_t>(X, ldx, rows, cols, out, amax_bits, scale, amax_only, mode, st);
   return cudaErrorInvalidValue;
 }
 

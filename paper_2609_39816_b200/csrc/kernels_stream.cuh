@@ -70,8 +70,11 @@ cudaError_t launch_encode(int storage, int product, const void* X, int64_t ldx, 
 // The same decisions for a whole operand taken as one block with coefficient 1 (the classical control): rows x cols
 // of `storage` -> `product` dtype, mode 0 / 1 / 2 as use_scale above (amax_bits, scale: one word, or one per row).
 cudaError_t launch_quantize_plain(int storage, int product, const void* X, int64_t ldx, int64_t rows, int64_t cols,
-                                  void* out, unsigned* amax_bits, float* scale, bool amax_only, int mode, int scale_rows,
-                                  int bf16_first, cudaStream_t st);
+                                  void* out, unsigned* amax_bits, float* scale, bool amax_only, int mode, cudaStream_t st);
+// and the model schedule's (use_scale 3) in one pass: e4m3 codes, scales [rows][ceil(cols/128)], or of blocks of 128 rows for
+// the weight, which is rounded to bf16 first.
+cudaError_t launch_quantize_groups(int storage, const void* X, int64_t ldx, int64_t rows, int64_t cols, void* out, float* scale, bool weight,
+                                   cudaStream_t st);
 
 // Two operands in one launch (A and B of one product, encoded side by side); b may be null.  Fields as the arguments
 // of launch_encode.

@@ -1,0 +1,41 @@
+"""Codes and scales of the model schedule's classical control, byte for byte against one fp32 division a code: operands smaller than
+a block of threads, ragged in both directions, zero groups, scales below the quotient rule's range, padded rows."""
+import pytest
+import torch
+
+import gpu_util as gu
+
+pytestmark = pytest.mark.gpu
+
+
+def _align(x):
+    return (x + 1023) // 1024 * 1024
+
+
+@pytest.mark.parametrize("storage", ["bf16", "f32"])
+@pytest.mark.parametrize("M,K,N", [(1, 16, 8), (33, 272, 136), (216, 1472, 800), (129, 8336, 264), (40, 128, 1032)])
+def test_codes(storage, M, K, N):
+    lib = gu.fmm()
+    td = torch.bfloat16 if storage == "bf16" else torch.float32
+    gen = torch.Generator(device="cuda").manual_seed(M + K)
+    A, W = torch.randn(M, K + 8, device="cuda", generator=gen), torch.randn(N, K, device="cuda", generator=gen)
+    A[:, ::53] *= 300.0
+    A[M // 2, :128] = 0.0
+    A[M // 3, K // 2 :] *= 2.0 ** -118
+    W[: N // 2, K // 2 :] *= 2.0 ** -115
+    A, W = A.to(td), W.to(td)
+    d = lib.GemmDesc.make(M, K, N, storage, "e4m3", "f32", weight_layout=True, scale_mode=3, lda=K + 8)
+    ws = gu.workspace(lib.classical_gemm_workspace(d))
+    lib.classical_gemm(d, A, W, torch.empty(M, N, device="cuda"), ws)
+    lib.device_status(ws)
+    end = ws.numel() - _align(N * K) - _align(M * K)              # the codes are the workspace's last two regions
+    for X, rows, at in ((A[:, :K], 1, end), (W, 128, end + _align(M * K))):
+        x = X.float() if rows == 1 else X.bfloat16().float()
+        R, C = x.shape
+        pad = torch.zeros(-(-R // rows) * rows, -(-C // 128) * 128, device="cuda")
+        pad[:R, :C] = x
+        b = pad.view(-1, rows, pad.shape[1] // 128, 128)
+        amax = b.abs().amax(dim=(1, 3), keepdim=True)
+        s = torch.where(amax > 0, amax / torch.full_like(amax, 448), torch.ones_like(amax))
+        want = (b / s).to(torch.float8_e4m3fn).view(torch.uint8).view(pad.shape)[:R, :C]
+        assert torch.equal(ws[at : at + R * C].view(R, C), want)
