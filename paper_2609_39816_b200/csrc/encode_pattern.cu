@@ -117,20 +117,21 @@ __device__ __forceinline__ void store_hint(char* p, const float2 (&a)[2], uint64
                ::"l"(p), "r"(*reinterpret_cast<const uint32_t*>(&lo)), "r"(*reinterpret_cast<const uint32_t*>(&hi)), "l"(policy) : "memory");
 }
 
-// weights are rounded to bf16 before they are quantised under the model schedule
+// weights are rounded to bf16 before they are quantised under the model schedule; kNegate: and negated
+template <bool kNegate>
 __device__ __forceinline__ void through_bf16(float2 (&a)[NP]) {
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
     const __nv_bfloat162 b = __floats2bfloat162_rn(a[i].x, a[i].y);
-    const uint32_t u = *reinterpret_cast<const uint32_t*>(&b);
+    const uint32_t u = *reinterpret_cast<const uint32_t*>(&b) ^ (kNegate ? 0x80008000u : 0u);
     a[i] = make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u));
   }
 }
 
 struct PatSmem {
   unsigned amax[kProducts];
-  // pairs (f, f, g, g).  kScaled: x / scale = (x * f) * g, both steps exact; groups: the scale's reciprocal and its negative
-  // (e4m3_quotient), of a warp's group (A) or the block's ([0], B)
+  // pairs (f, f, g, g).  kScaled: x / scale = (x * f) * g, both steps exact; groups: the scale's reciprocal and its negative,
+  // or their negatives (kMinusZero, e4m3_quotient), of a warp's group (A) or the block's ([0], B)
   float4 factors[kPatThreads / 32][kProducts];
 };
 
@@ -146,7 +147,7 @@ __device__ __noinline__ void exact_codes(const SrcT* src, const CellAt cell_at, 
     a[0] = __ffma2_rn(make_float2(w, w), make_float2(v.x, v.y), a[0]);
     a[1] = __ffma2_rn(make_float2(w, w), make_float2(v.z, v.w), a[1]);
   }
-  if (kB) through_bf16(a);
+  if (kB) through_bf16<false>(a);
   const float2 q[2] = {make_float2(__fdiv_rn(a[0].x, scale), __fdiv_rn(a[0].y, scale)), make_float2(__fdiv_rn(a[1].x, scale), __fdiv_rn(a[1].y, scale))};
   store_vec<2>(reinterpret_cast<__nv_fp8_storage_t*>(dst), q, false);
 }
@@ -218,6 +219,10 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
   constexpr bool kFindMax = kPass == kAmax || kPass == kGroupAmax;
   constexpr bool kLoop = kFindMax || kPass == kGroupScaled;
   constexpr bool kKeepMax = kFindMax && kKind == kScheme;     // maxima in registers until the end; coefficients leave no room for them
+  // Group quotients are taken of negated sums where a sum may be -0 (see e4m3_quotient).  Without factors it may not, but through
+  // bf16 it is where bf16 has nothing that small (bf16 cells add up to multiples of its smallest number).
+  constexpr bool kMinusZero = kKind != kScheme || (kB && sizeof(SrcT) == 4);
+  constexpr float kSign = kMinusZero ? -1.0f : 1.0f;
   static_assert(128 / E == 32 && (kB || (kPass != kGroupAmax && kPass != kGroupScaled)), "a group's columns are a warp's");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const SrcT* __restrict__ X = static_cast<const SrcT*>(j.X);
@@ -242,7 +247,7 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
   if (kPass == kGroupScaled) {
     if (tid < kProducts) {
       const float scale = group_scale(__uint_as_float(j.amax_bits[sidx + tid * sstep])), r = e4m3_reciprocal(scale);
-      sm.factors[0][tid] = make_float4(r, r, -scale, -scale);
+      sm.factors[0][tid] = make_float4(kSign * r, kSign * r, -kSign * scale, -kSign * scale);
       if ((rows0 & 127) == 0) j.scale_out[sidx + tid * sstep] = scale;
       odd = !e4m3_scale_ok(scale);
     }
@@ -302,7 +307,7 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
         const int r = u * 32 + lane;
         if (r < kProducts) {
           const float scale = group_scale(__uint_as_float(keep[u])), f = e4m3_reciprocal(scale);
-          sm.factors[warp][r] = make_float4(f, f, -scale, -scale);
+          sm.factors[warp][r] = make_float4(kSign * f, kSign * f, -kSign * scale, -kSign * scale);
           j.scale_out[sidx + r * sstep] = scale;
           odd = odd || !e4m3_scale_ok(scale);
         }
@@ -316,7 +321,7 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
       if (odd) {
         for (int r = 0; r < kProducts; ++r)
           exact_codes<SrcT, kB>(src, [&](int c) { return (int64_t)(c / kGrid) * j.br * j.ldx + (int64_t)(c % kGrid) * j.bc; },
-                                kKind == kScheme ? nullptr : coefs, r, -sm.factors[kB ? 0 : warp][r].w, dst + r * rbytes);
+                                kKind == kScheme ? nullptr : coefs, r, fabsf(sm.factors[kB ? 0 : warp][r].w), dst + r * rbytes);
         continue;
       }
     }
@@ -324,7 +329,12 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
       constexpr int r = decltype(rc)::value;
       float2 acc[NP];
       block_sum<kB, kKind, r>(acc, x, coefs);
-      if constexpr (kPass == kGroupScaled) through_bf16(acc);
+      if constexpr (kPass == kGroupScaled) {
+        through_bf16<kMinusZero>(acc);
+      } else if constexpr (kPass == kGroupOneRow && kMinusZero) {
+#pragma unroll
+        for (int i = 0; i < NP; ++i) acc[i] = make_float2(-acc[i].x, -acc[i].y);
+      }
       if constexpr (kFindMax && !kKeepMax) {
         const float a = max3(max3(0.0f, fabsf(acc[0].x), fabsf(acc[0].y)), fabsf(acc[1].x), fabsf(acc[1].y));
         const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(a));

@@ -200,8 +200,8 @@ quantize_groups_kernel(const SrcT* __restrict__ X, int64_t ldx, int64_t rows, in
       const float r = e4m3_reciprocal(s);
 #pragma unroll
       for (int i = 0; i < kPer; ++i) {
-        v[i][0] = e4m3_quotient(v[i][0], make_float2(r, r), make_float2(-s, -s));
-        v[i][1] = e4m3_quotient(v[i][1], make_float2(r, r), make_float2(-s, -s));
+        v[i][0] = e4m3_quotient(make_float2(-v[i][0].x, -v[i][0].y), make_float2(-r, -r), make_float2(s, s));
+        v[i][1] = e4m3_quotient(make_float2(-v[i][1].x, -v[i][1].y), make_float2(-r, -r), make_float2(s, s));
         store(i);
       }
     } else {

@@ -176,8 +176,10 @@ template <int NP> __device__ __forceinline__ void store_vec(__nv_fp8_storage_t* 
 // d r is off by less than 2^-24 of itself, and in units of 2^-27 of m s's binade d is a whole number and s / 2 units in the
 // last place of m a multiple of 2^-20 below 16, so the rounding to m or beside it goes wrong only if d is exactly half a unit,
 // which needs s to be a multiple of 1/8 of its binade, and r above 1 / s: there r is rounded towards zero instead.
-// For s from 2^-100 (below, d could underflow) to the largest float.
-__device__ __forceinline__ bool e4m3_scale_ok(float s) { return s >= 0x1p-100f && s <= 3.402823466e38f; }
+// For s from 2^-100 (below, d could underflow) to 2^126 (above, r is subnormal and short of bits; a largest magnitude over 448 is
+// below 2^120, so what is refused there is infinity).
+// x = -0 gives +0.  Where there may be one, callers pass -x, -r and s: the same numbers, and a zero keeps its sign.
+__device__ __forceinline__ bool e4m3_scale_ok(float s) { return s >= 0x1p-100f && s <= 0x1p126f; }
 __device__ __forceinline__ float e4m3_reciprocal(float s) { return (__float_as_uint(s) & 0xFFFFFu) == 0u ? __frcp_rz(s) : __frcp_rn(s); }
 __device__ __forceinline__ float2 e4m3_quotient(float2 x, float2 r, float2 minus_s) {      // r, -s twice each
   const float2 q = __fmul2_rn(x, r);
@@ -190,7 +192,7 @@ __device__ __forceinline__ void divide_for_e4m3(float2 (&a)[NP], float s) {
   if (e4m3_scale_ok(s)) {
     const float r = e4m3_reciprocal(s);
 #pragma unroll
-    for (int i = 0; i < NP; ++i) a[i] = e4m3_quotient(a[i], make_float2(r, r), make_float2(-s, -s));
+    for (int i = 0; i < NP; ++i) a[i] = e4m3_quotient(make_float2(-a[i].x, -a[i].y), make_float2(-r, -r), make_float2(s, s));
   } else {
 #pragma unroll
     for (int i = 0; i < NP; ++i) { a[i].x = __fdiv_rn(a[i].x, s); a[i].y = __fdiv_rn(a[i].y, s); }

@@ -26,18 +26,11 @@ def _codes(sums, rows, through_bf16):
     return q, s.squeeze(4).squeeze(2)
 
 
-@pytest.mark.parametrize("variant", [False, True])
-@pytest.mark.parametrize("storage,M,K,N", [("bf16", 20, 64, 32), ("bf16", 72, 1088, 1056), ("f32", 516, 576, 160), ("bf16", 8, 11008, 2080)])
-def test_model_schedule_codes(storage, M, K, N, variant):
+def _check(A, B, storage, variant, seen=None):
     lib = gu.fmm()
     o = oracle.sign_variant(S2, [1, -1, 1, 1], [1, 1, -1, 1], [-1, 1, 1, 1]) if variant else S2
     s = lib.scheme_load(o.U, o.V, o.W) if variant else lib.scheme_builtin("strassen444")
-    gen = torch.Generator(device="cuda").manual_seed(M + K + variant)
-    A = torch.randint(-63, 64, (M, K), device="cuda", generator=gen).float()
-    B = torch.randint(-63, 64, (N, K), device="cuda", generator=gen).float()
-    A[: M // 4, : min(K // 4, 128)] *= 2.0 ** -120            # groups whose scales are below the rule's range
-    A[M // 2 :, :: 37] = 0.0
-    B[:, K // 2 :] *= 2.0 ** -9
+    (M, K), N = A.shape, B.shape[0]
     td = torch.bfloat16 if storage == "bf16" else torch.float32
     A, B = A.to(td), B.to(td)
     d = lib.GemmDesc.make(M, K, N, storage, "e4m3", "bf16", weight_layout=True, scale_mode=3, flags=lib.FLAG_PRODUCTS_BF16)
@@ -59,5 +52,30 @@ def test_model_schedule_codes(storage, M, K, N, variant):
         want, scales = _codes(sums.view(49, br, bc), rows, rows == 128)
         got = torch.stack([ws[at + r * stride : at + r * stride + br * bc].view(br, bc) for r in range(49)])
         assert torch.equal(got, want)
+        assert X is A or seen is None or seen(want)
         n = scales.numel()
         assert torch.equal(ws[at_s : at_s + 4 * n].view(torch.float32).view(scales.shape), scales)
+
+
+@pytest.mark.parametrize("variant", [False, True])
+@pytest.mark.parametrize("storage,M,K,N", [("bf16", 20, 64, 32), ("bf16", 72, 1088, 1056), ("f32", 516, 576, 160), ("bf16", 8, 11008, 2080)])
+def test_model_schedule_codes(storage, M, K, N, variant):
+    gen = torch.Generator(device="cuda").manual_seed(M + K + variant)
+    A = torch.randint(-63, 64, (M, K), device="cuda", generator=gen).float()
+    B = torch.randint(-63, 64, (N, K), device="cuda", generator=gen).float()
+    A[: M // 4, : min(K // 4, 128)] *= 2.0 ** -120            # groups whose scales are below the rule's range
+    A[M // 2 :, :: 37] = 0.0
+    B[:, K // 2 :] *= 2.0 ** -9
+    _check(A, B, storage, variant)
+
+
+@pytest.mark.parametrize("variant", [False, True])
+@pytest.mark.parametrize("M,K,N", [(20, 64, 32), (72, 1088, 1056)])
+def test_weights_below_bf16_keep_their_sign(M, K, N, variant):
+    """Block sums of the weight that bf16 rounds to -0 have the code 0x80."""
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    A = torch.randn(M, K, device="cuda", generator=gen)
+    B = torch.randint(-3, 4, (N, K), device="cuda", generator=gen).float() * 2.0 ** -140
+    B.view(4, N // 4, 4, K // 4)[:, :, :, ::3] += 1.0
+    B.view(4, N // 4, 4, K // 4)[:, 0] = -2.0 ** -138
+    _check(A, B, "f32", variant, lambda codes: bool((codes == 0x80).any()))

@@ -39,3 +39,40 @@ def test_codes(storage, M, K, N):
         s = torch.where(amax > 0, amax / torch.full_like(amax, 448), torch.ones_like(amax))
         want = (b / s).to(torch.float8_e4m3fn).view(torch.uint8).view(pad.shape)[:R, :C]
         assert torch.equal(ws[at : at + R * C].view(R, C), want)
+
+
+@pytest.mark.parametrize("mode", [2, 3])
+@pytest.mark.parametrize("storage", ["bf16", "f32"])
+@pytest.mark.parametrize("M,K,N", [(5, 144, 24), (130, 1040, 200)])
+def test_zeros_keep_their_sign(storage, mode, M, K, N):
+    """A negative zero (a masked activation; a weight too small for bf16) has the code 0x80, as the division gives, in scales of
+    the quotient rule's range and below it.  Also with one scale a row (mode 2)."""
+    lib = gu.fmm()
+    td = torch.bfloat16 if storage == "bf16" else torch.float32
+    gen = torch.Generator(device="cuda").manual_seed(K)
+    A, W = torch.randn(M, K, device="cuda", generator=gen), torch.randn(N, K, device="cuda", generator=gen)
+    A *= torch.where(torch.rand(M, K, device="cuda", generator=gen) < 0.3, 0.0, 1.0)      # +0 and -0, by the sign under the mask
+    A[M // 2] *= 2.0 ** -120
+    W[:, ::5] *= 2.0 ** -137
+    W[:, ::7] = -0.0
+    A, W = A.to(td), W.to(td)
+    d = lib.GemmDesc.make(M, K, N, storage, "e4m3", "f32", weight_layout=True, scale_mode=mode)
+    ws = gu.workspace(lib.classical_gemm_workspace(d))
+    lib.classical_gemm(d, A, W, torch.empty(M, N, device="cuda"), ws)
+    lib.device_status(ws)
+    end = ws.numel() - _align(N * K) - _align(M * K)
+    for X, rows, at in ((A, 1, end), (W, 128, end + _align(M * K))):
+        x = X.float()
+        if mode == 3:
+            x = x if rows == 1 else x.bfloat16().float()
+            pad = torch.zeros(-(-x.shape[0] // rows) * rows, -(-K // 128) * 128, device="cuda")
+            pad[: x.shape[0], :K] = x
+            b = pad.view(-1, rows, pad.shape[1] // 128, 128)
+        else:
+            pad = x
+            b = x.view(-1, 1, 1, K)
+        amax = b.abs().amax(dim=(1, 3), keepdim=True)
+        s = torch.where(amax > 0, amax / torch.full_like(amax, 448), torch.ones_like(amax))
+        want = (b / s).to(torch.float8_e4m3fn).view(torch.uint8).view(pad.shape)[: x.shape[0], :K]
+        assert bool((want == 0x80).any())
+        assert torch.equal(ws[at : at + x.numel()].view(x.shape), want)
