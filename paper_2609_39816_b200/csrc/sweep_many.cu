@@ -108,9 +108,13 @@ gauge_tables_kernel(const double* __restrict__ data, const GaugeDims d, CoefTabl
 }
 
 // ------------------------------------------------------------------------------------------
-// Encode.  Block (r, copy, operand): the block sum of product r is formed once where a thread has one vector of it, else twice,
-// for its largest magnitude(s) and to be scaled and rounded; its cells come from L1 / L2 the second time.  The sums and roundings are those of
+// Encode.  Block (r, copy, operand): the block sum of product r is formed twice, once for its largest magnitude(s) and
+// once to be scaled and rounded; its cells come from L1 / L2 the second time.  The sums and roundings are those of
 // encode_kernel (scale modes 0, 1 and 2).
+// What bounds it: a block's chain of dependent loads (list offset, entries, cells), hidden by other blocks alone, eight of them an SM at
+// 32 registers.  Sums kept between the two passes and four cells' loads in flight take 39 and 48 registers and lose those blocks.
+// 512 sign variants, the whole encode, us so / as it is: 128^3 bf16 145 / 104, e4m3 row scales from bf16 187 / 154, from fp32
+// 185 / 189; 256^3 bf16 287 / 251, e4m3 row scales from bf16 490 / 456, from fp32 680 / 620.
 // ------------------------------------------------------------------------------------------
 constexpr int kManyThreads = 256;
 
@@ -142,36 +146,26 @@ encode_many_kernel(const EncodeManyJob ja, const EncodeManyJob jb, const CoefTab
     const SrcT* src = X + (int64_t)p * j.ldx + q * VE;
 #pragma unroll
     for (int i = 0; i < NP; ++i) acc[i] = make_float2(0.0f, 0.0f);
-    for (int e0 = 0; e0 < ne; e0 += 4) {              // four cells' loads in flight
-      uint4 raw[4];
+    for (int e = 0; e < ne; ++e) {
+      uint4 raw = make_uint4(0u, 0u, 0u, 0u);       // a padding entry: zero times zero
+      if (base[e] >= 0) raw = __ldg(reinterpret_cast<const uint4*>(src + base[e]));
+      float2 v[NP];
+      Vec16<SrcT>::unpack(raw, v);
+      const float c = cf[e];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        raw[u] = make_uint4(0u, 0u, 0u, 0u);          // a padding entry: zero times zero
-        if (e0 + u < ne && base[e0 + u] >= 0) raw[u] = __ldg(reinterpret_cast<const uint4*>(src + base[e0 + u]));
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (e0 + u < ne) {
-          float2 v[NP];
-          Vec16<SrcT>::unpack(raw[u], v);
-          const float c = cf[e0 + u];
-#pragma unroll
-          for (int i = 0; i < NP; ++i) acc[i] = __ffma2_rn(make_float2(c, c), v[i], acc[i]);
-        }
+      for (int i = 0; i < NP; ++i) acc[i] = __ffma2_rn(make_float2(c, c), v[i], acc[i]);
     }
   };
-  // a block of at most one vector a thread is summed once, the sums stay in registers between the two loops
-  const bool once = nvec <= kManyThreads;
-  float2 kept[NP];
   float scale = 1.0f, inv = 1.0f;
   bool use_mul = true;
   if (mode != 0) {
     for (int x = threadIdx.x; x < nvec; x += kManyThreads) {
       const int p = x / vpr;
-      sum(p, x - p * vpr, kept);
+      float2 acc[NP];
+      sum(p, x - p * vpr, acc);
       float a = 0.0f;
 #pragma unroll
-      for (int i = 0; i < NP; ++i) a = fmaxf(a, fmaxf(fabsf(kept[i].x), fabsf(kept[i].y)));   // fmaxf drops NaN
+      for (int i = 0; i < NP; ++i) a = fmaxf(a, fmaxf(fabsf(acc[i].x), fabsf(acc[i].y)));   // fmaxf drops NaN
       atomicMax(&row_max[mode == 2 ? p : 0], __float_as_uint(a));
     }
     __syncthreads();
@@ -190,12 +184,7 @@ encode_many_kernel(const EncodeManyJob ja, const EncodeManyJob jb, const CoefTab
   for (int x = threadIdx.x; x < nvec; x += kManyThreads) {
     const int p = x / vpr, q = x - p * vpr;
     float2 acc[NP];
-    if (once && mode != 0) {
-#pragma unroll
-      for (int i = 0; i < NP; ++i) acc[i] = kept[i];
-    } else {
-      sum(p, q, acc);
-    }
+    sum(p, q, acc);
     if (mode == 2) {
       const float amax = __uint_as_float(row_max[p]);
       if constexpr (sizeof(DstT) == 1) divide_for_e4m3<NP>(acc, amax > 0.0f ? __fdiv_rn(amax, 448.0f) : 1.0f);
