@@ -71,8 +71,10 @@ struct PatJob {
 // Passes of an operand; the last three are the model schedule's: A in one (its groups lie within a warp), B in two
 enum PatPass { kNoPass, kPlain, kAmax, kScaled, kGroupOneRow, kGroupAmax, kGroupScaled };
 // blocks per SM that the register allocation aims at: at the sizes above, 3 for the passes that look for maxima (49 of them a
-// thread) take 50 us where 4 take 38; 4 / 5 / 6 for kScaled 66 / 51 / 58
-template <int kPass, PatKind kKind> constexpr int kPatBlocksPerSm = kLevels == 1 ? 8 : kPass == kPlain || ((kPass == kAmax || kPass == kGroupAmax) && kKind == kScheme) ? 4 : 5;
+// thread) take 50 us where 4 take 38; 4 / 5 / 6 for kScaled 66 / 51 / 58.  kPlain lives on loads in flight: 6 (80 registers, no spills), where
+// 4 lets the compiler use 128 and, with coefficients of a dense pattern, spill; a copy of a sweep over general outer gauges, both
+// operands, 4 / 6: 18.5 / 16.9 us at 2048^3 from bf16, 20.9 / 19.1 from fp32, 10.8 / 9.6 at 1024^3.
+template <int kPass, PatKind kKind> constexpr int kPatBlocksPerSm = kLevels == 1 ? 8 : kPass == kPlain ? 6 : (kPass == kAmax || kPass == kGroupAmax) && kKind == kScheme ? 4 : 5;
 
 constexpr int E = 4, NP = 2;          // values of a thread: 16 cells x 4 fp32 registers
 __device__ __forceinline__ float4 load_values(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
