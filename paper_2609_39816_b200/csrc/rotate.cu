@@ -177,7 +177,7 @@ cudaError_t launch_rotate(const void* X, int64_t ldx, int64_t rows, int64_t K, i
 
 // ------------------------------------------------------------------------------------------
 // bf16, h from 32 to 1024: bits 0, 1, 3 and 4 of the column are transformed by mma.sync (m16n8k16 with a matrix of 1 and -1: exact
-// products, fp32 sums of sixteen), the rest by packed additions, none of the seven lower bits by a lane exchange.  (tcgen05 would
+// products, sums of sixteen in the tensor core's fp32), the rest by packed additions, none of the seven lower bits by a lane exchange.  (tcgen05 would
 // take the operand through shared memory and the result through tensor memory, for a contraction of sixteen.)
 // A warp works on 16 x 128 values: 16 rows where h <= 128; beyond, the row index of the fragment also counts the 128-column parts of
 // an h-block, bit 7 in a lane's two rows, bits 8 and 9 in the lane (one exchange of all values each).  A lane loads and stores 16 bytes
@@ -185,10 +185,16 @@ cudaError_t launch_rotate(const void* X, int64_t ldx, int64_t rows, int64_t K, i
 // half w % 2, for the value of bit 2 that w / 2 says; results come out in the same places.  Rows and columns past the end are zeros.
 // The number of warps is a multiple of the parts of a row: a warp stays in its columns, and the signs stay in registers.
 // What bounds it: the memory system.  8192 x 13824, L2 flushed before each, against the other form: h = 32 94 -> 77 us, 64 98 -> 77,
-// 128 90 -> 77 (5.9 TB/s), 256 101 -> 84, 512 115 -> 94; 8192 x 4096, h = 1024 52 -> 38.  The distance from 64-bit results is the
-// rounding to bf16 in either (1.661e-3); outputs that round otherwise than the 64-bit result: 6.0e-7 of them at h = 128 (5.8e-7 before).
+// 128 90 -> 77 (5.9 TB/s).  8192 x 13312, pass after pass: h = 128 83 -> 71, 256 95 -> 77, 512 108 -> 75, 1024 144 -> 75.
+// Registers: three blocks an SM up to h = 256 (at 128 4 bytes spill, at 256 72; two blocks without spills take 78.6 us there, not 77);
+// two beyond, where three spill up to 80 bytes and take 88 and 92 us.
+// Accuracy, measured: how the tensor core rounds inside a sum of sixteen is not documented.  Outputs that do not round as the 64-bit result
+// does, over six h and 4.9e8 outputs of heavy-tailed activations: 1694, the other form 1672 (the counts' own noise is 41); on
+// blocks spread over 2^20 or 2^40, and with two large entries that cancel, together fewer than the other form's, none further off than 1.1 2^-24
+// of its block's norm beside the rounding to bf16.  A block of zeros comes out as +0 whatever their signs.
 // ------------------------------------------------------------------------------------------
 constexpr int kMmaThreads = 128;
+template <int kH> constexpr int kMmaBlocksPerSm = kH > 256 ? 2 : 3;
 
 __device__ __forceinline__ void mma_16(float2 (&d)[2], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
@@ -202,7 +208,7 @@ __device__ __forceinline__ void butterfly(float2& a, float2& b) {
 }
 
 template <int kH>
-__global__ void __launch_bounds__(kMmaThreads, 3)
+__global__ void __launch_bounds__(kMmaThreads, kMmaBlocksPerSm<kH>)
 hadamard_rotate_mma_kernel(const __nv_bfloat16* X, int64_t rows, int64_t K, const signed char* __restrict__ signs, float inv_sqrt_h,
                            __nv_bfloat16* Y, int64_t ldx, int64_t ldy, int col_parts, int64_t row_step, int64_t warps) {
   constexpr int kParts = kH > 128 ? kH / 128 : 1, kRows = 16 / kParts;     // 128-column parts of an h-block, rows of a warp's unit
@@ -327,7 +333,7 @@ cudaError_t launch_rotate_mma(const void* X, int64_t ldx, int64_t rows, int64_t 
   if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
   if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return cudaErrorInvalidDevice;
   const int64_t col_parts = (K + kWidth - 1) / kWidth, groups = (rows + kRows - 1) / kRows;
-  const int64_t cap = std::max<int64_t>(1, (int64_t)sms * 3 * (kMmaThreads / 32) / col_parts), at_once = std::min(cap, groups), warps = at_once * col_parts;
+  const int64_t cap = std::max<int64_t>(1, (int64_t)sms * kMmaBlocksPerSm<kH> * (kMmaThreads / 32) / col_parts), at_once = std::min(cap, groups), warps = at_once * col_parts;
   hadamard_rotate_mma_kernel<kH><<<(unsigned)((warps + kMmaThreads / 32 - 1) / (kMmaThreads / 32)), kMmaThreads, 0, st>>>(
       (const __nv_bfloat16*)X, rows, K, signs, (float)(1.0 / std::sqrt((double)kH)), (__nv_bfloat16*)Y, ldx, ldy, (int)col_parts, at_once * kRows, warps);
   ++fmm_launch_counter();
