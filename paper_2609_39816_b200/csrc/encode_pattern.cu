@@ -74,7 +74,11 @@ enum PatPass { kNoPass, kPlain, kAmax, kScaled, kGroupOneRow, kGroupAmax, kGroup
 // thread) take 50 us where 4 take 38; 4 / 5 / 6 for kScaled 66 / 51 / 58.  kPlain lives on loads in flight: 6 (80 registers, no spills), where
 // 4 lets the compiler use 128 and, with coefficients of a dense pattern, spill; a copy of a sweep over general outer gauges, both
 // operands, 4 / 6: 18.5 / 16.9 us at 2048^3 from bf16, 20.9 / 19.1 from fp32, 10.8 / 9.6 at 1024^3.
-template <int kPass, PatKind kKind> constexpr int kPatBlocksPerSm = kLevels == 1 ? 8 : kPass == kPlain ? 6 : (kPass == kAmax || kPass == kGroupAmax) && kKind == kScheme ? 4 : 5;
+// The model schedule's codes of the built-in scheme keep more than the others: 5 spill 80 bytes from bf16 and take 229 us where 4 take 232
+// (the call at 2048 x 11008 x 4096); from fp32 5 spill 224 and take 255 where 4 take 250.
+template <int kPass, PatKind kKind, typename SrcT>
+constexpr int kPatBlocksPerSm = kLevels == 1 ? 8 : kPass == kPlain ? 6 : (kPass == kAmax || kPass == kGroupAmax) && kKind == kScheme ? 4
+                              : kPass == kGroupScaled && kKind == kScheme && sizeof(SrcT) == 4 ? 4 : 5;
 
 constexpr int E = 4, NP = 2;          // values of a thread: 16 cells x 4 fp32 registers
 __device__ __forceinline__ float4 load_values(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
@@ -383,7 +387,7 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
 
 // blocks [0, ja.blocks) make pass kPassA over A, the rest kPassB over B (kNoPass: B alone)
 template <typename SrcT, typename DstT, PatKind kKind, int kPassA, int kPassB>
-__global__ void __launch_bounds__(kPatThreads, (kPatBlocksPerSm<kPassB, kKind>))
+__global__ void __launch_bounds__(kPatThreads, (kPatBlocksPerSm<kPassB, kKind, SrcT>))
 encode_pattern_kernel(const __grid_constant__ PatJob ja, const __grid_constant__ PatJob jb, const __grid_constant__ PatCoefs coefs, int* status) {
   grid_launch_dependents();   // the next kernel may set up while this grid drains; it waits before reading
   grid_dependency_wait();     // the operands (and maxima) may come from the kernel before
