@@ -54,3 +54,28 @@ def test_model_schedule(M, K, N):
     a, b = _codes(A, 1), _codes(W, 128)
     bound = (K + 3 * (-(-K // 128))) * 2.0 ** -24 * (a.abs() @ b.abs().T) + 1e-30
     assert bool(((C.double() - a @ b.T).abs() <= bound).all())
+
+
+def _several_rounds_of_pairs(rows_a, rows_b, batches):
+    """The library's choice (pairs where 1.5 rounds of 256 x 256 tiles over the pairs are fewer than the rounds of 128 x 128 tiles over
+    the SMs), for shapes that give a pair more than one tile."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    tiles = {t: -(-rows_a // t) * -(-rows_b // t) * batches for t in (128, 256)}
+    rounds = -(-tiles[256] // (sms // 2))
+    return rounds > 1 and 1.5 * rounds < -(-tiles[128] // sms)
+
+
+@pytest.mark.parametrize("K", [272, 8320])
+def test_model_schedule_several_tiles_a_pair(K):
+    """Barrier phases over tiles; the next tile's scales beside this one's, and (65 groups) scales read where they lie."""
+    assert _several_rounds_of_pairs(3000, 2600, 1)
+    test_model_schedule(3000, K, 2600)
+
+
+@pytest.mark.parametrize("scheme,bound,M,K,N", [("strassen444", 31, 2000, 512, 4064), ("strassen444", 31, 2000, 7424, 4064),
+                                                ("strassen222", 63, 3016, 256, 3008), ("", 31, 3000, 8448, 2600)])
+def test_int8_several_tiles_a_pair(scheme, bound, M, K, N):
+    """Certified: tiles of several blocks of C one after the other, every other round backwards; signs beyond the first tile."""
+    g = {"strassen444": 4, "strassen222": 2, "": 1}[scheme]
+    assert _several_rounds_of_pairs(M // g, N // g, g * g)
+    test_int8(scheme, bound, M, K, N)

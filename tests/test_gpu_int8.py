@@ -293,7 +293,7 @@ def test_fine_group_control_on_the_device():
 def test_certified_at_the_edges_of_its_tiles_and_rings(M, K, N):
     """The certified realisation against the classical kernel, both bit-exact by the specification: blocks one row past a
     tile of 128 and 8 columns past two of them, 57 and 58 groups (column scales staged for 56), one group, and <1,1,1;2>
-    with weights of 3 and -2 (repeated MMAs into both accumulators, four steps of K per product)."""
+    with weights of 3 and -2 (repeated MMAs, the minus by operand tiles with turned signs, four steps of K per product)."""
     lib = fmm()
     At, A, Bt, B = _inputs(71, M, K, N)
     one = oracle.Scheme(np.ones((2, 1, 1)), np.ones((2, 1, 1)), np.array([3.0, -2.0]).reshape(2, 1, 1))

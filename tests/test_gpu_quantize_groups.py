@@ -76,3 +76,34 @@ def test_zeros_keep_their_sign(storage, mode, M, K, N):
         want = (b / s).to(torch.float8_e4m3fn).view(torch.uint8).view(pad.shape)[: x.shape[0], :K]
         assert bool((want == 0x80).any())
         assert torch.equal(ws[at : at + x.numel()].view(x.shape), want)
+
+
+@pytest.mark.parametrize("storage", ["bf16", "f32"])
+def test_nan_and_infinity_stay_in_their_group(storage):
+    """NaN is not part of a group's maximum and has a NaN code; infinity makes the scale infinite, so that finite values become zeros of
+    their sign and itself NaN.  Every other group is as it would be without them."""
+    lib = gu.fmm()
+    M, K, N = 70, 272, 136
+    td = torch.bfloat16 if storage == "bf16" else torch.float32
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    A, W = torch.randn(M, K, device="cuda", generator=gen), torch.randn(N, K, device="cuda", generator=gen)
+    for X in (A, W):
+        X[1, 5], X[69, 130], X[60, 271] = float("nan"), float("inf"), float("-inf")
+    A, W = A.to(td), W.to(td)
+    d = lib.GemmDesc.make(M, K, N, storage, "e4m3", "f32", weight_layout=True, scale_mode=3)
+    ws = gu.workspace(lib.classical_gemm_workspace(d))
+    lib.classical_gemm(d, A, W, torch.empty(M, N, device="cuda"), ws)
+    lib.device_status(ws)
+    end = ws.numel() - _align(N * K) - _align(M * K)
+    for X, rows, at in ((A, 1, end), (W, 128, end + _align(M * K))):
+        x = X.float() if rows == 1 else X.bfloat16().float()
+        pad = torch.zeros(-(-x.shape[0] // rows) * rows, 384, device="cuda")
+        pad[: x.shape[0], :K] = x
+        b = pad.view(-1, rows, 3, 128)
+        amax = b.abs().nan_to_num(0.0, float("inf")).amax(dim=(1, 3), keepdim=True)
+        s = torch.where(amax > 0, amax / torch.full_like(amax, 448), torch.ones_like(amax))
+        want = (b / s).to(torch.float8_e4m3fn).view(torch.uint8).view(pad.shape)[: x.shape[0], :K]
+        got = ws[at : at + x.numel()].view(x.shape)
+        nan = want & 0x7F == 0x7F
+        assert bool(nan.any()) and torch.equal(got & 0x7F == 0x7F, nan)
+        assert torch.equal(got[~nan], want[~nan])
