@@ -1237,7 +1237,7 @@ __device__ __forceinline__ void tc_mma_i8(uint32_t d_tmem, uint64_t a_desc, uint
 template <bool kPair> constexpr uint32_t kInt8Desc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(GroupShape<kPair>::BN >> 3) << 17) |
                                                      ((uint32_t)(GroupShape<kPair>::kRows >> 4) << 24);
 
-// The rescale role of the int8 kernels (warps 2..17): waits for a group's accumulator, converts it, applies the two scales
+// The rescale role of the int8 kernels (the sixteen warps from kFirstRescale on): waits for a group's accumulator, converts it, applies the two scales
 // and adds to the tile's fp32 sums, which a thread holds for one row and PN columns.
 // Its arithmetic is three rounded operations per element and group, in the order of the specification, and sets the pace of
 // the classical kernel.  The multiplications run as packed pairs.  A packed multiply followed by a packed add (__fmul2_rn,
@@ -1246,7 +1246,7 @@ template <bool kPair> constexpr uint32_t kInt8Desc = (2u << 4) | (1u << 7) | (1u
 // floats by a conversion: adding them to the bits of 1.5 * 2^23 and subtracting that took an instruction and a half.
 // Classical, 2048 x 4096 x 11008: 266 us with scalar additions and the bit trick, 253 with the packed additions, 196 with
 // the conversion too, 192 with the staged scales in a loop of their own (128 x 128 tiles), 167 as pairs, 155 with the registers
-// that keep a pair's 64 sums a thread out of local memory.  What bounds it now: issue slots (60 %, 268 instructions per 64 columns
+// that keep a pair's 64 sums a thread out of local memory.  What bounds it now: issue slots (67 %, 273 instructions per 64 columns
 // and group) and the latency of TMEM and scale loads behind four warps a scheduler.
 struct RescaleCtx {
   uint32_t tfull0, tempty0;     // accumulator barriers of the buffers (consecutive)
@@ -1266,7 +1266,7 @@ struct RescaleCtx {
 struct RescaleTile { int row0, rows, col0, cols; bool any; };   // this CTA's first row and the first column of the tile in C, its
                                                                 // extents; any: an MMA wrote the accumulators
 
-// kMove: the number of warps before the rescale warps; tile_at(k, &tile): the CTA's k-th tile, false after its last
+// kMove: a whole warpgroup stands before the rescale warps (kFirstRescale); tile_at(k, &tile): the CTA's k-th tile, false after its last
 template <bool kPair, int kMaxGroupsStaged, bool kMove, typename TileAt>
 __device__ __forceinline__ void int8_rescale_role(const RescaleCtx& c, const int warp, const int lane, const TileAt tile_at) {
   using S = GroupShape<kPair>;
@@ -1442,7 +1442,7 @@ int8_group_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __g
 // read where they lie, two groups ahead of their use and in a loop of their own (classical_gemm, 2048 x 11008 x 4096, 86 groups,
 // 128 x 128 tiles: 373 us fetched where they are used, 367 ahead of it beside the staged form in one loop, 343 so).
 // Pairs: 49 products of 512 x 2752 x 1024 119 -> 97 us (tensor pipe 44 % busy).  Registers moved to the rescale warps, as the int8
-// kernels do, make it slower (the call 191 -> 200 us): nothing that the loop touches is in local memory here.
+// kernels do, make it slower (the call 191 -> 200 us): 28 bytes spill here, touched by 0.4 % of the instructions.
 struct Fp8Layout : Int8Layout {
   static constexpr int kMaxGroups = 64;                                  // staged up to this many groups
   static constexpr int kScaleLd = BM + 1;                                // [group][row], padded against bank conflicts
@@ -1766,7 +1766,10 @@ fmm_status launch_block_products(const BlockProductArgs& a, cudaStream_t st) {
   // large problems: CTA pairs on 256 x 256 tiles (less L2 traffic per flop)
   if (a.rows_a > 128 && a.rows_b > 128 && !a.selftest_no_producer)
     return fp8 ? launch_pair<true>(a, st) : launch_pair<false>(a, st);
-  // small blocks, more products than SMs: several to a tile (8,400 products of 32 x 32 x 32, e4m3: 48 -> 20 us)
+  // small blocks, more products than SMs: several to a tile (8,400 products of 32 x 32 x 32, e4m3: 48 -> 20 us, bf16 40 -> 18; 64 x 64 x 64,
+  // bf16, 2,900: 22 -> 18).  From few products on it is no slower, one tile each / several: 196, 392 and 588 products in bf16 of 32 x 32 x 32
+  // 8.4 / 8.5, 8.9 / 8.5, 10.6 / 8.5, of 64 x 64 x 64 10.6 / 8.5, 10.6 / 10.6, 10.9 / 10.5, of 32 x 256 x 32 10.5 / 8.4, 12.7 / 8.9, 12.6 / 10.6,
+  // of 16 x 512 x 16 12.6 / 10.5, 14.7 / 10.6, 16.7 / 10.6.
   const int64_t side = std::max(a.rows_a, a.rows_b);
   if (side <= 64 && a.groups <= 1 && a.batches > sm_count() && !a.selftest_no_producer) {
     if (side <= 32) return fp8 ? launch_t<128, true, 4>(a, st) : launch_t<128, false, 4>(a, st);
