@@ -49,8 +49,9 @@ decode_pattern_kernel(const ProdT* __restrict__ prod, int64_t rstride, const __g
   __shared__ float w[P::value.off[kProducts]];
   __shared__ double red[8];
   const int tid = threadIdx.x;
-  // Not in a sweep: the next copy's blocks would hold registers and wait, while the encode and the products beside this grid want
-  // them (64 general outer gauges at 2048^3, bf16: 3.53 ms; with it 3.66, in some processes 4.0 to 4.2)
+  // Not in a sweep: the next kernel is the one block that adds the partial sums; started early it sits on an SM through the whole
+  // pass, where the products of the next copy, one block an SM, want in (64 general outer gauges at 2048^3, bf16: 3.53 ms; with it
+  // 3.66, in some processes 4.0 to 4.2; the cause as read, the times measured)
   if constexpr (!kErr) grid_launch_dependents();
   grid_dependency_wait();     // the products (and scales) come from the previous kernel of the stream
   for_each(std::make_integer_sequence<int, kProducts>{}, [&](auto rc) {

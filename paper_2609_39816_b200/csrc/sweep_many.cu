@@ -109,17 +109,19 @@ gauge_tables_kernel(const double* __restrict__ data, const GaugeDims d, CoefTabl
 
 // ------------------------------------------------------------------------------------------
 // Encode.  Block (r, copy, operand): the block sum of product r is formed twice, once for its largest magnitude(s) and
-// once to be scaled and rounded; its cells come from L1 / L2 the second time.  The sums and roundings are those of
-// encode_kernel (scale modes 0, 1 and 2).
+// once to be scaled and rounded; its cells come from L1 / L2 the second time.  A scaled block of at most one vector a thread is summed
+// once (kOnce).  The sums and roundings are those of encode_kernel (scale modes 0, 1 and 2).
 // What bounds it: a block's chain of dependent loads (list offset, entries, cells), hidden by other blocks alone, eight of them an SM at
-// 32 registers.  Sums kept between the two passes and four cells' loads in flight take 39 and 48 registers and lose those blocks.
-// 512 sign variants, the whole encode, us so / as it is: 128^3 bf16 145 / 104, e4m3 row scales from bf16 187 / 154, from fp32
-// 185 / 189; 256^3 bf16 287 / 251, e4m3 row scales from bf16 490 / 456, from fp32 680 / 620.
+// 32 registers, which either form keeps.  512 sign variants, e4m3, the whole encode, us with blocks summed twice / as it is: 128^3 row
+// scales from fp32 189 / 164, from bf16 154 / 150; one scale from bf16 167 / 160.  One kernel for both, with four cells' loads in
+// flight, took 39 and 48 registers and lost those blocks: 128^3 bf16 104 -> 144, 256^3 row scales from fp32 610 -> 670.
 // ------------------------------------------------------------------------------------------
 constexpr int kManyThreads = 256;
 
-template <typename SrcT, typename DstT>
-__global__ void __launch_bounds__(kManyThreads)
+// kOnce: a scaled block of at most one vector a thread; its sums stay in registers between the two steps.  (A bound of 8 blocks an SM
+// makes the other form 15 % slower, though it has them without.)
+template <typename SrcT, typename DstT, bool kOnce>
+__global__ void __launch_bounds__(kManyThreads, kOnce ? 8 : 0)
 encode_many_kernel(const EncodeManyJob ja, const EncodeManyJob jb, const CoefTable* __restrict__ tabs, int mode) {
   grid_launch_dependents();
   constexpr int VE = Vec16<SrcT>::kElems, NP = VE / 2;
@@ -158,6 +160,7 @@ encode_many_kernel(const EncodeManyJob ja, const EncodeManyJob jb, const CoefTab
   };
   float scale = 1.0f, inv = 1.0f;
   bool use_mul = true;
+  float2 kept[kOnce ? NP : 1];
   if (mode != 0) {
     for (int x = threadIdx.x; x < nvec; x += kManyThreads) {
       const int p = x / vpr;
@@ -167,6 +170,11 @@ encode_many_kernel(const EncodeManyJob ja, const EncodeManyJob jb, const CoefTab
 #pragma unroll
       for (int i = 0; i < NP; ++i) a = fmaxf(a, fmaxf(fabsf(acc[i].x), fabsf(acc[i].y)));   // fmaxf drops NaN
       atomicMax(&row_max[mode == 2 ? p : 0], __float_as_uint(a));
+      if constexpr (kOnce) {
+#pragma unroll
+        for (int i = 0; i < NP; ++i) kept[i] = acc[i];
+        break;
+      }
     }
     __syncthreads();
     if (mode == 1) {
@@ -184,7 +192,12 @@ encode_many_kernel(const EncodeManyJob ja, const EncodeManyJob jb, const CoefTab
   for (int x = threadIdx.x; x < nvec; x += kManyThreads) {
     const int p = x / vpr, q = x - p * vpr;
     float2 acc[NP];
-    sum(p, q, acc);
+    if constexpr (kOnce) {
+#pragma unroll
+      for (int i = 0; i < NP; ++i) acc[i] = kept[i];
+    } else {
+      sum(p, q, acc);
+    }
     if (mode == 2) {
       const float amax = __uint_as_float(row_max[p]);
       if constexpr (sizeof(DstT) == 1) divide_for_e4m3<NP>(acc, amax > 0.0f ? __fdiv_rn(amax, 448.0f) : 1.0f);
@@ -196,6 +209,7 @@ encode_many_kernel(const EncodeManyJob ja, const EncodeManyJob jb, const CoefTab
       }
     }
     store_vec<NP>(out + (int64_t)p * j.bc + q * VE, acc, false);
+    if (kOnce) break;
   }
 }
 
@@ -217,7 +231,15 @@ decode_many_kernel(const ProdT* __restrict__ prod, const CoefTable* __restrict__
 template <typename SrcT, typename DstT>
 void launch_encode_many_t(const EncodeManyJob& a, const EncodeManyJob& b, const CoefTable* tabs, int R, int copies, int mode,
                           cudaStream_t st) {
-  encode_many_kernel<SrcT, DstT><<<dim3(R, copies, 2), kManyThreads, 0, st>>>(a, b, tabs, mode);
+  const dim3 grid(R, copies, 2);
+  if constexpr (sizeof(DstT) == 1) {
+    constexpr int VE = Vec16<SrcT>::kElems;
+    if (mode != 0 && std::max(a.br * (a.bc / VE), b.br * (b.bc / VE)) <= kManyThreads) {
+      encode_many_kernel<SrcT, DstT, true><<<grid, kManyThreads, 0, st>>>(a, b, tabs, mode);
+      return;
+    }
+  }
+  encode_many_kernel<SrcT, DstT, false><<<grid, kManyThreads, 0, st>>>(a, b, tabs, mode);
 }
 
 template <typename OutT, typename ProdT>
