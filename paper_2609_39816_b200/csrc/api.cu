@@ -581,6 +581,36 @@ bool sweep_many_ok(const fmm_scheme* s, const fmm_gemm_desc* d, int G) {
   return work <= (batches == 1 ? 8192 : std::max<int64_t>(32768, 8192 * batches)) && work <= 32768 * (int64_t)many_layout(s, d, G).copies;
 }
 
+// Sweeps on small blocks that one kernel takes from the operands to the errors, given diagonal gauges.  Its blocks' partial sums
+// use the place of the decode's.  Whole calls, this kernel against the passes of sweep_many.cu, us: 512 copies at 64^3 279 / 410, 128^3 290 /
+// 539, 256^3 778 / 1254; 64 at 256^3 242 / 329, 512 x 64 x 512 317 / 462; one copy at 128^3 164 / 170.  Not where a tile is mostly
+// padding of one side (100 copies at 16 x 256 x 512 415 / 395), nor for a few copies of long rows, which it walks with one block of
+// threads a tile (2 at 256^3 190 / 176).
+bool sweep_variants_ok(const fmm_scheme* s, const fmm_gemm_desc* d, int G) {
+  const int64_t bm = d->M / s->m, bn = d->N / s->n, bk = d->K / s->k;
+  const int64_t tiles = sweep_variants_tiles(bm, bn);
+  if ((tiles > 1 && bm * bn < tiles * 256) || (bk > 32 && G < 8)) return false;
+  return s->R == 49 && d->product == FMM_E4M3 && d->scale_mode == 2 && !(d->flags & FMM_FLAG_PRODUCTS_BF16) &&
+         sweep_variants_sizes(bm, bn, bk) && tiles <= many_layout(s, d, G).blocks &&
+         sweep_variants_scheme(*fmm_packed_table(*s, 0), *fmm_packed_table(*s, 1), *fmm_packed_table(*s, 2));
+}
+
+// If all G matrices are diagonal and their entries far from fp32's limits: the diagonals and, half a stride behind them, the inverses'
+// (what fmm_gauge_pack finds).
+bool pack_diagonals(int G, int n, const double* X, double* out, size_t stride) {
+  for (int g = 0; g < G; ++g, X += n * n, out += stride) {
+    bool ok = true;
+    for (int i = 0; i < n; ++i)
+      for (int j = 0; j < n; ++j) {
+        const double x = X[i * n + j];
+        ok = ok && (i == j ? std::fabs(x) >= 0x1p-20 && std::fabs(x) <= 0x1p20 : x == 0.0);
+      }
+    if (!ok) return false;
+    for (int i = 0; i < n; ++i) { out[i] = X[i * n + i]; out[stride / 2 + i] = 1.0 / out[i]; }
+  }
+  return true;
+}
+
 struct SweepLayout {
   GemmLayout g; ClassicalLayout c;
   size_t gemm, gemm2, classical, cstar, cstar32, ccl, tables, sums, fpart, many, total;   // two GEMM workspaces: gauges are pipelined
@@ -858,16 +888,25 @@ fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P
   const bool many = sweep_many_ok(base, d, G);     // on the caller's stream alone: the same kernels and sums with and without `serial`
   // every gauge matrix is checked before the first launch: a singular one returns with nothing enqueued
   const size_t per_gauge = 2 * (size_t)(gm * gm + gk * gk + gn * gn);
+  const fmm_scheme* in = level == 1 ? base->inner.get() : nullptr;
+  const GaugeDims gd{gm, gk, gn, grid->R, in ? in->m : 1, in ? in->k : 1, in ? in->n : 1, in ? in->R : 1};
   std::vector<double> packed;           // small blocks: coefficients and gauges for the device (launch_gauge_tables)
+  bool variants = false;                // all gauges diagonal, and one kernel for the rest (launch_sweep_variants)
   if (many) {
-    const fmm_scheme* inner = level == 1 ? base->inner.get() : nullptr;
     const double one = 1.0;
     for (const auto* v : {&grid->U, &grid->V, &grid->W}) packed.insert(packed.end(), v->begin(), v->end());
-    if (inner) for (const auto* v : {&inner->U, &inner->V, &inner->W}) packed.insert(packed.end(), v->begin(), v->end());
+    if (in) for (const auto* v : {&in->U, &in->V, &in->W}) packed.insert(packed.end(), v->begin(), v->end());
     else packed.insert(packed.end(), 3, one);
-    const size_t head = packed.size();
-    packed.resize(head + G * per_gauge);
-    for (int g = 0; g < G; ++g)
+    const size_t head = packed.size(), diagonals = 2 * (size_t)(gm + gk + gn);
+    if (sweep_variants_ok(base, d, G)) {
+      packed.resize(head + G * diagonals + kVariantIndexBytes / 8);
+      double* x = packed.data() + head;
+      variants = pack_diagonals(G, gm, P, x, diagonals) && pack_diagonals(G, gk, Q, x + gm, diagonals) &&
+                 pack_diagonals(G, gn, S, x + gm + gk, diagonals);
+      if (variants) sweep_variants_index(gd, reinterpret_cast<unsigned short*>(x + G * diagonals));
+    }
+    if (!variants) packed.resize(head + G * per_gauge);
+    for (int g = 0; !variants && g < G; ++g)
       if (!fmm_gauge_pack(gm, gk, gn, P + (size_t)g * gm * gm, Q + (size_t)g * gk * gk, S + (size_t)g * gn * gn,
                           packed.data() + head + g * per_gauge))
         return FMM_ERR_SINGULAR;
@@ -934,13 +973,18 @@ fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P
   FMM_CUDA(launch_cstar_prepare(cstar, d->M * d->N, cstar32, part, &np, st));
   FMM_CUDA(launch_sum_partials(part, np, sums + 0, st));
 
-  // 3. classical product at the same dtypes and its error
-  fmm_gemm_desc dcl = *d;
-  dcl.ldc = d->N;
-  void* ccl = at<char>(ws, L.ccl);
-  FMM_TRY(run_classical(&dcl, L.c, dA, dB, ccl, cws, st));
-  FMM_CUDA(launch_frob_err(d->output, ccl, d->N, cstar, d->M, d->N, part, nullptr, &np, st));
-  FMM_CUDA(launch_sum_partials(part, np, sums + 1, st));
+  // 3. classical product at the same dtypes and its error.  One launch that fills the GPU (variants) goes first: the host enqueues
+  // the classical product's eight while it runs.
+  auto classical = [&]() -> fmm_status {
+    fmm_gemm_desc dcl = *d;
+    dcl.ldc = d->N;
+    void* ccl = at<char>(ws, L.ccl);
+    FMM_TRY(run_classical(&dcl, L.c, dA, dB, ccl, cws, st));
+    FMM_CUDA(launch_frob_err(d->output, ccl, d->N, cstar, d->M, d->N, part, nullptr, &np, st));
+    FMM_CUDA(launch_sum_partials(part, np, sums + 1, st));
+    return FMM_OK;
+  };
+  if (!variants) FMM_TRY(classical());
 
   // 4. the sweep: per gauge encode A, encode B, R products, decode + error reduction.
   // The three stages stress different parts of the machine (memory system, tensor cores + L2, memory system),
@@ -960,41 +1004,53 @@ fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P
     char* mws = ws + L.many;
     const int R = base->R, mode = d->scale_mode;
     const int64_t bm = d->M / base->m, bn = d->N / base->n, bk = d->K / base->k;
-    const fmm_scheme* inner = level == 1 ? base->inner.get() : nullptr;
-    const GaugeDims gd{gm, gk, gn, grid->R, inner ? inner->m : 1, inner ? inner->k : 1, inner ? inner->n : 1, inner ? inner->R : 1};
     {
       ProfScope ps(5, st);
       FMM_CUDA(cudaMemcpyAsync(mws + Lm.data, packed.data(), packed.size() * 8, cudaMemcpyHostToDevice, st));
-      FMM_CUDA(launch_gauge_tables(at<double>(mws, Lm.data), gd, G, d_tabs, st));
+      if (!variants) FMM_CUDA(launch_gauge_tables(at<double>(mws, Lm.data), gd, G, d_tabs, st));
     }
-    const EncodeManyJob ja{dA, d->lda, base->k, (int)bm, (int)bk, at<char>(mws, Lm.hat_a), L.g.sAhat, at<float>(mws, Lm.scale_a)};
-    const EncodeManyJob jb{bk_ptr, bk_ld, base->k, (int)bn, (int)bk, at<char>(mws, Lm.hat_b), L.g.sBhat, at<float>(mws, Lm.scale_b)};
-    const bool prod_bf16 = (d->flags & FMM_FLAG_PRODUCTS_BF16) != 0;
-    for (int g = 0; g < G; g += Lm.copies) {
-      const int copies = std::min(Lm.copies, G - g);
-      {
-        ProfScope ps(0, st);
-        FMM_CUDA(launch_encode_many(d->storage, d->product, ja, jb, d_tabs + 3 * g, R, copies, mode, st));
-      }
-      BlockProductArgs p{};
-      p.product = d->product;
-      p.A = ja.out; p.lda = bk; p.a_batch = L.g.sAhat;
-      p.B = jb.out; p.ldb = bk; p.b_batch = L.g.sBhat;
-      p.rows_a = bm; p.rows_b = bn; p.kdim = bk; p.batches = copies * R;
-      p.out = at<char>(mws, Lm.prod); p.ldo = bn; p.o_batch = L.g.sProd;
-      p.out_mode = prod_bf16 ? 1 : 0; p.output = prod_bf16 ? FMM_BF16 : FMM_F32;
-      if (mode == 2) { p.row_scale = ja.scale; p.rs_batch = bm; p.col_scale = jb.scale; p.cs_batch = bn; }
-      p.status = at<DeviceStatus>(gws, L.g.status);
+    if (variants) {
+      const int gauge_len = 2 * (gm + gk + gn);
+      const size_t at_index = packed.size() - kVariantIndexBytes / 8, coef_len = at_index - (size_t)G * gauge_len;
+      const double* data = at<double>(mws, Lm.data);
+      const SweepVariantArgs v{d->storage, d->output, dA, d->lda, bk_ptr, bk_ld, bm, bn, bk, G, data, (int)coef_len, gauge_len,
+                               data + at_index, cstar32, at<double>(mws, Lm.part)};
       {
         ProfScope ps(2, st);
-        FMM_TRY(launch_block_products(p, st));
+        FMM_CUDA(launch_sweep_variants(v, st));
       }
-      ProfScope ps(3, st);
-      FMM_CUDA(launch_decode_many(d->output, p.out, prod_bf16 ? FMM_BF16 : FMM_F32, L.g.sProd, d_tabs + 3 * g, R, copies,
-                                  mode == 1 ? ja.scale : nullptr, mode == 1 ? jb.scale : nullptr, base->m, base->n, bm, bn,
-                                  cstar32, at<double>(mws, Lm.part) + (size_t)g * Lm.blocks, Lm.blocks, Lm.tpb, st));
+      FMM_CUDA(launch_sum_partials(v.partials, sweep_variants_tiles(bm, bn), sums + 8, st, G));
+      FMM_TRY(classical());
+    } else {
+      const EncodeManyJob ja{dA, d->lda, base->k, (int)bm, (int)bk, at<char>(mws, Lm.hat_a), L.g.sAhat, at<float>(mws, Lm.scale_a)};
+      const EncodeManyJob jb{bk_ptr, bk_ld, base->k, (int)bn, (int)bk, at<char>(mws, Lm.hat_b), L.g.sBhat, at<float>(mws, Lm.scale_b)};
+      const bool prod_bf16 = (d->flags & FMM_FLAG_PRODUCTS_BF16) != 0;
+      for (int g = 0; g < G; g += Lm.copies) {
+        const int copies = std::min(Lm.copies, G - g);
+        {
+          ProfScope ps(0, st);
+          FMM_CUDA(launch_encode_many(d->storage, d->product, ja, jb, d_tabs + 3 * g, R, copies, mode, st));
+        }
+        BlockProductArgs p{};
+        p.product = d->product;
+        p.A = ja.out; p.lda = bk; p.a_batch = L.g.sAhat;
+        p.B = jb.out; p.ldb = bk; p.b_batch = L.g.sBhat;
+        p.rows_a = bm; p.rows_b = bn; p.kdim = bk; p.batches = copies * R;
+        p.out = at<char>(mws, Lm.prod); p.ldo = bn; p.o_batch = L.g.sProd;
+        p.out_mode = prod_bf16 ? 1 : 0; p.output = prod_bf16 ? FMM_BF16 : FMM_F32;
+        if (mode == 2) { p.row_scale = ja.scale; p.rs_batch = bm; p.col_scale = jb.scale; p.cs_batch = bn; }
+        p.status = at<DeviceStatus>(gws, L.g.status);
+        {
+          ProfScope ps(2, st);
+          FMM_TRY(launch_block_products(p, st));
+        }
+        ProfScope ps(3, st);
+        FMM_CUDA(launch_decode_many(d->output, p.out, prod_bf16 ? FMM_BF16 : FMM_F32, L.g.sProd, d_tabs + 3 * g, R, copies,
+                                    mode == 1 ? ja.scale : nullptr, mode == 1 ? jb.scale : nullptr, base->m, base->n, bm, bn,
+                                    cstar32, at<double>(mws, Lm.part) + (size_t)g * Lm.blocks, Lm.blocks, Lm.tpb, st));
+      }
+      FMM_CUDA(launch_sum_partials(at<double>(mws, Lm.part), Lm.blocks, sums + 8, st, G));
     }
-    FMM_CUDA(launch_sum_partials(at<double>(mws, Lm.part), Lm.blocks, sums + 8, st, G));
     next_gauge = G;
   }
   // Fused pipeline (unless FMM_FLAG_SWEEP_UNFUSED; bf16 storage and products, no scales, batches of four or eight one-level

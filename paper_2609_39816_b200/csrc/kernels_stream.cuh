@@ -171,6 +171,24 @@ cudaError_t launch_decode_many(int output, const void* prod, int prod_dtype, int
                                int copies, const float* sA, const float* sB, int m, int n, int64_t bm, int64_t bn,
                                const float* cstar32, double* partials, int blocks, int tiles_per_block, cudaStream_t st);
 
+// Sweeps over diagonal gauges of two-level Strassen on small blocks, e4m3 with scale mode 2 (sweep_variants.cu): error partials
+// [copy][sweep_variants_tiles].  A, B (K-major) as stored; data (DEVICE): coefficients as for launch_gauge_tables, then per copy
+// the diagonals of P, Q, S, P^-1, Q^-1, S^-1.
+struct SweepVariantArgs {
+  int storage, output;
+  const void* A; int64_t lda; const void* B; int64_t ldb;
+  int64_t bm, bn, bk; int copies;
+  const double* data; int coef_len, gauge_len;       // numbers of the coefficients, and of a copy's diagonals
+  const void* index;                                 // (DEVICE) sweep_variants_index
+  const float* cstar32; double* partials;
+};
+constexpr int kVariantIndexBytes = 784 * 8;
+void sweep_variants_index(const GaugeDims& d, unsigned short* out);
+int sweep_variants_tiles(int64_t bm, int64_t bn);
+bool sweep_variants_scheme(const CoefTable& a, const CoefTable& b, const CoefTable& w);    // are the (host) tables of the pattern?
+bool sweep_variants_sizes(int64_t bm, int64_t bn, int64_t bk);
+cudaError_t launch_sweep_variants(const SweepVariantArgs& a, cudaStream_t st);
+
 // out[0] = sum of partials[0..n) in a fixed order (single block).
 // out[b] = sum of partials[b*n .. b*n+n), b < count
 cudaError_t launch_sum_partials(const double* partials, int n, double* out, cudaStream_t st, int count = 1);
