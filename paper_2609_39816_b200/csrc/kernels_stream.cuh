@@ -102,6 +102,18 @@ inline bool fmm_encode_pattern(int storage, int product, const EncodeOperand* a,
   return ((a ? a : b)->h_tab->R == 7 ? fmm_encode_one_level : fmm_encode_two_level)(storage, product, a, b, mode, clear, clear_bytes, status, st, err);
 }
 
+// A whole scheme_gemm of one-level Strassen (and its diagonal gauges) on small blocks, bf16 products without scales, in one launch
+// (one_launch.cu).  False, with nothing enqueued, where it has no kernel for the tables or the sizes; else *err is the launch's result.
+struct OneLaunchArgs {
+  int storage, output, weight_layout;
+  const void* A; const void* B; void* C; int64_t lda, ldb, ldc;      // B as stored
+  const CoefTable* tab_a; const CoefTable* tab_b; const CoefTable* tab_w;      // host tables
+  void* ahat; void* bhat; void* prod; int64_t sAhat, sBhat, sProd;
+  int64_t bm, bn, bk;
+  int* status;                  // zeroed on the way
+};
+bool fmm_one_launch(const OneLaunchArgs& a, cudaStream_t st, cudaError_t* err);
+
 // One operand of an encode launch.  A launch carries up to two (A and B of one product): blocks [0, a.blocks) work
 // on the first, the rest on the second, so both operands are encoded side by side without a second stream.
 struct EncodeJob {

@@ -1,0 +1,86 @@
+"""scheme_gemm of one-level Strassen in one launch: block sums bit for bit those of the table-driven kernels (the same algorithm with
+its products renumbered), products against fp64 products of those sums (fp32 additions of bk terms), the result against the
+products in the workspace, combined in fp64 (at most four multiply-adds and the coefficient's rounding).  Nothing outside the
+operands is read, nothing outside the result written."""
+import numpy as np
+import pytest
+import torch
+
+import gpu_util as gu
+
+pytestmark = pytest.mark.gpu
+
+_TD = {"f32": torch.float32, "bf16": torch.bfloat16}
+
+
+@pytest.mark.parametrize("storage,output", [("f32", "f32"), ("bf16", "bf16"), ("f32", "bf16"), ("bf16", "f32")])
+@pytest.mark.parametrize("weight", [True, False])
+@pytest.mark.parametrize("M,K,N", [
+    (2, 32, 16),           # one row, one step of the tensor cores
+    (256, 256, 256),
+    (70, 96, 48),          # ragged tiles both ways
+    (34, 512, 352),        # the longest rows
+    (768, 128, 512),       # more blocks of threads than SMs
+    (514, 512, 416),       # beyond the line: the passes of their own
+])
+@pytest.mark.parametrize("gauged", [False, True])
+def test_one_launch(M, K, N, weight, storage, output, gauged):
+    lib = gu.fmm()
+    s = lib.scheme_builtin("strassen222")
+    if gauged:
+        s = lib.gauge_apply(s, np.diag([1.0, -0.5]), np.diag([3.0, 1.0]), np.diag([-1.0, 0.25]))
+    perm = list(range(6, -1, -1))
+    gen = torch.Generator(device="cuda").manual_seed(M + K + N)
+
+    def operand(rows, cols, dt, pad=16):
+        buf = torch.full((rows, cols + pad), float("nan"), dtype=dt, device="cuda")
+        buf[:, :cols] = torch.randn(rows, cols, generator=gen, device="cuda").to(dt)
+        return buf
+
+    A, B = operand(M, K, _TD[storage]), operand(*((N, K) if weight else (K, N)), _TD[storage])
+
+    def call(t, C):
+        d = lib.GemmDesc.make(M, K, N, storage, "bf16", output, weight_layout=weight, lda=A.shape[1], ldb=B.shape[1], ldc=C.shape[1])
+        ws = torch.full((lib.scheme_gemm_workspace(t, d),), 255, dtype=torch.uint8, device="cuda")
+        lib.scheme_gemm(t, d, A, B, C, ws)
+        lib.device_status(ws)
+        off = lib.scheme_gemm_workspace_layout(t, d)
+
+        def grab(o, stride, rows, cols, dt):
+            es = torch.empty((), dtype=dt).element_size()
+            return ws[o:o + 7 * stride * es].view(dt).view(7, stride)[:, :rows * cols].reshape(7, rows, cols)
+
+        bm, bk, bn = M // 2, K // 2, N // 2
+        return (grab(off["Ahat"], off["stride_Ahat"], bm, bk, torch.bfloat16), grab(off["Bhat"], off["stride_Bhat"], bn, bk, torch.bfloat16),
+                grab(off["M"], off["stride_M"], bm, bn, torch.float32))
+
+    before = lib.launch_count()
+    C = torch.full((M, N + 8), -7.0, dtype=_TD[output], device="cuda")
+    a, b, P = call(s, C)
+    launches = lib.launch_count() - before
+    assert launches == (1 if (M, K, N) != (514, 512, 416) else 3 + (not weight))
+    a2, b2, _ = call(lib.scheme_permute_products(s, perm), torch.empty_like(C))
+    assert torch.equal(a[perm], a2) and torch.equal(b[perm], b2)
+    exact = a.double() @ b.double().transpose(1, 2)
+    size = a.double().abs() @ b.double().abs().transpose(1, 2)
+    assert bool(((P.double() - exact).abs() <= (K // 2 + 1) * 2.0 ** -23 * size + 1e-30).all())
+    w = torch.from_numpy(s.coefficients()[2].astype(np.float32)).double().cuda()
+    ref = torch.einsum("rij,rpq->ipjq", w, P.double()).reshape(M, N)
+    size = torch.einsum("rij,rpq->ipjq", w.abs(), P.double().abs()).reshape(M, N)
+    out = 2.0 ** -9 if output == "bf16" else 0.0
+    assert bool(((C[:, :N].double() - ref).abs() <= (5 * 2.0 ** -24 + out) * size + out * ref.abs() + 1e-30).all())
+    assert bool((C[:, N:] == -7.0).all())
+
+
+def test_bhat_persists():
+    """The weight's block sums of such a call serve later calls that reuse them."""
+    lib = gu.fmm()
+    s = lib.scheme_builtin("strassen222")
+    A, B = torch.randn(64, 128, device="cuda"), torch.randn(128, 96, device="cuda")
+    d = lib.GemmDesc.make(64, 128, 96, "f32", "bf16", "f32")
+    ws = gu.workspace(lib.scheme_gemm_workspace(s, d))
+    C, R = torch.empty(64, 96, device="cuda"), torch.empty(64, 96, device="cuda")
+    lib.scheme_gemm(s, d, A, B, C, ws)
+    lib.scheme_gemm(s, lib.GemmDesc.make(64, 128, 96, "f32", "bf16", "f32", flags=lib.FLAG_REUSE_BHAT), A, B, R, ws)
+    # the other path's products are sums of 64 terms in another order
+    assert bool(((C - R).abs() <= 64 * 2.0 ** -22 * (A.abs() @ B.abs()) * 4).all())
