@@ -102,6 +102,13 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
+// a box from shared memory to a tensor, parts past the tensor's ends left out; one lane issues, commits and waits
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t src, int c0, int c1, int c2) {
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];"
+               ::"l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(src) : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -517,14 +524,39 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-struct PairLayout {
+template <bool kTma>
+struct PairLayoutT {
   static constexpr int BN = 256;                 // columns of the pair's tile
-  static constexpr int kStages = 6;
+  static constexpr int kStages = kTma ? 5 : 6;
   static constexpr int kABytes = BM * BKB;       // this CTA's 128 rows of A
   static constexpr int kBBytes = (BN / 2) * BKB; // this CTA's half of the B tile
   static constexpr int kStageBytes = kABytes + kBBytes;
   static constexpr int kBarBytes = 256;
-  static constexpr int kTotal = kStages * kStageBytes + kBarBytes + 1024;
+  static constexpr int kBoxBytes = 32 * 128;     // staging of the stores (StoreBox): two boxes of 32 rows x 128 bytes a warp, between ring and barriers
+  static constexpr int kStoreBytes = kTma ? 4 * 2 * kBoxBytes : 0;
+  static constexpr int kTotal = kStages * kStageBytes + kStoreBytes + kBarBytes + 1024;
+};
+using PairLayout = PairLayoutT<false>;
+
+// Products leave by TMA stores: a warp writes 32 rows x 32 columns of fp32 to shared memory (128-byte swizzle) and one lane sends them off,
+// whole lines, beside the copies of the operands.  49 products of 512 x 3072 x 1024 in e4m3, 74 pairs: 83 us; 97 with stores from registers, a
+// 32-byte sector of a row a lane (43 without stores, 67 with nothing but them).  A stage of the ring makes room for the boxes: beyond 200 KB
+// the decode's blocks, started ahead, find no place beside a CTA, and the call is no faster.
+struct StoreBox {
+  const CUtensorMap* map;
+  uint32_t boxes;             // this warp's, taken in turn
+  __device__ __forceinline__ void send(const uint32_t (&v)[32], int which, int lane, int col, int row, int r) const {
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");      // this box's previous contents are on their way
+    __syncwarp();
+    const uint32_t box = boxes + (uint32_t)((which & 1) * PairLayout::kBoxBytes), at = box + (uint32_t)(lane * 128);
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at + (uint32_t)((j ^ (lane & 7)) * 16)), "r"(v[4 * j]), "r"(v[4 * j + 1]),
+                   "r"(v[4 * j + 2]), "r"(v[4 * j + 3]) : "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) tma_store_3d(map, box, col, row, r);
+  }
 };
 
 // The three roles of one CTA of a pair (producer warp 0, MMA warp 1, epilogue warps 2..5), given the CTA's ring,
@@ -537,11 +569,13 @@ struct PairCtx {
   uint32_t rank;              // CTA rank in the pair (0 = leader)
 };
 
-template <bool kFp8>
+// kTma: fp32 products by TMA stores through map_out
+template <bool kFp8, bool kTma = false>
 __device__ __forceinline__ void pair_roles(const int warp, const int lane, const PairCtx& cx, const CUtensorMap& map_a,
                                            const CUtensorMap& map_b, void* __restrict__ out, const float* __restrict__ sA,
-                                           const float* __restrict__ sB, const TileParams& tp, DeviceStatus* status) {
-  using L = PairLayout;
+                                           const float* __restrict__ sB, const TileParams& tp, DeviceStatus* status,
+                                           const CUtensorMap* map_out = nullptr) {
+  using L = PairLayoutT<kTma>;
   constexpr int BN = L::BN;
   unsigned char* smem = cx.smem;
   const uint32_t bar_base = cx.bar_base;
@@ -675,7 +709,18 @@ __device__ __forceinline__ void pair_roles(const int warp, const int lane, const
         tc_ld32(taddr, v);
         tc_wait_ld();
         const int col0 = tn * BN + c * 32;
-        if (row_ok && col0 < tp.rows_b) {
+        if constexpr (kTma) {
+          if (col0 < tp.rows_b && row - lane < tp.rows_a) {       // whole warps
+            if (tp.row_scale != nullptr && row_ok)
+              apply_row_col_scale(v, tp.row_scale[(long long)r * tp.rs_batch + row],
+                                  tp.col_scale + (long long)r * tp.cs_batch + col0, min(32, tp.rows_b - col0));
+            if (alpha != 1.0f) {
+#pragma unroll
+              for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) * alpha);
+            }
+            StoreBox{map_out, smem_u32(smem) + (uint32_t)(L::kStages * L::kStageBytes + quad * 2 * L::kBoxBytes)}.send(v, c, lane, col0, row - lane, r);
+          }
+        } else if (row_ok && col0 < tp.rows_b) {
           if (tp.row_scale != nullptr)
             apply_row_col_scale(v, tp.row_scale[(long long)r * tp.rs_batch + row],
                                 tp.col_scale + (long long)r * tp.cs_batch + col0, min(32, tp.rows_b - col0));
@@ -687,18 +732,20 @@ __device__ __forceinline__ void pair_roles(const int warp, const int lane, const
       if (lane == 0) mbar_arrive_cluster(tempty_bar(acc) & kPeerBitMask);
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
+    if (kTma && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   }
 
 }
 
 // Set-up shared by every kernel that runs the pair roles: barrier block, TMEM allocation (warp 1 of the CTA), and the
 // CTA- and cluster-wide barriers that make them visible.  Every thread of the CTA calls it, and pair_teardown at the end.
+template <bool kTma = false>
 __device__ __forceinline__ PairCtx pair_setup(unsigned char* smem_raw, const int warp) {
-  using L = PairLayout;
+  using L = PairLayoutT<kTma>;
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t base = (raw_addr + 1023u) & ~1023u;
   unsigned char* smem = smem_raw + (base - raw_addr);
-  unsigned char* bar_mem = smem + L::kStages * L::kStageBytes;
+  unsigned char* bar_mem = smem + L::kStages * L::kStageBytes + L::kStoreBytes;
   const uint32_t bar_base = smem_u32(bar_mem);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_mem + 8 * (2 * L::kStages + 5));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_mem + 8 * (2 * L::kStages + 5) + 8);
@@ -740,18 +787,31 @@ __device__ __forceinline__ void pair_teardown(const PairCtx& cx, const int warp)
   }
 }
 
+template <bool kFp8, bool kTma>
+__device__ __forceinline__ void block_products_pair_body(const CUtensorMap& map_a, const CUtensorMap& map_b, const CUtensorMap* map_out,
+                                                         void* __restrict__ out, const float* __restrict__ sA, const float* __restrict__ sB,
+                                                         const TileParams& tp, DeviceStatus* status) {
+  grid_launch_dependents();   // the decode may set up while this grid drains; it waits before reading the products
+  extern __shared__ unsigned char smem_raw[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const PairCtx cx = pair_setup<kTma>(smem_raw, warp);
+  grid_dependency_wait();     // operands and scales come from the previous kernel of the stream
+  pair_roles<kFp8, kTma>(warp, lane, cx, map_a, map_b, out, sA, sB, tp, status, map_out);
+  pair_teardown(cx, warp);
+}
 template <bool kFp8>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kNumThreads, 1)
 block_products_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                            void* __restrict__ out, const float* __restrict__ sA, const float* __restrict__ sB,
                            TileParams tp, DeviceStatus* status) {
-  grid_launch_dependents();   // the decode may set up while this grid drains; it waits before reading the products
-  extern __shared__ unsigned char smem_raw[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const PairCtx cx = pair_setup(smem_raw, warp);
-  grid_dependency_wait();     // operands and scales come from the previous kernel of the stream
-  pair_roles<kFp8>(warp, lane, cx, map_a, map_b, out, sA, sB, tp, status);
-  pair_teardown(cx, warp);
+  block_products_pair_body<kFp8, false>(map_a, map_b, nullptr, out, sA, sB, tp, status);
+}
+template <bool kFp8>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kNumThreads, 1)
+block_products_pair_tma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
+                               const __grid_constant__ CUtensorMap map_out, const float* __restrict__ sA, const float* __restrict__ sB,
+                               TileParams tp, DeviceStatus* status) {
+  block_products_pair_body<kFp8, true>(map_a, map_b, &map_out, nullptr, sA, sB, tp, status);
 }
 
 // ---------------------------------------------------------------- fused sweep kernel
@@ -847,6 +907,17 @@ bool make_operand_map(CUtensorMap* map, bool fp8, const void* ptr, int64_t rows,
   return rc == CUDA_SUCCESS;
 }
 
+// fp32 output [batches][rows][cols], boxes of 32 rows x 32 columns; false where it has no such map (a batch's or row's alignment)
+bool make_output_map(CUtensorMap* map, const BlockProductArgs& a, int64_t batches) {
+  EncodeTiledFn fn = get_encode_fn();
+  if (!fn || reinterpret_cast<uintptr_t>(a.out) % 16 || a.ldo % 4 || a.o_batch % 4) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)a.rows_b, (cuuint64_t)a.rows_a, (cuuint64_t)batches};
+  cuuint64_t strides[2] = {(cuuint64_t)a.ldo * 4, (cuuint64_t)(batches > 1 ? a.o_batch : a.rows_a * a.ldo) * 4};
+  cuuint32_t box[3] = {32u, 32u, 1u}, estr[3] = {1u, 1u, 1u};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, a.out, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 int sm_count() {
   static int n = 0;
   if (n == 0) {
@@ -901,7 +972,7 @@ fmm_status launch_t(const BlockProductArgs& a, cudaStream_t st) {
 template <bool kFp8>
 fmm_status launch_pair(const BlockProductArgs& a, cudaStream_t st) {
   using L = PairLayout;
-  CUtensorMap ma, mb;
+  CUtensorMap ma, mb, mo;
   const int groups = a.groups > 1 ? a.groups : 1;
   if (!make_operand_map(&ma, kFp8, a.A, a.rows_a * groups, a.kdim, a.lda, a.a_batch, a.batches, BM)) return FMM_ERR_CUDA;
   if (!make_operand_map(&mb, kFp8, a.B, a.rows_b * groups, a.kdim, a.ldb, a.b_batch, a.batches, L::BN / 2)) return FMM_ERR_CUDA;
@@ -924,6 +995,21 @@ fmm_status launch_pair(const BlockProductArgs& a, cudaStream_t st) {
   const int sms = sm_count();
   if (sms < 2) return FMM_ERR_CUDA;
   const long long pairs = std::min<long long>(total, sms / 2);
+  // Products by TMA stores where stores hold the kernel up: 8-bit products of short inner dimensions.  Whole calls, from registers / by TMA, us:
+  // two-level e4m3 at 2048 x 4096 x 12288 268 / 260, 4096^3 171 / 162; 4096 x 13824 x 5120 438 / 445; bf16 at 4096^3 (products alone) 82.4 / 82.1,
+  // 8192 x 13824 x 5120 450 / 467.  Fewer rounds of tiles wait for their last stores alone.
+  if constexpr (kFp8) {
+    if ((a.out_mode == 0 || a.output == FMM_F32) && tp.kbytes <= 2048 && total >= 4 * pairs && make_output_map(&mo, a, (int64_t)a.batches * groups)) {
+      using LT = PairLayoutT<true>;
+      auto k = block_products_pair_tma_kernel<kFp8>;
+      static unsigned long long smem_ok = 0;
+      if (fmm_allow_dynamic_smem(k, LT::kTotal, &smem_ok) != cudaSuccess) return FMM_ERR_CUDA;
+      if (launch_dependent(k, dim3((unsigned)(2 * pairs)), dim3(kNumThreads), (size_t)LT::kTotal, st, ma, mb, mo, a.sA, a.sB, tp, a.status) != cudaSuccess)
+        return FMM_ERR_CUDA;
+      ++fmm_launch_counter();
+      return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+    }
+  }
   auto k = block_products_pair_kernel<kFp8>;
   static unsigned long long smem_ok = 0;
   if (fmm_allow_dynamic_smem(k, L::kTotal, &smem_ok) != cudaSuccess) return FMM_ERR_CUDA;
