@@ -384,10 +384,6 @@ cudaError_t launch_encode_split(const int8_t* codes, int64_t K, int gr, int gc, 
 // 2048 x 4096 x 11008.
 // ------------------------------------------------------------------------------------------
 constexpr int kCodesThreads = 256;
-struct CodesJob {
-  const int8_t* codes; const float* scales; const CoefTable* tab; int8_t* out; float* scales_t;
-  int gr, gc, tiles, blocks; int64_t br;      // grid, 128-row tiles of a block, thread blocks of the job, rows of a block
-};
 __device__ __forceinline__ uint32_t digits_of(uint32_t bytes) { return (bytes ^ 0x80808080u) - 0x80808080u; }
 __device__ __forceinline__ uint32_t bytes_of(uint32_t digits) { return (digits + 0x80808080u) ^ 0x80808080u; }
 
@@ -449,6 +445,8 @@ encode_codes_kernel(const CodesJob ja, const CodesJob jb, int64_t K, int G, int 
 }
 
 cudaError_t launch_encode_codes(CodesJob a, CodesJob b, const CoefTable& h_a, const CoefTable& h_b, int64_t K, int G, int h, cudaStream_t st) {
+  cudaError_t done = cudaSuccess;
+  if ((h_a.R == 7 ? fmm_encode_codes_one_level : fmm_encode_codes_two_level)(a, b, h_a, h_b, K, G, st, &done)) return done;
   size_t smem = 0;
   for (const CoefTable* t : {&h_a, &h_b})
     smem = std::max(smem, (size_t)(t->ncell + 1) * kCodesThreads * 16 + (size_t)t->off[t->R] * 8 + (size_t)(t->R + 1) * 4);

@@ -114,6 +114,17 @@ struct OneLaunchArgs {
 };
 bool fmm_one_launch(const OneLaunchArgs& a, cudaStream_t st, cudaError_t* err);
 
+// Block sums of int8 codes as int8 in the order that the certified kernel's MMAs read, and the rows' scales turned to group-major
+// (int8_path.cu): grid and 128-row tiles of a block, thread blocks of the job (set by the launch), rows of a block.
+struct CodesJob {
+  const int8_t* codes; const float* scales; const CoefTable* tab; int8_t* out; float* scales_t;
+  int gr, gc, tiles, blocks; int64_t br;
+};
+// The same for whole weights on the pattern of Strassen's algorithm, nested once or plain, in groups of 128 inner indices (encode_pattern.cu);
+// false, with nothing enqueued, where the tables are others
+bool fmm_encode_codes_two_level(CodesJob a, CodesJob b, const CoefTable& h_a, const CoefTable& h_b, int64_t K, int G, cudaStream_t st, cudaError_t* err);
+bool fmm_encode_codes_one_level(CodesJob a, CodesJob b, const CoefTable& h_a, const CoefTable& h_b, int64_t K, int G, cudaStream_t st, cudaError_t* err);
+
 // One operand of an encode launch.  A launch carries up to two (A and B of one product): blocks [0, a.blocks) work
 // on the first, the rest on the second, so both operands are encoded side by side without a second stream.
 struct EncodeJob {
