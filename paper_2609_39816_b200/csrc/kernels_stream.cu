@@ -427,6 +427,11 @@ decode_batch_kernel(const ProdT* __restrict__ prod, const CoefTable* __restrict_
 
 // ------------------------------------------------------------------------------------------
 // block b sums partials[b * n .. b * n + n) into out[b]
+__global__ void collect_status_kernel(const DeviceStatus* a, const DeviceStatus* b, const DeviceStatus* c, double* out) {
+  grid_dependency_wait();
+  out[0] = (double)(a->code != 0 ? a->code : b->code != 0 ? b->code : c->code);
+}
+
 __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restrict__ partials, int n,
                                                            double* __restrict__ out) {
   __shared__ double red[8];
@@ -846,6 +851,13 @@ cudaError_t launch_decode(int output, const void* prod, int prod_dtype, int64_t 
                                           cstar32, partials, n_partials, gauges, st);
   return launch_decode_p<float>(output, (const float*)prod, prod_stride, d_tab, h_tab, R, sA, sB, m, n, bm, bn, C, ldc, cstar32,
                                 partials, n_partials, gauges, st);
+}
+
+cudaError_t launch_collect_status(const DeviceStatus* a, const DeviceStatus* b, const DeviceStatus* c, double* out, cudaStream_t st) {
+  const cudaError_t e = launch_dependent(collect_status_kernel, dim3(1), dim3(1), 0, st, a, b, c, out);
+  if (e != cudaSuccess) return e;
+  ++fmm_launch_counter();
+  return cudaGetLastError();
 }
 
 cudaError_t launch_sum_partials(const double* partials, int n, double* out, cudaStream_t st, int count) {

@@ -216,6 +216,9 @@ cudaError_t launch_sweep_variants(const SweepVariantArgs& a, cudaStream_t st);
 // out[b] = sum of partials[b*n .. b*n+n), b < count
 cudaError_t launch_sum_partials(const double* partials, int n, double* out, cudaStream_t st, int count = 1);
 
+// out[0] = 0 if the three status blocks report nothing, else one of their codes
+cudaError_t launch_collect_status(const DeviceStatus* a, const DeviceStatus* b, const DeviceStatus* c, double* out, cudaStream_t st);
+
 // C*(fp64) -> fp32 copy, and partial sums of C*^2.
 cudaError_t launch_cstar_prepare(const double* cstar, int64_t count, float* cstar32, double* partials,
                                  int* n_partials, cudaStream_t st);
