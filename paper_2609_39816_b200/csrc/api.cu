@@ -170,16 +170,33 @@ T* at(void* ws, size_t off) { return reinterpret_cast<T*>(static_cast<char*>(ws)
 #define FMM_CUDA(x) do { if ((x) != cudaSuccess) return FMM_ERR_CUDA; } while (0)
 #define FMM_TRY(x) do { fmm_status _s = (x); if (_s != FMM_OK) return _s; } while (0)
 
+// The largest magnitudes that a pipelined sweep's encodes find (scale mode 1) lie in two workspaces by turns.  The encode of one copy zeroes
+// the other workspace's words on its way, where its kernels do that (fmm_encode_pattern): a memset between two launches would
+// keep the second from setting up while the first drains.
+struct AmaxClear {
+  unsigned* words[2][2];      // [workspace][operand A, B]
+  bool zero[2][2] = {};
+  int at = 0;                 // this copy's workspace
+  void use(EncodeOperand* o, bool b_side) {
+    o->amax_clear = zero[at][b_side];
+    o->clear_next = words[at ^ 1][b_side];
+    zero[at][b_side] = false;
+  }
+  void done(bool b_side) { zero[at ^ 1][b_side] = true; }
+};
+
 // Encode one operand: optional amax pass, then block sums -> product dtype.  status: zeroed on the way by the kernels of
 // fmm_encode_pattern (callers pass it only where those run).
 fmm_status encode_operand(const fmm_gemm_desc* d, const void* X, int64_t ldx, int gr, int gc, int64_t br, int64_t bc,
                           const CoefTable* d_tab, const CoefTable* h_tab, void* hat, int64_t hat_stride, unsigned* amax,
-                          float* scale, bool b_side, int* status, cudaStream_t st) {
+                          float* scale, bool b_side, int* status, cudaStream_t st, AmaxClear* clear = nullptr) {
   const int mode = d->scale_mode;   // 0 none, 1 per encoded tensor, 2 per row of it, 3 model schedule (128-groups)
-  const EncodeOperand o{X, ldx, gr, gc, br, bc, d_tab, h_tab, hat, hat_stride, amax, scale, b_side ? 128 : 1, b_side ? 1 : 0};
+  EncodeOperand o{X, ldx, gr, gc, br, bc, d_tab, h_tab, hat, hat_stride, amax, scale, b_side ? 128 : 1, b_side ? 1 : 0};
+  if (clear) clear->use(&o, b_side);
   cudaError_t e = cudaSuccess;
   if (fmm_encode_pattern(d->storage, d->product, b_side ? nullptr : &o, b_side ? &o : nullptr, mode, amax,
                          scale_words(mode, h_tab->R, br, bc, b_side) * 4, status, st, &e)) {
+    if (clear) clear->done(b_side);
     FMM_CUDA(e);
     return FMM_OK;
   }
@@ -216,6 +233,7 @@ struct SchemeRun {
   const CoefTable *hA, *hB, *hW;   // host tables (list lengths size the kernels' shared memory)
   const CoefTable *dA, *dB, *dW;   // device copies
   int* status = nullptr;           // to be zeroed by the encode
+  AmaxClear* clear = nullptr;
   float* sA() const { return d->scale_mode != 0 ? at<float>(ws, L.sA) : nullptr; }
   float* sB() const { return d->scale_mode != 0 ? at<float>(ws, L.sB) : nullptr; }
 };
@@ -224,27 +242,29 @@ fmm_status stage_encode_a(const SchemeRun& r, const void* A, cudaStream_t st) {
   const fmm_scheme* s = r.s;
   ProfScope ps(0, st);
   return encode_operand(r.d, A, r.d->lda, s->m, s->k, r.d->M / s->m, r.d->K / s->k, r.dA, r.hA, at<char>(r.ws, r.L.ahat),
-                        r.L.sAhat, at<unsigned>(r.ws, r.L.amaxA), r.sA(), false, r.status, st);
+                        r.L.sAhat, at<unsigned>(r.ws, r.L.amaxA), r.sA(), false, r.status, st, r.clear);
 }
 fmm_status stage_encode_b(const SchemeRun& r, const void* Bk, int64_t ldbk, cudaStream_t st) {
   const fmm_scheme* s = r.s;
   ProfScope ps(1, st);
   return encode_operand(r.d, Bk, ldbk, s->n, s->k, r.d->N / s->n, r.d->K / s->k, r.dB, r.hB, at<char>(r.ws, r.L.bhat),
-                        r.L.sBhat, at<unsigned>(r.ws, r.L.amaxB), r.sB(), true, r.status, st);
+                        r.L.sBhat, at<unsigned>(r.ws, r.L.amaxB), r.sB(), true, r.status, st, r.clear);
 }
 // Both operands in one launch per pass (amax pass if scaled, then the encode pass), on one stream.
 fmm_status stage_encode_pair(const SchemeRun& r, const void* A, const void* Bk, int64_t ldbk, cudaStream_t st) {
   const fmm_scheme* s = r.s;
   const fmm_gemm_desc* d = r.d;
   const int64_t bm = d->M / s->m, bk = d->K / s->k, bn = d->N / s->n;
-  const EncodeOperand oa{A, d->lda, s->m, s->k, bm, bk, r.dA, r.hA, at<char>(r.ws, r.L.ahat), r.L.sAhat,
-                         at<unsigned>(r.ws, r.L.amaxA), r.sA(), 1, 0};
-  const EncodeOperand ob{Bk, ldbk, s->n, s->k, bn, bk, r.dB, r.hB, at<char>(r.ws, r.L.bhat), r.L.sBhat,
-                         at<unsigned>(r.ws, r.L.amaxB), r.sB(), 128, 1};
+  EncodeOperand oa{A, d->lda, s->m, s->k, bm, bk, r.dA, r.hA, at<char>(r.ws, r.L.ahat), r.L.sAhat,
+                   at<unsigned>(r.ws, r.L.amaxA), r.sA(), 1, 0};
+  EncodeOperand ob{Bk, ldbk, s->n, s->k, bn, bk, r.dB, r.hB, at<char>(r.ws, r.L.bhat), r.L.sBhat,
+                   at<unsigned>(r.ws, r.L.amaxB), r.sB(), 128, 1};
+  if (r.clear) { r.clear->use(&oa, false); r.clear->use(&ob, true); }
   ProfScope ps(0, st);
   const int mode = d->scale_mode;
   cudaError_t e = cudaSuccess;
   if (fmm_encode_pattern(d->storage, d->product, &oa, &ob, mode, at<char>(r.ws, r.L.amaxA), r.L.sA - r.L.amaxA, r.status, st, &e)) {
+    if (r.clear) { r.clear->done(false); r.clear->done(true); }
     FMM_CUDA(e);
     return FMM_OK;
   }
@@ -1167,22 +1187,30 @@ fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P
     if (!stream_wait(side, st, sE) || !stream_wait(side, st, sD)) return FMM_ERR_CUDA;   // nothing of the sweep is enqueued yet
     if (sG != st && !stream_wait(side, st, sG)) return FMM_ERR_CUDA;
     cudaEvent_t evG[2] = {nullptr, nullptr}, evD[2] = {nullptr, nullptr};
+    AmaxClear clear{};
+    for (int b = 0; b < 2; ++b) {
+      clear.words[b][0] = at<unsigned>(b ? gws2 : gws, L.g.amaxA);
+      clear.words[b][1] = at<unsigned>(b ? gws2 : gws, L.g.amaxB);
+    }
     // One step of the pipeline; any failure leaves the loop through the joins below, so that the caller's stream is
     // ordered behind everything that was enqueued on the library's streams (the caller owns the workspace they use).
     auto step = [&](size_t c) -> fmm_status {
       const int b = (int)(c & 1);
       batched.R = base->R * chunks[c].count;
+      clear.at = b;
       const SchemeRun r{&batched, d, L.g, b ? gws2 : gws, &tabs[3 * c], &tabs[3 * c + 1], &tabs[3 * c + 2],
-                        d_tabs + 3 * c, d_tabs + 3 * c + 1, d_tabs + 3 * c + 2};
+                        d_tabs + 3 * c, d_tabs + 3 * c + 1, d_tabs + 3 * c + 2, nullptr, d->scale_mode == 1 ? &clear : nullptr};
       // encode: the products of batch c-2 must have finished reading this buffer's Ahat / Bhat.  With one scale per
       // encoded tensor (mode 1) the decode of batch c-2 still reads this buffer's scales, which the encode rewrites:
       // then the encode waits for that decode too (the other modes fold their scales into the products).
       if (evG[b] && cudaStreamWaitEvent(sE, evG[b], 0) != cudaSuccess) return FMM_ERR_CUDA;
       if (d->scale_mode == 1 && evD[b] && cudaStreamWaitEvent(sE, evD[b], 0) != cudaSuccess) return FMM_ERR_CUDA;
-      // Large operands: two launches, not the paired one — beside the products and decode of the neighbouring batches
-      // the two smaller kernels pack better.  Small operands are launch-bound: one paired launch.
-      const bool small_operands = (d->M + d->N) * d->K * (int64_t)esize(d->storage) < ((int64_t)16 << 20);
-      if (small_operands) {
+      // Small operands are launch-bound: one paired launch.  With a scale per block sum it is the better one at any size: two launches
+      // where four would each start and drain, half a chip's work at a time (a copy, us, paired / apart: 2048 x 3456 x 1280 66 / 75,
+      // 4096^3 193 / 199).  Large bf16 operands: two launches, beside the products and decode of the neighbouring batches the two smaller
+      // kernels pack better (2048^3 53 to 56 / 51).
+      const bool paired = d->scale_mode == 1 || (d->M + d->N) * d->K * (int64_t)esize(d->storage) < ((int64_t)16 << 20);
+      if (paired) {
         FMM_TRY(stage_encode_pair(r, dA, bk_ptr, bk_ld, sE));
       } else {
         FMM_TRY(stage_encode_b(r, bk_ptr, bk_ld, sE));

@@ -66,6 +66,7 @@ struct PatJob {
   const void* X; int64_t ldx; int br, bc; void* out; int64_t rstride;
   unsigned* amax_bits; float* scale_out; int evict_first; int blocks;
   int steps;      // positions that a thread works on, one after the other (kAmax, kGroupAmax, kGroupScaled)
+  unsigned* clear_next;      // EncodeOperand's
 };
 
 // Passes of an operand; the last three are the model schedule's: A in one (its groups lie within a warp), B in two
@@ -240,6 +241,7 @@ __device__ __forceinline__ void pattern_body(const PatJob& j, const float* coefs
     __syncthreads();
   }
   if (kPass == kScaled) {
+    if (bid == 0 && j.clear_next != nullptr && tid < FMM_MAX_R) j.clear_next[tid] = 0u;
     if (tid < kProducts) {
       const float s = pow2_scale_448(__uint_as_float(j.amax_bits[tid])), inv = 1.0f / s;   // s: at most 2^120
       sm.factors[0][tid] = isfinite(inv) ? make_float4(inv, inv, 1.0f, 1.0f)
@@ -439,7 +441,7 @@ bool is_scheme(const float* coefs, const Pattern& p) {
 
 PatJob make_pat_job(const EncodeOperand& o, int dst_bytes) {
   const bool evict = (int64_t)o.h_tab->R * o.out_stride * dst_bytes > ((int64_t)48 << 20);   // as encode_kernel
-  return PatJob{o.X, o.ldx, (int)o.br, (int)o.bc, o.out, o.out_stride, o.amax_bits, o.scale, evict ? 1 : 0, 0, 1};
+  return PatJob{o.X, o.ldx, (int)o.br, (int)o.bc, o.out, o.out_stride, o.amax_bits, o.scale, evict ? 1 : 0, 0, 1, o.clear_next};
 }
 
 // Blocks of a pass over an operand, and how many positions their threads work on.  Passes that keep 49 maxima a thread reduce them
@@ -485,7 +487,7 @@ bool run_pattern(const PatJob& a, const PatJob& b, bool have_a, bool have_b, con
     *e = launch_pass<SrcT, DstT, kKind, kPlain, kPlain>(a, b, have_a, have_b, c, status, st);
     return true;
   } else if (mode == 1) {
-    *e = cudaMemsetAsync(clear, 0, clear_bytes, st);
+    *e = clear != nullptr ? cudaMemsetAsync(clear, 0, clear_bytes, st) : cudaSuccess;
     if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kAmax, kAmax>(a, b, have_a, have_b, c, status, st);
     if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kScaled, kScaled>(a, b, have_a, have_b, c, nullptr, st);
     return true;
@@ -609,6 +611,7 @@ bool FMM_PATTERN(fmm_encode)(int storage, int product, const EncodeOperand* a, c
       c = numbers;
     }
   }
+  if (mode == 1 && (!a || a->amax_clear) && (!b || b->amax_clear)) clear = nullptr;
   const int dst = product == FMM_E4M3 ? 1 : 2;
   const PatJob ja = a ? make_pat_job(*a, dst) : PatJob{}, jb = b ? make_pat_job(*b, dst) : PatJob{};
   const bool ha = a != nullptr, hb = b != nullptr, f32 = storage == FMM_F32;

@@ -85,6 +85,9 @@ struct EncodeOperand {
   int bf16_first;   // use_scale 3 only: round the block sum to bf16 before it is quantised
   const float* pre_scale = nullptr;   // use_scale 1 only: DEVICE, one float; the source's codes are in units of it and
                                       // scale[r] receives (this pass's scale) * pre_scale[0]
+  unsigned* clear_next = nullptr;     // fmm_encode_pattern, use_scale 1: FMM_MAX_R amax words of a later encode of this operand in other
+                                      // memory, which the last pass zeroes on its way
+  int amax_clear = 0;                 // and this call's are zero already
 };
 cudaError_t launch_encode_pair(int storage, int product, const EncodeOperand& a, const EncodeOperand* b, bool amax_only,
                                int use_scale, cudaStream_t st);
