@@ -476,6 +476,21 @@ cudaError_t launch_pass(PatJob a, PatJob b, bool have_a, bool have_b, const PatC
   return cudaGetLastError();
 }
 
+// The amax words are zeroed by a kernel: unlike a memset it and the pass behind it set up while their predecessors drain.
+__global__ void __launch_bounds__(256) clear_words_kernel(unsigned* words, size_t count) {
+  grid_launch_dependents();
+  grid_dependency_wait();
+  const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+  if (i < count) words[i] = 0u;
+}
+cudaError_t clear_words(void* words, size_t bytes, cudaStream_t st) {
+  const size_t count = bytes / 4;
+  const cudaError_t e = launch_dependent(clear_words_kernel, dim3((unsigned)((count + 255) / 256)), dim3(256), 0, st, static_cast<unsigned*>(words), count);
+  if (e != cudaSuccess) return e;
+  ++fmm_launch_counter();
+  return cudaGetLastError();
+}
+
 // Which (types, pattern, mode) have a kernel: bf16 without scales and e4m3 with a scale per block sum, all patterns; the model
 // schedule for the scheme and its sign variants.  The rest (scale mode 2, e4m3 without scales, the model schedule
 // under a general gauge) stays with encode_kernel.
@@ -487,7 +502,7 @@ bool run_pattern(const PatJob& a, const PatJob& b, bool have_a, bool have_b, con
     *e = launch_pass<SrcT, DstT, kKind, kPlain, kPlain>(a, b, have_a, have_b, c, status, st);
     return true;
   } else if (mode == 1) {
-    *e = clear != nullptr ? cudaMemsetAsync(clear, 0, clear_bytes, st) : cudaSuccess;
+    *e = clear != nullptr ? clear_words(clear, clear_bytes, st) : cudaSuccess;
     if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kAmax, kAmax>(a, b, have_a, have_b, c, status, st);
     if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kScaled, kScaled>(a, b, have_a, have_b, c, nullptr, st);
     return true;
@@ -495,7 +510,7 @@ bool run_pattern(const PatJob& a, const PatJob& b, bool have_a, bool have_b, con
     if (mode != 3) return false;
     *e = cudaSuccess;
     if (have_b) {
-      *e = cudaMemsetAsync(clear, 0, clear_bytes, st);
+      *e = clear_words(clear, clear_bytes, st);
       if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kNoPass, kGroupAmax>(a, b, false, true, c, nullptr, st);
     }
     if (*e == cudaSuccess) *e = launch_pass<SrcT, DstT, kKind, kGroupOneRow, kGroupScaled>(a, b, have_a, have_b, c, status, st);
