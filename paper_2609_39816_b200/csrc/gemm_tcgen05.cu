@@ -691,6 +691,7 @@ __device__ __forceinline__ void pair_roles(const int warp, const int lane, const
     bool ok = true;
     float alpha = 1.0f;
     if (tp.out_mode == 1 && sA != nullptr && sB != nullptr) alpha = sA[0] * sB[0];
+    [[maybe_unused]] int sent = 0;      // the boxes' turn goes on from tile to tile: a tile cut by the last column may send an odd number
     for (int tile = pair_id; tile < total_tiles && ok; tile += num_pairs) {
       const int r = tile / tiles_per_batch;
       const int rem = tile - r * tiles_per_batch;
@@ -718,7 +719,7 @@ __device__ __forceinline__ void pair_roles(const int warp, const int lane, const
 #pragma unroll
               for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) * alpha);
             }
-            StoreBox{map_out, smem_u32(smem) + (uint32_t)(L::kStages * L::kStageBytes + quad * 2 * L::kBoxBytes)}.send(v, c, lane, col0, row - lane, r);
+            StoreBox{map_out, smem_u32(smem) + (uint32_t)(L::kStages * L::kStageBytes + quad * 2 * L::kBoxBytes)}.send(v, sent++, lane, col0, row - lane, r);
           }
         } else if (row_ok && col0 < tp.rows_b) {
           if (tp.row_scale != nullptr)

@@ -10,7 +10,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("mode", [1, 2])
-@pytest.mark.parametrize("M,K,N", [(1200, 512, 3104), (1028, 64, 4128)])
+@pytest.mark.parametrize("M,K,N", [
+    (1200, 512, 3104),      # rows and columns end inside a box
+    (1028, 64, 4128), (2308, 64, 2336),      # an odd number of boxes in the last tiles of a row, one step of the inner dimension
+])
 def test_block_products(M, K, N, mode):
     lib = gu.fmm()
     s = lib.scheme_builtin("strassen444")
