@@ -493,8 +493,9 @@ __global__ void __launch_bounds__(256) frob_err_kernel(const OutT* __restrict__ 
 // multiply-adds).  Four blocks per SM hide the staging (16 inner indices ahead, in registers); the fragments are read
 // without bank conflicts (row strides of 4 mod 16 doubles).  A 128 x 128 tile of plain multiply-adds, one block per SM,
 // left the pipe idle while it staged: 9.4 ms at 2048 x 4096 x 4096 where this takes 2.06.
-// Few tiles: a cluster of 2, 4 or 8 blocks shares one tile, each block takes a contiguous share of the inner dimension,
-// and the partial sums meet in distributed shared memory, added in ascending order of the shares.
+// Few tiles, and those left over by whole rounds of the chip: a cluster of 2, 4 or 8 blocks shares one tile, each block takes a
+// contiguous share of the inner dimension, and the partial sums meet in distributed shared memory, added in ascending order of the shares.
+// The leftover tiles are a launch of their own whose blocks fill in beside the whole tiles' (kBefore, kAfter).
 // ------------------------------------------------------------------------------------------
 constexpr int kExT = 64, kExK = 16, kExThreads = 128, kExBlocksPerSm = 4;
 constexpr int kExLdK = kExK + 4, kExLdN = kExT + 4;      // row strides of [row][k] and [k][column] staging
@@ -534,14 +535,19 @@ __device__ __forceinline__ void mma_f64(double (&c)[4], const double (&a)[4], co
       : "d"(a[0]), "d"(a[1]), "d"(a[2]), "d"(a[3]), "d"(b[0]), "d"(b[1]));
 }
 
+// two launches for one product: the first lets the second start beside it; one block of the second stays until the first is done, so that
+// what follows it in the stream follows both
+enum ExactTurn { kOnly, kBefore, kAfter };
+
 template <typename T, bool kWeight>
 __global__ void __launch_bounds__(kExThreads, kExBlocksPerSm)
 exact_f64_kernel(const T* __restrict__ A, int64_t lda, const T* __restrict__ B, int64_t ldb, int64_t M, int64_t K, int64_t N,
-                 double* __restrict__ C, int64_t tiles_n, int split, int vec_a, int vec_b) {
+                 double* __restrict__ C, int64_t tiles_n, int64_t first_tile, int split, ExactTurn turn, int vec_a, int vec_b) {
+  if (turn == kBefore) grid_launch_dependents();
   constexpr int VE = 16 / (int)sizeof(T), kLoads = kExT * kExK / VE / kExThreads;   // 16-byte vectors per thread and operand
   __shared__ __align__(16) double sm[2][2][kExOperand];
-  const int64_t tile = blockIdx.x / split;
-  const int share = (int)(blockIdx.x - tile * split);
+  const int64_t tile = first_tile + blockIdx.x / split;
+  const int share = (int)(blockIdx.x % split);
   const int64_t m0 = tile / tiles_n * kExT, n0 = tile % tiles_n * kExT;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3, wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
@@ -642,6 +648,7 @@ exact_f64_kernel(const T* __restrict__ A, int64_t lda, const T* __restrict__ B, 
     if (row < M && col < N) C[row * N + col] = sum;
   }
   cluster.sync();     // no block leaves while its partial sums may still be read
+  if (turn == kAfter && blockIdx.x == gridDim.x - 1) grid_dependency_wait();
 }
 
 template <typename T, bool kWeight>
@@ -658,16 +665,36 @@ cudaError_t launch_exact_t(const T* A, int64_t lda, const T* B, int64_t ldb, int
     const int64_t shares = (tiles * c + 147) / 148, load = shares * (K / c + 64) * (shares == 1 ? 4 : 3);
     if (load < least) { least = load; split = c; }
   }
+  // Two or more tiles an SM: whole rounds of the chip with a block a tile, and the tiles left over split among clusters of 4 or 8, beside them,
+  // where an SM's share of both comes out less.  A round that would leave one block to itself on its SM (a fifth, a ninth) is split too, and
+  // the last of four, after which an SM would have nothing but a rest.
+  // Measured, all tiles alike / rounds and rest, us: 1000 x 2112 x 1568 (2.70 tiles an SM) 245 -> 219, 844 x 1440 x 1488 (2.27) 170 -> 132,
+  // 328 x 1792 x 3920 (2.51) 211 -> 186, 1452 x 2992 x 2080 (5.13) 606 -> 571 (with a fifth round 661), 2048 x 3456 x 1280 (4.32), fp32
+  // 582 -> 581 (with a fourth round 591), 1500 x 1000 x 2950 (7.62) 304 -> 290; with one round and a rest 2048 x 1024 x 512 (1.73) 84 -> 90.
+  int64_t whole = 0;
+  const int64_t full = tiles / 148, rounds = full - (full % 4 == 1 || full == 4 ? 1 : 0);
+  if (rounds >= 2 && tiles > rounds * 148)
+    for (int c = 4; c <= 8 && K >= (int64_t)c * kExK; c *= 2) {
+      const int64_t share = K / c + 64, load = 3 * (rounds * (K + 64) + (tiles - rounds * 148) * c * share / 148 + share * 3 / 5);
+      if (load < least) { least = load; split = c; whole = rounds * 148; }
+    }
   if (tiles * split > 0x7fffffff) return cudaErrorInvalidValue;
   auto aligned = [](const void* p, int64_t ld) { return (reinterpret_cast<uintptr_t>(p) % 16 == 0) && (ld * (int64_t)sizeof(T)) % 16 == 0; };
+  const int vec_a = (int)aligned(A, lda), vec_b = (int)aligned(B, ldb);
+  if (whole != 0) {
+    exact_f64_kernel<T, kWeight><<<(unsigned)whole, kExThreads, 0, st>>>(A, lda, B, ldb, M, K, N, C, tiles_n, (int64_t)0, 1, kBefore, vec_a, vec_b);
+    ++fmm_launch_counter();
+  }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(tiles * split)); cfg.blockDim = dim3(kExThreads); cfg.stream = st;
-  cudaLaunchAttribute attr[1];
+  cfg.gridDim = dim3((unsigned)((tiles - whole) * split)); cfg.blockDim = dim3(kExThreads); cfg.stream = st;
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, exact_f64_kernel<T, kWeight>, A, lda, B, ldb, M, K, N, C, tiles_n, split,
-                                     (int)aligned(A, lda), (int)aligned(B, ldb));
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = whole != 0 ? 2 : 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, exact_f64_kernel<T, kWeight>, A, lda, B, ldb, M, K, N, C, tiles_n, whole, split,
+                                     whole != 0 ? kAfter : kOnly, vec_a, vec_b);
   if (e != cudaSuccess) return e;
   ++fmm_launch_counter();
   return cudaGetLastError();
