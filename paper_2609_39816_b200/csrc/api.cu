@@ -602,7 +602,8 @@ bool sweep_many_ok(const fmm_scheme* s, const fmm_gemm_desc* d, int G) {
 }
 
 // Sweeps on small blocks that one kernel takes from the operands to the errors, given diagonal gauges.  Its blocks' partial sums
-// use the place of the decode's.  Whole calls, this kernel against the passes of sweep_many.cu, us: 512 copies at 64^3 279 / 410, 128^3 290 /
+// use the place of the decode's.  Whole calls, this kernel against the passes of sweep_many.cu, both before statuses and sums came back in one
+// copy (30 us less), us: 512 copies at 64^3 279 / 410, 128^3 290 /
 // 539, 256^3 778 / 1254; 64 at 256^3 242 / 329, 512 x 64 x 512 317 / 462; one copy at 128^3 164 / 170.  Not where a tile is mostly
 // padding of one side (100 copies at 16 x 256 x 512 415 / 395), nor for a few copies of long rows, which it walks with one block of
 // threads a tile (2 at 256^3 190 / 176).

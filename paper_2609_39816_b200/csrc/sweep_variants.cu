@@ -9,7 +9,7 @@
 // is wanted in registers, where the sums over the products are; 49 of them would leave three quarters of a 128-row tile empty.
 // What bounds it: sixteen warps an SM on phases of instruction issue (block sums twice, for the maxima 10 and for the codes 13 thousand
 // cycles of a block's 48) and of shared memory (products and sums over them 12).  512 sign variants at 128^3 from fp32: 100 us,
-// the call 290, where the passes took 310 and the call 539.
+// the call 255, where the passes took 310 (the call 539 before this kernel, 290 with it before the statuses came back with the sums).
 //
 // The lists of A and B are one code: the places of Strassen's V are those of U for products in another order (kPartner), so
 // cells are kept by place in the coefficient matrix and block sums in the order of U.
