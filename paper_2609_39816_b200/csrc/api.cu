@@ -365,7 +365,7 @@ fmm_status stage_decode(const SchemeRun& r, void* C, const float* cstar32, doubl
   cudaError_t e = cudaSuccess;
   if (gauges == 1 &&
       fmm_decode_pattern(r.d->output, at<char>(r.ws, r.L.prod), (r.d->flags & FMM_FLAG_PRODUCTS_BF16) ? FMM_BF16 : FMM_F32, r.L.sProd,
-                         r.hW, per_product ? r.sA() : nullptr, per_product ? r.sB() : nullptr, r.d->M / s->m, r.d->N / s->n, C,
+                         r.hW, per_product ? r.sA() : nullptr, per_product ? r.sB() : nullptr, s->n, r.d->M / s->m, r.d->N / s->n, C,
                          r.d->ldc, cstar32, at<double>(r.ws, r.L.partials), &np, 148 * 4, st, &e))
     FMM_CUDA(e);
   else
@@ -414,11 +414,12 @@ bool pattern_gemm(const fmm_scheme* s, const fmm_gemm_desc* d, bool skip_b) {
   if (d->flags & FMM_FLAG_ROUND_PER_LEVEL) return false;
   EncodeOperand a{}, b{};
   a.br = d->M / s->m; b.br = d->N / s->n; a.bc = b.bc = d->K / s->k;
+  a.gr = s->m; b.gr = s->n; a.gc = b.gc = s->k;
   a.h_tab = fmm_packed_table(*s, 0); b.h_tab = fmm_packed_table(*s, 1);
   const CoefTable* w = fmm_packed_table(*s, 2);
   return a.h_tab->R == b.h_tab->R && a.h_tab->R == w->ncell &&
          fmm_encode_pattern(d->storage, d->product, &a, skip_b ? nullptr : &b, d->scale_mode, nullptr, 0, nullptr, nullptr, nullptr) &&
-         fmm_decode_pattern(d->output, nullptr, 0, 0, w, nullptr, nullptr, a.br, b.br, nullptr, 0, nullptr, nullptr, nullptr, 1, nullptr, nullptr);
+         fmm_decode_pattern(d->output, nullptr, 0, 0, w, nullptr, nullptr, s->n, a.br, b.br, nullptr, 0, nullptr, nullptr, nullptr, 1, nullptr, nullptr);
 }
 
 // B as a K-major matrix [N x K]: in place for the weight layout, else transposed into the workspace.

@@ -147,9 +147,10 @@ bool launch_out(const void* prod, bool prod_bf16, int64_t rstride, const PatCoef
 }  // namespace
 
 bool FMM_PATTERN(fmm_decode)(int output, const void* prod, int prod_dtype, int64_t prod_stride, const CoefTable* h_tab, const float* sA,
-                        const float* sB, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
+                        const float* sB, int n, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
                         int* n_partials, int max_partials, cudaStream_t st, cudaError_t* err) {
   if (err != nullptr && (C != nullptr) == (cstar32 != nullptr)) return false;
+  if (n != kGrid) return false;                                  // as fmm_encode
   const int64_t nvec = bm * (bn >> 2), tiles = (nvec + kPatThreads - 1) / kPatThreads;
   if (nvec >= ((int64_t)1 << 31) - 4096) return false;          // positions are 32-bit
   PatCoefs c;

@@ -605,8 +605,10 @@ bool FMM_PATTERN(fmm_encode)(int storage, int product, const EncodeOperand* a, c
                              size_t clear_bytes, int* status, cudaStream_t st, cudaError_t* err) {
   if (storage != FMM_F32 && storage != FMM_BF16) return false;
   if (product == FMM_BF16 ? mode != 0 : mode != 1 && mode != 3) return false;
-  for (const EncodeOperand* o : {a, b})
+  for (const EncodeOperand* o : {a, b}) {
+    if (o && (o->gr != kGrid || o->gc != kGrid)) return false;      // four cells may also be a row or a column: the same lists, other addresses
     if (o && o->br * (o->bc / E) >= ((int64_t)1 << 31) - 4096) return false;      // positions are 32-bit
+  }
   PatCoefs c;
   std::memset(&c, 0, sizeof(c));
   int dense = -1;
@@ -639,6 +641,8 @@ bool FMM_PATTERN(fmm_encode)(int storage, int product, const EncodeOperand* a, c
 
 bool FMM_PATTERN(fmm_encode_codes)(CodesJob a, CodesJob b, const CoefTable& h_a, const CoefTable& h_b, int64_t K, int G, cudaStream_t st, cudaError_t* err) {
   CodeWeights w;
+  for (const CodesJob* j : {&a, &b})
+    if (j->gr != kGrid || j->gc != kGrid) return false;      // as fmm_encode
   if (!whole_weights(h_a, Pat<false, false>::value, w.a) || !whole_weights(h_b, Pat<true, false>::value, w.b)) return false;
   constexpr int rows = kPatThreads / (128 / kGrid / 16);
   int64_t grid = 0;

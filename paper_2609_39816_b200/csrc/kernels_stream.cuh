@@ -164,19 +164,19 @@ cudaError_t launch_decode(int output, const void* prod, int prod_dtype, int64_t 
                           int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials, int* n_partials,
                           cudaStream_t st, int gauges = 1);
 int decode_grid(int64_t bm, int64_t bn);
-// The same for the patterns that fmm_encode_pattern takes (decode_pattern.cu), result or error; at most max_partials partial
+// The same for the patterns that fmm_encode_pattern takes (decode_pattern.cu), result or error, n blocks to a row of C; at most max_partials partial
 // sums.  False, with nothing enqueued, where it has no kernel; else *err is the launch's result.  With err null: would a result
 // of these tables have one?
 bool fmm_decode_two_level(int output, const void* prod, int prod_dtype, int64_t prod_stride, const CoefTable* h_tab, const float* sA,
-                          const float* sB, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
+                          const float* sB, int n, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
                           int* n_partials, int max_partials, cudaStream_t st, cudaError_t* err);
 bool fmm_decode_one_level(int output, const void* prod, int prod_dtype, int64_t prod_stride, const CoefTable* h_tab, const float* sA,
-                          const float* sB, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
+                          const float* sB, int n, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
                           int* n_partials, int max_partials, cudaStream_t st, cudaError_t* err);
 inline bool fmm_decode_pattern(int output, const void* prod, int prod_dtype, int64_t prod_stride, const CoefTable* h_tab, const float* sA,
-                               const float* sB, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
+                               const float* sB, int n, int64_t bm, int64_t bn, void* C, int64_t ldc, const float* cstar32, double* partials,
                                int* n_partials, int max_partials, cudaStream_t st, cudaError_t* err) {
-  return (h_tab->ncell == 7 ? fmm_decode_one_level : fmm_decode_two_level)(output, prod, prod_dtype, prod_stride, h_tab, sA, sB, bm, bn, C, ldc,
+  return (h_tab->ncell == 7 ? fmm_decode_one_level : fmm_decode_two_level)(output, prod, prod_dtype, prod_stride, h_tab, sA, sB, n, bm, bn, C, ldc,
                                                                            cstar32, partials, n_partials, max_partials, st, err);
 }
 
