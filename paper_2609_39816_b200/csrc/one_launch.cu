@@ -252,6 +252,7 @@ bool fmm_one_launch(const OneLaunchArgs& a, cudaStream_t st, cudaError_t* err) {
   // One round of blocks, or little work each: in a graph, us, one launch / four: 256^3 fp32 5.7 / 9.5 (64 tiles of 128 inner indices), 256 x 512 x
   // 512 5.9 / 12.4 (128 of 256), 1024 x 256 x 512 10.3 / 11.0 (512 of 128), 512^3 bf16 11.8 / 10.9 (256 of 256), 768 x 384 x 768 20 / 16.
   if (a.bk > 256 || a.bm > 65536 || a.bn > 65536 || tiles * a.bk > 49152) return false;
+  if (!a.weight_layout && reinterpret_cast<uintptr_t>(a.B) % (a.storage == FMM_F32 ? 16 : 8)) return false;      // the transpose reads B element by element then
   Coefs c;
   if (!take(*a.tab_a, Sums<false>::value, false, c.a) || !take(*a.tab_b, Sums<true>::value, true, c.b) || !take_cells(*a.tab_w, c.w)) return false;
   const Args p{a.A, a.B, a.C, a.lda, a.ldb, a.ldc, static_cast<__nv_bfloat16*>(a.ahat), static_cast<__nv_bfloat16*>(a.bhat), static_cast<float*>(a.prod),

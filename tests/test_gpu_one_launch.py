@@ -84,3 +84,29 @@ def test_bhat_persists():
     lib.scheme_gemm(s, lib.GemmDesc.make(64, 128, 96, "f32", "bf16", "f32", flags=lib.FLAG_REUSE_BHAT), A, B, R, ws)
     # the other path's products are sums of 64 terms in another order
     assert bool(((C - R).abs() <= 64 * 2.0 ** -22 * (A.abs() @ B.abs()) * 4).all())
+
+
+@pytest.mark.parametrize("storage,skip", [("f32", 1), ("f32", 2), ("bf16", 1), ("bf16", 2), ("bf16", 4)])
+def test_row_major_b_at_any_address(storage, skip):
+    """A row-major B that vectors of four do not reach keeps the passes with the transpose, which reads it element by element."""
+    lib = gu.fmm()
+    s = lib.scheme_builtin("strassen222")
+    M, K, N = 64, 128, 96
+    A = torch.randn(M, K, device="cuda").to(_TD[storage])
+    B = torch.randn(K, N, device="cuda").to(_TD[storage])
+    moved = torch.full((skip + K * N,), float("nan"), dtype=_TD[storage], device="cuda")[skip:].view(K, N)
+    moved.copy_(B)
+    d = lib.GemmDesc.make(M, K, N, storage, "bf16", "f32")
+    off = lib.scheme_gemm_workspace_layout(s, d)
+    out = []
+    for b in (B, moved):
+        ws, C = gu.workspace(lib.scheme_gemm_workspace(s, d)), torch.empty(M, N, device="cuda")
+        before = lib.launch_count()
+        lib.scheme_gemm(s, d, A, b, C, ws)
+        lib.device_status(ws)
+        out.append((lib.launch_count() - before, ws[off["Bhat"]:off["Bhat"] + 7 * off["stride_Bhat"] * 2].view(torch.bfloat16).view(7, -1)[:, :N * K // 4], C))
+    wide = moved.data_ptr() % (16 if storage == "f32" else 8) == 0
+    assert out[0][0] == 1 and out[1][0] == (1 if wide else 4)
+    assert torch.equal(out[0][1], out[1][1])
+    # products are sums of 64 terms in one of two orders
+    assert bool(((out[0][2] - out[1][2]).abs() <= 64 * 2.0 ** -22 * (A.float().abs() @ B.float().abs()) * 4).all())
