@@ -253,6 +253,16 @@ bool fmm_one_launch(const OneLaunchArgs& a, cudaStream_t st, cudaError_t* err) {
   // 512 5.9 / 12.4 (128 of 256), 1024 x 256 x 512 10.3 / 11.0 (512 of 128), 512^3 bf16 11.8 / 10.9 (256 of 256), 768 x 384 x 768 20 / 16.
   if (a.bk > 256 || a.bm > 65536 || a.bn > 65536 || tiles * a.bk > 49152) return false;
   if (!a.weight_layout && reinterpret_cast<uintptr_t>(a.B) % (a.storage == FMM_F32 ? 16 : 8)) return false;      // the transpose reads B element by element then
+  // Tiles of C are written while others still read A and B: a C that overlaps one of them keeps the passes, which read both first
+  const int es = a.storage == FMM_F32 ? 4 : 2, eo = a.output == FMM_F32 ? 4 : 2;
+  auto overlaps_c = [&](const void* x, int64_t rows, int64_t cols, int64_t ld) {
+    const char* at = static_cast<const char*>(x);
+    const char* c = static_cast<const char*>(a.C);
+    return at < c + ((2 * a.bm - 1) * a.ldc + 2 * a.bn) * eo && c < at + ((rows - 1) * ld + cols) * es;
+  };
+  if (overlaps_c(a.A, 2 * a.bm, 2 * a.bk, a.lda) ||
+      (a.weight_layout ? overlaps_c(a.B, 2 * a.bn, 2 * a.bk, a.ldb) : overlaps_c(a.B, 2 * a.bk, 2 * a.bn, a.ldb)))
+    return false;
   Coefs c;
   if (!take(*a.tab_a, Sums<false>::value, false, c.a) || !take(*a.tab_b, Sums<true>::value, true, c.b) || !take_cells(*a.tab_w, c.w)) return false;
   const Args p{a.A, a.B, a.C, a.lda, a.ldb, a.ldc, static_cast<__nv_bfloat16*>(a.ahat), static_cast<__nv_bfloat16*>(a.bhat), static_cast<float*>(a.prod),

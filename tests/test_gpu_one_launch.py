@@ -110,3 +110,36 @@ def test_row_major_b_at_any_address(storage, skip):
     assert torch.equal(out[0][1], out[1][1])
     # products are sums of 64 terms in one of two orders
     assert bool(((out[0][2] - out[1][2]).abs() <= 64 * 2.0 ** -22 * (A.float().abs() @ B.float().abs()) * 4).all())
+
+
+@pytest.mark.parametrize("storage", ["f32", "bf16"])
+@pytest.mark.parametrize("which", ["A", "B", "rows"])
+def test_result_over_an_operand(which, storage):
+    """C over A or B, whole or its last rows over A's first: the operands are read before C is written."""
+    lib = gu.fmm()
+    s = lib.scheme_builtin("strassen222")
+    n, td = 192, _TD[storage]
+    A, B = torch.randn(n, n, device="cuda").to(td), torch.randn(n, n, device="cuda").to(td)
+    d = lib.GemmDesc.make(n, n, n, storage, "bf16", storage)
+    ws = gu.workspace(lib.scheme_gemm_workspace(s, d))
+
+    def call(a, b, c):
+        before = lib.launch_count()
+        lib.scheme_gemm(s, d, a, b, c, ws)
+        lib.device_status(ws)
+        return lib.launch_count() - before
+
+    ref = torch.empty_like(A)
+    assert call(A, B, ref) == 1
+    both = torch.zeros(2 * n - 8, n, dtype=td, device="cuda")
+    a, b = A.clone(), B.clone()
+    C = {"A": a, "B": b, "rows": both[:n]}[which]
+    if which == "rows":
+        a = both[n - 8:]
+        a.copy_(A)
+    assert call(a, b, C) == 4
+    assert call(A, B, torch.empty_like(A)) == 1
+    # products are sums of 96 terms in one of two orders, C a sum of at most four of them, rounded
+    size = 4 * (A.float().abs() @ B.float().abs())
+    out = 2.0 ** -8 if storage == "bf16" else 0.0
+    assert bool(((C.float() - ref.float()).abs() <= 96 * 2.0 ** -22 * size + out * ref.float().abs()).all())
