@@ -249,9 +249,13 @@ cudaError_t launch_t(const Args& p, const Coefs& c, cudaStream_t st) {
 
 bool fmm_one_launch(const OneLaunchArgs& a, cudaStream_t st, cudaError_t* err) {
   const int64_t tiles = ((a.bm + kTile - 1) / kTile) * ((a.bn + kTile - 1) / kTile);
-  // One round of blocks, or little work each: in a graph, us, one launch / four: 256^3 fp32 5.7 / 9.5 (64 tiles of 128 inner indices), 256 x 512 x
-  // 512 5.9 / 12.4 (128 of 256), 1024 x 256 x 512 10.3 / 11.0 (512 of 128), 512^3 bf16 11.8 / 10.9 (256 of 256), 768 x 384 x 768 20 / 16.
-  if (a.bk > 256 || a.bm > 65536 || a.bn > 65536 || tiles * a.bk > 49152) return false;
+  // One round of blocks, or little work each: whole calls in a graph, us, one launch / the passes (four; weight layout: three).
+  // 256^3 fp32 5.7 / 9.5 (64 tiles of 128 inner indices), 512 x 256 x 512 6.4 / 12.4 (256 of 128), 512 x 256 x 768 10.4 / 14.0 (384 of 128), 512^3 bf16 11.8 /
+  // 10.9 (256 of 256), 768 x 384 x 768 20 / 16.  Many short tiles start and drain in rounds: 1024 x 96 x 1024 11.0 / 11.9 (1024 of 48), 1024 x 64 x 1536 14.4 /
+  // 11.4 (1536 of 32).  Beyond 224 inner indices a block has its SM to itself, and a second round costs more than the launches that the weight
+  // layout saves: 128 x 512 x 1536 11.8 / 9.0 (192 of 256), row-major 11.4 / 13.0, 192 x 512 x 768 6.5 / 9.3 (144 of 256).
+  if (a.bk > 256 || a.bm > 65536 || a.bn > 65536 || tiles * a.bk > 49152 || tiles > 1024) return false;
+  if (a.weight_layout && a.bk > 224 && tiles > 148) return false;
   if (!a.weight_layout && reinterpret_cast<uintptr_t>(a.B) % (a.storage == FMM_F32 ? 16 : 8)) return false;      // the transpose reads B element by element then
   // Tiles of C are written while others still read A and B: a C that overlaps one of them keeps the passes, which read both first
   const int es = a.storage == FMM_F32 ? 4 : 2, eo = a.output == FMM_F32 ? 4 : 2;
