@@ -997,10 +997,12 @@ fmm_status launch_pair(const BlockProductArgs& a, cudaStream_t st) {
   if (sms < 2) return FMM_ERR_CUDA;
   const long long pairs = std::min<long long>(total, sms / 2);
   // Products by TMA stores where stores hold the kernel up: 8-bit products of short inner dimensions.  Whole calls, from registers / by TMA, us:
-  // two-level e4m3 at 2048 x 4096 x 12288 268 / 260, 4096^3 171 / 162; 4096 x 13824 x 5120 438 / 445; bf16 at 4096^3 (products alone) 82.4 / 82.1,
-  // 8192 x 13824 x 5120 450 / 467.  Fewer rounds of tiles wait for their last stores alone.
+  // two-level e4m3 at 2048 x 4096 x 12288 (1024 bytes of K a product) 244 / 233, 4096^3 160 / 149, 2048 x 5120 x 4096 (1280) 111 / 107; classical products of
+  // codes, 8192^2 with K 512 74.7 / 53.6, 1024 82 / 72; 6144 x K x 4608 with K 1024 37.7 / 36.5, 1280 39.9 / 39.5, 1536 43.4 / 44.1, 2048 62 / 66.  bf16 at
+  // 4096^3 (products alone) 82.4 / 82.1, 8192 x 13824 x 5120 450 / 467.  Four rounds of tiles and more; fewer would gain
+  // as well (1024^3 27.1 / 25.8).
   if constexpr (kFp8) {
-    if ((a.out_mode == 0 || a.output == FMM_F32) && tp.kbytes <= 2048 && total >= 4 * pairs && make_output_map(&mo, a, (int64_t)a.batches * groups)) {
+    if ((a.out_mode == 0 || a.output == FMM_F32) && tp.kbytes <= 1280 && total >= 4 * pairs && make_output_map(&mo, a, (int64_t)a.batches * groups)) {
       using LT = PairLayoutT<true>;
       auto k = block_products_pair_tma_kernel<kFp8>;
       static unsigned long long smem_ok = 0;
