@@ -569,7 +569,7 @@ struct PairCtx {
   uint32_t rank;              // CTA rank in the pair (0 = leader)
 };
 
-// kTma: fp32 products by TMA stores through map_out
+// kTma: fp32 products without row and column scales by TMA stores through map_out
 template <bool kFp8, bool kTma = false>
 __device__ __forceinline__ void pair_roles(const int warp, const int lane, const PairCtx& cx, const CUtensorMap& map_a,
                                            const CUtensorMap& map_b, void* __restrict__ out, const float* __restrict__ sA,
@@ -712,9 +712,6 @@ __device__ __forceinline__ void pair_roles(const int warp, const int lane, const
         const int col0 = tn * BN + c * 32;
         if constexpr (kTma) {
           if (col0 < tp.rows_b && row - lane < tp.rows_a) {       // whole warps
-            if (tp.row_scale != nullptr && row_ok)
-              apply_row_col_scale(v, tp.row_scale[(long long)r * tp.rs_batch + row],
-                                  tp.col_scale + (long long)r * tp.cs_batch + col0, min(32, tp.rows_b - col0));
             if (alpha != 1.0f) {
 #pragma unroll
               for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) * alpha);
@@ -999,10 +996,11 @@ fmm_status launch_pair(const BlockProductArgs& a, cudaStream_t st) {
   // Products by TMA stores where stores hold the kernel up: 8-bit products of short inner dimensions.  Whole calls, from registers / by TMA, us:
   // two-level e4m3 at 2048 x 4096 x 12288 (1024 bytes of K a product) 244 / 233, 4096^3 160 / 149, 2048 x 5120 x 4096 (1280) 111 / 107; classical products of
   // codes, 8192^2 with K 512 74.7 / 53.6, 1024 82 / 72; 6144 x K x 4608 with K 1024 37.7 / 36.5, 1280 39.9 / 39.5, 1536 43.4 / 44.1, 2048 62 / 66.  bf16 at
-  // 4096^3 (products alone) 82.4 / 82.1, 8192 x 13824 x 5120 450 / 467.  Four rounds of tiles and more; fewer would gain
+  // 4096^3 (products alone) 82.4 / 82.1, 8192 x 13824 x 5120 450 / 467.  Not with row and column scales, which cost more here than the stores give:
+  // two-level 4096^3 from bf16 305 / 318, K 1024 193 / 207, one level 4096 x 512 x 4096 110 / 122.  Four rounds of tiles and more; fewer would gain
   // as well (1024^3 27.1 / 25.8).
   if constexpr (kFp8) {
-    if ((a.out_mode == 0 || a.output == FMM_F32) && tp.kbytes <= 1280 && total >= 4 * pairs && make_output_map(&mo, a, (int64_t)a.batches * groups)) {
+    if ((a.out_mode == 0 || a.output == FMM_F32) && a.row_scale == nullptr && tp.kbytes <= 1280 && total >= 4 * pairs && make_output_map(&mo, a, (int64_t)a.batches * groups)) {
       using LT = PairLayoutT<true>;
       auto k = block_products_pair_tma_kernel<kFp8>;
       static unsigned long long smem_ok = 0;
