@@ -685,10 +685,11 @@ cudaError_t launch_exact_t(const T* A, int64_t lda, const T* B, int64_t ldb, int
   // the last of four, after which an SM would have nothing but a rest.
   // Measured, all tiles alike / rounds and rest, us: 1000 x 2112 x 1568 (2.70 tiles an SM) 245 -> 219, 844 x 1440 x 1488 (2.27) 170 -> 132,
   // 328 x 1792 x 3920 (2.51) 211 -> 186, 1452 x 2992 x 2080 (5.13) 606 -> 571 (with a fifth round 661), 2048 x 3456 x 1280 (4.32), fp32
-  // 582 -> 581 (with a fourth round 591), 1500 x 1000 x 2950 (7.62) 304 -> 290; with one round and a rest 2048 x 1024 x 512 (1.73) 84 -> 90.
+  // 582 -> 581 (with a fourth round 591), 1500 x 1000 x 2950 (7.62) 304 -> 290; with one round and a rest 2048 x 1024 x 512 (1.73) 84 -> 90.  The second launch
+  // needs 128 inner indices to pay: 1216 x K x 4096 (8.22) 31.1 -> 32.4 with K 64, 52.4 -> 50.3 with 128.
   int64_t whole = 0;
   const int64_t full = tiles / 148, rounds = full - (full % 4 == 1 || full == 4 ? 1 : 0);
-  if (rounds >= 2 && tiles > rounds * 148)
+  if (K >= 128 && rounds >= 2 && tiles > rounds * 148)
     for (int c = 4; c <= 8 && K >= (int64_t)c * kExK; c *= 2) {
       const int64_t share = K / c + 64, load = 3 * (rounds * (K + 64) + (tiles - rounds * 148) * c * share / 148 + share * 3 / 5);
       if (load < least) { least = load; split = c; whole = rounds * 148; }

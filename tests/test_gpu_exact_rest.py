@@ -14,6 +14,7 @@ pytestmark = pytest.mark.gpu
     (1000, 2112, 1568),     # clusters of four
     (70, 520, 12160),       # 380 tiles in two rows
     (1452, 600, 2080),      # five rounds of which the last is split
+    (1216, 64, 4096),       # too short for a second launch
 ])
 def test_rounds_and_rest(M, K, N, storage, weight):
     td = torch.bfloat16 if storage == "bf16" else torch.float32
@@ -28,7 +29,9 @@ def test_rounds_and_rest(M, K, N, storage, weight):
         fmm.exact_gemm_f64(d, A, B, C)
         return C.clone()
 
+    before = fmm.launch_count()
     got = call()
+    assert fmm.launch_count() - before == (2 if K >= 128 else 1)
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph):
         captured = call()
