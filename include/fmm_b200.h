@@ -468,6 +468,7 @@ int64_t fmm_launch_count(void);
  * back on the caller's stream, as with FMM_FLAG_SWEEP_SERIAL).  Phases:
  *   0 encode A   1 encode B (incl. the transpose of a K x N operand)   2 block products (scheme)
  *   3 decode (+ error reduction)   4 block products of classical_gemm   5 everything else.
+ * A scheme_gemm, or an error_sweep's copies, that one kernel takes from the operands to the result counts under 2.
  * fmm_profile_collect synchronises the recorded events, adds their durations (milliseconds) to ms[8]
  * and the number of bracketed regions to count[8] (HOST arrays, overwritten), and clears the record. */
 void fmm_profile_enable(int on);

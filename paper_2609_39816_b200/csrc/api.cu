@@ -706,7 +706,6 @@ fmm_status scheme_gemm(const fmm_scheme* s, const fmm_gemm_desc* d, const void* 
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const bool skip_b = (d->flags & FMM_FLAG_REUSE_BHAT) != 0;
   if (s->R == 7 && d->product == FMM_BF16 && d->flags == 0) {
-    ProfScope ps(2, st);
     const OneLaunchArgs o{d->storage, d->output, d->b_is_weight_layout, dA, dB, dC, d->lda, d->ldb, d->ldc, fmm_packed_table(*s, 0), fmm_packed_table(*s, 1),
                           fmm_packed_table(*s, 2), at<char>(d_ws, L.ahat), at<char>(d_ws, L.bhat), at<char>(d_ws, L.prod), L.sAhat, L.sBhat, L.sProd,
                           d->M / s->m, d->N / s->n, d->K / s->k, at<int>(d_ws, L.status)};

@@ -269,6 +269,7 @@ bool fmm_one_launch(const OneLaunchArgs& a, cudaStream_t st, cudaError_t* err) {
     return false;
   Coefs c;
   if (!take(*a.tab_a, Sums<false>::value, false, c.a) || !take(*a.tab_b, Sums<true>::value, true, c.b) || !take_cells(*a.tab_w, c.w)) return false;
+  ProfScope ps(2, st);      // opened once the call is taken: a region counts
   const Args p{a.A, a.B, a.C, a.lda, a.ldb, a.ldc, static_cast<__nv_bfloat16*>(a.ahat), static_cast<__nv_bfloat16*>(a.bhat), static_cast<float*>(a.prod),
                a.sAhat, a.sBhat, a.sProd, (int)a.bm, (int)a.bn, (int)a.bk, (int)((a.bm + kTile - 1) / kTile), (int)((a.bn + kTile - 1) / kTile), a.status};
   const bool f32 = a.storage == FMM_F32, out32 = a.output == FMM_F32;

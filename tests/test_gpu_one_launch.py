@@ -146,3 +146,23 @@ def test_result_over_an_operand(which, storage):
     size = 4 * (A.float().abs() @ B.float().abs())
     out = 2.0 ** -8 if storage == "bf16" else 0.0
     assert bool(((C.float() - ref.float()).abs() <= 96 * 2.0 ** -22 * size + out * ref.float().abs()).all())
+
+
+@pytest.mark.parametrize("M,K,N,gauged,regions", [(256, 256, 256, False, (0, 0, 1, 0)), (514, 512, 416, False, (1, 1, 1, 1)), (256, 256, 256, True, (1, 1, 1, 1))])
+def test_phases_are_counted_once(M, K, N, gauged, regions):
+    """A call in one launch is one region of the products; one that the kernel declines has its passes' regions and no more."""
+    lib = gu.fmm()
+    s = lib.scheme_builtin("strassen222")
+    if gauged:
+        s = lib.gauge_apply(s, *(np.array([[1.0, 0.5], [0.25, 1.0]]) for _ in range(3)))
+    A, B, C = torch.randn(M, K, device="cuda"), torch.randn(K, N, device="cuda"), torch.empty(M, N, device="cuda")
+    d = lib.GemmDesc.make(M, K, N, "f32", "bf16", "f32")
+    ws = gu.workspace(lib.scheme_gemm_workspace(s, d))
+    lib.profile_enable(True)
+    try:
+        lib.profile_collect()
+        lib.scheme_gemm(s, d, A, B, C, ws)
+        counts = lib.profile_collect()
+    finally:
+        lib.profile_enable(False)
+    assert tuple(counts[p][1] for p in ("encode_a", "encode_b", "products", "decode")) == regions
