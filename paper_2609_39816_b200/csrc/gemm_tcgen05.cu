@@ -1839,7 +1839,7 @@ fmm_status launch_int8_certified(const Int8CertArgs& a, cudaStream_t st) {
   const long long total = (long long)p.tiles_m * p.tiles_n * p.blocks;
   const int units = pair ? sms / 2 : sms;
   // one round needs no plan, nine or more differ by less than a tile in ten (8192^3: 131 MMAs either way, 127 on average)
-  if (total > units && total <= 8 * units && total <= kMaxPlanned && units <= kMaxPlanners) plan_tiles(&p, cost, units, (int)total);
+  if (total > units && total <= kMaxOwn * units && total <= kMaxPlanned && units <= kMaxPlanners) plan_tiles(&p, cost, units, (int)total);
   // block sums as rows of 4 KB (a tile of 128 rows, 32 inner indices), copied whole
   CUtensorMap ma, mb;
   if (!make_sums_map(&ma, a.Ahat, (int64_t)a.R * a.G * p.ksteps * p.hat_tiles_m)) return FMM_ERR_CUDA;

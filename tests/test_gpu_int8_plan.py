@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
     ("strassen444", 31, 212, 256, 10912),     # single CTAs, three rounds
     ("strassen444", 31, 1276, 128, 3200),
     ("strassen222", 63, 1280, 128, 3200),     # in order: the busiest is no better off
-    ("strassen444", 31, 2000, 128, 4064),     # pairs, two rounds
+    ("strassen444", 31, 2000, 128, 4064),     # pairs, two rounds; in order: a pair would take a third tile
     ("strassen222", 63, 3072, 256, 5104),
     ("strassen444", 31, 4096, 128, 4096),
     ("strassen444", 31, 4092, 128, 10976),    # pairs, ten rounds
