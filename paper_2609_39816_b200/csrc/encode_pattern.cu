@@ -82,12 +82,6 @@ constexpr int kPatBlocksPerSm = kLevels == 1 ? 8 : kPass == kPlain ? 6 : (kPass 
                               : kPass == kGroupScaled && kKind == kScheme && sizeof(SrcT) == 4 ? 4 : 5;
 
 constexpr int E = 4, NP = 2;          // values of a thread: 16 cells x 4 fp32 registers
-__device__ __forceinline__ float4 load_values(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
-__device__ __forceinline__ float4 load_values(const __nv_bfloat16* p) {
-  const uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
-  return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xFFFF0000u), __uint_as_float(r.y << 16),
-                     __uint_as_float(r.y & 0xFFFF0000u));
-}
 
 __device__ __forceinline__ float max3(float a, float b, float c) {        // drops NaN, as fmaxf
   float d;
@@ -540,8 +534,6 @@ bool run_types(const PatJob& a, const PatJob& b, bool have_a, bool have_b, const
 // the whole call 337 -> 317, at 64 rows 186 -> 157, one level 253 -> 234.
 // ------------------------------------------------------------------------------------------
 struct CodeWeights { int a[kLevels == 2 ? 144 : 12], b[kLevels == 2 ? 144 : 12]; };
-__device__ __forceinline__ uint32_t digits_of(uint32_t bytes) { return (bytes ^ 0x80808080u) - 0x80808080u; }
-__device__ __forceinline__ uint32_t bytes_of(uint32_t digits) { return (digits + 0x80808080u) ^ 0x80808080u; }
 
 template <bool kB>
 __device__ __forceinline__ void codes_body(const CodesJob& j, const int* weights, int bid, int64_t K, int G, int vec) {

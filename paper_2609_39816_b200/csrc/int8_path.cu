@@ -384,8 +384,6 @@ cudaError_t launch_encode_split(const int8_t* codes, int64_t K, int gr, int gc, 
 // 2048 x 4096 x 11008.
 // ------------------------------------------------------------------------------------------
 constexpr int kCodesThreads = 256;
-__device__ __forceinline__ uint32_t digits_of(uint32_t bytes) { return (bytes ^ 0x80808080u) - 0x80808080u; }
-__device__ __forceinline__ uint32_t bytes_of(uint32_t digits) { return (digits + 0x80808080u) ^ 0x80808080u; }
 
 __global__ void __launch_bounds__(kCodesThreads)
 encode_codes_kernel(const CodesJob ja, const CodesJob jb, int64_t K, int G, int h) {

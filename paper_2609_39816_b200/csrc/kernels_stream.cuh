@@ -123,6 +123,11 @@ struct CodesJob {
   const int8_t* codes; const float* scales; const CoefTable* tab; int8_t* out; float* scales_t;
   int gr, gc, tiles, blocks; int64_t br;
 };
+#ifdef __CUDACC__
+// four int8 codes as one number with signed digits of base 256, and back
+__device__ __forceinline__ uint32_t digits_of(uint32_t bytes) { return (bytes ^ 0x80808080u) - 0x80808080u; }
+__device__ __forceinline__ uint32_t bytes_of(uint32_t digits) { return (digits + 0x80808080u) ^ 0x80808080u; }
+#endif
 // The same for whole weights on the pattern of Strassen's algorithm, nested once or plain, in groups of 128 inner indices (encode_pattern.cu);
 // false, with nothing enqueued, where the tables are others
 bool fmm_encode_codes_two_level(CodesJob a, CodesJob b, const CoefTable& h_a, const CoefTable& h_b, int64_t K, int G, cudaStream_t st, cudaError_t* err);

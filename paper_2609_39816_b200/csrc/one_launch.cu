@@ -51,12 +51,6 @@ struct Args {
   int* status;
 };
 
-__device__ __forceinline__ float4 load_values(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
-__device__ __forceinline__ float4 load_values(const __nv_bfloat16* p) {
-  const uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
-  return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xFFFF0000u), __uint_as_float(r.y << 16),
-                     __uint_as_float(r.y & 0xFFFF0000u));
-}
 __device__ __forceinline__ uint2 to_bf16(const float2 (&a)[NP]) {
   const __nv_bfloat162 lo = __floats2bfloat162_rn(a[0].x, a[0].y), hi = __floats2bfloat162_rn(a[1].x, a[1].y);
   return make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));

@@ -79,12 +79,6 @@ __device__ __forceinline__ int swizzled(int w, int row, int words) {
 }
 
 constexpr int NP = 2;
-__device__ __forceinline__ float4 load_values(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
-__device__ __forceinline__ float4 load_values(const __nv_bfloat16* p) {
-  const uint2 r = __ldg(reinterpret_cast<const uint2*>(p));
-  return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xFFFF0000u), __uint_as_float(r.y << 16),
-                     __uint_as_float(r.y & 0xFFFF0000u));
-}
 __device__ __forceinline__ unsigned codes_of(const float2 (&a)[2]) {
   return (unsigned)__nv_cvt_float2_to_fp8x2(a[0], __NV_SATFINITE, __NV_E4M3) |
          (unsigned)__nv_cvt_float2_to_fp8x2(a[1], __NV_SATFINITE, __NV_E4M3) << 16;
