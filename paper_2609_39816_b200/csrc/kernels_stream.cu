@@ -426,12 +426,12 @@ decode_batch_kernel(const ProdT* __restrict__ prod, const CoefTable* __restrict_
 
 
 // ------------------------------------------------------------------------------------------
-// block b sums partials[b * n .. b * n + n) into out[b]
 __global__ void collect_status_kernel(const DeviceStatus* a, const DeviceStatus* b, const DeviceStatus* c, double* out) {
   grid_dependency_wait();
   out[0] = (double)(a->code != 0 ? a->code : b->code != 0 ? b->code : c->code);
 }
 
+// block b sums partials[b * n .. b * n + n) into out[b]
 __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restrict__ partials, int n,
                                                            double* __restrict__ out) {
   __shared__ double red[8];
@@ -472,22 +472,18 @@ __global__ void __launch_bounds__(256) frob_err_kernel(const OutT* __restrict__ 
   int64_t i = ((int64_t)blockIdx.x * 256 + threadIdx.x) * E, r = i / N, c = i - r * N;
 #pragma unroll 4
   for (; i < count; i += step) {
-    double v[E];
-    OutT x[E];
+    auto add = [&](float x, double v) {
+      const double d = (double)x - v;
+      e += d * d;
+      s += v * v;
+    };
     if constexpr (E == 4) {
       const double2 lo = *reinterpret_cast<const double2*>(cstar + i), hi = *reinterpret_cast<const double2*>(cstar + i + 2);
-      v[0] = lo.x; v[1] = lo.y; v[2] = hi.x; v[3] = hi.y;
-      if constexpr (sizeof(OutT) == 4) *reinterpret_cast<float4*>(x) = *reinterpret_cast<const float4*>(C + r * ldc + c);
-      else *reinterpret_cast<uint2*>(x) = *reinterpret_cast<const uint2*>(C + r * ldc + c);
+      const float4 x = load_values(C + r * ldc + c);
+      add(x.x, lo.x); add(x.y, lo.y); add(x.z, hi.x); add(x.w, hi.y);
     } else {
-      v[0] = cstar[i];
-      x[0] = C[r * ldc + c];
-    }
-#pragma unroll
-    for (int u = 0; u < E; ++u) {
-      const double d = (double)(float)x[u] - v[u];
-      e += d * d;
-      s += v[u] * v[u];
+      const double v = cstar[i];
+      add((float)C[r * ldc + c], v);
     }
     r += step_r;
     c += step_c;
