@@ -175,28 +175,27 @@ T* at(void* ws, size_t off) { return reinterpret_cast<T*>(static_cast<char*>(ws)
 // keep the second from setting up while the first drains.
 struct AmaxClear {
   unsigned* words[2][2];      // [workspace][operand A, B]
-  bool zero[2][2] = {};
+  bool zero[2] = {};
   int at = 0;                 // this copy's workspace
-  void use(EncodeOperand* o, bool b_side) {
-    o->amax_clear = zero[at][b_side];
-    o->clear_next = words[at ^ 1][b_side];
-    zero[at][b_side] = false;
+  void use(EncodeOperand* a, EncodeOperand* b) {
+    a->amax_clear = b->amax_clear = zero[at];
+    a->clear_next = words[at ^ 1][0];
+    b->clear_next = words[at ^ 1][1];
+    zero[at] = false;
   }
-  void done(bool b_side) { zero[at ^ 1][b_side] = true; }
+  void done() { zero[at ^ 1] = true; }
 };
 
 // Encode one operand: optional amax pass, then block sums -> product dtype.  status: zeroed on the way by the kernels of
 // fmm_encode_pattern (callers pass it only where those run).
 fmm_status encode_operand(const fmm_gemm_desc* d, const void* X, int64_t ldx, int gr, int gc, int64_t br, int64_t bc,
                           const CoefTable* d_tab, const CoefTable* h_tab, void* hat, int64_t hat_stride, unsigned* amax,
-                          float* scale, bool b_side, int* status, cudaStream_t st, AmaxClear* clear = nullptr) {
+                          float* scale, bool b_side, int* status, cudaStream_t st) {
   const int mode = d->scale_mode;   // 0 none, 1 per encoded tensor, 2 per row of it, 3 model schedule (128-groups)
-  EncodeOperand o{X, ldx, gr, gc, br, bc, d_tab, h_tab, hat, hat_stride, amax, scale, b_side ? 128 : 1, b_side ? 1 : 0};
-  if (clear) clear->use(&o, b_side);
+  const EncodeOperand o{X, ldx, gr, gc, br, bc, d_tab, h_tab, hat, hat_stride, amax, scale, b_side ? 128 : 1, b_side ? 1 : 0};
   cudaError_t e = cudaSuccess;
   if (fmm_encode_pattern(d->storage, d->product, b_side ? nullptr : &o, b_side ? &o : nullptr, mode, amax,
                          scale_words(mode, h_tab->R, br, bc, b_side) * 4, status, st, &e)) {
-    if (clear) clear->done(b_side);
     FMM_CUDA(e);
     return FMM_OK;
   }
@@ -233,7 +232,7 @@ struct SchemeRun {
   const CoefTable *hA, *hB, *hW;   // host tables (list lengths size the kernels' shared memory)
   const CoefTable *dA, *dB, *dW;   // device copies
   int* status = nullptr;           // to be zeroed by the encode
-  AmaxClear* clear = nullptr;
+  AmaxClear* clear = nullptr;      // stage_encode_pair's
   float* sA() const { return d->scale_mode != 0 ? at<float>(ws, L.sA) : nullptr; }
   float* sB() const { return d->scale_mode != 0 ? at<float>(ws, L.sB) : nullptr; }
 };
@@ -242,13 +241,13 @@ fmm_status stage_encode_a(const SchemeRun& r, const void* A, cudaStream_t st) {
   const fmm_scheme* s = r.s;
   ProfScope ps(0, st);
   return encode_operand(r.d, A, r.d->lda, s->m, s->k, r.d->M / s->m, r.d->K / s->k, r.dA, r.hA, at<char>(r.ws, r.L.ahat),
-                        r.L.sAhat, at<unsigned>(r.ws, r.L.amaxA), r.sA(), false, r.status, st, r.clear);
+                        r.L.sAhat, at<unsigned>(r.ws, r.L.amaxA), r.sA(), false, r.status, st);
 }
 fmm_status stage_encode_b(const SchemeRun& r, const void* Bk, int64_t ldbk, cudaStream_t st) {
   const fmm_scheme* s = r.s;
   ProfScope ps(1, st);
   return encode_operand(r.d, Bk, ldbk, s->n, s->k, r.d->N / s->n, r.d->K / s->k, r.dB, r.hB, at<char>(r.ws, r.L.bhat),
-                        r.L.sBhat, at<unsigned>(r.ws, r.L.amaxB), r.sB(), true, r.status, st, r.clear);
+                        r.L.sBhat, at<unsigned>(r.ws, r.L.amaxB), r.sB(), true, r.status, st);
 }
 // Both operands in one launch per pass (amax pass if scaled, then the encode pass), on one stream.
 fmm_status stage_encode_pair(const SchemeRun& r, const void* A, const void* Bk, int64_t ldbk, cudaStream_t st) {
@@ -259,12 +258,12 @@ fmm_status stage_encode_pair(const SchemeRun& r, const void* A, const void* Bk, 
                    at<unsigned>(r.ws, r.L.amaxA), r.sA(), 1, 0};
   EncodeOperand ob{Bk, ldbk, s->n, s->k, bn, bk, r.dB, r.hB, at<char>(r.ws, r.L.bhat), r.L.sBhat,
                    at<unsigned>(r.ws, r.L.amaxB), r.sB(), 128, 1};
-  if (r.clear) { r.clear->use(&oa, false); r.clear->use(&ob, true); }
+  if (r.clear) r.clear->use(&oa, &ob);
   ProfScope ps(0, st);
   const int mode = d->scale_mode;
   cudaError_t e = cudaSuccess;
   if (fmm_encode_pattern(d->storage, d->product, &oa, &ob, mode, at<char>(r.ws, r.L.amaxA), r.L.sA - r.L.amaxA, r.status, st, &e)) {
-    if (r.clear) { r.clear->done(false); r.clear->done(true); }
+    if (r.clear) r.clear->done();
     FMM_CUDA(e);
     return FMM_OK;
   }

@@ -57,6 +57,30 @@ def test_pipelined_sweep_gives_the_bits_of_the_serial_one(lib, Pd, scale, level)
         assert np.array_equal(piped, serial)
 
 
+@pytest.mark.parametrize("level,order", [
+    (0, "g" * 35),              # batches of eight by tables, then two copies by tables and one by compiled-in lists
+    (1, "gttiggtigt"),          # full, triangular and identity gauges: lists of three kinds, the second by tables
+])
+def test_pipelined_copies_of_both_kinds(lib, level, order):
+    """One scale per encoded tensor: copies whose kernels zero the next copy's maxima take turns with copies that need a memset."""
+    M, K, N = 1024, 1536, 1280
+    At, Wt = _ops(7, M, K, N)
+    G = len(order)
+    full = _gauges(G)
+    tri, one = np.array([[1.0, 0.0], [0.75, 1.5]]), np.eye(2)
+    P, Q, S = (np.stack([{"g": x[g], "t": tri, "i": one}[kind] for g, kind in enumerate(order)]) for x in full)
+    s1 = lib.scheme_builtin("strassen222")
+    s = lib.scheme_kron(s1, s1) if level == 1 else s1
+    mk = lambda fl: lib.GemmDesc.make(M, K, N, "bf16", "e4m3", "bf16", weight_layout=True, scale_mode=1, flags=fl)
+    ws = gu.workspace(lib.error_sweep_workspace(s, mk(0), G))
+    ws.fill_(0xFF)
+    serial, _ = lib.error_sweep(s, level, P, Q, S, mk(lib.FLAG_SWEEP_SERIAL), At, Wt, ws)
+    for _ in range(3):
+        ws.fill_(0xFF)
+        piped, _ = lib.error_sweep(s, level, P, Q, S, mk(0), At, Wt, ws)
+        assert np.array_equal(piped, serial)
+
+
 @pytest.mark.parametrize("M,K,N,G,O", [(2048, 2048, 2048, 27, "bf16"), (1024, 512, 1536, 16, "f32"), (1024, 256, 2048, 17, "bf16")])
 def test_fused_sweep_launches_against_the_serial_path(lib, M, K, N, G, O):
     """The fused launches (default where they apply): products of a batch, decode of the batch before and encode of the batch after in one launch.
