@@ -602,15 +602,16 @@ bool sweep_many_ok(const fmm_scheme* s, const fmm_gemm_desc* d, int G) {
 }
 
 // Sweeps on small blocks that one kernel takes from the operands to the errors, given diagonal gauges.  Its blocks' partial sums
-// use the place of the decode's.  Whole calls, this kernel against the passes of sweep_many.cu, both before statuses and sums came back in one
-// copy (30 us less), us: 512 copies at 64^3 279 / 410, 128^3 290 /
-// 539, 256^3 778 / 1254; 64 at 256^3 242 / 329, 512 x 64 x 512 317 / 462; one copy at 128^3 164 / 170.  Not where a tile is mostly
-// padding of one side (100 copies at 16 x 256 x 512 415 / 395), nor for a few copies of long rows, which it walks with one block of
-// threads a tile (2 at 256^3 190 / 176).
-bool sweep_variants_ok(const fmm_scheme* s, const fmm_gemm_desc* d, int G) {
+// use the place of the decode's.  Whole calls, the passes of sweep_many.cu / this kernel, us: 512 copies at 128^3 503 / 255, 100 at 64^3 189 / 140, 64 at
+// 512 x 64 x 512 433 / 296, 64 at 512 x 256 x 512 581 / 436.  A block of threads walks a tile, 32 x 32 of a copy, on its own for some 30 us, twice that
+// beyond 32 inner indices; so few tiles stay with the passes: 4 copies at 128 x 256 x 128 139 / 158, 8 at 16 x 256 x 32 136 / 149, with 32 tiles
+// 8 at 256^3 170 / 166 (bf16 161 / 164), 32 at 128 x 256 x 128 164 / 160; up to 32 inner indices one copy at 64^3 134 / 132, 8 at 128^3 138 / 135.  With
+// gauges of the outer factor the passes have less to read before their first block sum: 4 at 64 x 128 x 64 124 / 130, 64 at 40 x 64 x 64 146 / 131,
+// 8 at 256^3 155 / 164, 48 at 64 x 192 x 64 148 / 152, 4 at 512 x 256 x 512 171 / 174.  Nor where a tile is mostly padding of one side.
+bool sweep_variants_ok(const fmm_scheme* s, int level, const fmm_gemm_desc* d, int G) {
   const int64_t bm = d->M / s->m, bn = d->N / s->n, bk = d->K / s->k;
-  const int64_t tiles = sweep_variants_tiles(bm, bn);
-  if ((tiles > 1 && bm * bn < tiles * 256) || (bk > 32 && G < 8)) return false;
+  const int64_t tiles = sweep_variants_tiles(bm, bn), least = bk > 32 ? (level == 1 ? 96 : 32) : level == 1 ? 32 : 1;
+  if ((tiles > 1 && bm * bn < tiles * 256) || G * tiles < least) return false;
   return s->R == 49 && d->product == FMM_E4M3 && d->scale_mode == 2 && !(d->flags & FMM_FLAG_PRODUCTS_BF16) &&
          sweep_variants_sizes(bm, bn, bk) && tiles <= many_layout(s, d, G).blocks &&
          sweep_variants_scheme(*fmm_packed_table(*s, 0), *fmm_packed_table(*s, 1), *fmm_packed_table(*s, 2));
@@ -929,7 +930,7 @@ fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P
     if (in) for (const auto* v : {&in->U, &in->V, &in->W}) packed.insert(packed.end(), v->begin(), v->end());
     else packed.insert(packed.end(), 3, one);
     const size_t head = packed.size(), diagonals = 2 * (size_t)(gm + gk + gn);
-    if (sweep_variants_ok(base, d, G)) {
+    if (sweep_variants_ok(base, level, d, G)) {
       packed.resize(head + G * diagonals + kVariantIndexBytes / 8);
       double* x = packed.data() + head;
       variants = pack_diagonals(G, gm, P, x, diagonals) && pack_diagonals(G, gk, Q, x + gm, diagonals) &&

@@ -92,3 +92,37 @@ def test_other_gauges_keep_their_kernels():
     singular[1, 2, 2] = 0.0
     with pytest.raises(lib.FmmError):
         lib.error_sweep(s, 0, singular, P, P, d, A, B, ws)
+
+
+@pytest.mark.parametrize("M,K,N,G,storage,weight,output,change", [
+    (64, 64, 64, 33, "f32", False, "f32", _zeros),         # as few tiles as one kernel takes with gauges of the outer factor
+    (140, 192, 160, 24, "bf16", True, "bf16", None), (256, 256, 256, 24, "f32", False, "f32", None),      # and with long rows
+])
+def test_gauges_of_the_outer_factor(M, K, N, G, storage, weight, output, change):
+    test_diagonal_gauges(1, M, K, N, G, storage, weight, output, change)
+
+
+@pytest.mark.parametrize("level,M,K,N,most", [
+    (0, 128, 128, 128, 0), (0, 128, 256, 128, 31), (0, 256, 256, 256, 7),
+    (1, 128, 128, 128, 31), (1, 64, 256, 64, 95), (1, 256, 256, 256, 23),
+])
+def test_few_tiles_stay_with_the_passes(level, M, K, N, most):
+    """`most` copies run as before, one more in one kernel: three launches fewer (tables and a batch's three passes against one)."""
+    lib = gu.fmm()
+    s = lib.scheme_builtin("strassen444")
+    A, B = torch.randn(M, K, device="cuda"), torch.randn(K, N, device="cuda")
+    d = lib.GemmDesc.make(M, K, N, "f32", "e4m3", "f32", scale_mode=2)
+    n = 2 if level else 4
+
+    def launches(G, general):
+        P = np.stack([np.eye(n)] * G)
+        Q = P.copy()
+        if general:
+            Q[0, 0, 1] = 0.25
+        ws = gu.workspace(lib.error_sweep_workspace(s, d, G))
+        before = lib.launch_count()
+        lib.error_sweep(s, level, P, Q, P, d, A, B, ws)
+        return lib.launch_count() - before
+
+    assert most == 0 or launches(most, False) == launches(most, True)
+    assert launches(most + 1, False) + 3 == launches(most + 1, True)
