@@ -22,7 +22,8 @@
  *   - out-parameters are written only when FMM_OK is returned;
  *   - scheme handles are created by the library (host memory only, no GPU needed),
  *     are immutable, and are released with scheme_free; gauge/kron results are
- *     independent objects;
+ *     independent objects; a captured graph may copy a handle's tables at every replay, so the
+ *     handle outlives the graph;
  *   - operand, result and workspace buffers are caller-owned DEVICE memory, 256-byte
  *     aligned, row-major, leading dimensions in elements and a multiple of 16 bytes;
  *   - calls that take a stream only enqueue work on it (no synchronisation, no device
@@ -219,7 +220,8 @@ fmm_status scheme_gemm_workspace_layout(const fmm_scheme* s, const fmm_gemm_desc
 
 /* C = scheme(A, B) as defined at the top of this file (Eq. 1 with rounded block sums).
  * dA, dB, dC: DEVICE.  d_ws: DEVICE, >= scheme_gemm_workspace bytes, 256-byte aligned; its
- * contents are scratch except that Bhat persists for FMM_FLAG_REUSE_BHAT.  Asynchronous on
+ * contents are scratch except that Bhat persists for FMM_FLAG_REUSE_BHAT (a small product that is then formed of kept block sums may
+ * add its fp32 terms in another order than the call that left them).  Asynchronous on
  * `cuda_stream` (a cudaStream_t passed as void*; NULL = default stream).  Device-side waits
  * are bounded; a wait that expires is reported by fmm_device_status.                       */
 fmm_status scheme_gemm(const fmm_scheme* s, const fmm_gemm_desc* d, const void* dA, const void* dB,
@@ -321,9 +323,12 @@ size_t error_sweep_workspace(const fmm_scheme* base, const fmm_gemm_desc* d, int
  * Execution: equivalent algorithms share their operands, so up to eight of them (as many as fit the table limits:
  * products of the batch <= FMM_MAX_R) run as one encode, one product launch and one error-only decode.  On small
  * blocks (up to 128 x 64 x 128 or 8 x 1024 x 8 in any sweep, up to 128 x 1024 x 128 where copies are many; scale modes
- * 0 to 2) up to 512 copies run that way, and their coefficients are transformed on the device.  Every
- * algorithm's arithmetic and summation order are those of a scheme_gemm call on it, and the call is bit-reproducible
- * run to run.                                                                                              */
+ * 0 to 2) up to 512 copies run that way, and their coefficients are transformed on the device.  Block
+ * sums, scales and codes of every algorithm are those of a scheme_gemm call on it bit for bit, and its products and combination
+ * add the same terms; products of small blocks may come from another unit of the tensor cores than that call's, and
+ * how many copies a call has, and whether all their gauges are diagonal, decides which: fp32 sums in another order (ratios
+ * agree to a few 2^-24 ||C*||_F over the error).
+ * A call is bit-reproducible run to run.                                                                   */
 fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P, const double* Q,
                        const double* S, const fmm_gemm_desc* d, const void* dA, const void* dB,
                        const double* dCstar, double* h_ratios, fmm_sweep_summary* out, void* d_ws,

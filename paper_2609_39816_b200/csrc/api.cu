@@ -1207,8 +1207,8 @@ fmm_status error_sweep(const fmm_scheme* base, int level, int G, const double* P
       if (evG[b] && cudaStreamWaitEvent(sE, evG[b], 0) != cudaSuccess) return FMM_ERR_CUDA;
       if (d->scale_mode == 1 && evD[b] && cudaStreamWaitEvent(sE, evD[b], 0) != cudaSuccess) return FMM_ERR_CUDA;
       // Small operands are launch-bound: one paired launch.  With a scale per block sum it is the better one at any size: two launches
-      // where four would each start and drain, half a chip's work at a time (a copy, us, paired / apart: 2048 x 3456 x 1280 66 / 75,
-      // 4096^3 193 / 199).  Large bf16 operands: two launches, beside the products and decode of the neighbouring batches the two smaller
+      // where four would each start and drain, half a chip's work at a time (two levels, a copy, us, paired / apart: 2048 x 3456 x 1280 66 / 75,
+      // 4096^3 193 / 199; one level, 32 copies from bf16: 2048^3 1560 / 1661, 4096^3 8025 / 8207).  Large bf16 operands: two launches, beside the products and decode of the neighbouring batches the two smaller
       // kernels pack better (2048^3 53 to 56 / 51).
       const bool paired = d->scale_mode == 1 || (d->M + d->N) * d->K * (int64_t)esize(d->storage) < ((int64_t)16 << 20);
       if (paired) {

@@ -3,7 +3,7 @@
 // (mma.sync: a tile is an eighth of tcgen05's rows) and the four cells of C.  Block sums and products go to the workspace as
 // from the passes that this replaces; which block of threads writes a block sum that several hold goes round by product.  Sums, roundings and the order of
 // the decode's additions are those of encode_kernel and decode_kernel.
-// What bounds it: latency, the operands' loads (each row of A by every tile of its row of tiles) and three barriers.  256^3 from fp32,
+// What bounds it: latency, the operands' loads (each row of A by every tile of its row of tiles) and two barriers.  256^3 from fp32,
 // B row-major: 5.7 us in a graph where transpose, encode, products and decode take 9.5.
 #define FMM_LEVELS 1
 #include <cstring>

@@ -9,7 +9,7 @@
 // is wanted in registers, where the sums over the products are; 49 of them would leave three quarters of a 128-row tile empty.
 // What bounds it: sixteen warps an SM on phases of instruction issue (block sums twice, for the maxima 10 and for the codes 13 thousand
 // cycles of a block's 48) and of shared memory (products and sums over them 12).  512 sign variants at 128^3 from fp32: 100 us,
-// the call 255, where the passes took 310 (the call 539 before this kernel, 290 with it before the statuses came back with the sums).
+// the call 255, where the passes take 310 and the call 503.
 //
 // The lists of A and B are one code: the places of Strassen's V are those of U for products in another order (kPartner), so
 // cells are kept by place in the coefficient matrix and block sums in the order of U.
@@ -52,8 +52,8 @@ constexpr bool lists_agree() {
   return true;
 }
 static_assert(lists_agree(), "lists");
-__device__ const unsigned char kMaskU[7] = {0b1001, 0b1100, 0b0001, 0b1000, 0b0011, 0b0101, 0b1010};
-__device__ const unsigned char kMaskW[7] = {0b1001, 0b1100, 0b1010, 0b0101, 0b0011, 0b1000, 0b0001};
+__device__ const unsigned char kMaskU[7] = {kU[0], kU[1], kU[2], kU[3], kU[4], kU[5], kU[6]};      // for loops over products at run time
+__device__ const unsigned char kMaskW[7] = {kW[0], kW[1], kW[2], kW[3], kW[4], kW[5], kW[6]};
 constexpr unsigned nibbles(const int (&v)[7]) {
   unsigned x = 0;
   for (int i = 0; i < 7; ++i) x |= (unsigned)v[i] << (4 * i);
