@@ -993,14 +993,16 @@ fmm_status launch_pair(const BlockProductArgs& a, cudaStream_t st) {
   const int sms = sm_count();
   if (sms < 2) return FMM_ERR_CUDA;
   const long long pairs = std::min<long long>(total, sms / 2);
-  // Products by TMA stores where stores hold the kernel up: 8-bit products of short inner dimensions.  Whole calls, from registers / by TMA, us:
-  // two-level e4m3 at 2048 x 4096 x 12288 (1024 bytes of K a product) 244 / 233, 4096^3 160 / 149, 2048 x 5120 x 4096 (1280) 111 / 107; classical products of
-  // codes, 8192^2 with K 512 74.7 / 53.6, 1024 82 / 72; 6144 x K x 4608 with K 1024 37.7 / 36.5, 1280 39.9 / 39.5, 1536 43.4 / 44.1, 2048 62 / 66.  bf16 at
-  // 4096^3 (products alone) 82.4 / 82.1, 8192 x 13824 x 5120 450 / 467.  Not with row and column scales, which cost more here than the stores give:
-  // two-level 4096^3 from bf16 305 / 318, K 1024 193 / 207, one level 4096 x 512 x 4096 110 / 122.  Four rounds of tiles and more; fewer would gain
-  // as well (1024^3 27.1 / 25.8).
+  // Products by TMA stores where stores hold the kernel up: 8-bit products of short inner dimensions, longer ones where a row of the operands is not
+  // whole lines of 128 bytes and its copies take more of the L2.  Whole calls, from registers / by TMA, us: two-level e4m3, bytes of K a product, 4096 x
+  // 4096: 1024 160 / 149, 1536 158.2 / 158.3, 1616 210 / 186, 1792 211 / 211.5, 1872 228 / 202, 2000 236 / 209, 2304 196 / 198; 2048 x 12288: 1024 244 / 233, 1888
+  // 242 / 228, 2048 361 / 369; 7248 x 2784: 1296 276 / 230, 1856 280 / 250, 1920 255 / 249; classical products of codes, 8192^2: 512 74.7 / 53.6, 1024 82 / 72,
+  // 1536 98.9 / 94.3, 1792 107 / 110, 1680 145 / 129, 2000 177 / 159; 6144 x 4608: 1024 37.7 / 36.5, 1536 43.4 / 44.1, 2048 62 / 66.  bf16 at 4096^3 (products
+  // alone) 82.4 / 82.1, 8192 x 13824 x 5120 450 / 467.  Not with row and column scales, which cost more here than the stores give: two-level 4096^3 from
+  // bf16 305 / 318, K 1024 193 / 207, one level 4096 x 512 x 4096 110 / 122.  Four rounds of tiles and more, up to 2048 bytes; fewer rounds and longer
+  // rows of broken lines would gain as well (1024^3 27.1 / 25.8, 2608 bytes at 4096 x 4096 272 / 242).
   if constexpr (kFp8) {
-    if ((a.out_mode == 0 || a.output == FMM_F32) && a.row_scale == nullptr && tp.kbytes <= 1280 && total >= 4 * pairs && make_output_map(&mo, a, (int64_t)a.batches * groups)) {
+    if ((a.out_mode == 0 || a.output == FMM_F32) && a.row_scale == nullptr && tp.kbytes <= (tp.kbytes % BKB ? 2048 : 1536) && total >= 4 * pairs && make_output_map(&mo, a, (int64_t)a.batches * groups)) {
       using LT = PairLayoutT<true>;
       auto k = block_products_pair_tma_kernel<kFp8>;
       static unsigned long long smem_ok = 0;

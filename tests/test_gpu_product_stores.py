@@ -59,3 +59,8 @@ def test_one_matrix_with_scales():
     a, b = rounded(A), rounded(B)
     assert bool(((C[:, :N].double() - a @ b.T).abs() <= (K + 2) * 2.0 ** -23 * (a.abs() @ b.abs().T)).all())
     assert bool((C[:, N:] == -7.0).all())
+
+
+@pytest.mark.parametrize("K", [6208, 7552, 8064])      # rows of the operands that are not whole lines: 1552, 1888, 2016 bytes
+def test_rows_of_broken_lines(K):
+    test_block_products(1200, K, 3104, 1)
