@@ -531,7 +531,8 @@ bool run_types(const PatJob& a, const PatJob& b, bool have_a, bool have_b, const
 // a word as signed digits of base 256 (exact while a result's digits fit int8), and forms the products' sums one after the other: a
 // multiply-add of a list entry for four sums, no staging in shared memory, no table walk.
 // What bounds it: its writes.  Both operands at 2048 x 4096 x 11008, two-level: 43 us (218 MB, 5.1 TB/s), where the kernel that walks tables takes 62;
-// the whole call 337 -> 317, at 64 rows 186 -> 157, one level 253 -> 234.
+// the whole call 337 -> 317, at 64 rows 186 -> 157, one level 253 -> 234; few blocks, which that kernel's launch shares out by products:
+// 4 x 128 x 32 20.8 -> 14.7, 512^3 28.5 -> 22.9, 64 x 4096 x 64 68 -> 60, one level 15 -> 11.6, 18.8 -> 16.7, 43 -> 41.
 // ------------------------------------------------------------------------------------------
 struct CodeWeights { int a[kLevels == 2 ? 144 : 12], b[kLevels == 2 ? 144 : 12]; };
 
