@@ -93,7 +93,7 @@ cudaError_t launch_encode_pair(int storage, int product, const EncodeOperand& a,
                                int use_scale, cudaStream_t st);
 
 // The whole encode of one or both operands (a or b may be null; amax passes included) for tables of the pattern of Strassen's
-// algorithm, nested once or plain (encode_pattern.cu).  False, with nothing enqueued, where it has no kernel for the tables, types
+// algorithm, nested once or plain, on a square grid of blocks (encode_pattern.cu).  False, with nothing enqueued, where it has no kernel for the tables, types
 // or mode; else *err is the launches' result.  clear: the amax words of the operands (zeroed first where they are accumulated);
 // status: a DeviceStatus that the launches zero, or null.  With err null nothing is enqueued: the answer alone.
 bool fmm_encode_two_level(int storage, int product, const EncodeOperand* a, const EncodeOperand* b, int mode, void* clear,
@@ -106,7 +106,8 @@ inline bool fmm_encode_pattern(int storage, int product, const EncodeOperand* a,
 }
 
 // A whole scheme_gemm of one-level Strassen (and its diagonal gauges) on small blocks, bf16 products without scales, in one launch
-// (one_launch.cu).  False, with nothing enqueued, where it has no kernel for the tables or the sizes; else *err is the launch's result.
+// (one_launch.cu).  False, with nothing enqueued, where it does not take the tables, the sizes, B's address or a C over A or B; else *err
+// is the launch's result.
 struct OneLaunchArgs {
   int storage, output, weight_layout;
   const void* A; const void* B; void* C; int64_t lda, ldb, ldc;      // B as stored
@@ -129,7 +130,7 @@ __device__ __forceinline__ uint32_t digits_of(uint32_t bytes) { return (bytes ^ 
 __device__ __forceinline__ uint32_t bytes_of(uint32_t digits) { return (digits + 0x80808080u) ^ 0x80808080u; }
 #endif
 // The same for whole weights on the pattern of Strassen's algorithm, nested once or plain, in groups of 128 inner indices (encode_pattern.cu);
-// false, with nothing enqueued, where the tables are others
+// false, with nothing enqueued, where the tables or the grid are others
 bool fmm_encode_codes_two_level(CodesJob a, CodesJob b, const CoefTable& h_a, const CoefTable& h_b, int64_t K, int G, cudaStream_t st, cudaError_t* err);
 bool fmm_encode_codes_one_level(CodesJob a, CodesJob b, const CoefTable& h_a, const CoefTable& h_b, int64_t K, int G, cudaStream_t st, cudaError_t* err);
 
